@@ -37,7 +37,8 @@ __global__ void k_wait_selftest(int*);
 cudaError_t sweep_setup_attributes();
 int sweep_num_variants();
 int sweep_blocks_per_sm(int v);
-std::vector<int4> sweep_items(int64_t n, int v);
+SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk);
+std::vector<int4> sweep_items(int64_t n, const SweepPlan& pl, int v);
 cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row_end, bool bgt,
                          bool ll);
 cudaError_t launch_sweep_list(hawkes_ctx* c, const int4* items, int nitems, bool bgt, bool ll);
@@ -165,7 +166,8 @@ bool params_ok(const hawkes_params* p) {
 int ensure_items(hawkes_ctx* c) {
     if (c->items && c->items_variant == c->variant) return HAWKES_OK;
     dfree(c->items);
-    const std::vector<int4> items = sweep_items(c->n, c->variant);
+    c->plan = sweep_plan({c->n}, c->sms, c->variant, 0);
+    const std::vector<int4> items = sweep_items(c->n, c->plan, c->variant);
     HK_TRY(dalloc(&c->items, items.size()));
     HK_CUDA(cudaMemcpyAsync(c->items, items.data(), items.size() * sizeof(int4),
                             cudaMemcpyHostToDevice, c->stream));
@@ -615,7 +617,10 @@ int hawkes_shard_moments(hawkes_ctx* c, const hawkes_params* d_params, uint32_t 
         HK_TRY(hawkes_shard_bounds(c->n, tr, nshards, b.data()));
         const int64_t I0 = b[shard] / tr, I1 = (b[shard + 1] + tr - 1) / tr;
         std::vector<int4> mine;
-        for (const int4& it : sweep_items(c->n, c->variant))
+        // (row tiles in the whole sweep's item lengths, where it runs on row tiles:
+        // the same FP32 partial sums)
+        const SweepPlan pl{false, c->plan.split ? CHUNK : c->plan.chunk};
+        for (const int4& it : sweep_items(c->n, pl, c->variant))
             if (it.x >= I0 && it.x < I1) mine.push_back(it);
         HK_TRY(dalloc(&c->shard_items, mine.size()));
         HK_CUDA(cudaMemcpyAsync(c->shard_items, mine.data(), mine.size() * sizeof(int4),

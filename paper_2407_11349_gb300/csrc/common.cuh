@@ -104,6 +104,14 @@ struct ProbDesc {
     int64_t n, npad;
 };
 
+// How the symmetric sweep of a problem (or of a batch) is cut into work items
+// of `chunk` column tiles: by the row-tile kernel of the selected variant
+// (k_sweep), or by the column-split kernel (k_sweep_cs).
+struct SweepPlan {
+    bool split;
+    int chunk;
+};
+
 // A group of chains with identical event times, swept kc at a time by the
 // group kernel (sweep_group.cu): the group's tile records (TC / 2 + 3 kc TC
 // float4 per tile of TC events: the shared time plane, then three planes per
@@ -269,6 +277,7 @@ struct hawkes_ctx {
     int4* items = nullptr;     // symmetric-sweep work list
     int nitems = 0;
     int items_variant = -1;    // variant the work list was built for
+    hk::SweepPlan plan{false, 0};  // how the work list cuts the symmetric sweep
     int variant = 0;           // sweep kernel variant in use
     int variant_bpsm = 1;      // its resident CTAs per SM
     double* acc = nullptr;     // [6 * npad] per-row moment sums (natural units)

@@ -20,6 +20,7 @@
 // work overlaps on the GPU (other streams, other host threads) race on it.
 #include <cmath>
 #include <mutex>
+#include <vector>
 
 #include "common.cuh"
 
@@ -40,6 +41,8 @@ __global__ void k_reduce(const double*, int, const double*, double*, int64_t, do
 cudaError_t sweep_setup_attributes();
 int sweep_blocks_per_sm(int v);
 int sweep_variant_rows(int v);
+int split_rows();
+SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk);
 cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row_end, bool bgt,
                          bool ll);
 }  // namespace hk
@@ -52,7 +55,7 @@ namespace {
 constexpr int64_t kMaxN = HAWKES_NOALLOC_MAX_N;
 static_assert(kMaxN % NPAD_MULT == 0, "scratch holds whole row tiles");
 constexpr int kMaxFinalBlocks = 512;
-constexpr int kMaxItems = 4096;
+constexpr int kMaxItems = 16384;
 constexpr int kVariant = 0;  // sweep variant used by this entry point
 
 constexpr size_t align256(size_t b) { return (b + 255) / 256 * 256; }
@@ -133,16 +136,21 @@ __global__ void k_na_setup(const double* __restrict__ t_in, const double* __rest
     }
 }
 
-// Symmetric work list (row tile, column tiles [jb, je)), largest row tiles first.
-__global__ void k_na_items(int64_t n, int tr, int4* items) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    const int64_t nI = (n + tr - 1) / tr;
-    int k = 0;
-    for (int64_t I = nI - 1; I >= 0; --I) {
-        const int64_t last = (I + 1) * tr < n ? (I + 1) * tr : n;
-        const int nJ = static_cast<int>((last + TC - 1) / TC);
-        for (int jb = 0; jb < nJ && k < kMaxItems; jb += CHUNK)
-            items[k++] = make_int4(static_cast<int>(I), jb, jb + CHUNK < nJ ? jb + CHUNK : nJ, 0);
+// Symmetric work list (row tile, column tiles [jb, je)), largest row tiles
+// first: one thread per row tile counts the items of the later tiles and
+// writes its own.
+__global__ void k_na_items(int64_t n, int tr, int chunk, int4* items) {
+    const int nI = static_cast<int>((n + tr - 1) / tr);
+    auto tiles_of = [&](int I) {
+        const int64_t last = (I + 1) * static_cast<int64_t>(tr) < n ? (I + 1) * static_cast<int64_t>(tr) : n;
+        return static_cast<int>((last + TC - 1) / TC);
+    };
+    for (int I = blockIdx.x * blockDim.x + threadIdx.x; I < nI; I += gridDim.x * blockDim.x) {
+        int k = 0;
+        for (int L = nI - 1; L > I; --L) k += (tiles_of(L) + chunk - 1) / chunk;
+        const int nJ = tiles_of(I);
+        for (int jb = 0; jb < nJ && k < kMaxItems; jb += chunk)
+            items[k++] = make_int4(I, jb, jb + chunk < nJ ? jb + chunk : nJ, 0);
     }
 }
 
@@ -151,13 +159,13 @@ __global__ void k_na_nan_on_error(const int* ctr, double* out) {
         for (int q = 0; q < 7; ++q) out[q] = nan("");
 }
 
-int items_for(int64_t n, int tr) {
+int items_for(int64_t n, int tr, int chunk) {
     const int64_t nI = (n + tr - 1) / tr;
     int64_t k = 0;
     for (int64_t I = 0; I < nI; ++I) {
         const int64_t last = (I + 1) * tr < n ? (I + 1) * tr : n;
         const int64_t nJ = (last + TC - 1) / TC;
-        k += (nJ + CHUNK - 1) / CHUNK;
+        k += (nJ + chunk - 1) / chunk;
     }
     return static_cast<int>(k);
 }
@@ -213,7 +221,9 @@ extern "C" int hawkes_loglik_grad_noalloc(const double* d_t, const double* d_x, 
 
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     unsigned char* base = d->scratch;
-    const int tr = sweep_variant_rows(kVariant);
+    SweepPlan plan = sweep_plan({n}, d->sms, kVariant, 0);
+    const int tr = plan.split ? split_rows() : sweep_variant_rows(kVariant);
+    while (items_for(n, tr, plan.chunk) > kMaxItems) plan.chunk *= 2;
     const int64_t npad = (n + NPAD_MULT - 1) / NPAD_MULT * NPAD_MULT;
 
     // A context on the stack that points into the scratch array; only the
@@ -240,11 +250,11 @@ extern "C" int hawkes_loglik_grad_noalloc(const double* d_t, const double* d_x, 
     c.ctr = reinterpret_cast<int*>(base + OFF_CTR);
     c.cc = reinterpret_cast<double*>(base + OFF_CC);
     c.items = reinterpret_cast<int4*>(base + OFF_ITEMS);
-    c.nitems = items_for(n, tr);
+    c.plan = plan;
+    c.nitems = items_for(n, tr, plan.chunk);
     c.variant = kVariant;
     c.variant_bpsm = d->bpsm;
     c.final_blocks = 2 * d->sms < kMaxFinalBlocks ? 2 * d->sms : kMaxFinalBlocks;
-    if (c.nitems > kMaxItems) return HAWKES_ERR_TOO_LARGE;
     const int model = static_cast<int>(flags & (HAWKES_MODEL1 | HAWKES_BG_TIME));
     int grid = static_cast<int>((npad + 255) / 256);
     if (grid > 8 * c.sms) grid = 8 * c.sms;
@@ -253,7 +263,7 @@ extern "C" int hawkes_loglik_grad_noalloc(const double* d_t, const double* d_x, 
     if (cudaMemsetAsync(c.ctr, 0, CT_COUNT * sizeof(int), st) != cudaSuccess) return HAWKES_ERR_CUDA;
     k_na_setup<<<grid, 256, 0, st>>>(d_t, d_x, d_y, d_s, n, npad, c.t, c.x, c.y, c.s, c.lo, c.hi,
                                      c.tb, c.ctr);
-    k_na_items<<<1, 32, 0, st>>>(n, tr, c.items);
+    k_na_items<<<8, 64, 0, st>>>(n, tr, plan.chunk, c.items);
     k_prep<<<grid, 256, 0, st>>>(c.t, c.x, c.y, c.s, c.tb, d_params, model, 1, 0, n, npad, c.rec,
                                  c.acc, c.cc, c.ctr, c.fix7);
     if (launch_sweep(&c, true, 0, n, (flags & HAWKES_BG_TIME) != 0, false) != cudaSuccess) return HAWKES_ERR_CUDA;

@@ -9,6 +9,12 @@
 
 namespace hk {
 
+// The column-split kernels (sweep_split.cu).
+cudaError_t split_setup_attributes();
+int split_rows();
+cudaError_t launch_sweep_split(cudaStream_t st, int sms, const ProbDesc& one, const ProbDesc* probs,
+                               int nprobs, const int4* items, int nitems, int* ctr, bool bgt, bool ll);
+
 static const Variant kVariants[] = HK_SWEEP_VARIANTS(false, false);
 static_assert(sizeof(kVariants) / sizeof(kVariants[0]) == kNumVariants, "variant count");
 
@@ -32,7 +38,7 @@ cudaError_t sweep_setup_attributes() {
             if (e != cudaSuccess) return e;
         }
     }
-    return cudaSuccess;
+    return split_setup_attributes();
 }
 
 int sweep_blocks_per_sm(int v) {
@@ -43,14 +49,57 @@ int sweep_blocks_per_sm(int v) {
     return nb > 0 ? nb : 1;
 }
 
-// Symmetric work list over problems of sizes ns[] for variant v: items
-// (row tile, column tiles [jb, je), problem) in chunks of `chunk` column
-// tiles.  order 0: all items longest first (ties: later row tiles first);
+// Column tiles of all row tiles of `tr` rows in the causal triangle of n events.
+static int64_t plan_units(int64_t n, int tr) {
+    int64_t u = 0;
+    for (int64_t r = 0; r < n; r += tr) u += (std::min<int64_t>(r + tr, n) + TC - 1) / TC;
+    return u;
+}
+
+static int pow2_floor(double v, int cap) {
+    int p = 1;
+    while (2 * p <= cap && 2 * p <= v) p *= 2;
+    return p;
+}
+
+// The plan for problems of sizes ns[] swept in one launch on variant v.
+//   chunk > 0: that many column tiles per item; 0: chosen here.
+// Kernel: a row tile's units that lie partly above the diagonal leave warps
+// idle.  Where the row tiles cover more than 1.1 times the pairs that the
+// column-split kernel's 128-row items cover (N below about 36,000), the
+// latter runs: 0.402 against 0.434 ms at N = 30,000; at N = 50,000 (1.08
+// times) it would be 1.056 against 1.042.  30 chains of 20,000 events (1.14
+// times): 4.29 against 4.52 ms per step.
+// Chunk: small enough for 16 items per SM (the tail), large enough to
+// amortise an item's row flush.  Row tiles: N = 100,000 3.95 ms with 4 against
+// 4.07 with 16; 250,000 23.2 with 16 against 23.5 with 4.  Column split: from
+// three items per SM up to 4 tiles (N = 17,103: 0.144 ms with 4, 0.163 with
+// 1; N = 5,000: 0.023 with 1, 0.028 with 2), and 8 where 64 items per SM are
+// left (30 x 20,000: 4.29 with 8, 4.44 with 4).
+SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk) {
+    double rows = 0.0, split = 0.0;
+    for (int64_t n : ns) {
+        rows += static_cast<double>(plan_units(n, kVariants[v].tr)) * kVariants[v].tr;
+        split += static_cast<double>(plan_units(n, split_rows())) * split_rows();
+    }
+    SweepPlan pl{rows > 1.1 * split, chunk};
+    if (chunk <= 0) {
+        const double u = pl.split ? split / split_rows() : rows / kVariants[v].tr;  // items of one tile
+        pl.chunk = pl.split ? std::max(pow2_floor(u / (3.0 * sms), 4), pow2_floor(u / (64.0 * sms), 8))
+                            : pow2_floor(u / (16.0 * sms), CHUNK);
+    }
+    return pl;
+}
+
+// Symmetric work list over problems of sizes ns[] for plan pl (variant v on
+// the row-tile kernel): items (row tile, column tiles [jb, je), problem) in
+// chunks of pl.chunk column tiles.  order 0: all items longest first (ties: later row tiles first);
 // order 1: problem by problem, largest problem first, each problem's items
 // longest first, so that the source tiles and accumulators of the problems
 // in flight stay in L2 while the tail still ends on the smallest items.
-std::vector<int4> sweep_items_batch(const std::vector<int64_t>& ns, int v, int chunk, int order) {
-    const int tr = kVariants[v].tr;
+std::vector<int4> sweep_items_batch(const std::vector<int64_t>& ns, const SweepPlan& pl, int v,
+                                    int order) {
+    const int tr = pl.split ? split_rows() : kVariants[v].tr, chunk = pl.chunk;
     auto longest_first = [](const int4& a, const int4& b) {
         return (a.z - a.y) > (b.z - b.y) || ((a.z - a.y) == (b.z - b.y) && a.x > b.x);
     };
@@ -75,14 +124,16 @@ std::vector<int4> sweep_items_batch(const std::vector<int64_t>& ns, int v, int c
     return items;
 }
 
-std::vector<int4> sweep_items(int64_t n, int v) { return sweep_items_batch({n}, v, CHUNK, 0); }
+std::vector<int4> sweep_items(int64_t n, const SweepPlan& pl, int v) {
+    return sweep_items_batch({n}, pl, v, 0);
+}
 
 static ProbDesc desc_of(const hawkes_ctx* c) {
     return ProbDesc{c->t, c->rec, c->lo, c->hi, c->tb, c->cc, c->acc, c->n, c->npad};
 }
 
-// Symmetric sweep of one problem over the work list items[0, nitems) (the
-// whole list, or one shard's part of it).
+// Row-tile sweep of one problem over the work list items[0, nitems) (the whole
+// list, or one shard's part of it).
 cudaError_t launch_sweep_list(hawkes_ctx* c, const int4* items, int nitems, bool bgt, bool ll) {
     const Variant& v = variant_of(c->variant, bgt, ll);
     const int grid_cap = c->sms * c->variant_bpsm;
@@ -98,7 +149,10 @@ cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row
     const Variant& v = variant_of(c->variant, bgt, ll);
     const int grid_cap = c->sms * c->variant_bpsm;
     const ProbDesc one = desc_of(c);
-    if (sym) {
+    if (sym && c->plan.split) {
+        return launch_sweep_split(c->stream, c->sms, one, nullptr, 0, c->items, c->nitems, c->ctr, bgt,
+                                  ll);
+    } else if (sym) {
         return launch_sweep_list(c, c->items, c->nitems, bgt, ll);
     } else {
         const int item0 = static_cast<int>(row_begin / v.tr);
@@ -116,9 +170,11 @@ cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row
 
 // One persistent launch over the items of many problems; ctr[CT_WORK] must be
 // zero when it starts.
-cudaError_t launch_sweep_batch(cudaStream_t st, int variant, int grid, const ProbDesc* probs,
-                               int nprobs, const int4* items, int nitems, int* ctr, bool bgt,
-                               bool ll) {
+cudaError_t launch_sweep_batch(cudaStream_t st, const SweepPlan& pl, int sms, int variant, int grid,
+                               const ProbDesc* probs, int nprobs, const int4* items, int nitems,
+                               int* ctr, bool bgt, bool ll) {
+    if (pl.split)
+        return launch_sweep_split(st, sms, ProbDesc{}, probs, nprobs, items, nitems, ctr, bgt, ll);
     const Variant& v = variant_of(variant, bgt, ll);
     if (grid > nitems) grid = nitems;
     if (grid <= 0) return cudaSuccess;

@@ -99,6 +99,96 @@ __device__ __forceinline__ void fold_rows(Rows<RP>& rr, float4* __restrict__ rac
     }
 }
 
+// One 32-column chunk `ch` of a tile; on return (COL) lane k holds the column
+// sums (B, B r~^2, B dt~^2) of column ch * 32 + k over the warp's rows.
+template <int RP, int UNROLL, int MASK, bool EXC, bool COL, bool BGT, bool LL>
+__device__ __forceinline__ void chunk_pass(const float4* __restrict__ tile, int ch, int j0, int lane,
+                                           Rows<RP>& rr, float2 nomt,
+                                           const int* __restrict__ rlo,
+                                           const int* __restrict__ rhi, float2& cB, float2& cBr,
+                                           float2& cBt) {
+    cB = cBr = cBt = f2(0.f, 0.f);
+#pragma unroll UNROLL
+    for (int s = 0; s < 32; ++s) {
+        const int c = ch * 32 + ((lane + s) & 31);
+        const float4 q0 = tile[0 * TC + c];  // -t, -t, -xh, -xh
+        const float4 q1 = tile[1 * TC + c];  // -xl, -xl, -yh, -yh
+        const float4 q2 = tile[2 * TC + c];  // -yl, -yl, -beta, -beta
+        const float4 q3 = tile[3 * TC + c];  // ce, ce, -, -
+        const float2 nT = f2(q0.x, q0.y), nXH = f2(q0.z, q0.w);
+        const float2 nXL = f2(q1.x, q1.y), nYH = f2(q1.z, q1.w);
+        const float2 nYL = f2(q2.x, q2.y), NB = f2(q2.z, q2.w);
+        const float2 CE = f2(q3.x, q3.y);
+        const int j = j0 + c;
+        float2 pB, pBt;  // BGT: this step's column partial over the lane's rows
+#pragma unroll
+        for (int p = 0; p < RP; ++p) {
+            const float2 dt = add2(rr.tp[p], nT);
+            const float2 dx = add2(add2(rr.xh[p], nXH), add2(rr.xl[p], nXL));
+            const float2 dy = add2(add2(rr.yh[p], nYH), add2(rr.yl[p], nYL));
+            const float2 r2 = fma2(dy, dy, mul2(dx, dx));
+            const float2 dt2 = mul2(dt, dt);
+            const float2 aB = BGT ? dt2 : add2(dt2, r2);
+            float2 B = f2(ex2(-aB.x), ex2(-aB.y));
+            if (MASK != M_NONE) {
+                const int l0 = rlo[2 * p], l1 = rlo[2 * p + 1];
+                if (MASK == M_LOWER) {
+                    B.x = (j < l0) ? B.x : 0.f;
+                    B.y = (j < l1) ? B.y : 0.f;
+                } else {
+                    B.x = (j < l0 || j >= rhi[2 * p]) ? B.x : 0.f;
+                    B.y = (j < l1 || j >= rhi[2 * p + 1]) ? B.y : 0.f;
+                }
+            }
+            rr.sB[p] = add2(rr.sB[p], B);
+            if (!BGT && !LL) rr.sBr[p] = fma2(B, r2, rr.sBr[p]);
+            if (!LL) rr.sBt[p] = fma2(B, dt2, rr.sBt[p]);
+            if (COL && !BGT) {
+                cB = add2(cB, B);
+                if (!LL) {
+                    cBr = fma2(B, r2, cBr);
+                    cBt = fma2(B, dt2, cBt);
+                }
+            }
+            if (COL && BGT) {  // per-step partial (no SBr moment here)
+                pB = (p == 0) ? B : add2(pB, B);
+                if (!LL) pBt = (p == 0) ? mul2(B, dt2) : fma2(B, dt2, pBt);
+            }
+            if (EXC) {
+                const float2 nv = mul2(NB, r2);                  // -beta r~^2
+                const float2 arg = add2(fma2(nomt, dt, nv), CE); // ce - omega~ dt - beta r~^2
+                float2 E = f2(ex2(arg.x), ex2(arg.y));
+                if (MASK != M_NONE) {
+                    E.x = (j < rlo[2 * p]) ? E.x : 0.f;
+                    E.y = (j < rlo[2 * p + 1]) ? E.y : 0.f;
+                }
+                rr.sE[p] = add2(rr.sE[p], E);
+                if (!LL) {
+                    rr.sEt[p] = fma2(E, dt, rr.sEt[p]);
+                    rr.sEq[p] = fma2(E, nv, rr.sEq[p]);  // accumulates -sum E beta r~^2
+                }
+            }
+        }
+        if (COL) {
+            if (BGT) {
+                cB = add2(cB, pB);
+                if (!LL) cBt = add2(cBt, pBt);
+            }
+            const int src = (lane + 1) & 31;
+            cB.x = __shfl_sync(0xffffffffu, cB.x, src);
+            cB.y = __shfl_sync(0xffffffffu, cB.y, src);
+            if (!BGT && !LL) {
+                cBr.x = __shfl_sync(0xffffffffu, cBr.x, src);
+                cBr.y = __shfl_sync(0xffffffffu, cBr.y, src);
+            }
+            if (!LL) {
+                cBt.x = __shfl_sync(0xffffffffu, cBt.x, src);
+                cBt.y = __shfl_sync(0xffffffffu, cBt.y, src);
+            }
+        }
+    }
+}
+
 template <int RP, int UNROLL, int MASK, bool EXC, bool COL, bool BGT, bool LL>
 __device__ __forceinline__ void tile_pass(const float4* __restrict__ tile, int j0, int lane,
                                           Rows<RP>& rr, float2 nomt,
@@ -107,86 +197,8 @@ __device__ __forceinline__ void tile_pass(const float4* __restrict__ tile, int j
                                           float4* __restrict__ racc) {
 #pragma unroll 1
     for (int ch = 0; ch < TC / 32; ++ch) {
-        float2 cB = f2(0.f, 0.f), cBr = f2(0.f, 0.f), cBt = f2(0.f, 0.f);
-#pragma unroll UNROLL
-        for (int s = 0; s < 32; ++s) {
-            const int c = ch * 32 + ((lane + s) & 31);
-            const float4 q0 = tile[0 * TC + c];  // -t, -t, -xh, -xh
-            const float4 q1 = tile[1 * TC + c];  // -xl, -xl, -yh, -yh
-            const float4 q2 = tile[2 * TC + c];  // -yl, -yl, -beta, -beta
-            const float4 q3 = tile[3 * TC + c];  // ce, ce, -, -
-            const float2 nT = f2(q0.x, q0.y), nXH = f2(q0.z, q0.w);
-            const float2 nXL = f2(q1.x, q1.y), nYH = f2(q1.z, q1.w);
-            const float2 nYL = f2(q2.x, q2.y), NB = f2(q2.z, q2.w);
-            const float2 CE = f2(q3.x, q3.y);
-            const int j = j0 + c;
-            float2 pB, pBt;  // BGT: this step's column partial over the lane's rows
-#pragma unroll
-            for (int p = 0; p < RP; ++p) {
-                const float2 dt = add2(rr.tp[p], nT);
-                const float2 dx = add2(add2(rr.xh[p], nXH), add2(rr.xl[p], nXL));
-                const float2 dy = add2(add2(rr.yh[p], nYH), add2(rr.yl[p], nYL));
-                const float2 r2 = fma2(dy, dy, mul2(dx, dx));
-                const float2 dt2 = mul2(dt, dt);
-                const float2 aB = BGT ? dt2 : add2(dt2, r2);
-                float2 B = f2(ex2(-aB.x), ex2(-aB.y));
-                if (MASK != M_NONE) {
-                    const int l0 = rlo[2 * p], l1 = rlo[2 * p + 1];
-                    if (MASK == M_LOWER) {
-                        B.x = (j < l0) ? B.x : 0.f;
-                        B.y = (j < l1) ? B.y : 0.f;
-                    } else {
-                        B.x = (j < l0 || j >= rhi[2 * p]) ? B.x : 0.f;
-                        B.y = (j < l1 || j >= rhi[2 * p + 1]) ? B.y : 0.f;
-                    }
-                }
-                rr.sB[p] = add2(rr.sB[p], B);
-                if (!BGT && !LL) rr.sBr[p] = fma2(B, r2, rr.sBr[p]);
-                if (!LL) rr.sBt[p] = fma2(B, dt2, rr.sBt[p]);
-                if (COL && !BGT) {
-                    cB = add2(cB, B);
-                    if (!LL) {
-                        cBr = fma2(B, r2, cBr);
-                        cBt = fma2(B, dt2, cBt);
-                    }
-                }
-                if (COL && BGT) {  // per-step partial (no SBr moment here)
-                    pB = (p == 0) ? B : add2(pB, B);
-                    if (!LL) pBt = (p == 0) ? mul2(B, dt2) : fma2(B, dt2, pBt);
-                }
-                if (EXC) {
-                    const float2 nv = mul2(NB, r2);                  // -beta r~^2
-                    const float2 arg = add2(fma2(nomt, dt, nv), CE); // ce - omega~ dt - beta r~^2
-                    float2 E = f2(ex2(arg.x), ex2(arg.y));
-                    if (MASK != M_NONE) {
-                        E.x = (j < rlo[2 * p]) ? E.x : 0.f;
-                        E.y = (j < rlo[2 * p + 1]) ? E.y : 0.f;
-                    }
-                    rr.sE[p] = add2(rr.sE[p], E);
-                    if (!LL) {
-                        rr.sEt[p] = fma2(E, dt, rr.sEt[p]);
-                        rr.sEq[p] = fma2(E, nv, rr.sEq[p]);  // accumulates -sum E beta r~^2
-                    }
-                }
-            }
-            if (COL) {
-                if (BGT) {
-                    cB = add2(cB, pB);
-                    if (!LL) cBt = add2(cBt, pBt);
-                }
-                const int src = (lane + 1) & 31;
-                cB.x = __shfl_sync(0xffffffffu, cB.x, src);
-                cB.y = __shfl_sync(0xffffffffu, cB.y, src);
-                if (!BGT && !LL) {
-                    cBr.x = __shfl_sync(0xffffffffu, cBr.x, src);
-                    cBr.y = __shfl_sync(0xffffffffu, cBr.y, src);
-                }
-                if (!LL) {
-                    cBt.x = __shfl_sync(0xffffffffu, cBt.x, src);
-                    cBt.y = __shfl_sync(0xffffffffu, cBt.y, src);
-                }
-            }
-        }
+        float2 cB, cBr, cBt;
+        chunk_pass<RP, UNROLL, MASK, EXC, COL, BGT, LL>(tile, ch, j0, lane, rr, nomt, rlo, rhi, cB, cBr, cBt);
         if (COL) {  // lane k now holds column ch*32 + k, summed over the warp's rows
             atomicAdd(colacc + 0 * TC + ch * 32 + lane, cB.x + cB.y);
             if (!BGT && !LL) atomicAdd(colacc + 1 * TC + ch * 32 + lane, cBr.x + cBr.y);
