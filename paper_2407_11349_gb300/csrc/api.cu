@@ -12,26 +12,20 @@
 namespace hk {
 // kernels.cu
 __global__ void k_setup(double*, double*, double*, const int32_t*, int32_t, const double*, int64_t,
-                        int64_t, int, double*, int32_t*, int32_t*, double*, int*);
-__global__ void k_prep(const double*, const double*, const double*, const double*, const double*,
-                       const hawkes_params*, int, int, int, int64_t, int64_t, Rec*, double*, double*,
-                       int*, double*);
-__global__ void k_finalize(const double*, const double*, const int32_t*, const int32_t*,
-                           const double*, int64_t, int64_t, int64_t, int64_t, int, int*, int*,
-                           double*, double*);
-__global__ void k_flushfix(const double*, const double*, const double*, const double*,
-                           const double*, const int32_t*, const int32_t*, const double*, int,
-                           int64_t, int64_t, int64_t, int64_t, int*, double*, double*, double*);
-__global__ void k_rows64(const double*, const double*, const double*, const double*,
-                         const int32_t*, const int32_t*, const double*, int, int64_t, int64_t,
-                         int64_t, int64_t, int, const int*, int*, double*, double*, double*);
-__global__ void k_reduce(const double*, int, const double*, double*, int64_t, double*, int*);
+                        int64_t, int, double*, float*, int32_t*, int32_t*, double*, int*);
+__global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const hawkes_params*,
+                       const __grid_constant__ hawkes_params,
+                       int, int, int, int, const uint64_t*, int*);
+void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
+                     double*, double*, double*);
+__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, int, double*,
+                         double*);
+__global__ void k_flushfix(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, double*, double*,
+                           double*);
 __global__ void k_tri_area(const double*, int32_t, double*, int*);
 __global__ void k_tri_county(const int32_t*, int32_t, int32_t, double*, int32_t*, int32_t*, int*);
 __global__ void k_tri_check(const int32_t*, int32_t, int32_t, int*);
-__global__ void k_resample(const int32_t*, int64_t, const double*, const double*, const int32_t*,
-                           const int32_t*, uint64_t, uint64_t, uint64_t, const uint64_t*, double*,
-                           double*);
+__global__ void k_resample(const __grid_constant__ EvalDesc, uint64_t);
 __global__ void k_wait_selftest(int*);
 // sweep.cu
 cudaError_t sweep_setup_attributes();
@@ -128,7 +122,7 @@ void drop_shard_items(hawkes_ctx* c) {
 }
 
 void free_events(hawkes_ctx* c) {
-    dfree(c->t); dfree(c->x); dfree(c->y); dfree(c->s); dfree(c->scale_c); dfree(c->county);
+    dfree(c->t); dfree(c->x); dfree(c->y); dfree(c->is2); dfree(c->ce); dfree(c->scale_c); dfree(c->county);
     dfree(c->lo); dfree(c->hi); dfree(c->tb); dfree(c->rec); dfree(c->acc); dfree(c->fixlist);
     dfree(c->items);
     drop_shard_items(c);
@@ -184,37 +178,52 @@ int select_variant(hawkes_ctx* c, int v) {
     return c->n ? ensure_items(c) : HAWKES_OK;
 }
 
-// Queue the FP32 path's finalisation of rows [rb, re) from the moment sums in
-// c->acc: per-row terms (rows near the FP32 floor recomputed in FP64), the
-// global reduction, and the FP64 recomputation of the rows whose flushed FP32
-// terms could matter to an output.
-int enqueue_finalize32(hawkes_ctx* c, int model, int64_t rb, int64_t re, double* d_out,
-                       double* d_rows9) {
-    HK_TRY(timed(c, HAWKES_K_FINAL, [&] {
-        k_finalize<<<c->final_blocks, 256, 0, c->stream>>>(c->acc, c->t, c->lo, c->hi, c->cc, c->n,
-                                                           c->npad, rb, re, 1, c->fixlist, c->ctr,
-                                                           c->partials, d_rows9);
-    }));
-    HK_TRY(timed(c, HAWKES_K_ROWS64, [&] {
-        k_rows64<<<c->sms, 256, 0, c->stream>>>(c->t, c->x, c->y, c->s, c->lo, c->hi, c->cc, model,
-                                                c->n, c->npad, 0, 0, 1, c->fixlist, c->ctr, c->acc,
-                                                c->fix7, d_rows9);
-    }));
-    HK_TRY(timed(c, HAWKES_K_REDUCE, [&] {
-        k_reduce<<<1, 256, 0, c->stream>>>(c->partials, c->final_blocks, c->fix7, c->cc, re - rb,
-                                           d_out, c->ctr);
-    }));
-    return timed(c, HAWKES_K_ROWS64, [&] {
-        k_flushfix<<<grid_for(c, re - rb, 2), 256, 0, c->stream>>>(
-            c->acc, c->t, c->x, c->y, c->s, c->lo, c->hi, c->cc, model, c->n, c->npad, rb, re,
-            c->ctr, c->fix7, d_out, d_rows9);
+// The parameters of a call: on the device, or (synchronous calls) by value.
+struct CallParams {
+    const hawkes_params* dev;
+    hawkes_params val;
+};
+
+// Queue the per-call constants, cleared accumulators and (stage) FP32 records.
+int enqueue_prep(hawkes_ctx* c, const CallParams& cp, int model, int stage, int skip) {
+    const EventGrid g = event_grid(c->npad, c->sms);
+    return timed(c, HAWKES_K_PREP, [&] {
+        k_prep<<<g.blocks, g.threads, 0, c->stream>>>(eval_desc(c), nullptr, cp.dev, cp.val, model, stage,
+                                                      skip, 0, nullptr, nullptr);
     });
 }
 
-// Queue one log-likelihood evaluation over rows [rb, re).  d_params: device
-// parameters; d_out: 7 doubles; d_rows9: optional per-row output [9 n].
-int enqueue_loglik(hawkes_ctx* c, const hawkes_params* d_params, uint32_t flags, int64_t rb,
-                   int64_t re, double* d_out, double* d_rows9) {
+int enqueue_rows(hawkes_ctx* c, int64_t rb, int64_t re, int check, double* d_out, double* d_rows9,
+                 double* d_err) {
+    return timed(c, HAWKES_K_FINAL, [&] {
+        launch_finalize(c->stream, final_grid(re - rb, c->sms), eval_desc(c), nullptr, rb, re, check, d_out,
+                        d_rows9, d_err);
+    });
+}
+
+// Queue the FP32 path's finalisation of rows [rb, re) from the moment sums in
+// c->acc: per-row terms and the global reduction (k_finalize), the rows near
+// the FP32 floor recomputed in FP64 (k_rows64), and the FP64 recomputation of
+// the rows whose flushed FP32 terms could matter to an output (k_flushfix);
+// the last two return at once when there are none.  d_err (optional): receives
+// the latched error status as a double.
+int enqueue_finalize32(hawkes_ctx* c, int model, int64_t rb, int64_t re, double* d_out,
+                       double* d_rows9, double* d_err) {
+    const EvalDesc d = eval_desc(c);
+    HK_TRY(enqueue_rows(c, rb, re, 1, d_out, d_rows9, nullptr));
+    HK_TRY(timed(c, HAWKES_K_ROWS64, [&] {
+        k_rows64<<<c->sms, 256, 0, c->stream>>>(d, nullptr, model, 0, re - rb, 1, d_out, d_rows9);
+    }));
+    return timed(c, HAWKES_K_ROWS64, [&] {
+        k_flushfix<<<grid_for(c, re - rb, 2), 256, 0, c->stream>>>(d, nullptr, model, rb, re, d_out,
+                                                                   d_rows9, d_err);
+    });
+}
+
+// Queue one log-likelihood evaluation over rows [rb, re).  d_out: 7 doubles;
+// d_rows9: optional per-row output [9 n]; d_err as above.
+int enqueue_loglik(hawkes_ctx* c, const CallParams& cp, uint32_t flags, int64_t rb, int64_t re,
+                   double* d_out, double* d_rows9, double* d_err) {
     const bool f64 = (flags & HAWKES_F64) != 0;
     const int model = static_cast<int>(flags & kModelBits);
     const bool bgt = (flags & HAWKES_BG_TIME) != 0;
@@ -222,12 +231,7 @@ int enqueue_loglik(hawkes_ctx* c, const hawkes_params* d_params, uint32_t flags,
     if (spatial && (f64 || bgt || rb != 0 || re != c->n)) return HAWKES_ERR_ARG;
     if (spatial) HK_TRY(spatial_build(c));  // synchronous on first use after set_events
     const int skip = (!f64 && !spatial && (flags & HAWKES_SKIP_UNDERFLOW)) ? 1 : 0;
-    const int prep_grid = grid_for(c, c->npad);
-    HK_TRY(timed(c, HAWKES_K_PREP, [&] {
-        k_prep<<<prep_grid, 256, 0, c->stream>>>(c->t, c->x, c->y, c->s, c->tb, d_params, model,
-                                                  (f64 || spatial) ? 0 : 1, skip, c->n, c->npad, c->rec,
-                                                  c->acc, c->cc, c->ctr, c->fix7);
-    }));
+    HK_TRY(enqueue_prep(c, cp, model, (f64 || spatial) ? 0 : 1, skip));
     if (!f64) {
         const bool sym = (rb == 0 && re == c->n);
         cudaError_t se = cudaSuccess;
@@ -238,35 +242,22 @@ int enqueue_loglik(hawkes_ctx* c, const hawkes_params* d_params, uint32_t flags,
                 launch_sweep(c, sym, rb, re, bgt, (flags & HAWKES_LOGLIK_ONLY) != 0);
         }));
         HK_CUDA(se);
-        return enqueue_finalize32(c, model, rb, re, d_out, d_rows9);
-    } else {
-        const int64_t count = re - rb;
-        int g = static_cast<int>(count < static_cast<int64_t>(c->sms) * 16 ? count : c->sms * 16);
-        if (g < 1) g = 1;
-        HK_TRY(timed(c, HAWKES_K_ROWS64, [&] {
-            k_rows64<<<g, 256, 0, c->stream>>>(c->t, c->x, c->y, c->s, c->lo, c->hi, c->cc, model,
-                                               c->n, c->npad, rb, count, 0, c->fixlist, c->ctr,
-                                               c->acc, c->fix7, d_rows9);
-        }));
-        HK_TRY(timed(c, HAWKES_K_FINAL, [&] {
-            k_finalize<<<c->final_blocks, 256, 0, c->stream>>>(c->acc, c->t, c->lo, c->hi, c->cc,
-                                                               c->n, c->npad, rb, re, 0, c->fixlist,
-                                                               c->ctr, c->partials, d_rows9);
-        }));
+        return enqueue_finalize32(c, model, rb, re, d_out, d_rows9, d_err);
     }
-    HK_TRY(timed(c, HAWKES_K_REDUCE, [&] {
-        k_reduce<<<1, 256, 0, c->stream>>>(c->partials, c->final_blocks, c->fix7, c->cc, re - rb,
-                                           d_out, c->ctr);
+    const EvalDesc d = eval_desc(c);
+    const int64_t count = re - rb;
+    int g = static_cast<int>(count < static_cast<int64_t>(c->sms) * 16 ? count : c->sms * 16);
+    if (g < 1) g = 1;
+    HK_TRY(timed(c, HAWKES_K_ROWS64, [&] {
+        k_rows64<<<g, 256, 0, c->stream>>>(d, nullptr, model, rb, count, 0, nullptr, nullptr);
     }));
-    return HAWKES_OK;
+    return enqueue_rows(c, rb, re, 0, d_out, d_rows9, d_err);
 }
 
 int sync_loglik(hawkes_ctx* c, const hawkes_params* p, uint32_t flags, int64_t rb, int64_t re,
                 double* out7, double* rows_host) {
     if (!params_ok(p)) return HAWKES_ERR_ARG;
     if ((flags & ~kFlagsAll) != 0) return HAWKES_ERR_ARG;
-    HK_CUDA(cudaMemcpyAsync(c->params_dev, p, sizeof(hawkes_params), cudaMemcpyHostToDevice,
-                            c->stream));
     double* d_rows9 = nullptr;
     if (rows_host) {
         if (c->rows9_cap < c->n) {
@@ -276,15 +267,19 @@ int sync_loglik(hawkes_ctx* c, const hawkes_params* p, uint32_t flags, int64_t r
         }
         d_rows9 = c->rows9;
     }
-    HK_TRY(enqueue_loglik(c, c->params_dev, flags, rb, re, c->out_dev, d_rows9));
-    HK_CUDA(cudaMemcpyAsync(c->out_host, c->out_dev, 7 * sizeof(double), cudaMemcpyDeviceToHost,
+    // The parameters go by value and the error status comes back behind the
+    // outputs: no copy in, one copy out, one wait.
+    HK_TRY(enqueue_loglik(c, CallParams{nullptr, *p}, flags, rb, re, c->out_dev, d_rows9, c->out_dev + 7));
+    HK_CUDA(cudaMemcpyAsync(c->out_host, c->out_dev, 8 * sizeof(double), cudaMemcpyDeviceToHost,
                             c->stream));
     if (rows_host)
         HK_CUDA(cudaMemcpyAsync(rows_host, d_rows9, sizeof(double) * 9 * c->n,
                                 cudaMemcpyDeviceToHost, c->stream));
     HK_CUDA(cudaStreamSynchronize(c->stream));
-    const int err = take_device_error(c);
-    if (err != 0) return err;
+    if (c->out_host[7] != 0.0) {
+        const int err = take_device_error(c);  // reads and clears it
+        return err != 0 ? err : static_cast<int>(c->out_host[7]);
+    }
     std::memcpy(out7, c->out_host, 7 * sizeof(double));
     return HAWKES_OK;
 }
@@ -341,13 +336,11 @@ int hawkes_create(hawkes_ctx** out, int device, void* cuda_stream) {
         if (sweep_setup_attributes() != cudaSuccess) { rc = HAWKES_ERR_CUDA; break; }
         c->variant = 0;
         c->variant_bpsm = sweep_blocks_per_sm(0);
-        c->final_blocks = 2 * c->sms;
         if ((rc = dalloc(&c->ctr, CT_COUNT)) != HAWKES_OK) break;
         if ((rc = dalloc(&c->cc, CC_COUNT)) != HAWKES_OK) break;
-        if ((rc = dalloc(&c->params_dev, 1)) != HAWKES_OK) break;
         if ((rc = dalloc(&c->out_dev, 8)) != HAWKES_OK) break;
         if ((rc = dalloc(&c->fix7, FIX_DOUBLES)) != HAWKES_OK) break;
-        if ((rc = dalloc(&c->partials, static_cast<size_t>(PART_STRIDE * c->final_blocks))) != HAWKES_OK)
+        if ((rc = dalloc(&c->partials, static_cast<size_t>(PART_STRIDE * BPSM * c->sms))) != HAWKES_OK)
             break;
         if (cudaMallocHost(reinterpret_cast<void**>(&c->out_host), 8 * sizeof(double)) != cudaSuccess) {
             rc = HAWKES_ERR_OOM;
@@ -381,7 +374,7 @@ void hawkes_destroy(hawkes_ctx* c) {
     free_events(c);
     free_counties(c);
     spatial_free(c);
-    dfree(c->ctr); dfree(c->cc); dfree(c->params_dev); dfree(c->out_dev); dfree(c->fix7);
+    dfree(c->ctr); dfree(c->cc); dfree(c->out_dev); dfree(c->fix7);
     dfree(c->partials);
     if (c->out_host) cudaFreeHost(c->out_host);
     for (auto& e : c->pev)
@@ -417,7 +410,8 @@ int hawkes_set_events(hawkes_ctx* c, int64_t n, const double* t, const double* x
         c->nblk = npad / TB;
         c->n_counties = n_counties;
         if ((rc = dalloc(&c->t, npad)) || (rc = dalloc(&c->x, npad)) || (rc = dalloc(&c->y, npad)) ||
-            (rc = dalloc(&c->s, npad)) || (rc = dalloc(&c->scale_c, n_counties)) ||
+            (rc = dalloc(&c->is2, npad)) || (rc = dalloc(&c->ce, npad)) ||
+            (rc = dalloc(&c->scale_c, n_counties)) ||
             (rc = dalloc(&c->county, n)) || (rc = dalloc(&c->lo, npad)) ||
             (rc = dalloc(&c->hi, npad)) || (rc = dalloc(&c->tb, c->nblk)) ||
             (rc = dalloc(&c->rec, npad)) || (rc = dalloc(&c->acc, 6 * npad)) ||
@@ -436,7 +430,7 @@ int hawkes_set_events(hawkes_ctx* c, int64_t n, const double* t, const double* x
         return fail(HAWKES_ERR_CUDA);
     rc = timed(c, HAWKES_K_OTHER, [&] {
         k_setup<<<grid_for(c, npad), 256, 0, st>>>(c->t, c->x, c->y, c->county, n_counties,
-                                                   c->scale_c, n, npad, x ? 1 : 0, c->s, c->lo,
+                                                   c->scale_c, n, npad, x ? 1 : 0, c->is2, c->ce, c->lo,
                                                    c->hi, c->tb, c->ctr);
     });
     if (rc != HAWKES_OK) return fail(rc);
@@ -500,11 +494,12 @@ int hawkes_resample_locations(hawkes_ctx* c, uint64_t seed, uint64_t stream, uin
     if (!c) return HAWKES_ERR_ARG;
     if (c->n == 0 || !c->counties_ok) return HAWKES_ERR_STATE;
     DeviceGuard g(c->device);
-    return timed(c, HAWKES_K_RESAMPLE, [&] {
-        k_resample<<<grid_for(c, c->n), 256, 0, c->stream>>>(c->county, c->n, c->tri_xy, c->tri_cum,
-                                                             c->cfirst, c->clast, seed, stream,
-                                                             iteration, nullptr, c->x, c->y);
-    });
+    EvalDesc d = eval_desc(c);
+    d.seed = seed;
+    d.stream = stream;
+    const EventGrid eg = event_grid(c->n, c->sms);
+    return timed(c, HAWKES_K_RESAMPLE,
+                 [&] { k_resample<<<eg.blocks, eg.threads, 0, c->stream>>>(d, iteration); });
 }
 
 int hawkes_get_locations(hawkes_ctx* c, double* x, double* y) {
@@ -539,7 +534,7 @@ int hawkes_loglik_grad_async(hawkes_ctx* c, const hawkes_params* d_params, uint3
     if ((flags & ~kFlagsAll) != 0) return HAWKES_ERR_ARG;
     if (c->n == 0) return HAWKES_ERR_STATE;
     DeviceGuard g(c->device);
-    return enqueue_loglik(c, d_params, flags, 0, c->n, d_out, nullptr);
+    return enqueue_loglik(c, CallParams{d_params, {}}, flags, 0, c->n, d_out, nullptr, nullptr);
 }
 
 int hawkes_loglik_rows(hawkes_ctx* c, const hawkes_params* p, uint32_t flags, double* out7,
@@ -631,11 +626,7 @@ int hawkes_shard_moments(hawkes_ctx* c, const hawkes_params* d_params, uint32_t 
     }
     const int model = static_cast<int>(flags & kModelBits);
     const int skip = (flags & HAWKES_SKIP_UNDERFLOW) ? 1 : 0;
-    HK_TRY(timed(c, HAWKES_K_PREP, [&] {
-        k_prep<<<grid_for(c, c->npad), 256, 0, c->stream>>>(c->t, c->x, c->y, c->s, c->tb, d_params,
-                                                            model, 1, skip, c->n, c->npad, c->rec,
-                                                            c->acc, c->cc, c->ctr, c->fix7);
-    }));
+    HK_TRY(enqueue_prep(c, CallParams{d_params, {}}, model, 1, skip));
     cudaError_t se = cudaSuccess;
     HK_TRY(timed(c, HAWKES_K_SWEEP, [&] {
         se = launch_sweep_list(c, c->shard_items, c->shard_nitems, (flags & HAWKES_BG_TIME) != 0,
@@ -658,14 +649,10 @@ int hawkes_finalize_moments(hawkes_ctx* c, const hawkes_params* d_params, uint32
     if (c->n == 0) return HAWKES_ERR_STATE;
     DeviceGuard g(c->device);
     const int model = static_cast<int>(flags & kModelBits);
-    HK_TRY(timed(c, HAWKES_K_PREP, [&] {  // constants and counters (nothing staged)
-        k_prep<<<grid_for(c, c->npad), 256, 0, c->stream>>>(c->t, c->x, c->y, c->s, c->tb, d_params,
-                                                            model, 0, 0, c->n, c->npad, c->rec,
-                                                            c->acc, c->cc, c->ctr, c->fix7);
-    }));
+    HK_TRY(enqueue_prep(c, CallParams{d_params, {}}, model, 0, 0));  // constants, counters
     HK_CUDA(cudaMemcpy2DAsync(c->acc, c->npad * sizeof(double), d_moments, c->n * sizeof(double),
                               c->n * sizeof(double), 6, cudaMemcpyDeviceToDevice, c->stream));
-    return enqueue_finalize32(c, model, 0, c->n, d_out, nullptr);
+    return enqueue_finalize32(c, model, 0, c->n, d_out, nullptr, nullptr);
 }
 
 int hawkes_sweep_variants(void) { return sweep_num_variants(); }

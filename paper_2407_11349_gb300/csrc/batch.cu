@@ -18,21 +18,14 @@
 #include "common.cuh"
 
 namespace hk {
-__global__ void k_prep(const double*, const double*, const double*, const double*, const double*,
-                       const hawkes_params*, int, int, int, int64_t, int64_t, Rec*, double*, double*,
-                       int*, double*);
-__global__ void k_finalize(const double*, const double*, const int32_t*, const int32_t*,
-                           const double*, int64_t, int64_t, int64_t, int64_t, int, int*, int*,
-                           double*, double*);
-__global__ void k_flushfix(const double*, const double*, const double*, const double*,
-                           const double*, const int32_t*, const int32_t*, const double*, int,
-                           int64_t, int64_t, int64_t, int64_t, int*, double*, double*, double*);
-__global__ void k_rows64(const double*, const double*, const double*, const double*,
-                         const int32_t*, const int32_t*, const double*, int, int64_t, int64_t,
-                         int64_t, int64_t, int, const int*, int*, double*, double*, double*);
-__global__ void k_reduce(const double*, int, const double*, double*, int64_t, double*, int*);
-__global__ void k_resample(const int32_t*, int64_t, const double*, const double*, const int32_t*,
-                           const int32_t*, uint64_t, uint64_t, uint64_t, const uint64_t*, double*,
+__global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const hawkes_params*,
+                       const __grid_constant__ hawkes_params,
+                       int, int, int, int, const uint64_t*, int*);
+void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
+                     double*, double*, double*);
+__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, int, double*,
+                         double*);
+__global__ void k_flushfix(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, double*, double*,
                            double*);
 int sweep_num_variants();
 int sweep_blocks_per_sm(int v);
@@ -56,6 +49,25 @@ cudaError_t launch_sweep_batch(cudaStream_t st, const SweepPlan& pl, int sms, in
 __global__ void k_set_u64(uint64_t* dst, uint64_t v) {
     if (threadIdx.x == 0 && blockIdx.x == 0) *dst = v;
 }
+
+// First latched error of the batch (its own counters, then the problems' in
+// order); clears them all.  One warp.
+__global__ void k_take_errors(int* bctr, const EvalDesc* __restrict__ probs, int P, int* out) {
+    const int lane = threadIdx.x;
+    int err = 0;
+    if (lane == 0) {
+        err = atomicExch(bctr + CT_ERR, 0);
+        const int g = atomicExch(bctr + CT_COUNT + CT_ERR, 0);
+        if (err == 0) err = g;
+    }
+    err = __shfl_sync(0xffffffffu, err, 0);
+    for (int p0 = 0; p0 < P; p0 += 32) {
+        const int e = p0 + lane < P ? atomicExch(probs[p0 + lane].ctr + CT_ERR, 0) : 0;
+        const unsigned any = __ballot_sync(0xffffffffu, e != 0);
+        if (err == 0 && any) err = __shfl_sync(0xffffffffu, e, __ffs(any) - 1);
+    }
+    if (lane == 0) *out = err;
+}
 int tune_cache_get(const char* path, const char* key, int* variant, int* chunk, int* order,
                    double* ms, int* kc);
 int tune_cache_put(const char* path, const char* key, int variant, int chunk, int order, double ms,
@@ -75,7 +87,9 @@ struct hawkes_batch {
     std::vector<hawkes_ctx*> probs;
     std::vector<uint64_t> seeds, streams;
     bool resample = false;
-    ProbDesc* d_probs = nullptr;
+    ProbDesc* d_probs = nullptr;  // the problems as the sweep and the O(N) kernels see them
+    EvalDesc* d_eval = nullptr;
+    std::vector<EvalDesc> h_eval;  // what d_eval holds
     int4* d_items = nullptr;
     int nitems = 0;
     int variant = 0;
@@ -90,12 +104,8 @@ struct hawkes_batch {
     const hawkes_params* g_params = nullptr;  // pointers the graph was captured with
     double* g_out = nullptr;
     cudaEvent_t ev[2] = {nullptr, nullptr};
-    // the per-problem O(N) kernels run on NAUX side streams forked from and
-    // joined back into `stream` (branches of the captured graph)
-    static constexpr int NAUX = 4;
-    cudaStream_t aux[NAUX] = {nullptr, nullptr, nullptr, nullptr};
-    cudaEvent_t fork_ev = nullptr;
-    cudaEvent_t join_ev[NAUX] = {nullptr, nullptr, nullptr, nullptr};
+    int* d_err = nullptr;        // first latched error and its pinned host copy
+    int* h_err = nullptr;
     // chains per CTA (sweep_group.cu)
     int kc = 1;
     std::vector<std::vector<int>> tclass;  // problems with identical event times, in input order
@@ -273,106 +283,79 @@ int build_items(hawkes_batch* b, int variant, int chunk, int order) {
     return HAWKES_OK;
 }
 
-// Make the side streams wait for the work queued so far on the batch's stream,
-// and the batch's stream wait for the side streams.
-int fork_side(hawkes_batch* b) {
-    HB_CUDA(cudaEventRecord(b->fork_ev, b->stream));
-    for (cudaStream_t s : b->aux) HB_CUDA(cudaStreamWaitEvent(s, b->fork_ev, 0));
-    return HAWKES_OK;
-}
-int join_side(hawkes_batch* b) {
-    for (int k = 0; k < hawkes_batch::NAUX; ++k) {
-        HB_CUDA(cudaEventRecord(b->join_ev[k], b->aux[k]));
-        HB_CUDA(cudaStreamWaitEvent(b->stream, b->join_ev[k], 0));
+static_assert(sizeof(EvalDesc) % 8 == 0, "compared as bytes: no padding");
+
+// Bring the device's problem descriptors up to date (hawkes_set_counties on a
+// member replaces its triangles).  Not under stream capture.
+int refresh_eval(hawkes_batch* b) {
+    std::vector<EvalDesc> now;
+    for (size_t p = 0; p < b->probs.size(); ++p) {
+        if (b->resample && !b->probs[p]->counties_ok) return HAWKES_ERR_STATE;
+        EvalDesc d = eval_desc(b->probs[p]);
+        if (b->resample) {
+            d.seed = b->seeds[p];
+            d.stream = b->streams[p];
+        }
+        now.push_back(d);
     }
+    if (now.size() == b->h_eval.size() &&
+        std::memcmp(now.data(), b->h_eval.data(), now.size() * sizeof(EvalDesc)) == 0)
+        return HAWKES_OK;
+    HB_CUDA(cudaStreamSynchronize(b->stream));
+    HB_CUDA(cudaMemcpyAsync(b->d_eval, now.data(), now.size() * sizeof(EvalDesc), cudaMemcpyHostToDevice,
+                            b->stream));
+    HB_CUDA(cudaStreamSynchronize(b->stream));
+    b->h_eval = now;
     return HAWKES_OK;
 }
 
 // Queue one batched evaluation.  d_params[P], d_out[7 P]; the iteration is read
-// from b->d_iter by the resample kernels.  The problems' resample and staging
-// kernels, and after the sweep their finalisation, are spread over the side
-// streams (problems are independent there); the sweep launches run on the
-// batch's stream, which also ends the whole evaluation.
+// from b->d_iter.  One launch per stage covers all problems (blockIdx.y): the
+// resample and staging, the sweeps, the finalisation and its two fix-ups.  (As
+// one kernel per problem and stage over four side streams, 30 chains of 20,000
+// events took 180 launches, 0.5 ms of a 4.4 ms evaluation.)
 int enqueue(hawkes_batch* b, const hawkes_params* d_params, double* d_out, bool time_sweep) {
     const int model = static_cast<int>(b->flags & kModelBits);
     const bool bgt = (b->flags & HAWKES_BG_TIME) != 0;
     const int skip = (b->flags & HAWKES_SKIP_UNDERFLOW) ? 1 : 0;
     const int P = static_cast<int>(b->probs.size());
-    HB_TRY(fork_side(b));
-    for (int p = 0; p < P; ++p) {
-        cudaStream_t st = b->aux[p % hawkes_batch::NAUX];
-        hawkes_ctx* c = b->probs[p];
-        int g = static_cast<int>((c->npad + 255) / 256);
-        if (g > 8 * b->sms) g = 8 * b->sms;
-        if (b->resample)
-            k_resample<<<g, 256, 0, st>>>(c->county, c->n, c->tri_xy, c->tri_cum, c->cfirst, c->clast,
-                                          b->seeds[p], b->streams[p], 0, b->d_iter, c->x, c->y);
-        k_prep<<<g, 256, 0, st>>>(c->t, c->x, c->y, c->s, c->tb, d_params + p, model, 1, skip,
-                                  c->n, c->npad, c->rec, c->acc, c->cc, c->ctr, c->fix7);
-    }
-    HB_TRY(join_side(b));
     cudaStream_t st = b->stream;
+    int64_t nmax = 0;
+    for (const hawkes_ctx* c : b->probs) nmax = std::max(nmax, c->n);
+    const EventGrid g = event_grid(nmax, b->sms, P);
+    const dim3 grid(g.blocks, P);
+    k_prep<<<grid, g.threads, 0, st>>>(EvalDesc{}, b->d_eval, d_params, hawkes_params{}, model, 1, skip,
+                                       b->resample ? 1 : 0, b->d_iter, b->d_ctr);
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
         const Rec* recs[KMAX] = {nullptr, nullptr, nullptr, nullptr};
         for (int k = 0; k < b->kc; ++k) recs[k] = b->probs[b->groups[gi][k]]->rec;
         HB_CUDA(launch_group_stage(st, b->sms, b->h_groups[gi], recs, b->probs[b->groups[gi][0]]->t,
                                    b->kc, b->d_gtiles + b->gtile_off[gi]));
     }
-    HB_CUDA(cudaMemsetAsync(b->d_ctr + CT_WORK, 0, sizeof(int), st));
-    HB_CUDA(cudaMemsetAsync(b->d_ctr + CT_COUNT + CT_WORK, 0, sizeof(int), st));
     if (time_sweep) HB_CUDA(cudaEventRecord(b->ev[0], st));
     if (b->ngitems > 0)
         HB_CUDA(launch_sweep_group(st, b->kc, b->ggrid, b->d_groups,
                                    static_cast<int>(b->h_groups.size()), b->d_gitems, b->ngitems,
                                    b->d_ctr + CT_COUNT));
-    HB_CUDA(launch_sweep_batch(st, b->plan, b->sms, b->variant, b->grid, b->d_probs, static_cast<int>(P), b->d_items,
-                               b->nitems, b->d_ctr, bgt,
-                               (b->flags & HAWKES_LOGLIK_ONLY) != 0));
+    HB_CUDA(launch_sweep_batch(st, b->plan, b->sms, b->variant, b->grid, b->d_probs, P, b->d_items,
+                               b->nitems, b->d_ctr, bgt, (b->flags & HAWKES_LOGLIK_ONLY) != 0));
     if (time_sweep) HB_CUDA(cudaEventRecord(b->ev[1], st));
-    HB_TRY(fork_side(b));
-    for (int p = 0; p < P; ++p) {
-        cudaStream_t st = b->aux[p % hawkes_batch::NAUX];
-        hawkes_ctx* c = b->probs[p];
-        k_finalize<<<c->final_blocks, 256, 0, st>>>(c->acc, c->t, c->lo, c->hi, c->cc, c->n,
-                                                    c->npad, 0, c->n, 1, c->fixlist, c->ctr,
-                                                    c->partials, nullptr);
-        k_rows64<<<b->sms, 256, 0, st>>>(c->t, c->x, c->y, c->s, c->lo, c->hi, c->cc, model, c->n,
-                                         c->npad, 0, 0, 1, c->fixlist, c->ctr, c->acc, c->fix7,
-                                         nullptr);
-        k_reduce<<<1, 256, 0, st>>>(c->partials, c->final_blocks, c->fix7, c->cc, c->n,
-                                    d_out + 7 * p, c->ctr);
-        int gf = static_cast<int>((c->n + 255) / 256);
-        if (gf > 2 * b->sms) gf = 2 * b->sms;
-        k_flushfix<<<gf, 256, 0, st>>>(c->acc, c->t, c->x, c->y, c->s, c->lo, c->hi, c->cc, model,
-                                       c->n, c->npad, 0, c->n, c->ctr, c->fix7, d_out + 7 * p,
-                                       nullptr);
-    }
+    launch_finalize(st, dim3(final_grid(nmax, b->sms, P), P), EvalDesc{}, b->d_eval, 0, 0, 1, d_out,
+                    nullptr, nullptr);
+    const int fix = std::max(2 * b->sms / P, 8);  // blocks per problem for the fix-ups (usually idle)
+    k_rows64<<<dim3(fix, P), 256, 0, st>>>(EvalDesc{}, b->d_eval, model, 0, 0, 1, d_out, nullptr);
+    k_flushfix<<<dim3(fix, P), 256, 0, st>>>(EvalDesc{}, b->d_eval, model, 0, 0, d_out, nullptr, nullptr);
     HB_CUDA(cudaGetLastError());
-    return join_side(b);
+    return HAWKES_OK;
 }
 
+// Wait for the queued work; the first latched error, cleared.
 int latched_errors(hawkes_batch* b) {
-    int err = 0, gerr = 0;
-    HB_CUDA(cudaMemcpyAsync(&err, b->d_ctr + CT_ERR, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
-    HB_CUDA(cudaMemcpyAsync(&gerr, b->d_ctr + CT_COUNT + CT_ERR, sizeof(int), cudaMemcpyDeviceToHost,
-                            b->stream));
+    k_take_errors<<<1, 32, 0, b->stream>>>(b->d_ctr, b->d_eval, static_cast<int>(b->probs.size()), b->d_err);
+    HB_CUDA(cudaGetLastError());
+    HB_CUDA(cudaMemcpyAsync(b->h_err, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
     HB_CUDA(cudaStreamSynchronize(b->stream));
-    if (gerr != 0) {
-        HB_CUDA(cudaMemsetAsync(b->d_ctr + CT_COUNT + CT_ERR, 0, sizeof(int), b->stream));
-        if (err == 0) err = gerr;
-    }
-    for (auto* c : b->probs) {
-        int e = 0;
-        HB_CUDA(cudaMemcpyAsync(&e, c->ctr + CT_ERR, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
-        HB_CUDA(cudaStreamSynchronize(b->stream));
-        if (e != 0) {
-            HB_CUDA(cudaMemsetAsync(c->ctr + CT_ERR, 0, sizeof(int), b->stream));
-            if (err == 0) err = e;
-        }
-    }
-    HB_CUDA(cudaStreamSynchronize(b->stream));
-    if (err != 0) HB_CUDA(cudaMemsetAsync(b->d_ctr + CT_ERR, 0, sizeof(int), b->stream));
-    return err;
+    return *b->h_err;
 }
 
 }  // namespace
@@ -418,12 +401,9 @@ int hawkes_batch_create(hawkes_batch** out, hawkes_ctx* const* problems, int32_t
             b->own_stream = true;
         }
         if ((rc = st_of(cudaEventCreate(&b->ev[0]))) || (rc = st_of(cudaEventCreate(&b->ev[1])))) break;
-        if ((rc = st_of(cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming)))) break;
-        for (int k = 0; k < hawkes_batch::NAUX && rc == HAWKES_OK; ++k) {
-            rc = st_of(cudaStreamCreateWithFlags(&b->aux[k], cudaStreamNonBlocking));
-            if (rc == HAWKES_OK) rc = st_of(cudaEventCreateWithFlags(&b->join_ev[k], cudaEventDisableTiming));
-        }
-        if (rc) break;
+        if ((rc = st_of(cudaMalloc(&b->d_err, sizeof(int)))) ||
+            (rc = st_of(cudaMallocHost(reinterpret_cast<void**>(&b->h_err), sizeof(int)))))
+            break;
         if ((rc = st_of(cudaMalloc(&b->d_ctr, 2 * CT_COUNT * sizeof(int))))) break;
         if ((rc = st_of(cudaMalloc(&b->d_iter, sizeof(uint64_t))))) break;
         if ((rc = st_of(cudaMemsetAsync(b->d_ctr, 0, 2 * CT_COUNT * sizeof(int), b->stream)))) break;
@@ -436,6 +416,8 @@ int hawkes_batch_create(hawkes_batch** out, hawkes_ctx* const* problems, int32_t
         if ((rc = st_of(cudaMemcpyAsync(b->d_probs, descs.data(), descs.size() * sizeof(ProbDesc),
                                         cudaMemcpyHostToDevice, b->stream))))
             break;
+        if ((rc = st_of(cudaMalloc(&b->d_eval, b->probs.size() * sizeof(EvalDesc))))) break;
+        if ((rc = refresh_eval(b))) break;
         // the contexts' own queued work must finish before the batch touches their buffers
         for (auto* c : b->probs)
             if ((rc = st_of(cudaStreamSynchronize(c->stream)))) break;
@@ -466,13 +448,9 @@ void hawkes_batch_destroy(hawkes_batch* b) {
     if (b->d_iter) cudaFree(b->d_iter);
     for (auto& e : b->ev)
         if (e) cudaEventDestroy(e);
-    for (cudaStream_t s : b->aux)
-        if (s) cudaStreamSynchronize(s);
-    for (int k = 0; k < hawkes_batch::NAUX; ++k) {
-        if (b->join_ev[k]) cudaEventDestroy(b->join_ev[k]);
-        if (b->aux[k]) cudaStreamDestroy(b->aux[k]);
-    }
-    if (b->fork_ev) cudaEventDestroy(b->fork_ev);
+    if (b->d_eval) cudaFree(b->d_eval);
+    if (b->d_err) cudaFree(b->d_err);
+    if (b->h_err) cudaFreeHost(b->h_err);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     cudaGetLastError();
     delete b;
@@ -483,6 +461,7 @@ int hawkes_batch_run(hawkes_batch* b, const hawkes_params* d_params, uint64_t it
     HK_NVTX("hawkes_batch_run");
     if (!b || !d_params || !d_out || !aligned8(d_params) || !aligned8(d_out)) return HAWKES_ERR_ARG;
     DeviceGuard g(b->device);
+    HB_TRY(refresh_eval(b));
     k_set_u64<<<1, 32, 0, b->stream>>>(b->d_iter, iteration);
     HB_CUDA(cudaGetLastError());
     if (b->exec && b->g_params == d_params && b->g_out == d_out)
@@ -496,6 +475,7 @@ int hawkes_batch_capture(hawkes_batch* b, const hawkes_params* d_params, double*
     DeviceGuard g(b->device);
     HB_CUDA(cudaStreamSynchronize(b->stream));
     drop_graph(b);
+    HB_TRY(refresh_eval(b));
     HB_CUDA(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     const int rc = enqueue(b, d_params, d_out, false);
     cudaGraph_t graph = nullptr;
@@ -520,7 +500,6 @@ int hawkes_batch_wait(hawkes_batch* b) {
     HK_NVTX("hawkes_batch_wait");
     if (!b) return HAWKES_ERR_ARG;
     DeviceGuard g(b->device);
-    HB_CUDA(cudaStreamSynchronize(b->stream));
     return latched_errors(b);
 }
 
@@ -547,6 +526,7 @@ int hawkes_batch_tune(hawkes_batch* b, const hawkes_params* d_params, double* d_
         *t = tot / reps;
         return HAWKES_OK;
     };
+    HB_TRY(refresh_eval(b));
     // one problem per CTA: sweep variant x item order x chunk length
     b->kc = 1;
     for (int v = 0; v < sweep_num_variants(); ++v) {
@@ -583,7 +563,6 @@ int hawkes_batch_tune(hawkes_batch* b, const hawkes_params* d_params, double* d_
     }
     b->kc = bk;
     HB_TRY(build_items(b, bv, bc, bo));
-    HB_CUDA(cudaStreamSynchronize(b->stream));
     if (variant) *variant = bv;
     if (chunk) *chunk = bc;
     if (order) *order = bo;

@@ -104,6 +104,65 @@ struct ProbDesc {
     int64_t n, npad;
 };
 
+// One problem as the O(N) kernels see it (device pointers).  They take one by
+// value, or an array of them with the problem in blockIdx.y (batches).
+struct EvalDesc {
+    const double* t;
+    double* x;
+    double* y;
+    const double* is2;   // 1 / s_j^2
+    const float* ce;     // -2 log2 s_j
+    const double* tb;
+    const int32_t* lo;
+    const int32_t* hi;
+    Rec* rec;
+    double* acc;
+    double* cc;
+    int* ctr;
+    double* fix7;
+    int* fixlist;
+    double* partials;
+    int64_t n, npad;
+    // location resample
+    const int32_t* county;
+    const double* tri_xy;
+    const double* tri_cum;
+    const int32_t* cfirst;
+    const int32_t* clast;
+    uint64_t seed, stream;
+};
+
+// Threads per block and blocks per problem of the O(N) kernels (events: of the
+// largest problem), one thread per event up to BPSM blocks per SM.  An FP64 instruction
+// takes a warp about 19 cycles of its SM (1.7 lanes per clock measured), so the
+// warps of few events are spread over the SMs in blocks of 64; each block's
+// constants (k_prep) and partial sums (k_finalize) make more blocks dear.
+constexpr int BPSM = 4;
+struct EventGrid {
+    int threads, blocks;
+};
+inline EventGrid event_grid(int64_t events, int sms, int problems = 1) {
+    const int th = events * problems <= 256ll * sms ? 64 : 256;
+    const int64_t most = static_cast<int64_t>(sms) * BPSM;
+    int64_t cap = most / problems, big = (events + 1023) / 1024;  // at most 4 events a thread
+    if (big > most) big = most;
+    if (cap < big) cap = big;
+    int64_t g = (events + th - 1) / th;
+    if (g > cap) g = cap;
+    return EventGrid{th, g < 1 ? 1 : static_cast<int>(g)};
+}
+
+// k_finalize: four warps per 32 rows (see there).
+constexpr int FINAL_THREADS = 128;
+inline int final_grid(int64_t rows, int sms, int problems = 1) {
+    const int64_t most = static_cast<int64_t>(sms) * BPSM;
+    int64_t cap = most / problems, big = (rows + 511) / 512, g = (rows + 31) / 32;
+    if (big > most) big = most;
+    if (cap < big) cap = big;
+    if (g > cap) g = cap;
+    return g < 1 ? 1 : static_cast<int>(g);
+}
+
 // How the symmetric sweep of a problem (or of a batch) is cut into work items
 // of `chunk` column tiles: by the row-tile kernel of the selected variant
 // (k_sweep), or by the column-split kernel (k_sweep_cs).
@@ -149,14 +208,24 @@ enum {
     CC_BGT,         // 1 for the time-only background
     CC_LLONLY,      // 1 when only the log-likelihood is evaluated
     CC_FTHR,        // [7] flush-bound thresholds per output (< 0: nothing to recompute)
-    CC_COUNT = CC_FTHR + 7
+    // Row finalisation, linear in the raw moment sums S (see row_eval):
+    CC_LB = CC_FTHR + 7,  // lambda = LB SB + LE SE
+    CC_LE,
+    CC_A1, CC_B1,   // d/dtau_x numerator A1 SBr - B1 SB
+    CC_A2, CC_B2,   // d/dtau_t           A2 SBt - B2 SB
+    CC_A4,          // d/domega           A4 SE - LE SEt
+    CC_A5, CC_B5,   // d/dh               A5 SEq - B5 SE
+    CC_ITT,         // 1 / tau_t
+    CC_F0,          // flush bounds of the numerators per source: 6, then LE F
+    CC_COUNT = CC_F0 + 7
 };
 
 // Per-block partials of k_finalize: the 7 outputs, then the 7 flush bounds.
 constexpr int PART_STRIDE = 16;
 // fix7 buffer: [0, 8) sums over rows recomputed because their rate is near the
-// FP32 floor, [8, 16) corrections of rows recomputed because of the flush bound.
-constexpr int FIX_DOUBLES = 16;
+// FP32 floor, [8, 16) corrections of rows recomputed because of the flush bound,
+// [16, 32) the totals over the other rows, kept until those sums are complete.
+constexpr int FIX_DOUBLES = 32;
 // Relative share of an output's magnitude that the bound on the FP32 sweep's
 // flushed terms may reach before the rows that carry it are recomputed in FP64.
 constexpr double FLUSH_TAU = 1e-8;
@@ -168,12 +237,15 @@ enum {
     CT_ERR,         // latched error status (0 or a HAWKES_ERR_* value)
     CT_DONE,        // finished-block counter
     CT_CEMAX,       // bits of max(0, max_j -2 log2 s_j), set when the events are loaded
+    CT_FDONE,       // finished blocks of k_finalize
+    CT_RDONE,       // finished blocks of k_rows64 (fix-up rows)
     CT_COUNT = 8
 };
 
 constexpr double LOG2E = 1.4426950408889634;
 constexpr double CLIP = 1e-40;
 constexpr double TWO_PI = 6.283185307179586;
+constexpr double SQRT_TWO_PI = 2.5066282746310002;
 
 // Bounded waits: a wait on an mbarrier gives up after WAIT_CYCLES SM clock
 // cycles (about 2 s at 2 GHz) or SPIN_LIMIT polls, whichever comes first.
@@ -267,7 +339,8 @@ struct hawkes_ctx {
     double* t = nullptr;       // [npad] FP64 times (padding = t_N)
     double* x = nullptr;       // [npad] current locations
     double* y = nullptr;
-    double* s = nullptr;       // [npad] per-event source scale
+    double* is2 = nullptr;     // [npad] 1 / s_j^2 of the per-event source scale
+    float* ce = nullptr;       // [npad] -2 log2 s_j
     double* scale_c = nullptr; // [n_counties]
     int32_t* county = nullptr; // [n]
     int32_t* lo = nullptr;     // [npad] first index with t_j == t_i
@@ -281,17 +354,15 @@ struct hawkes_ctx {
     int variant = 0;           // sweep kernel variant in use
     int variant_bpsm = 1;      // its resident CTAs per SM
     double* acc = nullptr;     // [6 * npad] per-row moment sums (natural units)
-    double* partials = nullptr;// [final_blocks * 8]
-    double* fix7 = nullptr;    // [8] sums over FP64-recomputed rows
+    double* partials = nullptr;// [BPSM * sms * PART_STRIDE]
+    double* fix7 = nullptr;    // [FIX_DOUBLES]
     int* fixlist = nullptr;    // [npad]
     int* ctr = nullptr;        // [CT_COUNT]
     double* cc = nullptr;      // [CC_COUNT]
-    hawkes_params* params_dev = nullptr;
     double* out_dev = nullptr; // [8]
     double* out_host = nullptr;// pinned [8]
     double* rows9 = nullptr;   // [9 * n] optional per-row output (allocated on demand)
     int64_t rows9_cap = 0;
-    int final_blocks = 0;
 
     int32_t n_tri = 0;
     bool counties_ok = false;
@@ -313,3 +384,16 @@ struct hawkes_ctx {
     int shard_nitems = 0;
     int shard_key[3] = {-1, -1, -1};
 };
+
+namespace hk {
+inline EvalDesc eval_desc(const hawkes_ctx* c) {
+    EvalDesc d{};
+    d.t = c->t; d.x = c->x; d.y = c->y; d.is2 = c->is2; d.ce = c->ce; d.tb = c->tb;
+    d.lo = c->lo; d.hi = c->hi; d.rec = c->rec; d.acc = c->acc; d.cc = c->cc; d.ctr = c->ctr;
+    d.fix7 = c->fix7; d.fixlist = c->fixlist; d.partials = c->partials;
+    d.n = c->n; d.npad = c->npad;
+    d.county = c->county; d.tri_xy = c->tri_xy; d.tri_cum = c->tri_cum;
+    d.cfirst = c->cfirst; d.clast = c->clast;
+    return d;
+}
+}  // namespace hk

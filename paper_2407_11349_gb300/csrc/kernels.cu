@@ -30,7 +30,7 @@ __device__ __forceinline__ int64_t upper_bound_d(const double* a, int64_t n, dou
 }
 
 __global__ void k_setup(double* t, double* x, double* y, const int32_t* county, int32_t nc,
-                        const double* scale_c, int64_t n, int64_t npad, int xy_given, double* s,
+                        const double* scale_c, int64_t n, int64_t npad, int xy_given, double* is2, float* ces,
                         int32_t* lo, int32_t* hi, double* tb, int* ctr) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < npad;
          e += (int64_t)gridDim.x * blockDim.x) {
@@ -43,8 +43,9 @@ __global__ void k_setup(double* t, double* x, double* y, const int32_t* county, 
             if (c < 0 || c >= nc) set_error(ctr, HAWKES_ERR_ARG);
             else se = scale_c[c];
             if (!(se > 0.0) || !isfinite(se)) set_error(ctr, HAWKES_ERR_ARG);
-            s[e] = se;
+            is2[e] = 1.0 / (se * se);
             const float ce = static_cast<float>(-2.0 * log2(se));
+            ces[e] = ce;
             if (ce > 0.f) atomicMax(ctr + CT_CEMAX, __float_as_int(ce));
             if (xy_given) {
                 if (!isfinite(x[e]) || !isfinite(y[e])) set_error(ctr, HAWKES_ERR_ARG);
@@ -58,7 +59,8 @@ __global__ void k_setup(double* t, double* x, double* y, const int32_t* county, 
             t[e] = t[n - 1];
             x[e] = 0.0;
             y[e] = 0.0;
-            s[e] = 1.0;
+            is2[e] = 1.0;
+            ces[e] = 0.f;
             lo[e] = 0;
             hi[e] = 0;
         }
@@ -67,160 +69,291 @@ __global__ void k_setup(double* t, double* x, double* y, const int32_t* county, 
 }
 
 // ---------------------------------------------------------------------------
-// Per-call constants (every thread derives them; block 0 publishes them).
+// Per-call constants.
 // ---------------------------------------------------------------------------
 struct Consts {
     double mu, tx, tt, th, om, h;
-    double kx, kt, omt, sr, st, set, seq, cB, cE;
+    double kx, kt, omt, sr, st, set, seq, cB, cE, itx, itt, iom, ih, beta0;
     bool valid;
 };
 
-__device__ __forceinline__ Consts make_consts(const hawkes_params* P, bool bg_time) {
+// One warp forms the constants: the quotients side by side, one per lane, then
+// the square roots.  (An FP64 division is a chain of a dozen instructions of
+// about 40 cycles; one thread forming them in turn took 6 us.)
+__device__ __forceinline__ Consts make_consts(const hawkes_params& P, bool bg_time) {
     Consts k;
-    k.mu = P->mu; k.tx = P->tau_x; k.tt = P->tau_t; k.th = P->theta; k.om = P->omega; k.h = P->h;
+    k.mu = P.mu; k.tx = P.tau_x; k.tt = P.tau_t; k.th = P.theta; k.om = P.omega; k.h = P.h;
     k.valid = isfinite(k.mu) && isfinite(k.tx) && isfinite(k.tt) && isfinite(k.th) &&
               isfinite(k.om) && isfinite(k.h) && k.mu >= 0.0 && k.th >= 0.0 && k.tx > 0.0 &&
               k.tt > 0.0 && k.om > 0.0 && k.h > 0.0;
-    const double ax = LOG2E / (2.0 * k.tx * k.tx), at = LOG2E / (2.0 * k.tt * k.tt);
-    k.kx = sqrt(ax);
-    k.kt = sqrt(at);
-    k.omt = k.om * LOG2E / k.kt;
-    k.sr = 1.0 / ax;
-    k.st = 1.0 / at;
-    k.set = 1.0 / k.kt;
-    k.seq = 2.0 * k.h * k.h / LOG2E;
-    // Space-time background phi2(r; tau_x) phi1(dt; tau_t), or the time-only
-    // background phi1(dt; tau_t) / tau_x^2 (eq. 2, tau_x^2 read as the area).
-    k.cB = bg_time ? 1.0 / (sqrt(TWO_PI) * k.tx * k.tx * k.tt)
-                   : 1.0 / (TWO_PI * sqrt(TWO_PI) * k.tx * k.tx * k.tt);
-    k.cE = k.om / (TWO_PI * k.h * k.h);
+    const int lane = threadIdx.x & 31;
+    const double tx2 = k.tx * k.tx, tt2 = k.tt * k.tt, h2 = k.h * k.h;
+    double num = 1.0, den = 1.0;
+    switch (lane) {
+        case 0: num = LOG2E; den = 2.0 * tx2; break;       // a_x
+        case 1: num = LOG2E; den = 2.0 * tt2; break;       // a_t
+        case 2: num = 2.0 * tx2; den = LOG2E; break;       // 1 / a_x
+        case 3: num = 2.0 * tt2; den = LOG2E; break;       // 1 / a_t
+        case 4: num = 2.0 * h2; den = LOG2E; break;
+        // Space-time background phi2(r; tau_x) phi1(dt; tau_t), or the time-only
+        // background phi1(dt; tau_t) / tau_x^2 (eq. 2, tau_x^2 read as the area).
+        case 5: den = (bg_time ? 1.0 : TWO_PI) * SQRT_TWO_PI * tx2 * k.tt; break;
+        case 6: num = k.om; den = TWO_PI * h2; break;
+        case 7: den = k.tx; break;
+        case 8: den = k.tt; break;
+        case 9: den = k.om; break;
+        case 10: den = k.h; break;
+        case 11: num = tx2; den = h2; break;
+    }
+    const double q = num / den, r = sqrt(q);
+    auto of = [](double v, int l) { return __shfl_sync(0xffffffffu, v, l); };
+    k.kx = of(r, 0);
+    k.kt = of(r, 1);
+    k.sr = of(q, 2);
+    k.st = of(q, 3);
+    k.set = of(r, 3);
+    k.omt = k.om * LOG2E * k.set;
+    k.seq = of(q, 4);
+    k.cB = of(q, 5);
+    k.cE = of(q, 6);
+    k.itx = of(q, 7);
+    k.itt = of(q, 8);
+    k.iom = of(q, 9);
+    k.ih = of(q, 10);
+    k.beta0 = of(q, 11);
     return k;
 }
 
-// Zero the accumulators, reset the counters and (FP32 path) stage the event table.
+// Location draw of event i (cut posterior, Sec. 2.2); below.
+__device__ __forceinline__ void draw_location(const EvalDesc& d, int64_t i, uint64_t iteration,
+                                              double& x, double& y);
+
+// Zero the accumulators, reset the counters and (FP32 path) stage the event
+// table; with `resample`, first draw every event's location (batches: one pass
+// over the events instead of two).
+// P: device parameters (one per problem), or null to take `pv`.
 // model: the HAWKES_MODEL1, HAWKES_BG_TIME and HAWKES_LOGLIK_ONLY bits of the
 // call's flags.
 // skip: evaluate only tiles whose terms can be nonzero in FP32 (see CC_SKIPDT).
-__global__ void k_prep(const double* __restrict__ t, const double* __restrict__ x,
-                       const double* __restrict__ y, const double* __restrict__ s,
-                       const double* __restrict__ tb, const hawkes_params* P, int model,
-                       int stage, int skip, int64_t n, int64_t npad, Rec* __restrict__ rec,
-                       double* __restrict__ acc, double* __restrict__ cc, int* ctr,
-                       double* fix7) {
+// bctr: the batch's two sweep work cursors to reset, or null.
+// Bound by HBM at large n (156 MB at n = 1,000,000); the FP64 constants are
+// formed by one warp of each block, because in every warp they would cost more
+// than the staging itself.
+__global__ void k_prep(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs,
+                       const hawkes_params* __restrict__ P, const __grid_constant__ hawkes_params pv,
+                       int model, int stage, int skip, int resample, const uint64_t* d_iteration,
+                       int* bctr) {
+    const EvalDesc& d = probs ? probs[blockIdx.y] : one;
     const bool model1 = (model & HAWKES_MODEL1) != 0;
-    const Consts k = make_consts(P, (model & HAWKES_BG_TIME) != 0);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        cc[CC_KX] = k.kx; cc[CC_KT] = k.kt; cc[CC_OMT] = k.omt;
-        cc[CC_SR] = k.sr; cc[CC_ST] = k.st; cc[CC_SET] = k.set; cc[CC_SEQ] = k.seq;
-        cc[CC_CB] = k.cB; cc[CC_CE] = k.cE;
-        cc[CC_MU] = k.mu; cc[CC_TX] = k.tx; cc[CC_TT] = k.tt;
-        cc[CC_TH] = k.th; cc[CC_OM] = k.om; cc[CC_H] = k.h;
-        cc[CC_TN] = t[n - 1];
-        // Terms below 2^-126 flush to zero in the FP32 path; rows whose rate is
-        // within 1e9 x (n such terms) of that are recomputed in FP64.
-        cc[CC_FLAGTHR] = 1e9 * (double)n * 1.1754943508222875e-38 * (k.mu * k.cB + k.th * k.cE);
-        // A background term is exactly 0 in FP32 (flush to zero) when its
-        // base-2 exponent dt~^2 + r~^2 exceeds 126; an excitation term when
-        // omega~ dt~ + beta r~^2 - ce exceeds 126.  With 2 units of margin, a
-        // tile whose smallest scaled time gap exceeds both bounds contributes
-        // exactly nothing.
-        const double cemax = model1 ? 0.0 : static_cast<double>(__int_as_float(ctr[CT_CEMAX]));
-        cc[CC_SKIPDTB] = skip ? sqrt(128.0) : 0.0;
-        cc[CC_SKIPDT] = skip ? fmax(sqrt(128.0), (cemax + 128.0) / k.omt) : 0.0;
-        cc[CC_VALID] = k.valid ? 1.0 : 0.0;
-        cc[CC_CEMAX] = cemax;
-        cc[CC_BGT] = (model & HAWKES_BG_TIME) ? 1.0 : 0.0;
-        cc[CC_LLONLY] = (model & HAWKES_LOGLIK_ONLY) ? 1.0 : 0.0;
-        for (int q = 0; q < 7; ++q) cc[CC_FTHR + q] = -1.0;
-        ctr[CT_WORK] = 0;
-        ctr[CT_FIX] = 0;
-        ctr[CT_DONE] = 0;
-        for (int q = 0; q < FIX_DOUBLES; ++q) fix7[q] = 0.0;
-        if (!k.valid) set_error(ctr, HAWKES_ERR_ARG);
+    const int64_t n = d.n, npad = d.npad;
+    __shared__ double s_kx, s_kt, s_beta0;
+    if (threadIdx.x < 32) {
+        const bool bgt = (model & HAWKES_BG_TIME) != 0;
+        const Consts k = make_consts(P ? P[blockIdx.y] : pv, bgt);
+        s_kx = k.kx;
+        s_kt = k.kt;
+        s_beta0 = k.beta0;
+        if (threadIdx.x == 0 && bctr && blockIdx.x == 0 && blockIdx.y == 0) {
+            bctr[CT_WORK] = 0;
+            bctr[CT_COUNT + CT_WORK] = 0;
+        }
+        if (threadIdx.x == 0 && blockIdx.x == 0) {
+            double* cc = d.cc;
+            int* ctr = d.ctr;
+            cc[CC_KX] = k.kx; cc[CC_KT] = k.kt; cc[CC_OMT] = k.omt;
+            cc[CC_SR] = k.sr; cc[CC_ST] = k.st; cc[CC_SET] = k.set; cc[CC_SEQ] = k.seq;
+            cc[CC_CB] = k.cB; cc[CC_CE] = k.cE;
+            cc[CC_MU] = k.mu; cc[CC_TX] = k.tx; cc[CC_TT] = k.tt;
+            cc[CC_TH] = k.th; cc[CC_OM] = k.om; cc[CC_H] = k.h;
+            cc[CC_TN] = d.t[n - 1];
+            // Terms below 2^-126 flush to zero in the FP32 path; rows whose rate is
+            // within 1e9 x (n such terms) of that are recomputed in FP64.
+            cc[CC_FLAGTHR] = 1e9 * (double)n * 1.1754943508222875e-38 * (k.mu * k.cB + k.th * k.cE);
+            // A background term is exactly 0 in FP32 (flush to zero) when its
+            // base-2 exponent dt~^2 + r~^2 exceeds 126; an excitation term when
+            // omega~ dt~ + beta r~^2 - ce exceeds 126.  With 2 units of margin, a
+            // tile whose smallest scaled time gap exceeds both bounds contributes
+            // exactly nothing.
+            const double cemax = model1 ? 0.0 : static_cast<double>(__int_as_float(ctr[CT_CEMAX]));
+            cc[CC_SKIPDTB] = skip ? sqrt(128.0) : 0.0;
+            cc[CC_SKIPDT] = skip ? fmax(sqrt(128.0), (cemax + 128.0) / k.omt) : 0.0;
+            cc[CC_VALID] = k.valid ? 1.0 : 0.0;
+            cc[CC_CEMAX] = cemax;
+            cc[CC_BGT] = bgt ? 1.0 : 0.0;
+            cc[CC_LLONLY] = (model & HAWKES_LOGLIK_ONLY) ? 1.0 : 0.0;
+            for (int q = 0; q < 7; ++q) cc[CC_FTHR + q] = -1.0;
+            // coefficients of the row finalisation (see row_eval)
+            const double LB = k.mu * k.cB, LE = k.th * k.cE;
+            const double itx = k.itx, itt = k.itt, iom = k.iom, ih = k.ih;
+            const double itx3 = itx * itx * itx, itt3 = itt * itt * itt, ih3 = ih * ih * ih;
+            cc[CC_LB] = LB;
+            cc[CC_LE] = LE;
+            cc[CC_A1] = LB * itx3; cc[CC_B1] = 2.0 * LB * itx;
+            cc[CC_A2] = LB * itt3; cc[CC_B2] = LB * itt;
+            cc[CC_A4] = LE * iom;
+            cc[CC_A5] = LE * ih3; cc[CC_B5] = 2.0 * LE * ih;
+            cc[CC_ITT] = itt;
+            constexpr double F = 1.2e-38;  // 2^-126 = 1.1755e-38, with margin
+            cc[CC_F0 + 0] = k.cB * F;
+            cc[CC_F0 + 1] = LB * F * ((bgt ? 0.0 : 126.0 * k.sr * itx3) + 2.0 * itx);
+            cc[CC_F0 + 2] = LB * F * (126.0 * k.st * itt3 + itt);
+            cc[CC_F0 + 3] = k.cE * F;
+            cc[CC_F0 + 4] = LE * F * iom;
+            cc[CC_F0 + 5] = LE * F * ((cemax + 127.0) * k.seq * ih3 + 2.0 * ih);
+            cc[CC_F0 + 6] = LE * F;
+            ctr[CT_WORK] = 0;
+            ctr[CT_FIX] = 0;
+            ctr[CT_DONE] = 0;
+            ctr[CT_FDONE] = 0;
+            ctr[CT_RDONE] = 0;
+            for (int q = 0; q < FIX_DOUBLES; ++q) d.fix7[q] = 0.0;
+            if (!k.valid) set_error(ctr, HAWKES_ERR_ARG);
+        }
     }
-    const double beta0 = (k.tx * k.tx) / (k.h * k.h);
+    __syncthreads();
+    const double kx = s_kx, kt = s_kt, beta0 = s_beta0;
+    const uint64_t iteration = resample ? *d_iteration : 0;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < npad;
          e += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
-        for (int q = 0; q < 6; ++q) acc[q * npad + e] = 0.0;
+        for (int q = 0; q < 6; ++q) d.acc[q * npad + e] = 0.0;
+        double xe = 0.0, ye = 0.0;
+        if (e < n) {
+            if (resample) {
+                draw_location(d, e, iteration, xe, ye);
+                d.x[e] = xe;
+                d.y[e] = ye;
+            } else if (stage) {
+                xe = d.x[e];
+                ye = d.y[e];
+            }
+        }
         if (!stage) continue;
         float nt, nxh, nxl, nyh, nyl, nb, ce;
         if (e < n) {
-            const double tt = (t[e] - tb[e / TB]) * k.kt;
-            const double xs = x[e] * k.kx, ys = y[e] * k.kx;
+            const double tt = (d.t[e] - d.tb[e / TB]) * kt;
+            const double xs = xe * kx, ys = ye * kx;
             const float xh = static_cast<float>(xs), yh = static_cast<float>(ys);
-            const double se = model1 ? 1.0 : s[e];
             nt = -static_cast<float>(tt);
             nxh = -xh;
             nyh = -yh;
             nxl = -static_cast<float>(xs - static_cast<double>(xh));
             nyl = -static_cast<float>(ys - static_cast<double>(yh));
-            nb = -static_cast<float>(beta0 / (se * se));
-            ce = static_cast<float>(-2.0 * log2(se));
+            nb = -static_cast<float>(model1 ? beta0 : beta0 * d.is2[e]);
+            ce = model1 ? 0.f : d.ce[e];
         } else {
             nt = -PAD_T;
             nxh = nyh = nxl = nyl = 0.f;
             nb = 0.f;
             ce = 0.f;
         }
-        *rec_q(rec, e, 0) = make_float4(nt, nt, nxh, nxh);
-        *rec_q(rec, e, 1) = make_float4(nxl, nxl, nyh, nyh);
-        *rec_q(rec, e, 2) = make_float4(nyl, nyl, nb, nb);
-        *rec_q(rec, e, 3) = make_float4(ce, ce, 0.f, 0.f);
+        *rec_q(d.rec, e, 0) = make_float4(nt, nt, nxh, nxh);
+        *rec_q(d.rec, e, 1) = make_float4(nxl, nxl, nyh, nyh);
+        *rec_q(d.rec, e, 2) = make_float4(nyl, nyl, nb, nb);
+        *rec_q(d.rec, e, 3) = make_float4(ce, ce, 0.f, 0.f);
     }
 }
 
 // ---------------------------------------------------------------------------
 // Row finalisation: lambda_i, clip, Lambda_i and the gradient (FP64).
-// sums = SB, SBr, SBt, SE, SEt, SEq in natural units (unnormalised).
+// S = SB, SBr, SBt, SE, SEt, SEq of row i in natural units (unnormalised).
+//
+// FP64 arithmetic is the cost (1.7 lanes per clock and SM): the parameters'
+// quotients are formed once per call (k_prep), so a row needs one division,
+// one logarithm, the exponentials, and the normal CDF only near the ends of
+// the time range, where it is not 0 or 1 to the last bit: Phi(a) rounds to 1
+// for a > 8.5, and Phi(b) for b < -8.5 is below half an ulp of Phi(a) >= 1/2.
+// An exponential whose argument is below -746 is exactly 0.
+//
+// row_lambda: log lambda_i and the partials of log lambda_i.  With BOUND, b[7] receives a bound on what the FP32 sweep's flushed terms can
+// move in the row's outputs.  ex2.approx.ftz returns 0 for every term below
+// 2^-126, and a product below 2^-126 in an accumulation flushes too, so each
+// FP32 moment sum of row i lacks a nonnegative part that is at most (per
+// source, natural units):
+//   SB  : F                         SE  : F
+//   SBr : F 126 / a_x               SEt : F max(t_i - t_1, 1 / sqrt(a_t))
+//   SBt : F 126 / a_t               SEq : F (ce_max + 127) 2 h^2 / log2(e)
+// with F = 2^-126 (plus margin for the approximation), summed over the row's
+// nb background sources (t_j != t_i) and ne excitation sources (t_j < t_i).
+// The r^2 and dt^2 factors follow from 2^-a a <= 126 2^-126 for a >= 126; the
+// excitation's from 2^g (ce_max - g) <= 2^-126 (ce_max + 126) for g <= -126.
+// The row's outputs are N_k / lambda with N_k linear in the moments, so each
+// output moves by at most (|dN_k| + |N_k| dlambda / lambda) / lambda, and the
+// log-likelihood by dlambda / lambda.  A clipped row whose true rate could
+// reach the clip gets an infinite bound.
 // ---------------------------------------------------------------------------
-__device__ void row_terms(const double* sums, double ti, const double* __restrict__ cc,
-                          double out[9]) {
-    const double mu = cc[CC_MU], tx = cc[CC_TX], tt = cc[CC_TT];
-    const double th = cc[CC_TH], om = cc[CC_OM], h = cc[CC_H];
-    const double cB = cc[CC_CB], cE = cc[CC_CE], tN = cc[CC_TN];
-    const double SB = cB * sums[0], SBr = cB * sums[1], SBt = cB * sums[2];
-    const double SE = cE * sums[3], SEt = cE * sums[4], SEq = cE * sums[5];
-    const double lam = mu * SB + th * SE;
-    double d[6] = {0, 0, 0, 0, 0, 0};
-    double loglam;
-    if (cc[CC_LLONLY] != 0.0) {  // the sweep formed SB and SE only: no gradient
-        loglam = lam < CLIP ? log(CLIP) : log(lam);
-        const double a = (tN - ti) / tt, b = -ti / tt;
-        const double Lam = mu * (normcdf(a) - normcdf(b)) + th * (1.0 - exp(-om * (tN - ti)));
-        out[0] = loglam - Lam;
-        for (int q = 1; q < 7; ++q) out[q] = CUDART_NAN;
-        out[7] = loglam;
-        out[8] = Lam;
-        return;
-    }
+template <bool BOUND>
+__device__ __forceinline__ void row_lambda(const double* S, double ti, double t1, double nb, double ne,
+                                           const double* __restrict__ cc, double& loglam, double d[6],
+                                           double b[7]) {
+    const double lam = cc[CC_LB] * S[0] + cc[CC_LE] * S[3];
+    for (int q = 0; q < 6; ++q) d[q] = 0.0;
+    const double dlam = BOUND ? cc[CC_MU] * cc[CC_F0] * nb + cc[CC_F0 + 6] * ne : 0.0;
     if (lam < CLIP) {
         loglam = log(CLIP);
+        if (BOUND)
+            for (int q = 0; q < 7; ++q) b[q] = (lam + dlam >= CLIP) ? CUDART_INF : 0.0;
     } else {
         loglam = log(lam);
         const double il = 1.0 / lam;
-        d[0] = SB * il;
-        d[1] = mu * (SBr / (tx * tx * tx) - 2.0 * SB / tx) * il;
-        d[2] = mu * (SBt / (tt * tt * tt) - SB / tt) * il;
-        d[3] = SE * il;
-        d[4] = th * (SE / om - SEt) * il;
-        d[5] = th * (SEq / (h * h * h) - 2.0 * SE / h) * il;
+        d[0] = cc[CC_CB] * S[0] * il;
+        d[1] = (cc[CC_A1] * S[1] - cc[CC_B1] * S[0]) * il;
+        d[2] = (cc[CC_A2] * S[2] - cc[CC_B2] * S[0]) * il;
+        d[3] = cc[CC_CE] * S[3] * il;
+        d[4] = (cc[CC_A4] * S[3] - cc[CC_LE] * S[4]) * il;
+        d[5] = (cc[CC_A5] * S[5] - cc[CC_B5] * S[3]) * il;
+        if (BOUND) {
+            const double r = dlam * il, nbl = nb * il, nel = ne * il;
+            b[0] = r;
+            b[1] = cc[CC_F0] * nbl + fabs(d[0]) * r;
+            b[2] = cc[CC_F0 + 1] * nbl + fabs(d[1]) * r;
+            b[3] = cc[CC_F0 + 2] * nbl + fabs(d[2]) * r;
+            b[4] = cc[CC_F0 + 3] * nel + fabs(d[3]) * r;
+            b[5] = (cc[CC_F0 + 4] + cc[CC_F0 + 6] * fmax(ti - t1, cc[CC_SET])) * nel + fabs(d[4]) * r;
+            b[6] = cc[CC_F0 + 5] * nel + fabs(d[5]) * r;
+        }
     }
-    const double a = (tN - ti) / tt, b = -ti / tt;
-    const double Pa = normcdf(a), Pb = normcdf(b);
-    const double pa = exp(-0.5 * a * a) * 0.3989422804014327;
-    const double pb = exp(-0.5 * b * b) * 0.3989422804014327;
-    const double ea = exp(-om * (tN - ti));
-    const double Lam = mu * (Pa - Pb) + th * (1.0 - ea);
-    out[0] = loglam - Lam;
+    if (cc[CC_LLONLY] != 0.0)  // the sweep formed SB and SE only: no gradient
+        for (int q = 0; q < 6; ++q) d[q] = CUDART_NAN;
+}
+
+// Lambda_i's three parts (Sec. 2.1) and their derivatives: the Gaussian end
+// terms z = Phi(a), w = phi(a) a for a = (t_N - t_i)/tau_t (upper) or
+// -t_i/tau_t (lower), and the exponential e^{-omega (t_N - t_i)}.
+__device__ __forceinline__ void lambda_upper(double ti, const double* __restrict__ cc, double& z, double& w) {
+    const double a = (cc[CC_TN] - ti) * cc[CC_ITT], x = 0.5 * a * a;
+    z = a > 8.5 ? 1.0 : normcdf(a);
+    w = x > 746.0 ? 0.0 : exp(-x) * 0.3989422804014327 * a;
+}
+__device__ __forceinline__ void lambda_lower(double ti, const double* __restrict__ cc, double& z, double& w) {
+    const double b = -ti * cc[CC_ITT], x = 0.5 * b * b;
+    z = b < -8.5 ? 0.0 : normcdf(b);
+    w = x > 746.0 ? 0.0 : exp(-x) * 0.3989422804014327 * b;
+}
+__device__ __forceinline__ double lambda_exp(double ti, const double* __restrict__ cc, double& gap) {
+    gap = cc[CC_TN] - ti;
+    const double x = cc[CC_OM] * gap;
+    return x > 746.0 ? 0.0 : exp(-x);
+}
+
+// A whole row: ell_i, its six partials, log lambda_i, Lambda_i.
+template <bool BOUND>
+__device__ __forceinline__ void row_eval(const double* S, double ti, double t1, double nb, double ne,
+                                         const double* __restrict__ cc, double out[9], double b[7]) {
+    double d[6], Pa, Pb, wa, wb, gap;
+    row_lambda<BOUND>(S, ti, t1, nb, ne, cc, out[7], d, b);
+    lambda_upper(ti, cc, Pa, wa);
+    lambda_lower(ti, cc, Pb, wb);
+    const double ea = lambda_exp(ti, cc, gap);
+    const double mu = cc[CC_MU], th = cc[CC_TH];
+    out[8] = mu * (Pa - Pb) + th * (1.0 - ea);
+    out[0] = out[7] - out[8];
     out[1] = d[0] - (Pa - Pb);
     out[2] = d[1];
-    out[3] = d[2] - mu * (-pa * a + pb * b) / tt;
+    out[3] = d[2] - mu * (wb - wa) * cc[CC_ITT];
     out[4] = d[3] - (1.0 - ea);
-    out[5] = d[4] - th * (tN - ti) * ea;
+    out[5] = d[4] - th * gap * ea;
     out[6] = d[5];
-    out[7] = loglam;
-    out[8] = Lam;
 }
 
 template <int NV>
@@ -243,120 +376,198 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NV], double* dst)
     }
 }
 
-// ---------------------------------------------------------------------------
-// Bound on what the FP32 sweep's flushed terms can move in a row.
-//
-// ex2.approx.ftz returns 0 for every term below 2^-126, and a product below
-// 2^-126 in an accumulation flushes too, so each FP32 moment sum of row i
-// lacks a nonnegative part that is at most (per source, natural units):
-//   SB  : F                         SE  : F
-//   SBr : F 126 / a_x               SEt : F max(t_i - t_1, 1 / sqrt(a_t))
-//   SBt : F 126 / a_t               SEq : F (ce_max + 127) 2 h^2 / log2(e)
-// with F = 2^-126 (plus margin for the approximation), summed over the row's
-// background sources (t_j != t_i) and excitation sources (t_j < t_i).  The
-// r^2 and dt^2 factors follow from 2^-a a <= 126 2^-126 for a >= 126; the
-// excitation's from 2^g (ce_max - g) <= 2^-126 (ce_max + 126) for g <= -126.
-// The row's outputs are N_k / lambda with N_k linear in the moments, so each
-// output moves by at most (|dN_k| + |N_k| dlambda / lambda) / lambda, and the
-// log-likelihood by dlambda / lambda.  A clipped row whose true rate could
-// reach the clip gets an infinite bound.
-// ---------------------------------------------------------------------------
-__device__ void row_flush_bound(const double* sums, double ti, double t1, int64_t nb, int64_t ne,
-                                const double* __restrict__ cc, double b[7]) {
-    constexpr double F = 1.2e-38;  // 2^-126 = 1.1755e-38, with margin
-    const double mu = cc[CC_MU], tx = cc[CC_TX], tt = cc[CC_TT];
-    const double th = cc[CC_TH], om = cc[CC_OM], h = cc[CC_H];
-    const double cB = cc[CC_CB], cE = cc[CC_CE];
-    const double fb = F * static_cast<double>(nb), fe = F * static_cast<double>(ne);
-    const double DB = cB * fb;
-    const double DBr = cc[CC_BGT] != 0.0 ? 0.0 : cB * fb * 126.0 * cc[CC_SR];
-    const double DBt = cB * fb * 126.0 * cc[CC_ST];
-    const double DE = cE * fe;
-    const double DEt = cE * fe * fmax(ti - t1, cc[CC_SET]);
-    const double DEq = cE * fe * (cc[CC_CEMAX] + 127.0) * cc[CC_SEQ];
-    const double SB = cB * sums[0], SBr = cB * sums[1], SBt = cB * sums[2];
-    const double SE = cE * sums[3], SEt = cE * sums[4], SEq = cE * sums[5];
-    const double lam = mu * SB + th * SE, dlam = mu * DB + th * DE;
-    if (lam < CLIP) {
-        const double inf = CUDART_INF;
-        for (int q = 0; q < 7; ++q) b[q] = (lam + dlam >= CLIP) ? inf : 0.0;
-        return;
+// Sums of 16 values over a warp with 16 FP64 additions per lane instead of 80:
+// each exchange halves the values a lane still carries.  Lane l returns the
+// total of value l >> 1.
+__device__ __forceinline__ double warp_sum16(double (&v)[16]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 8, m = 16; h >= 1; h >>= 1, m >>= 1) {
+        const bool up = (lane & m) != 0;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const double keep = up ? v[k + h] : v[k], send = up ? v[k] : v[k + h];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+        }
     }
-    const double il = 1.0 / lam, r = dlam * il;
-    const double N[6] = {SB, mu * (SBr / (tx * tx * tx) - 2.0 * SB / tx),
-                         mu * (SBt / (tt * tt * tt) - SB / tt), SE, th * (SE / om - SEt),
-                         th * (SEq / (h * h * h) - 2.0 * SE / h)};
-    const double dN[6] = {DB, mu * (DBr / (tx * tx * tx) + 2.0 * DB / tx),
-                          mu * (DBt / (tt * tt * tt) + DB / tt), DE, th * (DE / om + DEt),
-                          th * (DEq / (h * h * h) + 2.0 * DE / h)};
-    b[0] = r;
-    for (int q = 0; q < 6; ++q) b[1 + q] = (dN[q] + fabs(N[q]) * r) * il;
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-// Finalise rows [rb, re).  With `check` (FP32 sweep), rows whose rate could be
-// moved by FP32 underflow are queued for FP64 recomputation instead, and each
-// block's partials also carry the summed flush bounds of its other rows.
-__global__ void k_finalize(const double* __restrict__ acc, const double* __restrict__ t,
-                           const int32_t* __restrict__ lo, const int32_t* __restrict__ hi,
-                           const double* __restrict__ cc, int64_t n, int64_t npad, int64_t rb,
-                           int64_t re, int check, int* fixlist, int* ctr, double* partials,
-                           double* rows9) {
-    double v[14] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+// The 7 outputs from the totals tot[14] over all rows (outputs, flush bounds)
+// and the FP64-recomputed rows' sums; called by one whole block.  The summed
+// flush bounds of the FP32 sweep (zero on the FP64 path) decide, per output,
+// whether rows must be recomputed by k_flushfix: when an output's bound exceeds
+// FLUSH_TAU of its magnitude, every row whose own bound is above FLUSH_TAU
+// |output| / nrows is, so the rows left in FP32 can move it by at most
+// FLUSH_TAU of its magnitude.
+__device__ __forceinline__ void finish_outputs(const double* tot, const volatile double* fix7,
+                                               double* cc, int64_t nrows, double* out, int* ctr) {
+    const int q = threadIdx.x;
+    if (q < 7) {
+        const bool valid = cc[CC_VALID] != 0.0, llonly = cc[CC_LLONLY] != 0.0;
+        const double r = valid ? tot[q] + fix7[q] : CUDART_NAN;
+        out[q] = r;
+        const double g = fabs(r), bound = tot[7 + q];
+        const bool used = valid && (q == 0 || !llonly);
+        if (used && !isfinite(r)) set_error(ctr, HAWKES_ERR_NONFINITE);
+        cc[CC_FTHR + q] = (used && bound > FLUSH_TAU * g)
+                              ? FLUSH_TAU * g / static_cast<double>(nrows > 0 ? nrows : 1)
+                              : -1.0;
+    }
+}
+
+// Finalise rows [rb, re) (batches: all rows).  With `check` (FP32 sweep), the
+// lambda terms of rows whose rate could be moved by FP32 underflow are left
+// out and the rows queued for FP64 recomputation, and each block's partials
+// also carry the summed flush bounds of its other rows.  The last block to
+// finish adds the blocks' partials in a fixed order and writes the 7 outputs
+// to out (7 per problem), unless rows were queued: then it keeps the totals for
+// k_rows64's last block.
+//
+// Without per-row outputs (ROWS false) four warps share 32 rows, each forming
+// one additive part of their sums: the lambda terms, the two Gaussian end
+// terms and the exponential of Lambda.  A warp's chain of FP64 instructions is
+// then a third as long, which is what few rows wait for (N = 2,000: 57 us as
+// 8 blocks of 256 whole rows, 19.5 in blocks of 64); many rows are bound by
+// the FP64 rate either way.
+// err_out (optional): receives the latched error status as a double.
+template <bool ROWS>
+__global__ void __launch_bounds__(FINAL_THREADS)
+    k_finalize(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs, int64_t rb,
+               int64_t re, int check, double* out, double* rows9, double* err_out) {
+    const EvalDesc& d = probs ? probs[blockIdx.y] : one;
+    if (probs) {
+        rb = 0;
+        re = d.n;
+        out += 7 * blockIdx.y;
+    }
+    const int64_t n = d.n, npad = d.npad;
+    double* cc = d.cc;
+    int* ctr = d.ctr;
+    double v[16] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     const bool valid = cc[CC_VALID] != 0.0;
-    const double thr = cc[CC_FLAGTHR];
-    const double mu = cc[CC_MU], th = cc[CC_TH], cB = cc[CC_CB], cE = cc[CC_CE];
-    const double t1 = t[0];
-    for (int64_t i = rb + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; valid && i < re;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        double sums[6];
+    const double thr = cc[CC_FLAGTHR], LB = cc[CC_LB], LE = cc[CC_LE];
+    const double t1 = d.t[0];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int SPAN = ROWS ? FINAL_THREADS : FINAL_THREADS / 4;  // rows per block and step
+    const int part = ROWS ? 0 : warp & 3;
+    for (int64_t i = rb + static_cast<int64_t>(blockIdx.x) * SPAN + (ROWS ? tid : (warp >> 2) * 32 + lane);
+         valid && i < re; i += static_cast<int64_t>(gridDim.x) * SPAN) {
+        const double ti = d.t[i], mu = cc[CC_MU], th = cc[CC_TH];
+        if (part == 0) {
+            double S[6];
 #pragma unroll
-        for (int q = 0; q < 6; ++q) sums[q] = acc[q * npad + i];
-        if (check) {
-            const double lam = mu * cB * sums[0] + th * cE * sums[3];
-            if (lam < thr) {
+            for (int q = 0; q < 6; ++q) S[q] = d.acc[q * npad + i];
+            const bool queue = check && LB * S[0] + LE * S[3] < thr;
+            if (queue) {
                 const int k = atomicAdd(ctr + CT_FIX, 1);
-                if (kDebug && !(k >= 0 && k < npad)) {
+                if (kDebug && !(k >= 0 && k < npad))
                     set_error(ctr, HAWKES_ERR_BOUNDS);
-                    continue;
+                else
+                    d.fixlist[k] = static_cast<int>(i);
+            } else {
+                double loglam, dl[6], bd[7] = {0, 0, 0, 0, 0, 0, 0};
+                if (check) {
+                    const int64_t l = d.lo[i];
+                    row_lambda<true>(S, ti, t1, static_cast<double>(l + (n - d.hi[i])),
+                                     static_cast<double>(l), cc, loglam, dl, bd);
+                } else {
+                    row_lambda<false>(S, ti, t1, 0.0, 0.0, cc, loglam, dl, bd);
                 }
-                fixlist[k] = static_cast<int>(i);
-                continue;
+                v[0] += loglam;
+#pragma unroll
+                for (int q = 0; q < 6; ++q) v[1 + q] += dl[q];
+                if (check)
+#pragma unroll
+                    for (int q = 0; q < 7; ++q) v[7 + q] += bd[q];
+            }
+            if (ROWS && !queue) {  // queued rows are written by k_rows64
+                double o[9], b[7];
+                row_eval<false>(S, ti, t1, 0.0, 0.0, cc, o, b);
+                for (int q = 0; q < 9; ++q) rows9[9 * i + q] = o[q];
             }
         }
-        double o[9];
-        row_terms(sums, t[i], cc, o);
-#pragma unroll
-        for (int q = 0; q < 7; ++q) v[q] += o[q];
-        if (check) {
-            double bd[7];
-            const int64_t l = lo[i];
-            row_flush_bound(sums, t[i], t1, l + (n - hi[i]), l, cc, bd);
-#pragma unroll
-            for (int q = 0; q < 7; ++q) v[7 + q] += bd[q];
+        if (ROWS || part == 1) {
+            double z, w;
+            lambda_upper(ti, cc, z, w);
+            v[0] -= mu * z;
+            v[1] -= z;
+            v[3] += mu * w * cc[CC_ITT];
         }
-        if (rows9)
-            for (int q = 0; q < 9; ++q) rows9[9 * i + q] = o[q];
+        if (ROWS || part == 2) {
+            double z, w;
+            lambda_lower(ti, cc, z, w);
+            v[0] += mu * z;
+            v[1] += z;
+            v[3] -= mu * w * cc[CC_ITT];
+        }
+        if (ROWS || part == 3) {
+            double gap;
+            const double ea = lambda_exp(ti, cc, gap);
+            v[0] -= th * (1.0 - ea);
+            v[4] -= 1.0 - ea;
+            v[5] -= th * gap * ea;
+        }
     }
-    block_reduce_store<14>(v, partials + PART_STRIDE * blockIdx.x);
+    constexpr int NW = FINAL_THREADS / 32;
+    __shared__ double red[NW][16];  // per warp; then the totals in red[0]
+    __shared__ bool s_last;
+    const double w = warp_sum16(v);
+    if ((lane & 1) == 0) red[warp][lane >> 1] = w;
+    __syncthreads();
+    if (tid < 16) {
+        double u = red[0][tid];
+        for (int k = 1; k < NW; ++k) u += red[k][tid];
+        d.partials[PART_STRIDE * blockIdx.x + tid] = u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(ctr + CT_FDONE, 1) == static_cast<int>(gridDim.x) - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // last block: value tid & 15, every (FINAL_THREADS / 16)-th partial
+    const int parts = gridDim.x;
+    double u = 0.0;
+    for (int b = tid >> 4; b < parts; b += FINAL_THREADS / 16) u += __ldcg(d.partials + PART_STRIDE * b + (tid & 15));
+    u += __shfl_xor_sync(0xffffffffu, u, 16);
+    if (lane < 16) red[warp][lane] = u;
+    __syncthreads();
+    if (tid < 16) {
+        double s = red[0][tid];
+        for (int k = 1; k < NW; ++k) s += red[k][tid];
+        red[0][tid] = s;
+    }
+    __syncthreads();
+    const bool queued = valid && *static_cast<volatile int*>(ctr + CT_FIX) > 0;
+    if (queued) {
+        if (tid < 16) d.fix7[16 + tid] = red[0][tid];
+        return;
+    }
+    finish_outputs(red[0], d.fix7, cc, re - rb, out, ctr);
+    __syncthreads();
+    if (err_out && tid == 0) *err_out = static_cast<double>(*static_cast<volatile int*>(ctr + CT_ERR));
+}
+
+void launch_finalize(cudaStream_t st, dim3 grid, const EvalDesc& one, const EvalDesc* probs, int64_t rb,
+                     int64_t re, int check, double* out, double* rows9, double* err_out) {
+    if (rows9)
+        k_finalize<true><<<grid, FINAL_THREADS, 0, st>>>(one, probs, rb, re, check, out, rows9, err_out);
+    else
+        k_finalize<false><<<grid, FINAL_THREADS, 0, st>>>(one, probs, rb, re, check, out, rows9, err_out);
 }
 
 // This thread's share (sources j = threadIdx.x + k blockDim.x) of row i's six
 // FP64 moment sums, in natural units: the pair terms of eqs. 2-3 written out.
 // ix2 = 1/(2 tau_x^2) (0 for the time-only background), it2 = 1/(2 tau_t^2),
 // ih2 = 1/(2 h^2).
-__device__ __forceinline__ void row_sums64(int64_t i, const double* __restrict__ t,
-                                           const double* __restrict__ x,
-                                           const double* __restrict__ y,
-                                           const double* __restrict__ s,
-                                           const int32_t* __restrict__ lo,
-                                           const int32_t* __restrict__ hi, bool model1, int64_t n,
-                                           double ix2, double it2, double ih2, double om,
-                                           double v[6]) {
-    const double ti = t[i], xi = x[i], yi = y[i];
-    const int64_t li = lo[i], hj = hi[i];
+__device__ __forceinline__ void row_sums64(const EvalDesc& d, int64_t i, bool model1, double ix2,
+                                           double it2, double ih2, double om, double v[6]) {
+    const double ti = d.t[i], xi = d.x[i], yi = d.y[i];
+    const int64_t li = d.lo[i], hj = d.hi[i];
     for (int q = 0; q < 6; ++q) v[q] = 0.0;
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-        const double dt = ti - t[j], dx = xi - x[j], dy = yi - y[j];
+    for (int64_t j = threadIdx.x; j < d.n; j += blockDim.x) {
+        const double dt = ti - d.t[j], dx = xi - d.x[j], dy = yi - d.y[j];
         const double r2 = dx * dx + dy * dy;
         if (j < li || j >= hj) {
             const double b = exp(-r2 * ix2 - dt * dt * it2);
@@ -365,8 +576,7 @@ __device__ __forceinline__ void row_sums64(int64_t i, const double* __restrict__
             v[2] += b * dt * dt;
         }
         if (j < li) {
-            const double sj = model1 ? 1.0 : s[j];
-            const double is2 = 1.0 / (sj * sj);
+            const double is2 = model1 ? 1.0 : d.is2[j];
             const double e = is2 * exp(-om * dt - r2 * ih2 * is2);
             v[3] += e;
             v[4] += e * dt;
@@ -378,107 +588,98 @@ __device__ __forceinline__ void row_sums64(int64_t i, const double* __restrict__
 // ---------------------------------------------------------------------------
 // FP64 pair rows: one CTA per row, threads stride over all sources.
 // mode 0: rows row_begin + [0, count) -> write natural-unit sums to acc
-// mode 1: rows fixlist[0 .. ctr[CT_FIX]) -> finalise and add into fix7
+// mode 1: the queued rows fixlist[0 .. ctr[CT_FIX]) -> finalise, add into fix7;
+//         the last block then writes the outputs (see k_finalize).  Returns at
+//         once when no row is queued.
 // ---------------------------------------------------------------------------
-__global__ void k_rows64(const double* __restrict__ t, const double* __restrict__ x,
-                         const double* __restrict__ y, const double* __restrict__ s,
-                         const int32_t* __restrict__ lo, const int32_t* __restrict__ hi,
-                         const double* __restrict__ cc, int model, int64_t n, int64_t npad,
-                         int64_t row_begin, int64_t count, int mode, const int* fixlist, int* ctr,
-                         double* acc, double* fix7, double* rows9) {
-    if (cc[CC_VALID] == 0.0) return;
+__global__ void k_rows64(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs,
+                         int model, int64_t row_begin, int64_t count, int mode, double* out,
+                         double* rows9) {
+    const EvalDesc& d = probs ? probs[blockIdx.y] : one;
+    const int64_t n = d.n, npad = d.npad;
+    double* cc = d.cc;
+    int* ctr = d.ctr;
+    const int64_t total = mode ? static_cast<int64_t>(ctr[CT_FIX]) : count;
+    if (cc[CC_VALID] == 0.0 || total == 0) return;
     const bool model1 = (model & HAWKES_MODEL1) != 0;
     const double tx = cc[CC_TX], tt = cc[CC_TT], om = cc[CC_OM], h = cc[CC_H];
     // Time-only background: no spatial factor in B and no r^2 moment.
     const double ix2 = (model & HAWKES_BG_TIME) ? 0.0 : 1.0 / (2.0 * tx * tx);
     const double it2 = 1.0 / (2.0 * tt * tt), ih2 = 1.0 / (2.0 * h * h);
-    const int64_t total = mode ? static_cast<int64_t>(ctr[CT_FIX]) : count;
+    __shared__ double sums[8];
     for (int64_t k = blockIdx.x; k < total; k += gridDim.x) {
-        const int64_t i = mode ? fixlist[k] : row_begin + k;
+        const int64_t i = mode ? d.fixlist[k] : row_begin + k;
         if (kDebug && !(i >= 0 && i < n && (mode || k < npad))) {
             if (threadIdx.x == 0) set_error(ctr, HAWKES_ERR_BOUNDS);
             continue;  // uniform over the block: i depends on k only
         }
-        const double ti = t[i];
         double v[6];
-        row_sums64(i, t, x, y, s, lo, hi, model1, n, ix2, it2, ih2, om, v);
-        __shared__ double sums[8];
+        row_sums64(d, i, model1, ix2, it2, ih2, om, v);
         block_reduce_store<6>(v, sums);
         __syncthreads();
         if (threadIdx.x == 0) {
             if (mode == 0) {
-                for (int q = 0; q < 6; ++q) acc[q * npad + i] = sums[q];
+                for (int q = 0; q < 6; ++q) d.acc[q * npad + i] = sums[q];
             } else {
-                double o[9];
-                row_terms(sums, ti, cc, o);
-                for (int q = 0; q < 7; ++q) atomicAdd(fix7 + q, o[q]);
-                if (rows9)
+                // (k_finalize has the row's Lambda terms)
+                double o[9], b[7], loglam, dl[6];
+                row_lambda<false>(sums, d.t[i], 0.0, 0.0, 0.0, cc, loglam, dl, b);
+                atomicAdd(d.fix7, loglam);
+                for (int q = 0; q < 6; ++q) atomicAdd(d.fix7 + 1 + q, dl[q]);
+                if (rows9) {
+                    row_eval<false>(sums, d.t[i], 0.0, 0.0, 0.0, cc, o, b);
                     for (int q = 0; q < 9; ++q) rows9[9 * i + q] = o[q];
+                }
             }
         }
         __syncthreads();
     }
-}
-
-// Sum the per-block partials in a fixed order, add the FP64-recomputed rows,
-// write the 7 outputs.  One CTA.  The summed flush bounds of the FP32 sweep
-// (zero on the FP64 path) decide, per output, whether rows must be recomputed
-// by k_flushfix: when an output's bound exceeds FLUSH_TAU of its magnitude,
-// every row whose own bound exceeds FLUSH_TAU |output| / nrows is, so the rows
-// left in FP32 can move it by at most FLUSH_TAU of its magnitude.
-__global__ void k_reduce(const double* __restrict__ partials, int nparts,
-                         const double* __restrict__ fix7, double* __restrict__ cc, int64_t nrows,
-                         double* out, int* ctr) {
-    double v[14] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int b = threadIdx.x; b < nparts; b += blockDim.x)
-        for (int q = 0; q < 14; ++q) v[q] += partials[PART_STRIDE * b + q];
-    __shared__ double tot[16];
-    block_reduce_store<14>(v, tot);
-    __syncthreads();
+    if (mode == 0) return;
+    __shared__ bool s_last;
     if (threadIdx.x == 0) {
-        const bool valid = cc[CC_VALID] != 0.0;
-        const bool llonly = cc[CC_LLONLY] != 0.0;
-        bool finite = true;
-        for (int q = 0; q < 7; ++q) {
-            const double r = valid ? tot[q] + fix7[q] : CUDART_NAN;
-            if (q == 0 || !llonly) finite = finite && isfinite(r);
-            out[q] = r;
-            const double g = fabs(r), bound = tot[7 + q];
-            cc[CC_FTHR + q] = (valid && (q == 0 || !llonly) && bound > FLUSH_TAU * g)
-                                  ? FLUSH_TAU * g / static_cast<double>(nrows > 0 ? nrows : 1)
-                                  : -1.0;
-        }
-        if (valid && !finite) set_error(ctr, HAWKES_ERR_NONFINITE);
+        __threadfence();
+        s_last = atomicAdd(ctr + CT_RDONE, 1) == static_cast<int>(gridDim.x) - 1;
+        __threadfence();
     }
+    __syncthreads();
+    if (s_last) finish_outputs(d.fix7 + 16, d.fix7, cc, probs ? n : count, out + (probs ? 7 * blockIdx.y : 0), ctr);
 }
 
-// Recompute in FP64 the rows that k_reduce's thresholds select (a row whose
-// flush bound for some output exceeds that output's threshold; rows already
-// recomputed for their low rate are left out), replace their FP32 values by
-// the FP64 ones in the outputs, and write their per-row values.  Each block
-// takes 256-row chunks; the last block to finish adds the corrections to out.
-// Returns at once when no output needs it (the usual case).
-__global__ void k_flushfix(const double* __restrict__ acc, const double* __restrict__ t,
-                           const double* __restrict__ x, const double* __restrict__ y,
-                           const double* __restrict__ s, const int32_t* __restrict__ lo,
-                           const int32_t* __restrict__ hi, const double* __restrict__ cc,
-                           int model, int64_t n, int64_t npad, int64_t rb, int64_t re, int* ctr,
-                           double* fix7, double* out, double* rows9) {
-    if (cc[CC_VALID] == 0.0) return;
+// Recompute in FP64 the rows that the flush thresholds (finish_outputs) select
+// (a row whose flush bound for some output exceeds that output's threshold;
+// rows already recomputed for their low rate are left out), replace their FP32
+// values by the FP64 ones in the outputs, and write their per-row values.  Each
+// block takes 256-row chunks; the last block to finish adds the corrections to
+// out.  Returns at once when no output needs it (the usual case).
+// err_out (optional): receives the latched error status as a double.
+__global__ void k_flushfix(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs,
+                           int model, int64_t rb, int64_t re, double* out, double* rows9,
+                           double* err_out) {
+    const EvalDesc& d = probs ? probs[blockIdx.y] : one;
+    if (probs) {
+        rb = 0;
+        re = d.n;
+        out += 7 * blockIdx.y;
+    }
+    const int64_t n = d.n, npad = d.npad;
+    const double* cc = d.cc;
+    int* ctr = d.ctr;
     double thr[7];
     bool any = false;
     for (int q = 0; q < 7; ++q) {
         thr[q] = cc[CC_FTHR + q];
         any = any || thr[q] >= 0.0;
     }
-    if (!any) return;  // uniform over the grid
+    if (cc[CC_VALID] == 0.0 || !any) {  // uniform over the grid
+        if (err_out && blockIdx.x == 0 && threadIdx.x == 0) *err_out = static_cast<double>(ctr[CT_ERR]);
+        return;
+    }
     const bool model1 = (model & HAWKES_MODEL1) != 0;
     const double tx = cc[CC_TX], tt = cc[CC_TT], om = cc[CC_OM], h = cc[CC_H];
     const double ix2 = cc[CC_BGT] != 0.0 ? 0.0 : 1.0 / (2.0 * tx * tx);
     const double it2 = 1.0 / (2.0 * tt * tt), ih2 = 1.0 / (2.0 * h * h);
-    const double flagthr = cc[CC_FLAGTHR];
-    const double mu = cc[CC_MU], th = cc[CC_TH], cB = cc[CC_CB], cE = cc[CC_CE];
-    const double t1 = t[0];
+    const double flagthr = cc[CC_FLAGTHR], LB = cc[CC_LB], LE = cc[CC_LE];
+    const double t1 = d.t[0];
     __shared__ int list[256];
     __shared__ int cnt;
     __shared__ double sums[8];
@@ -490,12 +691,13 @@ __global__ void k_flushfix(const double* __restrict__ acc, const double* __restr
         __syncthreads();
         const int64_t i = base + threadIdx.x;
         if (threadIdx.x < 256 && i < re) {
-            double sm[6];
-            for (int q = 0; q < 6; ++q) sm[q] = acc[q * npad + i];
-            if (!(mu * cB * sm[0] + th * cE * sm[3] < flagthr)) {
-                double bd[7];
-                const int64_t l = lo[i];
-                row_flush_bound(sm, t[i], t1, l + (n - hi[i]), l, cc, bd);
+            double S[6];
+            for (int q = 0; q < 6; ++q) S[q] = d.acc[q * npad + i];
+            if (!(LB * S[0] + LE * S[3] < flagthr)) {
+                double loglam, dl[6], bd[7];
+                const int64_t l = d.lo[i];
+                row_lambda<true>(S, d.t[i], t1, static_cast<double>(l + (n - d.hi[i])),
+                                 static_cast<double>(l), cc, loglam, dl, bd);
                 bool f = false;
                 for (int q = 0; q < 7; ++q) f = f || (thr[q] >= 0.0 && bd[q] > thr[q]);
                 if (f) list[atomicAdd(&cnt, 1)] = threadIdx.x;
@@ -506,30 +708,34 @@ __global__ void k_flushfix(const double* __restrict__ acc, const double* __restr
         for (int k = 0; k < m; ++k) {
             const int64_t r = base + list[k];
             double v[6];
-            row_sums64(r, t, x, y, s, lo, hi, model1, n, ix2, it2, ih2, om, v);
+            row_sums64(d, r, model1, ix2, it2, ih2, om, v);
             block_reduce_store<6>(v, sums);
             if (threadIdx.x == 0) {
-                double s32[6], o64[9], o32[9];
-                for (int q = 0; q < 6; ++q) s32[q] = acc[q * npad + r];
-                row_terms(sums, t[r], cc, o64);
-                row_terms(s32, t[r], cc, o32);
-                for (int q = 0; q < 7; ++q) mine[q] += o64[q] - o32[q];
-                if (rows9)
+                double s32[6], d64[6], d32[6], l64, l32, b[7];
+                for (int q = 0; q < 6; ++q) s32[q] = d.acc[q * npad + r];
+                row_lambda<false>(sums, d.t[r], 0.0, 0.0, 0.0, cc, l64, d64, b);
+                row_lambda<false>(s32, d.t[r], 0.0, 0.0, 0.0, cc, l32, d32, b);
+                mine[0] += l64 - l32;
+                for (int q = 0; q < 6; ++q) mine[1 + q] += d64[q] - d32[q];
+                if (rows9) {
+                    double o64[9];
+                    row_eval<false>(sums, d.t[r], 0.0, 0.0, 0.0, cc, o64, b);
                     for (int q = 0; q < 9; ++q) rows9[9 * r + q] = o64[q];
+                }
             }
             __syncthreads();
         }
     }
     if (threadIdx.x == 0) {
         for (int q = 0; q < 7; ++q)
-            if (mine[q] != 0.0) atomicAdd(fix7 + 8 + q, mine[q]);
+            if (mine[q] != 0.0) atomicAdd(d.fix7 + 8 + q, mine[q]);
         __threadfence();
         last = atomicAdd(ctr + CT_DONE, 1) == static_cast<int>(gridDim.x) - 1;
     }
     __syncthreads();
     if (last && threadIdx.x == 0) {
         __threadfence();
-        const volatile double* fb = fix7 + 8;
+        const volatile double* fb = d.fix7 + 8;
         const bool llonly = cc[CC_LLONLY] != 0.0;
         bool finite = true;
         for (int q = 0; q < 7; ++q) {
@@ -538,6 +744,7 @@ __global__ void k_flushfix(const double* __restrict__ acc, const double* __restr
             if (q == 0 || !llonly) finite = finite && isfinite(r);
         }
         if (!finite) set_error(ctr, HAWKES_ERR_NONFINITE);
+        if (err_out) *err_out = static_cast<double>(*static_cast<volatile int*>(ctr + CT_ERR));
     }
 }
 
@@ -619,32 +826,35 @@ __device__ __forceinline__ double unit53(uint64_t w) {
     return __dmul_rn(static_cast<double>(w >> 11), 1.0 / 9007199254740992.0);
 }
 
-__global__ void k_resample(const int32_t* __restrict__ county, int64_t n,
-                           const double* __restrict__ tri_xy, const double* __restrict__ cum,
-                           const int32_t* __restrict__ first, const int32_t* __restrict__ last,
-                           uint64_t seed, uint64_t stream, uint64_t iteration,
-                           const uint64_t* d_iteration, double* x, double* y) {
-    if (d_iteration) iteration = *d_iteration;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+__device__ __forceinline__ void draw_location(const EvalDesc& d, int64_t i, uint64_t iteration,
+                                              double& x, double& y) {
+    const int32_t c = d.county[i];
+    uint64_t w[4] = {static_cast<uint64_t>(i), iteration, 0ull, 0ull};
+    philox4x64_10(w, d.seed, d.stream);
+    const double u0 = unit53(w[0]), u1 = unit53(w[1]), u2 = unit53(w[2]);
+    int32_t a = d.cfirst[c], b = d.clast[c];
+    const double target = __dmul_rn(u0, d.tri_cum[b]);
+    // first k in [a, b] with target < cum[k]; b if there is none
+    while (a < b) {
+        const int32_t mid = (a + b) >> 1;
+        if (target < d.tri_cum[mid]) b = mid; else a = mid + 1;
+    }
+    const double* v = d.tri_xy + 6 * (int64_t)a;
+    const double r1 = __dsqrt_rn(u1);
+    const double w0 = __dsub_rn(1.0, r1);
+    const double w1 = __dmul_rn(r1, __dsub_rn(1.0, u2));
+    const double w2 = __dmul_rn(r1, u2);
+    x = __dadd_rn(__dadd_rn(__dmul_rn(w0, v[0]), __dmul_rn(w1, v[2])), __dmul_rn(w2, v[4]));
+    y = __dadd_rn(__dadd_rn(__dmul_rn(w0, v[1]), __dmul_rn(w1, v[3])), __dmul_rn(w2, v[5]));
+}
+
+__global__ void k_resample(const __grid_constant__ EvalDesc d, uint64_t iteration) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d.n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t c = county[i];
-        uint64_t w[4] = {static_cast<uint64_t>(i), iteration, 0ull, 0ull};
-        philox4x64_10(w, seed, stream);
-        const double u0 = unit53(w[0]), u1 = unit53(w[1]), u2 = unit53(w[2]);
-        int32_t a = first[c], b = last[c];
-        const double target = __dmul_rn(u0, cum[b]);
-        // first k in [a, b] with target < cum[k]; b if there is none
-        while (a < b) {
-            const int32_t mid = (a + b) >> 1;
-            if (target < cum[mid]) b = mid; else a = mid + 1;
-        }
-        const double* v = tri_xy + 6 * (int64_t)a;
-        const double r1 = __dsqrt_rn(u1);
-        const double w0 = __dsub_rn(1.0, r1);
-        const double w1 = __dmul_rn(r1, __dsub_rn(1.0, u2));
-        const double w2 = __dmul_rn(r1, u2);
-        x[i] = __dadd_rn(__dadd_rn(__dmul_rn(w0, v[0]), __dmul_rn(w1, v[2])), __dmul_rn(w2, v[4]));
-        y[i] = __dadd_rn(__dadd_rn(__dmul_rn(w0, v[1]), __dmul_rn(w1, v[3])), __dmul_rn(w2, v[5]));
+        double x, y;
+        draw_location(d, i, iteration, x, y);
+        d.x[i] = x;
+        d.y[i] = y;
     }
 }
 

@@ -25,19 +25,15 @@
 #include "common.cuh"
 
 namespace hk {
-__global__ void k_prep(const double*, const double*, const double*, const double*, const double*,
-                       const hawkes_params*, int, int, int, int64_t, int64_t, Rec*, double*, double*,
-                       int*, double*);
-__global__ void k_finalize(const double*, const double*, const int32_t*, const int32_t*,
-                           const double*, int64_t, int64_t, int64_t, int64_t, int, int*, int*,
-                           double*, double*);
-__global__ void k_flushfix(const double*, const double*, const double*, const double*,
-                           const double*, const int32_t*, const int32_t*, const double*, int,
-                           int64_t, int64_t, int64_t, int64_t, int*, double*, double*, double*);
-__global__ void k_rows64(const double*, const double*, const double*, const double*,
-                         const int32_t*, const int32_t*, const double*, int, int64_t, int64_t,
-                         int64_t, int64_t, int, const int*, int*, double*, double*, double*);
-__global__ void k_reduce(const double*, int, const double*, double*, int64_t, double*, int*);
+__global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const hawkes_params*,
+                       const __grid_constant__ hawkes_params,
+                       int, int, int, int, const uint64_t*, int*);
+void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
+                     double*, double*, double*);
+__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, int, double*,
+                         double*);
+__global__ void k_flushfix(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, double*, double*,
+                           double*);
 cudaError_t sweep_setup_attributes();
 int sweep_blocks_per_sm(int v);
 int sweep_variant_rows(int v);
@@ -54,7 +50,7 @@ namespace {
 // Largest event count the fixed scratch holds (a multiple of NPAD_MULT).
 constexpr int64_t kMaxN = HAWKES_NOALLOC_MAX_N;
 static_assert(kMaxN % NPAD_MULT == 0, "scratch holds whole row tiles");
-constexpr int kMaxFinalBlocks = 512;
+constexpr int kMaxSms = 256;
 constexpr int kMaxItems = 16384;
 constexpr int kVariant = 0;  // sweep variant used by this entry point
 
@@ -64,14 +60,15 @@ constexpr size_t OFF_T = 0;
 constexpr size_t OFF_X = OFF_T + align256(kMaxN * sizeof(double));
 constexpr size_t OFF_Y = OFF_X + align256(kMaxN * sizeof(double));
 constexpr size_t OFF_S = OFF_Y + align256(kMaxN * sizeof(double));
-constexpr size_t OFF_LO = OFF_S + align256(kMaxN * sizeof(double));
+constexpr size_t OFF_CE = OFF_S + align256(kMaxN * sizeof(double));
+constexpr size_t OFF_LO = OFF_CE + align256(kMaxN * sizeof(float));
 constexpr size_t OFF_HI = OFF_LO + align256(kMaxN * sizeof(int32_t));
 constexpr size_t OFF_TB = OFF_HI + align256(kMaxN * sizeof(int32_t));
 constexpr size_t OFF_REC = OFF_TB + align256((kMaxN / TB) * sizeof(double));
 constexpr size_t OFF_ACC = OFF_REC + align256(kMaxN * sizeof(Rec));
 constexpr size_t OFF_FIX = OFF_ACC + align256(6 * kMaxN * sizeof(double));
 constexpr size_t OFF_PART = OFF_FIX + align256(kMaxN * sizeof(int));
-constexpr size_t OFF_FIX7 = OFF_PART + align256(PART_STRIDE * kMaxFinalBlocks * sizeof(double));
+constexpr size_t OFF_FIX7 = OFF_PART + align256(PART_STRIDE * BPSM * kMaxSms * sizeof(double));
 constexpr size_t OFF_CTR = OFF_FIX7 + align256(FIX_DOUBLES * sizeof(double));
 constexpr size_t OFF_CC = OFF_CTR + align256(CT_COUNT * sizeof(int));
 constexpr size_t OFF_ITEMS = OFF_CC + align256(CC_COUNT * sizeof(double));
@@ -93,8 +90,8 @@ std::mutex g_setup_mutex;
 // build the tie ranges and block time bases (same rules as hawkes_set_events).
 __global__ void k_na_setup(const double* __restrict__ t_in, const double* __restrict__ x_in,
                            const double* __restrict__ y_in, const double* __restrict__ s_in,
-                           int64_t n, int64_t npad, double* t, double* x, double* y, double* s,
-                           int32_t* lo, int32_t* hi, double* tb, int* ctr) {
+                           int64_t n, int64_t npad, double* t, double* x, double* y, double* is2,
+                           float* ces, int32_t* lo, int32_t* hi, double* tb, int* ctr) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < npad;
          e += (int64_t)gridDim.x * blockDim.x) {
         if (e < n) {
@@ -110,7 +107,8 @@ __global__ void k_na_setup(const double* __restrict__ t_in, const double* __rest
             t[e] = te;
             x[e] = x_in[e];
             y[e] = y_in[e];
-            s[e] = se;
+            is2[e] = 1.0 / (se * se);
+            ces[e] = ce;
             int64_t a = 0, b = n;  // first index with t >= te
             while (a < b) {
                 const int64_t m = (a + b) >> 1;
@@ -128,7 +126,8 @@ __global__ void k_na_setup(const double* __restrict__ t_in, const double* __rest
             t[e] = t_in[n - 1];
             x[e] = 0.0;
             y[e] = 0.0;
-            s[e] = 1.0;
+            is2[e] = 1.0;
+            ces[e] = 0.f;
             lo[e] = 0;
             hi[e] = 0;
         }
@@ -238,7 +237,8 @@ extern "C" int hawkes_loglik_grad_noalloc(const double* d_t, const double* d_x, 
     c.t = reinterpret_cast<double*>(base + OFF_T);
     c.x = reinterpret_cast<double*>(base + OFF_X);
     c.y = reinterpret_cast<double*>(base + OFF_Y);
-    c.s = reinterpret_cast<double*>(base + OFF_S);
+    c.is2 = reinterpret_cast<double*>(base + OFF_S);
+    c.ce = reinterpret_cast<float*>(base + OFF_CE);
     c.lo = reinterpret_cast<int32_t*>(base + OFF_LO);
     c.hi = reinterpret_cast<int32_t*>(base + OFF_HI);
     c.tb = reinterpret_cast<double*>(base + OFF_TB);
@@ -254,26 +254,21 @@ extern "C" int hawkes_loglik_grad_noalloc(const double* d_t, const double* d_x, 
     c.nitems = items_for(n, tr, plan.chunk);
     c.variant = kVariant;
     c.variant_bpsm = d->bpsm;
-    c.final_blocks = 2 * d->sms < kMaxFinalBlocks ? 2 * d->sms : kMaxFinalBlocks;
     const int model = static_cast<int>(flags & (HAWKES_MODEL1 | HAWKES_BG_TIME));
-    int grid = static_cast<int>((npad + 255) / 256);
-    if (grid > 8 * c.sms) grid = 8 * c.sms;
-
     // Counters and the error flag start at zero on every call.
     if (cudaMemsetAsync(c.ctr, 0, CT_COUNT * sizeof(int), st) != cudaSuccess) return HAWKES_ERR_CUDA;
-    k_na_setup<<<grid, 256, 0, st>>>(d_t, d_x, d_y, d_s, n, npad, c.t, c.x, c.y, c.s, c.lo, c.hi,
-                                     c.tb, c.ctr);
+    const EventGrid g = event_grid(npad, d->sms < kMaxSms ? d->sms : kMaxSms);
+    const EvalDesc e = eval_desc(&c);
+    k_na_setup<<<g.blocks, g.threads, 0, st>>>(d_t, d_x, d_y, d_s, n, npad, c.t, c.x, c.y, c.is2, c.ce,
+                                               c.lo, c.hi, c.tb, c.ctr);
     k_na_items<<<8, 64, 0, st>>>(n, tr, plan.chunk, c.items);
-    k_prep<<<grid, 256, 0, st>>>(c.t, c.x, c.y, c.s, c.tb, d_params, model, 1, 0, n, npad, c.rec,
-                                 c.acc, c.cc, c.ctr, c.fix7);
+    k_prep<<<g.blocks, g.threads, 0, st>>>(e, nullptr, d_params, hawkes_params{}, model, 1, 0, 0, nullptr,
+                                           nullptr);
     if (launch_sweep(&c, true, 0, n, (flags & HAWKES_BG_TIME) != 0, false) != cudaSuccess) return HAWKES_ERR_CUDA;
-    k_finalize<<<c.final_blocks, 256, 0, st>>>(c.acc, c.t, c.lo, c.hi, c.cc, n, npad, 0, n, 1,
-                                               c.fixlist, c.ctr, c.partials, nullptr);
-    k_rows64<<<c.sms, 256, 0, st>>>(c.t, c.x, c.y, c.s, c.lo, c.hi, c.cc, model, n, npad, 0, 0, 1,
-                                    c.fixlist, c.ctr, c.acc, c.fix7, nullptr);
-    k_reduce<<<1, 256, 0, st>>>(c.partials, c.final_blocks, c.fix7, c.cc, n, d_out, c.ctr);
-    k_flushfix<<<c.sms, 256, 0, st>>>(c.acc, c.t, c.x, c.y, c.s, c.lo, c.hi, c.cc, model, n, npad,
-                                      0, n, c.ctr, c.fix7, d_out, nullptr);
+    launch_finalize(st, final_grid(n, d->sms < kMaxSms ? d->sms : kMaxSms), e, nullptr, 0, n, 1, d_out,
+                    nullptr, nullptr);
+    k_rows64<<<c.sms, 256, 0, st>>>(e, nullptr, model, 0, n, 1, d_out, nullptr);
+    k_flushfix<<<c.sms, 256, 0, st>>>(e, nullptr, model, 0, n, d_out, nullptr, nullptr);
     k_na_nan_on_error<<<1, 32, 0, st>>>(c.ctr, d_out);
     return cudaGetLastError() == cudaSuccess ? HAWKES_OK : HAWKES_ERR_CUDA;
 }

@@ -100,8 +100,9 @@ int spatial_build(hawkes_ctx* c) {
         cudaMemcpy(t.data(), c->t, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
         cudaMemcpy(x.data(), c->x, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
         cudaMemcpy(y.data(), c->y, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
-        cudaMemcpy(s.data(), c->s, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
+        cudaMemcpy(s.data(), c->is2, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
         return HAWKES_ERR_CUDA;
+    for (double& v : s) v = 1.0 / std::sqrt(v);
     double x0 = x[0], x1 = x[0], y0 = y[0], y1 = y[0];
     for (int64_t i = 1; i < n; ++i) {
         x0 = std::min(x0, x[i]); x1 = std::max(x1, x[i]);
@@ -160,8 +161,8 @@ int spatial_build(hawkes_ctx* c) {
 // in the last word (padding: an index no row ever admits).
 __global__ void k_sp_prep(const int32_t* __restrict__ perm, const double* __restrict__ tmeta,
                           const double* __restrict__ t, const double* __restrict__ x,
-                          const double* __restrict__ y, const double* __restrict__ s,
-                          const double* __restrict__ cc, int model1, int64_t npad, Rec* rec) {
+                          const double* __restrict__ y, const double* __restrict__ is2,
+                          const float* __restrict__ ces, const double* __restrict__ cc, int model1, int64_t npad, Rec* rec) {
     if (cc[CC_VALID] == 0.0) return;
     const double kx = cc[CC_KX], kt = cc[CC_KT];
     const double beta0 = (cc[CC_TX] * cc[CC_TX]) / (cc[CC_H] * cc[CC_H]);
@@ -176,9 +177,8 @@ __global__ void k_sp_prep(const int32_t* __restrict__ perm, const double* __rest
             const float xh = static_cast<float>(xs), yh = static_cast<float>(ys);
             const float xl = static_cast<float>(xs - static_cast<double>(xh));
             const float yl = static_cast<float>(ys - static_cast<double>(yh));
-            const double se = model1 ? 1.0 : s[e];
-            const float nb = -static_cast<float>(beta0 / (se * se));
-            const float ce = static_cast<float>(-2.0 * log2(se));
+            const float nb = -static_cast<float>(model1 ? beta0 : beta0 * is2[e]);
+            const float ce = model1 ? 0.f : ces[e];
             q0 = make_float4(-th, -th, -xh, -xh);
             q1 = make_float4(-xl, -xl, -yh, -yh);
             q2 = make_float4(-yl, -yl, nb, nb);
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_sweep_sp(SpArgs a, int* __restri
 cudaError_t spatial_launch(hawkes_ctx* c, int model1) {
     SpatialState* sp = c->sp;
     const int g = c->sms * 8;
-    k_sp_prep<<<g, 256, 0, c->stream>>>(sp->perm, sp->tmeta, c->t, c->x, c->y, c->s, c->cc, model1, c->npad,
+    k_sp_prep<<<g, 256, 0, c->stream>>>(sp->perm, sp->tmeta, c->t, c->x, c->y, c->is2, c->ce, c->cc, model1, c->npad,
                                          c->rec);
     k_sp_box<<<(sp->ntiles * 32 + 255) / 256, 256, 0, c->stream>>>(sp->perm, c->x, c->y, sp->ntiles, sp->box);
     SpArgs a;
