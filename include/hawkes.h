@@ -108,15 +108,16 @@ enum {
     /*
      * FP32 path, whole sum only (no row window), space-time background:
      * evaluate only the pairs that can be nonzero in FP32.  Events are
-     * ordered by location (a Morton curve) inside time windows cut between
-     * distinct times (hawkes_set_spatial_window); tiles of 256 events in that
-     * order whose every background and excitation term is provably an exact
-     * FP32 zero against a tile of rows (by bounding boxes of the current
-     * locations and time ranges, with 2 units of margin on each base-2
-     * exponent) are skipped.  The rest is evaluated pair by pair with exact
-     * tie and causality indicators, so the result is the full sum up to
-     * FP32 summation order.  The first call after hawkes_set_events builds
-     * the order on the host (synchronous: make it outside stream capture).
+     * ordered by place and time (time windows, hawkes_set_spatial_window,
+     * each split by a k-d tree); columns whose every background or excitation
+     * term is provably an exact FP32 zero against a group of 32 rows (by the
+     * bounding boxes of the current locations and times, with 2 units of
+     * margin on each base-2 exponent) are skipped.  The rest is evaluated pair
+     * by pair with exact tie and causality indicators, so the result is the
+     * full sum up to FP32 summation order.  The first call after
+     * hawkes_set_events builds the order on the host (synchronous: make it
+     * outside stream capture), weighing space against time by that call's
+     * tau_x and tau_t; a later call with other values gives the same result.
      * Not for batches, HAWKES_F64, HAWKES_BG_TIME or row windows
      * (HAWKES_ERR_ARG).
      */
@@ -573,11 +574,10 @@ int hawkes_check_bounded_wait(hawkes_ctx* ctx, double* seconds);
  */
 /*
  * Events per time window of the HAWKES_SKIP_SPATIAL order (>= 256; default
- * 131,072).  Longer windows make tiles more compact in space and skip more
- * pairs, at the cost of a wider time span per tile (times are carried in two
- * FP32 words, so precision holds).  At N = 1,000,000 over 1,200 days the
- * sweep took 99, 65, 47, 38 and 41 ms with windows of 16k, 32k, 64k, 128k
- * and 256k events.  Takes effect at the next evaluation with the flag.
+ * 131,072).  Windows are split in space and time, so their length matters
+ * little; short ones (below about 16,384 events at N = 1,000,000 over 1,200
+ * days) make groups of rows wide in space and skip fewer pairs.  Takes effect
+ * at the next evaluation with the flag.
  */
 int hawkes_set_spatial_window(hawkes_ctx* ctx, int64_t events);
 

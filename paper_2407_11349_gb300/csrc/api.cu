@@ -38,8 +38,8 @@ cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row
 cudaError_t launch_sweep_list(hawkes_ctx* c, const int4* items, int nitems, bool bgt, bool ll);
 int sweep_variant_rows(int v);
 // sweep_spatial.cu
-int spatial_build(hawkes_ctx* c);
-cudaError_t spatial_launch(hawkes_ctx* c, int model1);
+int spatial_build(hawkes_ctx* c, const hawkes_params* p, const hawkes_params* d_p);
+cudaError_t spatial_launch(hawkes_ctx* c, int model1, int llonly);
 void spatial_free(hawkes_ctx* c);
 int spatial_set_window(hawkes_ctx* c, int64_t window);
 void spatial_invalidate(hawkes_ctx* c);
@@ -229,7 +229,7 @@ int enqueue_loglik(hawkes_ctx* c, const CallParams& cp, uint32_t flags, int64_t 
     const bool bgt = (flags & HAWKES_BG_TIME) != 0;
     const bool spatial = (flags & HAWKES_SKIP_SPATIAL) != 0;
     if (spatial && (f64 || bgt || rb != 0 || re != c->n)) return HAWKES_ERR_ARG;
-    if (spatial) HK_TRY(spatial_build(c));  // synchronous on first use after set_events
+    if (spatial) HK_TRY(spatial_build(c, cp.dev ? nullptr : &cp.val, cp.dev));  // synchronous on first use after set_events
     const int skip = (!f64 && !spatial && (flags & HAWKES_SKIP_UNDERFLOW)) ? 1 : 0;
     HK_TRY(enqueue_prep(c, cp, model, (f64 || spatial) ? 0 : 1, skip));
     if (!f64) {
@@ -237,7 +237,8 @@ int enqueue_loglik(hawkes_ctx* c, const CallParams& cp, uint32_t flags, int64_t 
         cudaError_t se = cudaSuccess;
         HK_TRY(timed(c, HAWKES_K_SWEEP, [&] {
             if (spatial)
-                se = spatial_launch(c, (flags & HAWKES_MODEL1) ? 1 : 0);
+                se = spatial_launch(c, (flags & HAWKES_MODEL1) ? 1 : 0,
+                                    (flags & HAWKES_LOGLIK_ONLY) ? 1 : 0);
             else
                 launch_sweep(c, sym, rb, re, bgt, (flags & HAWKES_LOGLIK_ONLY) != 0);
         }));

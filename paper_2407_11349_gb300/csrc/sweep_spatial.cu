@@ -3,58 +3,78 @@
 // At the sizes of the paper most pair terms are exact FP32 zeros because the
 // two events are far apart: a background term B' = 2^-(dt~^2 + r~^2) flushes
 // to zero once its exponent passes 126, and an excitation term once
-// omega~ dt~ + beta r~^2 - ce passes 126 (ex2.approx.ftz).  The symmetric
-// sweep visits 256-event tiles in time order, and such a tile spans the whole
-// map, so no tile pair is ever entirely zero by distance.  This path orders
-// the events so that tiles are compact in space and time, and skips every
-// tile pair whose terms are all provably zero:
-//   - time windows of about `window` consecutive events, cut only between
-//     distinct times (a tie group never straddles two windows);
-//   - inside each window, events ordered along a Morton curve of their
-//     locations at the time the order is built;
-//   - per 256-event tile of that order: the time range and the smallest and
-//     largest s_j (fixed), and the bounding box of the current locations
-//     (recomputed every call, so a resample moves it with the events);
-//   - a tile pair is skipped when, with 2 units of margin, the smallest
-//     possible background exponent exceeds 128 and the smallest possible
-//     excitation exponent (or the absence of an earlier source) makes every
-//     excitation term zero as well.
-// The kept pairs are evaluated without the symmetric shortcut (each row
-// against the kept column tiles); the tie and causality indicators come from
-// each event's index in the time order, carried in its record, so the masks
-// are exact.  Times are split into FP32 hi + lo parts like the coordinates,
-// because a tile now spans many days.  Row sums go to the FP64 accumulators
-// of the events' original indices; finalisation is shared with the other
-// paths.  The result equals the full sweep's up to FP32 summation order.
+// omega~ dt~ + beta r~^2 - ce passes 126 (ex2.approx.ftz).  This path orders
+// the events so that neighbours in the order are neighbours in space and time,
+// and evaluates, for each group of 32 rows, only the columns that can hold a
+// nonzero term:
+//   - Order (host, on first use): time windows of about `window` events, each
+//     split by a k-d tree over (x, y, t) down to chunks of 32 events (tiles of
+//     256).  Space and time are weighed by tau_x and tau_t of the call that
+//     builds the order.  Locations that will be redrawn inside their counties
+//     say little beyond the county, so they enter as the county's mean plus a
+//     fifth of the offset from it.
+//   - Per call: records in that order and the bounding box, time range and
+//     largest excitation reach of every chunk and tile (a resample moves them
+//     with the events).
+//   - Sweep: one warp per group of 32 rows (one chunk of the order, a row per
+//     lane).  It tests tiles, then chunks, against its rows' box, then the
+//     chunk's 32 events, one per lane, and appends the survivors to two small
+//     buffers in shared memory (background, excitation).  A full buffer is
+//     evaluated, two columns per packed f32x2 register.
+// Every test keeps 2 units of margin on the base-2 exponent, and the boxes are
+// widened by the FP32 rounding of the coordinates, so what is left out is an
+// exact FP32 zero; the rest is the full sweep's sum in another order.
+//
+// What bounds it: shared-memory reads (a column's 24 bytes go to every lane;
+// 74% of the wavefronts) and instruction issue (67%) in the evaluation of the
+// columns that pass the point test; the FP32 pipe is 46% busy.  Two rows per
+// lane would halve the reads, but the box of 64 rows keeps 48% more columns.
+// At N = 1,000,000 (3,143 counties, 1,200 days) a row has 1,811
+// columns with a nonzero background and 14 with a nonzero excitation; point
+// tests against the box of 32 rows leave 4,070 and 1,210, in 4.1 ms.  (The former
+// design, 256 x 256 tile pairs kept whole by box tests and swept through
+// shared-memory tiles, left about 40,000 with both terms: 45 ms.)
+// Tie and causality indicators come from each event's index in the time order,
+// carried beside its record, and are only tested for columns that can share a
+// time with the rows.  Row sums go to the FP64 accumulators of the events'
+// original indices; finalisation is shared with the other paths.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <new>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "sweep_kernel.cuh"
 
 namespace hk {
 
+constexpr int SP_CH = 32;              // events per chunk: a row group, and the finest column unit
+constexpr int SP_WARPS = 8, SP_THREADS = 32 * SP_WARPS;
+// Resident CTAs per SM.  At N = 1,000,000: 2 4.30 ms, 3 4.07, 4 (64 registers,
+// spills) 4.52, 5 6.3.
+constexpr int SP_BPSM = 3;
+constexpr int SP_BUF = 64;             // buffered columns (32 evaluated at a time)
+constexpr int SP_LIST = 128;           // chunks listed before they are read
+constexpr int SP_B_PLANES = 7, SP_E_PLANES = 9;
+constexpr int32_t SP_TIED = 1 << 30;   // flag in a position's rank: other events share the time
+constexpr float SP_ZERO = 128.f;       // exponent beyond which a term counts as zero (126 + margin)
+static_assert(NPAD_MULT % TC == 0 && TC == 8 * SP_CH, "a tile is 8 chunks");
+
 struct SpatialState {
     int64_t window = 131072;  // target events per time window
     bool built = false;
     int ntiles = 0;           // npad / TC
-    int32_t* perm = nullptr;  // [npad] time-order index at each position (-1: padding)
-    double* tmeta = nullptr;  // [4 ntiles] time min, time max, s min, s max of each tile
-    double* box = nullptr;    // [4 ntiles] x min, x max, y min, y max of the current locations
+    int32_t* rank = nullptr;  // [npad] time-order index at each position, | SP_TIED (-1: padding)
+    float4* meta = nullptr;   // [2 x chunks], then [2 x tiles]: SpBox of each
 };
-
-constexpr int SP_CH = THREADS;  // column tiles per work item (one per thread when listing)
-constexpr int SP_RP = 4, SP_R = 2 * SP_RP, SP_WROWS = 32 * SP_R, SP_TR = WARPS * SP_WROWS;
-static_assert(SP_WROWS == TC, "a warp's rows are one tile of the spatial order");
-constexpr int32_t SP_PAD_RANK = 0x7fffffff;
 
 void spatial_free(hawkes_ctx* c) {
     if (!c->sp) return;
     SpatialState* s = c->sp;
-    if (s->perm) cudaFree(s->perm);
-    if (s->tmeta) cudaFree(s->tmeta);
-    if (s->box) cudaFree(s->box);
+    if (s->rank) cudaFree(s->rank);
+    if (s->meta) cudaFree(s->meta);
     delete s;
     c->sp = nullptr;
 }
@@ -76,476 +96,536 @@ int spatial_set_window(hawkes_ctx* c, int64_t window) {
     return HAWKES_OK;
 }
 
-static uint32_t spread16(uint32_t v) {
-    v &= 0xFFFFu;
-    v = (v | (v << 8)) & 0x00FF00FFu;
-    v = (v | (v << 4)) & 0x0F0F0F0Fu;
-    v = (v | (v << 2)) & 0x33333333u;
-    v = (v | (v << 1)) & 0x55555555u;
-    return v;
+// Split [a, b) of the permutation at medians of its widest side, down to
+// chunks; parts stay whole tiles while larger than a tile.
+struct SpPoint {
+    float c[3];
+    int32_t e;
+};
+static void sp_split(SpPoint* a, SpPoint* b) {
+    while (b - a > SP_CH) {
+        const int64_t len = b - a, unit = len > TC ? TC : SP_CH;
+        float lo[3], hi[3];
+        for (int k = 0; k < 3; ++k) lo[k] = hi[k] = a->c[k];
+        for (const SpPoint* p = a + 1; p < b; ++p)
+            for (int k = 0; k < 3; ++k) {
+                lo[k] = std::min(lo[k], p->c[k]);
+                hi[k] = std::max(hi[k], p->c[k]);
+            }
+        int ax = 0;
+        for (int k = 1; k < 3; ++k)
+            if (hi[k] - lo[k] > hi[ax] - lo[ax]) ax = k;
+        SpPoint* m = a + std::min((len / 2 + unit - 1) / unit * unit, (len - 1) / unit * unit);
+        std::nth_element(a, m, b, [ax](const SpPoint& u, const SpPoint& v) {
+            return u.c[ax] < v.c[ax] || (u.c[ax] == v.c[ax] && u.e < v.e);
+        });
+        sp_split(m, b);
+        b = m;
+    }
 }
 
-// Build the order and its fixed tile data from the current events
-// (synchronous; the locations used for the order are the current ones).
-int spatial_build(hawkes_ctx* c) {
-    if (!c->sp) {
-        const int rc = spatial_set_window(c, 131072);
-        if (rc != HAWKES_OK) return rc;
-    }
+static int build_order(hawkes_ctx* c, double tau_x, double tau_t) {
     SpatialState* sp = c->sp;
-    if (sp->built) return HAWKES_OK;
     const int64_t n = c->n, npad = c->npad;
-    std::vector<double> t(n), x(n), y(n), s(n);
+    std::vector<double> t(n), x(n), y(n);
+    std::vector<int32_t> cty(n), lo(n), hi(n);
     if (cudaStreamSynchronize(c->stream) != cudaSuccess ||
         cudaMemcpy(t.data(), c->t, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
         cudaMemcpy(x.data(), c->x, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
         cudaMemcpy(y.data(), c->y, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
-        cudaMemcpy(s.data(), c->is2, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
+        cudaMemcpy(cty.data(), c->county, n * sizeof(int32_t), cudaMemcpyDeviceToHost) != cudaSuccess ||
+        cudaMemcpy(lo.data(), c->lo, n * sizeof(int32_t), cudaMemcpyDeviceToHost) != cudaSuccess ||
+        cudaMemcpy(hi.data(), c->hi, n * sizeof(int32_t), cudaMemcpyDeviceToHost) != cudaSuccess)
         return HAWKES_ERR_CUDA;
-    for (double& v : s) v = 1.0 / std::sqrt(v);
-    double x0 = x[0], x1 = x[0], y0 = y[0], y1 = y[0];
-    for (int64_t i = 1; i < n; ++i) {
-        x0 = std::min(x0, x[i]); x1 = std::max(x1, x[i]);
-        y0 = std::min(y0, y[i]); y1 = std::max(y1, y[i]);
+    if (c->counties_ok) {  // a resample can move the events inside their counties
+        std::vector<double> mx(c->n_counties, 0.0), my(c->n_counties, 0.0), cnt(c->n_counties, 0.0);
+        for (int64_t i = 0; i < n; ++i) {
+            mx[cty[i]] += x[i];
+            my[cty[i]] += y[i];
+            cnt[cty[i]] += 1.0;
+        }
+        for (int64_t i = 0; i < n; ++i) {
+            const double cx = mx[cty[i]] / cnt[cty[i]], cy = my[cty[i]] / cnt[cty[i]];
+            x[i] = cx + 0.2 * (x[i] - cx);
+            y[i] = cy + 0.2 * (y[i] - cy);
+        }
     }
-    const double gx = 65535.0 / std::max(x1 - x0, 1e-300), gy = 65535.0 / std::max(y1 - y0, 1e-300);
-    std::vector<uint64_t> key(n);
-    for (int64_t i = 0; i < n; ++i) {
-        const uint32_t cx = static_cast<uint32_t>(std::min(65535.0, std::max(0.0, (x[i] - x0) * gx)));
-        const uint32_t cy = static_cast<uint32_t>(std::min(65535.0, std::max(0.0, (y[i] - y0) * gy)));
-        key[i] = (static_cast<uint64_t>(spread16(cx) | (spread16(cy) << 1)) << 32) | static_cast<uint64_t>(i);
+    std::vector<SpPoint> pt(n);
+    for (int64_t i = 0; i < n; ++i)
+        pt[i] = SpPoint{{static_cast<float>((x[i] - x[0]) / tau_x), static_cast<float>((y[i] - y[0]) / tau_x),
+                         static_cast<float>((t[i] - t[0]) / tau_t)},
+                        static_cast<int32_t>(i)};
+    // time windows (whole tiles), split independently on a few host threads
+    const int64_t w = (sp->window + TC - 1) / TC * TC;
+    const int64_t nw = (n + w - 1) / w;
+    auto work = [&](int64_t k0, int64_t step) {
+        for (int64_t k = k0; k < nw; k += step) sp_split(pt.data() + k * w, pt.data() + std::min(n, (k + 1) * w));
+    };
+    const int64_t nth = std::min<int64_t>(nw, n > 50000 ? 8 : 1);
+    std::vector<std::thread> th;
+    int64_t started = 1;  // this thread takes window 0, nth, 2 nth, ...
+    try {
+        for (; started < nth; ++started) th.emplace_back(work, started, nth);
+    } catch (const std::system_error&) {  // no more threads: the rest runs here
     }
-    std::vector<int32_t> perm(npad, -1);
-    for (int64_t a = 0; a < n;) {  // windows cut between distinct times only
-        int64_t b = std::min(n, a + sp->window);
-        while (b < n && t[b] == t[b - 1]) ++b;
-        std::sort(key.begin() + a, key.begin() + b);
-        for (int64_t p = a; p < b; ++p) perm[p] = static_cast<int32_t>(key[p] & 0xFFFFFFFFu);
-        a = b;
+    work(0, nth);
+    for (int64_t k = started; k < nth; ++k) work(k, nth);
+    for (std::thread& q : th) q.join();
+    std::vector<int32_t> rank(npad, -1);
+    for (int64_t p = 0; p < n; ++p) {
+        const int32_t e = pt[p].e;
+        rank[p] = hi[e] - lo[e] > 1 ? (e | SP_TIED) : e;
     }
     const int ntiles = static_cast<int>(npad / TC);
-    std::vector<double> meta(4 * static_cast<size_t>(ntiles));
-    for (int k = 0; k < ntiles; ++k) {
-        double t0 = 1e300, t1 = -1e300, s0 = 1e300, s1 = -1e300;
-        for (int q = 0; q < TC; ++q) {
-            const int32_t e = perm[static_cast<size_t>(k) * TC + q];
-            if (e < 0) continue;
-            t0 = std::min(t0, t[e]); t1 = std::max(t1, t[e]);
-            s0 = std::min(s0, s[e]); s1 = std::max(s1, s[e]);
-        }
-        meta[4 * k + 0] = t0; meta[4 * k + 1] = t1; meta[4 * k + 2] = s0; meta[4 * k + 3] = s1;
-    }
-    if (sp->ntiles != ntiles || !sp->perm) {
-        if (sp->perm) cudaFree(sp->perm);
-        if (sp->tmeta) cudaFree(sp->tmeta);
-        if (sp->box) cudaFree(sp->box);
-        sp->perm = nullptr; sp->tmeta = nullptr; sp->box = nullptr;
-        if (cudaMalloc(&sp->perm, npad * sizeof(int32_t)) != cudaSuccess ||
-            cudaMalloc(&sp->tmeta, 4 * static_cast<size_t>(ntiles) * sizeof(double)) != cudaSuccess ||
-            cudaMalloc(&sp->box, 4 * static_cast<size_t>(ntiles) * sizeof(double)) != cudaSuccess) {
+    if (sp->ntiles != ntiles || !sp->rank || !sp->meta) {
+        if (sp->rank) cudaFree(sp->rank);
+        if (sp->meta) cudaFree(sp->meta);
+        sp->rank = nullptr;
+        sp->meta = nullptr;
+        if (cudaMalloc(&sp->rank, npad * sizeof(int32_t)) != cudaSuccess ||
+            cudaMalloc(&sp->meta, 2 * static_cast<size_t>(9 * ntiles) * sizeof(float4)) != cudaSuccess) {
             cudaGetLastError();
             return HAWKES_ERR_OOM;
         }
         sp->ntiles = ntiles;
     }
-    if (cudaMemcpy(sp->perm, perm.data(), npad * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(sp->tmeta, meta.data(), meta.size() * sizeof(double), cudaMemcpyHostToDevice) !=
-            cudaSuccess)
+    if (cudaMemcpy(sp->rank, rank.data(), npad * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess)
         return HAWKES_ERR_CUDA;
     sp->built = true;
     return HAWKES_OK;
 }
 
-// Stage the records in the spatial order: times relative to their tile's
-// earliest time, split into FP32 hi + lo; the time-order index of the event
-// in the last word (padding: an index no row ever admits).
-__global__ void k_sp_prep(const int32_t* __restrict__ perm, const double* __restrict__ tmeta,
-                          const double* __restrict__ t, const double* __restrict__ x,
-                          const double* __restrict__ y, const double* __restrict__ is2,
-                          const float* __restrict__ ces, const double* __restrict__ cc, int model1, int64_t npad, Rec* rec) {
-    if (cc[CC_VALID] == 0.0) return;
-    const double kx = cc[CC_KX], kt = cc[CC_KT];
-    const double beta0 = (cc[CC_TX] * cc[CC_TX]) / (cc[CC_H] * cc[CC_H]);
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npad;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t e = perm[p];
-        float4 q0, q1, q2, q3;
-        if (e >= 0) {
-            const double tt = (t[e] - tmeta[4 * (p / TC)]) * kt;
-            const float th = static_cast<float>(tt), tl = static_cast<float>(tt - static_cast<double>(th));
-            const double xs = x[e] * kx, ys = y[e] * kx;
-            const float xh = static_cast<float>(xs), yh = static_cast<float>(ys);
-            const float xl = static_cast<float>(xs - static_cast<double>(xh));
-            const float yl = static_cast<float>(ys - static_cast<double>(yh));
-            const float nb = -static_cast<float>(model1 ? beta0 : beta0 * is2[e]);
-            const float ce = model1 ? 0.f : ces[e];
-            q0 = make_float4(-th, -th, -xh, -xh);
-            q1 = make_float4(-xl, -xl, -yh, -yh);
-            q2 = make_float4(-yl, -yl, nb, nb);
-            q3 = make_float4(ce, ce, -tl, __int_as_float(e));
-        } else {
-            q0 = make_float4(-PAD_T, -PAD_T, 0.f, 0.f);
-            q1 = make_float4(0.f, 0.f, 0.f, 0.f);
-            q2 = make_float4(0.f, 0.f, 0.f, 0.f);
-            q3 = make_float4(0.f, 0.f, 0.f, __int_as_float(SP_PAD_RANK));
-        }
-        *rec_q(rec, p, 0) = q0;
-        *rec_q(rec, p, 1) = q1;
-        *rec_q(rec, p, 2) = q2;
-        *rec_q(rec, p, 3) = q3;
+// Build the order from the current events (synchronous; the locations used for
+// the order are the current ones).  p: the call's parameters on the host, or
+// null with d_p on the device; they only weigh space against time.
+int spatial_build(hawkes_ctx* c, const hawkes_params* p, const hawkes_params* d_p) {
+    if (!c->sp) {
+        const int rc = spatial_set_window(c, 131072);
+        if (rc != HAWKES_OK) return rc;
+    }
+    if (c->sp->built) return HAWKES_OK;
+    if (c->n >= SP_TIED) return HAWKES_ERR_ARG;
+    hawkes_params q{};
+    if (p)
+        q = *p;
+    else if (cudaStreamSynchronize(c->stream) != cudaSuccess ||
+             cudaMemcpy(&q, d_p, sizeof(q), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return HAWKES_ERR_CUDA;
+    auto usable = [](double v) { return v > 1e-30 && v < 1e30; };
+    if (!usable(q.tau_x) || !usable(q.tau_t)) q.tau_x = q.tau_t = 1.0;
+    try {
+        return build_order(c, q.tau_x, q.tau_t);
+    } catch (const std::bad_alloc&) {
+        return HAWKES_ERR_OOM;
     }
 }
 
-// Bounding box of the current locations of each tile of the order (one warp
-// per tile).  Tiles of padding only get an empty box (min > max).
-__global__ void k_sp_box(const int32_t* __restrict__ perm, const double* __restrict__ x,
-                         const double* __restrict__ y, int ntiles, double* box) {
-    const int lane = threadIdx.x & 31;
-    for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < ntiles;
-         k += (gridDim.x * blockDim.x) >> 5) {
-        double x0 = 1e300, x1 = -1e300, y0 = 1e300, y1 = -1e300;
-        for (int q = lane; q < TC; q += 32) {
-            const int32_t e = perm[static_cast<int64_t>(k) * TC + q];
-            if (e < 0) continue;
-            x0 = fmin(x0, x[e]); x1 = fmax(x1, x[e]);
-            y0 = fmin(y0, y[e]); y1 = fmax(y1, y[e]);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            x0 = fmin(x0, __shfl_xor_sync(0xffffffffu, x0, o));
-            x1 = fmax(x1, __shfl_xor_sync(0xffffffffu, x1, o));
-            y0 = fmin(y0, __shfl_xor_sync(0xffffffffu, y0, o));
-            y1 = fmax(y1, __shfl_xor_sync(0xffffffffu, y1, o));
-        }
-        if (lane == 0) {
-            box[4 * k + 0] = x0; box[4 * k + 1] = x1;
-            box[4 * k + 2] = y0; box[4 * k + 3] = y1;
-        }
-    }
-}
-
-// Everything the sweep needs to know about a set of tiles for the zero test.
-struct SpRange {
-    double x0, x1, y0, y1;  // bounding box (km)
-    double t0, t1;          // time range (days)
-    double s0, s1;          // s_j range
-    bool empty;
+// Bounds of a set of events, in scaled units: box, time range, largest ce,
+// smallest beta.  Empty: x0 > x1.
+struct SpBox {
+    float x0, x1, y0, y1, t0, t1, ce, beta;
 };
 
-__device__ __forceinline__ SpRange sp_tile(const double* __restrict__ tmeta,
-                                           const double* __restrict__ box, int k) {
-    SpRange r;
-    r.x0 = box[4 * k + 0]; r.x1 = box[4 * k + 1]; r.y0 = box[4 * k + 2]; r.y1 = box[4 * k + 3];
-    r.t0 = tmeta[4 * k + 0]; r.t1 = tmeta[4 * k + 1];
-    r.s0 = tmeta[4 * k + 2]; r.s1 = tmeta[4 * k + 3];
-    r.empty = !(r.t0 <= r.t1);
-    return r;
+__device__ __forceinline__ SpBox sp_load(const float4* __restrict__ meta, int k) {
+    const float4 a = meta[2 * k], b = meta[2 * k + 1];
+    return SpBox{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+}
+__device__ __forceinline__ void sp_store(float4* meta, int k, const SpBox& v) {
+    meta[2 * k] = make_float4(v.x0, v.x1, v.y0, v.y1);
+    meta[2 * k + 1] = make_float4(v.t0, v.t1, v.ce, v.beta);
+}
+__device__ __forceinline__ SpBox sp_empty() {
+    return SpBox{1e30f, -1e30f, 1e30f, -1e30f, 1e30f, -1e30f, -1e30f, 1e30f};
+}
+__device__ __forceinline__ void sp_join(SpBox& a, const SpBox& b) {
+    a.x0 = fminf(a.x0, b.x0); a.x1 = fmaxf(a.x1, b.x1);
+    a.y0 = fminf(a.y0, b.y0); a.y1 = fmaxf(a.y1, b.y1);
+    a.t0 = fminf(a.t0, b.t0); a.t1 = fmaxf(a.t1, b.t1);
+    a.ce = fmaxf(a.ce, b.ce); a.beta = fminf(a.beta, b.beta);
+}
+// Widen [lo, hi] by 2^-22 of its magnitude: more than the rounding to FP32 of
+// its own ends and of any point compared with it nearby.
+__device__ __forceinline__ void sp_widen(float& lo, float& hi) {
+    const float s = 2.384185791015625e-07f * fmaxf(fabsf(lo), fabsf(hi));
+    lo -= s;
+    hi += s;
 }
 
-__device__ __forceinline__ void sp_union(SpRange& a, const SpRange& b) {
-    if (b.empty) return;
-    if (a.empty) {
-        a = b;
-        return;
-    }
-    a.x0 = fmin(a.x0, b.x0); a.x1 = fmax(a.x1, b.x1);
-    a.y0 = fmin(a.y0, b.y0); a.y1 = fmax(a.y1, b.y1);
-    a.t0 = fmin(a.t0, b.t0); a.t1 = fmax(a.t1, b.t1);
-    a.s0 = fmin(a.s0, b.s0); a.s1 = fmax(a.s1, b.s1);
-}
-
-// True if every background and excitation term of a row in `rw` against a
-// source in `col` is an exact FP32 zero (2 units of margin on each exponent).
-__device__ __forceinline__ bool sp_all_zero(const SpRange& rw, const SpRange& col,
-                                            const double* __restrict__ cc, int model1) {
-    if (rw.empty || col.empty) return true;
-    const double ax = cc[CC_KX] * cc[CC_KX], kt = cc[CC_KT], omt = cc[CC_OMT];
-    const double dx = fmax(0.0, fmax(col.x0 - rw.x1, rw.x0 - col.x1));
-    const double dy = fmax(0.0, fmax(col.y0 - rw.y1, rw.y0 - col.y1));
-    const double r2 = (dx * dx + dy * dy) * ax;
-    const double gap = fmax(0.0, fmax(col.t0 - rw.t1, rw.t0 - col.t1)) * kt;
-    if (gap * gap + r2 <= 128.0) return false;
-    if (col.t0 >= rw.t1) return true;  // no source earlier than any row: no excitation
-    const double causal = fmax(0.0, rw.t0 - col.t1) * kt;
-    const double smin = model1 ? 1.0 : col.s0, smax = model1 ? 1.0 : col.s1;
-    const double ce_max = -2.0 * log2(smin);
-    const double beta_min = (cc[CC_TX] * cc[CC_TX]) / (cc[CC_H] * cc[CC_H] * smax * smax);
-    return ce_max - omt * causal - beta_min * r2 < -128.0;
-}
-
-// One tile of the spatial order against the warp's rows (no symmetry).
-//   MASK  per-pair indicators from the time-order indices (rows' tie ranges
-//         [lo, hi) against the source's index); else every pair counts and
-//   EXC   says whether the sources are all earlier (excitation) or all later.
-template <int UNROLL, bool MASK, bool EXC>
-__device__ __forceinline__ void sp_tile_pass(const float4* __restrict__ tile, int lane,
-                                             Rows<SP_RP>& rr, const float2 (&tl)[SP_RP],
-                                             float2 nomt, const int (&lo)[SP_R],
-                                             const int (&hi)[SP_R]) {
-#pragma unroll 1
-    for (int ch = 0; ch < TC / 32; ++ch) {
-#pragma unroll UNROLL
-        for (int s = 0; s < 32; ++s) {
-            const int c = ch * 32 + ((lane + s) & 31);
-            const float4 q0 = tile[0 * TC + c];  // -t, -t, -xh, -xh
-            const float4 q1 = tile[1 * TC + c];  // -xl, -xl, -yh, -yh
-            const float4 q2 = tile[2 * TC + c];  // -yl, -yl, -beta, -beta
-            const float4 q3 = tile[3 * TC + c];  // ce, ce, -t lo, time-order index
-            const float2 nT = f2(q0.x, q0.y), nXH = f2(q0.z, q0.w);
-            const float2 nXL = f2(q1.x, q1.y), nYH = f2(q1.z, q1.w);
-            const float2 nYL = f2(q2.x, q2.y), NB = f2(q2.z, q2.w);
-            const float2 CE = f2(q3.x, q3.y), nTL = f2(q3.z, q3.z);
-            const int rank = __float_as_int(q3.w);
-#pragma unroll
-            for (int p = 0; p < SP_RP; ++p) {
-                const float2 dt = add2(add2(rr.tp[p], nT), add2(tl[p], nTL));
-                const float2 dx = add2(add2(rr.xh[p], nXH), add2(rr.xl[p], nXL));
-                const float2 dy = add2(add2(rr.yh[p], nYH), add2(rr.yl[p], nYL));
-                const float2 r2 = fma2(dy, dy, mul2(dx, dx));
-                const float2 dt2 = mul2(dt, dt);
-                const float2 aB = add2(dt2, r2);
-                float2 B = f2(ex2(-aB.x), ex2(-aB.y));
-                if (MASK) {
-                    B.x = (rank < lo[2 * p] || rank >= hi[2 * p]) ? B.x : 0.f;
-                    B.y = (rank < lo[2 * p + 1] || rank >= hi[2 * p + 1]) ? B.y : 0.f;
-                }
-                rr.sB[p] = add2(rr.sB[p], B);
-                rr.sBr[p] = fma2(B, r2, rr.sBr[p]);
-                rr.sBt[p] = fma2(B, dt2, rr.sBt[p]);
-                if (MASK || EXC) {
-                    const float2 nv = mul2(NB, r2);
-                    const float2 arg = add2(fma2(nomt, dt, nv), CE);
-                    float2 E = f2(ex2(arg.x), ex2(arg.y));
-                    if (MASK) {
-                        E.x = rank < lo[2 * p] ? E.x : 0.f;
-                        E.y = rank < lo[2 * p + 1] ? E.y : 0.f;
-                    }
-                    rr.sE[p] = add2(rr.sE[p], E);
-                    rr.sEt[p] = fma2(E, dt, rr.sEt[p]);
-                    rr.sEq[p] = fma2(E, nv, rr.sEq[p]);
-                }
-            }
+// Stage the records in the spatial order (negated column values): planes
+// ra[npad] = (-x hi, -x lo, -y hi, -y lo), rb[npad] = (-t hi, -t lo, -beta, ce),
+// with t~ = (t - t_1) sqrt(a_t) in two FP32 words like the coordinates, and
+// the boxes of the chunks and tiles (one block per tile).
+__global__ void __launch_bounds__(TC) k_sp_prep(EvalDesc d, const int32_t* __restrict__ rank, int model1,
+                                                float4* __restrict__ ra, float4* __restrict__ rb,
+                                                float4* __restrict__ meta, int ntiles) {
+    if (d.cc[CC_VALID] == 0.0) return;
+    const double kx = d.cc[CC_KX], kt = d.cc[CC_KT], tf = d.t[0];
+    const double beta0 = (d.cc[CC_TX] * d.cc[CC_TX]) / (d.cc[CC_H] * d.cc[CC_H]);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ SpBox boxes[TC / SP_CH];
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t p = static_cast<int64_t>(tile) * TC + threadIdx.x;
+        const int32_t r = rank[p];
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = make_float4(-PAD_T, 0.f, 0.f, -1e30f);
+        SpBox box = sp_empty();
+        if (r >= 0) {
+            const int32_t e = r & ~SP_TIED;
+            const double ts = (d.t[e] - tf) * kt, xs = d.x[e] * kx, ys = d.y[e] * kx;
+            const float th = static_cast<float>(ts), xh = static_cast<float>(xs), yh = static_cast<float>(ys);
+            const float beta = static_cast<float>(model1 ? beta0 : beta0 * d.is2[e]);
+            const float ce = model1 ? 0.f : d.ce[e];
+            a = make_float4(-xh, -static_cast<float>(xs - static_cast<double>(xh)), -yh,
+                            -static_cast<float>(ys - static_cast<double>(yh)));
+            b = make_float4(-th, -static_cast<float>(ts - static_cast<double>(th)), -beta, ce);
+            box = SpBox{xh, xh, yh, yh, th, th, ce, beta};
         }
+        ra[p] = a;
+        rb[p] = b;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            SpBox q;
+            q.x0 = __shfl_xor_sync(0xffffffffu, box.x0, o); q.x1 = __shfl_xor_sync(0xffffffffu, box.x1, o);
+            q.y0 = __shfl_xor_sync(0xffffffffu, box.y0, o); q.y1 = __shfl_xor_sync(0xffffffffu, box.y1, o);
+            q.t0 = __shfl_xor_sync(0xffffffffu, box.t0, o); q.t1 = __shfl_xor_sync(0xffffffffu, box.t1, o);
+            q.ce = __shfl_xor_sync(0xffffffffu, box.ce, o); q.beta = __shfl_xor_sync(0xffffffffu, box.beta, o);
+            sp_join(box, q);
+        }
+        if (lane == 0) {
+            if (box.x0 <= box.x1) {
+                sp_widen(box.x0, box.x1);
+                sp_widen(box.y0, box.y1);
+                sp_widen(box.t0, box.t1);
+            }
+            boxes[warp] = box;
+            sp_store(meta, tile * (TC / SP_CH) + warp, box);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int k = 1; k < TC / SP_CH; ++k) sp_join(box, boxes[k]);
+            sp_store(meta, ntiles * (TC / SP_CH) + tile, box);
+        }
+        __syncthreads();
     }
 }
 
 struct SpArgs {
-    const Rec* rec;
+    const float4* ra;
+    const float4* rb;
+    const int32_t* rank;
     const int32_t* lo;
     const int32_t* hi;
     const double* cc;
     double* acc;
-    const double* tmeta;
-    const double* box;
-    int64_t n, npad;
-    int ntiles, nI, nch, model1;
-    int chunk;  // column tiles per item (<= SP_CH)
+    const float4* cmeta;
+    const float4* tmeta;
+    int64_t npad;
+    int ntiles, groups, parts;
 };
 
-// Persistent sweep over items (row tile I of the spatial order x a chunk of
-// SP_CH column tiles).  The CTA first lists the chunk's column tiles that are
-// not entirely zero against its 8 row tiles, then streams only those through
-// shared memory (TMA, double-buffered); each warp re-tests them against its
-// own row tile.
-__global__ void __launch_bounds__(THREADS, 1) k_sweep_sp(SpArgs a, int* __restrict__ ctr, int nitems) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    Rec* tiles = reinterpret_cast<Rec*>(smem);
-    __shared__ __align__(8) uint64_t bars[2];
-    __shared__ int s_item, s_abort, s_nlist;
-    __shared__ int s_list[SP_CH];
-    __shared__ int s_wcount[WARPS];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (a.cc[CC_VALID] == 0.0) return;
-    if (tid == 0) {
-        mbar_init(&bars[0], 1);
-        mbar_init(&bars[1], 1);
-        fence_barrier_init();
-        s_abort = 0;
+// Can a column of box (or point) c hold a nonzero background / excitation term
+// for some row of box w?
+__device__ __forceinline__ float sp_gap(float lo, float hi, float a0, float a1) {
+    return fmaxf(0.f, fmaxf(a0 - hi, lo - a1));
+}
+__device__ __forceinline__ void sp_near(const SpBox& w, const SpBox& c, float omt, bool& nb, bool& ne) {
+    const float dx = sp_gap(w.x0, w.x1, c.x0, c.x1), dy = sp_gap(w.y0, w.y1, c.y0, c.y1);
+    const float r2 = fmaf(dx, dx, dy * dy), g = sp_gap(w.t0, w.t1, c.t0, c.t1);
+    nb = !(fmaf(g, g, r2) > SP_ZERO);  // (negated: a NaN is kept, and reported as ever)
+    ne = c.t0 <= w.t1 && !(c.ce - omt * fmaxf(0.f, w.t0 - c.t1) - c.beta * r2 < -SP_ZERO);
+}
+
+// A lane's row (values doubled for packed arithmetic) and its sums over the
+// even and odd columns.
+struct SpRow {
+    float2 th, tl, xh, xl, yh, yl;
+    float2 sB, sBr, sBt, sE, sEt, sEq;
+    int lo, hi;
+};
+
+__device__ __forceinline__ float2 half4(const float4& v, int h) { return h ? f2(v.z, v.w) : f2(v.x, v.y); }
+
+// Background of `quads` x 4 buffered columns against the lane's row.
+template <bool MASK, bool LL>
+__device__ __forceinline__ void sp_eval_b(const float* __restrict__ buf, int quads, SpRow& w) {
+#pragma unroll 4
+    for (int q = 0; q < quads; ++q) {
+        const float4* p = reinterpret_cast<const float4*>(buf) + q;
+        const float4 xh = p[0 * SP_BUF / 4], xl = p[1 * SP_BUF / 4], yh = p[2 * SP_BUF / 4],
+                     yl = p[3 * SP_BUF / 4], th = p[4 * SP_BUF / 4], tl = p[5 * SP_BUF / 4];
+        int4 rk;
+        if (MASK) rk = *reinterpret_cast<const int4*>(p + 6 * SP_BUF / 4);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 dt = add2(add2(w.th, half4(th, h)), add2(w.tl, half4(tl, h)));
+            const float2 dx = add2(add2(w.xh, half4(xh, h)), add2(w.xl, half4(xl, h)));
+            const float2 dy = add2(add2(w.yh, half4(yh, h)), add2(w.yl, half4(yl, h)));
+            const float2 r2 = fma2(dy, dy, mul2(dx, dx));
+            const float2 dt2 = mul2(dt, dt);
+            const float2 aB = add2(dt2, r2);
+            float2 B = f2(ex2(-aB.x), ex2(-aB.y));
+            if (MASK) {  // t_j != t_i
+                const int r0 = h ? rk.z : rk.x, r1 = h ? rk.w : rk.y;
+                B.x = (r0 < w.lo || r0 >= w.hi) ? B.x : 0.f;
+                B.y = (r1 < w.lo || r1 >= w.hi) ? B.y : 0.f;
+            }
+            w.sB = add2(w.sB, B);
+            if (!LL) {
+                w.sBr = fma2(B, r2, w.sBr);
+                w.sBt = fma2(B, dt2, w.sBt);
+            }
+        }
     }
-    __syncthreads();
-    uint32_t parbits = 0u, pendbits = 0u;
+}
+
+// Excitation of `quads` x 4 buffered columns (planes as above, then -beta, ce).
+template <bool MASK, bool LL>
+__device__ __forceinline__ void sp_eval_e(const float* __restrict__ buf, int quads, float2 nomt, SpRow& w) {
+#pragma unroll 1
+    for (int q = 0; q < quads; ++q) {
+        const float4* p = reinterpret_cast<const float4*>(buf) + q;
+        const float4 xh = p[0 * SP_BUF / 4], xl = p[1 * SP_BUF / 4], yh = p[2 * SP_BUF / 4],
+                     yl = p[3 * SP_BUF / 4], th = p[4 * SP_BUF / 4], tl = p[5 * SP_BUF / 4],
+                     nb = p[7 * SP_BUF / 4], ce = p[8 * SP_BUF / 4];
+        int4 rk;
+        if (MASK) rk = *reinterpret_cast<const int4*>(p + 6 * SP_BUF / 4);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 dt = add2(add2(w.th, half4(th, h)), add2(w.tl, half4(tl, h)));
+            const float2 dx = add2(add2(w.xh, half4(xh, h)), add2(w.xl, half4(xl, h)));
+            const float2 dy = add2(add2(w.yh, half4(yh, h)), add2(w.yl, half4(yl, h)));
+            const float2 r2 = fma2(dy, dy, mul2(dx, dx));
+            const float2 nv = mul2(half4(nb, h), r2);
+            const float2 arg = add2(fma2(nomt, dt, nv), half4(ce, h));
+            float2 E = f2(ex2(arg.x), ex2(arg.y));
+            if (MASK) {  // t_j < t_i
+                const int r0 = h ? rk.z : rk.x, r1 = h ? rk.w : rk.y;
+                E.x = r0 < w.lo ? E.x : 0.f;
+                E.y = r1 < w.lo ? E.y : 0.f;
+            }
+            w.sE = add2(w.sE, E);
+            if (!LL) {
+                w.sEt = fma2(E, dt, w.sEt);
+                w.sEq = fma2(E, nv, w.sEq);
+            }
+        }
+    }
+}
+
+// Shared memory of a warp: the two column buffers and the chunk list.
+struct SpWarp {
+    float b[SP_B_PLANES * SP_BUF];
+    float e[SP_E_PLANES * SP_BUF];
+    int list[SP_LIST];
+};
+
+// Persistent warps over items (row group, part of the column tiles).
+template <bool LL>
+__global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int* __restrict__ ctr, int nitems) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31;
+    SpWarp& sw = reinterpret_cast<SpWarp*>(smem)[threadIdx.x >> 5];
     const double* cc = a.cc;
+    if (cc[CC_VALID] == 0.0) return;
     const float omt = static_cast<float>(cc[CC_OMT]);
     const float2 nomt = f2(-omt, -omt);
-    const double kt = cc[CC_KT];
+    const unsigned below = (1u << lane) - 1u;
+    constexpr unsigned ALL = 0xffffffffu;
 
     for (;;) {
-        if (tid == 0) s_item = atomicAdd(ctr + CT_WORK, 1);
-        __syncthreads();
-        const int item = s_item;
-        if (item >= nitems || s_abort) break;
-        const int I = item / a.nch;
-        const int cb = (item % a.nch) * a.chunk;
-        const int cend = min(cb + a.chunk, a.ntiles);
-        // the CTA's rows: tiles 8 I .. 8 I + 7 of the order
-        SpRange rows;
-        rows.empty = true;
-        for (int w = 0; w < WARPS; ++w) sp_union(rows, sp_tile(a.tmeta, a.box, I * WARPS + w));
-        // list the chunk's column tiles that can hold a nonzero term
-        const int jt_mine = cb + tid;
-        const bool keep = jt_mine < cend && !sp_all_zero(rows, sp_tile(a.tmeta, a.box, jt_mine), cc, a.model1);
-        const unsigned bal = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) s_wcount[warp] = __popc(bal);
-        __syncthreads();
-        int base = 0;
-        for (int w = 0; w < warp; ++w) base += s_wcount[w];
-        if (keep) s_list[base + __popc(bal & ((1u << lane) - 1u))] = jt_mine;
-        if (tid == 0) {
-            int tot = 0;
-            for (int w = 0; w < WARPS; ++w) tot += s_wcount[w];
-            s_nlist = tot;
+        int item = 0;
+        if (lane == 0) item = atomicAdd(ctr + CT_WORK, 1);
+        item = __shfl_sync(ALL, item, 0);
+        if (item >= nitems) return;
+        const int g = item / a.parts, part = item % a.parts;
+        const int64_t p0 = static_cast<int64_t>(g) * SP_CH;
+        const SpBox box = sp_load(a.cmeta, g);
+        if (!(box.x0 <= box.x1)) continue;  // padding only
+        SpRow w;
+        const int rr = a.rank[p0 + lane];
+        const int e = rr >= 0 ? rr & ~SP_TIED : -1;
+        {
+            const float4 qa = a.ra[p0 + lane], qb = a.rb[p0 + lane];
+            w.xh = f2(-qa.x, -qa.x); w.xl = f2(-qa.y, -qa.y);
+            w.yh = f2(-qa.z, -qa.z); w.yl = f2(-qa.w, -qa.w);
+            w.th = f2(-qb.x, -qb.x); w.tl = f2(-qb.y, -qb.y);
         }
-        __syncthreads();
-        const int nJ = s_nlist;
-        if (nJ == 0) continue;  // the next item is fetched after the barrier at the loop top
+        w.lo = e >= 0 ? a.lo[e] : 0;
+        w.hi = e >= 0 ? a.hi[e] : 0;
+        w.sB = w.sBr = w.sBt = w.sE = w.sEt = w.sEq = f2(0.f, 0.f);
+        // time-order indices that some row must be compared with one by one
+        const int lo_min = __reduce_min_sync(ALL, e >= 0 ? w.lo : 0x7fffffff);
+        const int hi_max = __reduce_max_sync(ALL, e >= 0 ? w.hi : 0);
 
-        // rows of this warp: one tile of the order
-        const int wtile = I * WARPS + warp;
-        const int64_t r0 = static_cast<int64_t>(wtile) * TC;
-        const SpRange mine = sp_tile(a.tmeta, a.box, wtile);
-        const bool live = !mine.empty;
-        Rows<SP_RP> rr;
-        float t0h[SP_R], t0l[SP_R];
-        int lo[SP_R], hi[SP_R], rk[SP_R];
-#pragma unroll
-        for (int p = 0; p < SP_RP; ++p) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int64_t i = r0 + lane + 64 * p + 32 * h;
-                const float4 qa = *rec_q(a.rec, i, 0), qb = *rec_q(a.rec, i, 1);
-                const float4 qc = *rec_q(a.rec, i, 2), qd = *rec_q(a.rec, i, 3);
-                const int e = __float_as_int(qd.w);
-                rk[2 * p + h] = e;
-                const bool real = e >= 0 && e < a.n;
-                lo[2 * p + h] = real ? a.lo[e] : 0;
-                hi[2 * p + h] = real ? a.hi[e] : 0;
-                t0h[2 * p + h] = -qa.x;
-                t0l[2 * p + h] = -qd.z;
-                if (h == 0) {
-                    rr.xh[p].x = -qa.z; rr.xl[p].x = -qb.x; rr.yh[p].x = -qb.z; rr.yl[p].x = -qc.x;
-                } else {
-                    rr.xh[p].y = -qa.z; rr.xl[p].y = -qb.x; rr.yh[p].y = -qb.z; rr.yl[p].y = -qc.x;
+        int nB = 0, nE = 0;            // buffered columns
+        bool maskB = false, maskE = false;
+        int tile0 = 0;                 // next round of 32 tiles (of this part)
+        unsigned mT = 0;               // surviving tiles of the current round
+        int nlist = 0;
+        for (;;) {
+            // list chunks that can hold a nonzero term
+            while (nlist <= SP_LIST - 32) {
+                if (mT == 0) {
+                    const int first = tile0 * a.parts + part;
+                    if (first >= a.ntiles) break;
+                    const int t = (tile0 + lane) * a.parts + part;
+                    bool nb = false, ne = false;
+                    if (t < a.ntiles) sp_near(box, sp_load(a.tmeta, t), omt, nb, ne);
+                    mT = __ballot_sync(ALL, nb || ne);
+                    if (mT == 0) tile0 += 32;
+                    continue;
                 }
+                // the 8 chunks of the next (up to) 4 surviving tiles
+                unsigned m = mT;
+                for (int k = 0; k < 4; ++k) mT &= mT - 1;
+                for (int k = 0; k < (lane >> 3); ++k) m &= m - 1;
+                const bool has = m != 0;
+                const int t = has ? (tile0 + __ffs(m) - 1) * a.parts + part : 0;
+                const int ch = t * (TC / SP_CH) + (lane & 7);
+                bool nb = false, ne = false;
+                if (has) sp_near(box, sp_load(a.cmeta, ch), omt, nb, ne);
+                const unsigned keep = __ballot_sync(ALL, nb || ne);
+                if (nb || ne) sw.list[nlist + __popc(keep & below)] = ch | (nb ? 1 << 29 : 0) | (ne ? 1 << 30 : 0);
+                nlist += __popc(keep);
+                if (mT == 0) tile0 += 32;
             }
-            rr.sB[p] = rr.sBr[p] = rr.sBt[p] = rr.sE[p] = rr.sEt[p] = rr.sEq[p] = f2(0.f, 0.f);
-        }
-
-        if (tid == 0) {
-            for (int q = 0; q < 2 && q < nJ; ++q) {
-                mbar_arrive_expect_tx(&bars[q], TC * sizeof(Rec));
-                tma_load_1d(tiles + q * TC, a.rec + static_cast<int64_t>(s_list[q]) * TC, TC * sizeof(Rec),
-                            &bars[q]);
-                pendbits |= 1u << q;
-            }
-        }
-        for (int J = 0; J < nJ; ++J) {
-            const int buf = J & 1;
-            if (!mbar_wait(&bars[buf], (parbits >> buf) & 1u)) {
-                set_error(ctr, HAWKES_ERR_TIMEOUT);
-                s_abort = 1;
-            }
-            parbits ^= 1u << buf;
-            pendbits &= ~(1u << buf);
-            const int jt = s_list[J];
-            const SpRange col = sp_tile(a.tmeta, a.box, jt);
-            if (live && !s_abort && !sp_all_zero(mine, col, cc, a.model1)) {
-                // row times against this tile's base: two-word sums, exact in the hi part
-                const double dT = (mine.t0 - col.t0) * kt;
-                const float dTh = static_cast<float>(dT), dTl = static_cast<float>(dT - static_cast<double>(dTh));
-                float2 tl[SP_RP];
-#pragma unroll
-                for (int p = 0; p < SP_RP; ++p) {
-                    float hv[2], lv[2];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const float u = t0h[2 * p + h], v = dTh;
-                        const float sm = __fadd_rn(u, v);
-                        const float vb = __fsub_rn(sm, u);
-                        const float ua = __fsub_rn(sm, vb);
-                        const float err = __fadd_rn(__fsub_rn(u, ua), __fsub_rn(v, vb));
-                        hv[h] = sm;
-                        lv[h] = __fadd_rn(err, __fadd_rn(t0l[2 * p + h], dTl));
-                    }
-                    rr.tp[p] = f2(hv[0], hv[1]);
-                    tl[p] = f2(lv[0], lv[1]);
+            __syncwarp();
+            if (nlist == 0) break;
+            // read the listed chunks, one event per lane, the next one ahead
+            int cur = sw.list[0];
+            int64_t p = static_cast<int64_t>(cur & ((1 << 29) - 1)) * SP_CH + lane;
+            float4 qa = a.ra[p], qb = a.rb[p];
+            int rk = a.rank[p];
+            for (int k = 0; k < nlist; ++k) {
+                const int id = cur;
+                const float4 ca = qa, cb = qb;
+                const int rank = rk & ~SP_TIED;
+                const bool real = rk >= 0;
+                const bool tied = (rk & SP_TIED) != 0 || (id & ((1 << 29) - 1)) == g;
+                if (k + 1 < nlist) {
+                    cur = sw.list[k + 1];
+                    p = static_cast<int64_t>(cur & ((1 << 29) - 1)) * SP_CH + lane;
+                    qa = a.ra[p];
+                    qb = a.rb[p];
+                    rk = a.rank[p];
                 }
-                const float4* tile = reinterpret_cast<const float4*>(tiles + buf * TC);
-                const bool partial = (static_cast<int64_t>(jt) + 1) * TC > a.n;
-                if (!partial && col.t1 < mine.t0)  // every source strictly earlier
-                    sp_tile_pass<8, false, true>(tile, lane, rr, tl, nomt, lo, hi);
-                else if (!partial && col.t0 > mine.t1)  // every source strictly later
-                    sp_tile_pass<8, false, false>(tile, lane, rr, tl, nomt, lo, hi);
-                else
-                    sp_tile_pass<8, true, true>(tile, lane, rr, tl, nomt, lo, hi);
-            }
-            __syncthreads();
-            if (tid == 0 && J + 2 < nJ && !s_abort) {
-                mbar_arrive_expect_tx(&bars[buf], TC * sizeof(Rec));
-                tma_load_1d(tiles + buf * TC, a.rec + static_cast<int64_t>(s_list[J + 2]) * TC,
-                            TC * sizeof(Rec), &bars[buf]);
-                pendbits |= 1u << buf;
-            }
-            if (s_abort) break;
-        }
-        if (live && !s_abort) {
-            const double sr = cc[CC_SR], st = cc[CC_ST], set = cc[CC_SET], seq = cc[CC_SEQ];
-#pragma unroll
-            for (int p = 0; p < SP_RP; ++p) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int e = rk[2 * p + h];
-                    if (e < 0 || e >= a.n) continue;
-                    const float vB = h ? rr.sB[p].y : rr.sB[p].x, vBr = h ? rr.sBr[p].y : rr.sBr[p].x;
-                    const float vBt = h ? rr.sBt[p].y : rr.sBt[p].x, vE = h ? rr.sE[p].y : rr.sE[p].x;
-                    const float vEt = h ? rr.sEt[p].y : rr.sEt[p].x, vEq = h ? rr.sEq[p].y : rr.sEq[p].x;
-                    if (vB != 0.f || vBr != 0.f || vBt != 0.f) {
-                        atomicAdd(a.acc + 0 * a.npad + e, static_cast<double>(vB));
-                        atomicAdd(a.acc + 1 * a.npad + e, static_cast<double>(vBr) * sr);
-                        atomicAdd(a.acc + 2 * a.npad + e, static_cast<double>(vBt) * st);
+                const float dx = sp_gap(box.x0, box.x1, -ca.x, -ca.x), dy = sp_gap(box.y0, box.y1, -ca.z, -ca.z);
+                const float r2 = fmaf(dx, dx, dy * dy);
+                if (id & (1 << 29)) {
+                    const float gap = sp_gap(box.t0, box.t1, -cb.x, -cb.x);
+                    const bool keep = real && !(fmaf(gap, gap, r2) > SP_ZERO);
+                    const unsigned bal = __ballot_sync(ALL, keep);
+                    maskB |= __any_sync(ALL, keep && tied && rank >= lo_min && rank < hi_max);
+                    if (keep) {
+                        float* b = sw.b + nB + __popc(bal & below);
+                        b[0 * SP_BUF] = ca.x; b[1 * SP_BUF] = ca.y; b[2 * SP_BUF] = ca.z; b[3 * SP_BUF] = ca.w;
+                        b[4 * SP_BUF] = cb.x; b[5 * SP_BUF] = cb.y; b[6 * SP_BUF] = __int_as_float(rank);
                     }
-                    if (vE != 0.f || vEt != 0.f || vEq != 0.f) {
-                        atomicAdd(a.acc + 3 * a.npad + e, static_cast<double>(vE));
-                        atomicAdd(a.acc + 4 * a.npad + e, static_cast<double>(vEt) * set);
-                        atomicAdd(a.acc + 5 * a.npad + e, -static_cast<double>(vEq) * seq);
+                    nB += __popc(bal);
+                    if (nB >= 32) {
+                        __syncwarp();
+                        if (maskB) sp_eval_b<true, LL>(sw.b, 8, w);
+                        else sp_eval_b<false, LL>(sw.b, 8, w);
+                        nB -= 32;
+                        maskB = maskB && nB > 0;
+                        __syncwarp();
+                        if (lane < nB)
+#pragma unroll
+                            for (int q = 0; q < SP_B_PLANES; ++q) sw.b[q * SP_BUF + lane] = sw.b[q * SP_BUF + 32 + lane];
+                        __syncwarp();
+                    }
+                }
+                if (id & (1 << 30)) {
+                    const float tj = -cb.x;
+                    const bool keep = real && tj <= box.t1 &&
+                                      !(cb.w - omt * fmaxf(0.f, box.t0 - tj) + cb.z * r2 < -SP_ZERO);
+                    const unsigned bal = __ballot_sync(ALL, keep);
+                    maskE |= __any_sync(ALL, keep && rank >= lo_min);
+                    if (keep) {
+                        float* b = sw.e + nE + __popc(bal & below);
+                        b[0 * SP_BUF] = ca.x; b[1 * SP_BUF] = ca.y; b[2 * SP_BUF] = ca.z; b[3 * SP_BUF] = ca.w;
+                        b[4 * SP_BUF] = cb.x; b[5 * SP_BUF] = cb.y; b[6 * SP_BUF] = __int_as_float(rank);
+                        b[7 * SP_BUF] = cb.z; b[8 * SP_BUF] = cb.w;
+                    }
+                    nE += __popc(bal);
+                    if (nE >= 32) {
+                        __syncwarp();
+                        if (maskE) sp_eval_e<true, LL>(sw.e, 8, nomt, w);
+                        else sp_eval_e<false, LL>(sw.e, 8, nomt, w);
+                        nE -= 32;
+                        maskE = maskE && nE > 0;
+                        __syncwarp();
+                        if (lane < nE)
+#pragma unroll
+                            for (int q = 0; q < SP_E_PLANES; ++q) sw.e[q * SP_BUF + lane] = sw.e[q * SP_BUF + 32 + lane];
+                        __syncwarp();
                     }
                 }
             }
+            nlist = 0;
+            __syncwarp();
         }
-        __syncthreads();
-        if (s_abort) break;
+        // what is left in the buffers, filled up to quads with columns whose
+        // terms are zero
+        const int qB = (nB + 3) >> 2, qE = (nE + 3) >> 2;
+        if (nB + lane < 4 * qB) {
+            for (int q = 0; q < SP_B_PLANES; ++q) sw.b[q * SP_BUF + nB + lane] = 0.f;
+            sw.b[4 * SP_BUF + nB + lane] = -PAD_T;
+        }
+        if (nE + lane < 4 * qE) {
+            for (int q = 0; q < SP_E_PLANES; ++q) sw.e[q * SP_BUF + nE + lane] = 0.f;
+            sw.e[8 * SP_BUF + nE + lane] = -1e30f;
+        }
+        __syncwarp();
+        if (maskB) sp_eval_b<true, LL>(sw.b, qB, w);
+        else sp_eval_b<false, LL>(sw.b, qB, w);
+        if (maskE) sp_eval_e<true, LL>(sw.e, qE, nomt, w);
+        else sp_eval_e<false, LL>(sw.e, qE, nomt, w);
+        __syncwarp();
+        if (e >= 0) {
+            const float v[6] = {w.sB.x + w.sB.y, w.sBr.x + w.sBr.y, w.sBt.x + w.sBt.y,
+                                w.sE.x + w.sE.y, w.sEt.x + w.sEt.y, w.sEq.x + w.sEq.y};
+            double* acc = a.acc + e;
+            if (v[0] != 0.f) atomicAdd(acc, static_cast<double>(v[0]));
+            if (v[3] != 0.f) atomicAdd(acc + 3 * a.npad, static_cast<double>(v[3]));
+            if (!LL) {
+                if (v[1] != 0.f) atomicAdd(acc + 1 * a.npad, static_cast<double>(v[1]) * cc[CC_SR]);
+                if (v[2] != 0.f) atomicAdd(acc + 2 * a.npad, static_cast<double>(v[2]) * cc[CC_ST]);
+                if (v[4] != 0.f) atomicAdd(acc + 4 * a.npad, static_cast<double>(v[4]) * cc[CC_SET]);
+                if (v[5] != 0.f) atomicAdd(acc + 5 * a.npad, -static_cast<double>(v[5]) * cc[CC_SEQ]);
+            }
+        }
     }
-    // A wait that gave up may leave bulk copies in flight: let them land
-    // (bounded) before the CTA's shared memory is released.
-    if (tid == 0)
-        for (int q = 0; q < 2; ++q)
-            if ((pendbits >> q) & 1u) (void)mbar_wait(&bars[q], (parbits >> q) & 1u);
 }
 
 // Queue the spatial path's staging and sweep (after k_prep has written the
-// per-call constants and zeroed the accumulators).
-cudaError_t spatial_launch(hawkes_ctx* c, int model1) {
+// per-call constants and zeroed the accumulators).  The records take the place
+// of the staged records of the other paths.
+cudaError_t spatial_launch(hawkes_ctx* c, int model1, int llonly) {
     SpatialState* sp = c->sp;
-    const int g = c->sms * 8;
-    k_sp_prep<<<g, 256, 0, c->stream>>>(sp->perm, sp->tmeta, c->t, c->x, c->y, c->is2, c->ce, c->cc, model1, c->npad,
-                                         c->rec);
-    k_sp_box<<<(sp->ntiles * 32 + 255) / 256, 256, 0, c->stream>>>(sp->perm, c->x, c->y, sp->ntiles, sp->box);
+    float4* ra = reinterpret_cast<float4*>(c->rec);
+    float4* rb = ra + c->npad;
+    k_sp_prep<<<std::min(sp->ntiles, 8 * c->sms), TC, 0, c->stream>>>(eval_desc(c), sp->rank, model1, ra, rb,
+                                                                      sp->meta, sp->ntiles);
     SpArgs a;
-    a.rec = c->rec; a.lo = c->lo; a.hi = c->hi; a.cc = c->cc; a.acc = c->acc;
-    a.tmeta = sp->tmeta; a.box = sp->box; a.n = c->n; a.npad = c->npad;
+    a.ra = ra; a.rb = rb; a.rank = sp->rank; a.lo = c->lo; a.hi = c->hi; a.cc = c->cc; a.acc = c->acc;
+    a.cmeta = sp->meta;
+    a.tmeta = sp->meta + 2 * static_cast<size_t>(sp->ntiles) * (TC / SP_CH);
+    a.npad = c->npad;
     a.ntiles = sp->ntiles;
-    a.nI = static_cast<int>(c->npad / SP_TR);
-    // column chunks of up to SP_CH tiles, halved until there are at least 4
-    // items per SM (smaller problems would otherwise leave SMs idle)
-    a.chunk = SP_CH;
-    while (a.chunk > 32 && static_cast<int64_t>(a.nI) * ((sp->ntiles + a.chunk - 1) / a.chunk) <
-                               4LL * c->sms)
-        a.chunk /= 2;
-    a.nch = (sp->ntiles + a.chunk - 1) / a.chunk;
-    a.model1 = model1;
-    const int nitems = a.nI * a.nch;
-    const size_t smem = 2 * TC * sizeof(Rec);  // 32 KB: below the default dynamic limit
-    const int grid = std::min(nitems, c->sms);
-    if (grid <= 0) return cudaSuccess;
-    k_sweep_sp<<<grid, THREADS, smem, c->stream>>>(a, c->ctr, nitems);
+    a.groups = static_cast<int>((c->n + SP_CH - 1) / SP_CH);
+    // Few rows: several warps share a group's columns, until there are a
+    // resident CTA's worth of warps for every SM.
+    const size_t smem = SP_WARPS * sizeof(SpWarp);
+    auto* kern = llonly ? k_sweep_sp<true> : k_sweep_sp<false>;
+    static_assert(SP_WARPS * sizeof(SpWarp) <= 48 * 1024, "below the default dynamic limit");
+    a.parts = 1;
+    while (a.parts < 64 && 2 * a.parts <= a.ntiles &&
+           static_cast<int64_t>(a.groups) * a.parts < static_cast<int64_t>(c->sms) * SP_BPSM * SP_WARPS)
+        a.parts *= 2;
+    const int64_t nitems = static_cast<int64_t>(a.groups) * a.parts;
+    const int grid = static_cast<int>(std::min<int64_t>((nitems + SP_WARPS - 1) / SP_WARPS,
+                                                        static_cast<int64_t>(c->sms) * SP_BPSM));
+    kern<<<grid, SP_THREADS, smem, c->stream>>>(a, c->ctr, static_cast<int>(nitems));
     return cudaGetLastError();
 }
 
