@@ -17,9 +17,8 @@ __global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const 
                        const __grid_constant__ hawkes_params,
                        int, int, int, int, const uint64_t*, int*);
 void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
-                     double*, double*, double*);
-__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, int, double*,
-                         double*);
+                     const double*, int, double*, double*, double*);
+__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, double*, double*);
 __global__ void k_flushfix(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, double*, double*,
                            double*);
 __global__ void k_tri_area(const double*, int32_t, double*, int*);
@@ -37,6 +36,10 @@ cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row
                          bool ll);
 cudaError_t launch_sweep_list(hawkes_ctx* c, const int4* items, int nitems, bool bgt, bool ll);
 int sweep_variant_rows(int v);
+// rows64.cu
+int rows64_segments(int64_t rows, int sms);
+size_t rows64_scratch(int sms);
+cudaError_t launch_pairs64(const hawkes_ctx* c, bool model1, bool bgt, int64_t rb, int64_t re, double* out);
 // sweep_spatial.cu
 int spatial_build(hawkes_ctx* c, const hawkes_params* p, const hawkes_params* d_p);
 cudaError_t spatial_launch(hawkes_ctx* c, int model1, int llonly);
@@ -193,11 +196,11 @@ int enqueue_prep(hawkes_ctx* c, const CallParams& cp, int model, int stage, int 
     });
 }
 
-int enqueue_rows(hawkes_ctx* c, int64_t rb, int64_t re, int check, double* d_out, double* d_rows9,
-                 double* d_err) {
+int enqueue_rows(hawkes_ctx* c, int64_t rb, int64_t re, int check, int nparts, double* d_out,
+                 double* d_rows9, double* d_err) {
     return timed(c, HAWKES_K_FINAL, [&] {
-        launch_finalize(c->stream, final_grid(re - rb, c->sms), eval_desc(c), nullptr, rb, re, check, d_out,
-                        d_rows9, d_err);
+        launch_finalize(c->stream, final_grid(re - rb, c->sms), eval_desc(c), nullptr, rb, re, check,
+                        c->parts64, nparts, d_out, d_rows9, d_err);
     });
 }
 
@@ -210,9 +213,9 @@ int enqueue_rows(hawkes_ctx* c, int64_t rb, int64_t re, int check, double* d_out
 int enqueue_finalize32(hawkes_ctx* c, int model, int64_t rb, int64_t re, double* d_out,
                        double* d_rows9, double* d_err) {
     const EvalDesc d = eval_desc(c);
-    HK_TRY(enqueue_rows(c, rb, re, 1, d_out, d_rows9, nullptr));
+    HK_TRY(enqueue_rows(c, rb, re, 1, 1, d_out, d_rows9, nullptr));
     HK_TRY(timed(c, HAWKES_K_ROWS64, [&] {
-        k_rows64<<<c->sms, 256, 0, c->stream>>>(d, nullptr, model, 0, re - rb, 1, d_out, d_rows9);
+        k_rows64<<<c->sms, 256, 0, c->stream>>>(d, nullptr, model, re - rb, d_out, d_rows9);
     }));
     return timed(c, HAWKES_K_ROWS64, [&] {
         k_flushfix<<<grid_for(c, re - rb, 2), 256, 0, c->stream>>>(d, nullptr, model, rb, re, d_out,
@@ -245,14 +248,13 @@ int enqueue_loglik(hawkes_ctx* c, const CallParams& cp, uint32_t flags, int64_t 
         HK_CUDA(se);
         return enqueue_finalize32(c, model, rb, re, d_out, d_rows9, d_err);
     }
-    const EvalDesc d = eval_desc(c);
-    const int64_t count = re - rb;
-    int g = static_cast<int>(count < static_cast<int64_t>(c->sms) * 16 ? count : c->sms * 16);
-    if (g < 1) g = 1;
+    const int nparts = rows64_segments(re - rb, c->sms);
+    cudaError_t e64 = cudaSuccess;
     HK_TRY(timed(c, HAWKES_K_ROWS64, [&] {
-        k_rows64<<<g, 256, 0, c->stream>>>(d, nullptr, model, rb, count, 0, nullptr, nullptr);
+        e64 = launch_pairs64(c, (flags & HAWKES_MODEL1) != 0, bgt, rb, re, nparts > 1 ? c->parts64 : c->acc);
     }));
-    return enqueue_rows(c, rb, re, 0, d_out, d_rows9, d_err);
+    HK_CUDA(e64);
+    return enqueue_rows(c, rb, re, 0, nparts, d_out, d_rows9, d_err);
 }
 
 int sync_loglik(hawkes_ctx* c, const hawkes_params* p, uint32_t flags, int64_t rb, int64_t re,
@@ -341,6 +343,7 @@ int hawkes_create(hawkes_ctx** out, int device, void* cuda_stream) {
         if ((rc = dalloc(&c->cc, CC_COUNT)) != HAWKES_OK) break;
         if ((rc = dalloc(&c->out_dev, 8)) != HAWKES_OK) break;
         if ((rc = dalloc(&c->fix7, FIX_DOUBLES)) != HAWKES_OK) break;
+        if ((rc = dalloc(&c->parts64, rows64_scratch(c->sms))) != HAWKES_OK) break;
         if ((rc = dalloc(&c->partials, static_cast<size_t>(PART_STRIDE * BPSM * c->sms))) != HAWKES_OK)
             break;
         if (cudaMallocHost(reinterpret_cast<void**>(&c->out_host), 8 * sizeof(double)) != cudaSuccess) {
@@ -377,6 +380,7 @@ void hawkes_destroy(hawkes_ctx* c) {
     spatial_free(c);
     dfree(c->ctr); dfree(c->cc); dfree(c->out_dev); dfree(c->fix7);
     dfree(c->partials);
+    dfree(c->parts64);
     if (c->out_host) cudaFreeHost(c->out_host);
     for (auto& e : c->pev)
         if (e) cudaEventDestroy(e);

@@ -22,9 +22,8 @@ __global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const 
                        const __grid_constant__ hawkes_params,
                        int, int, int, int, const uint64_t*, int*);
 void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
-                     double*, double*, double*);
-__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, int, double*,
-                         double*);
+                     const double*, int, double*, double*, double*);
+__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, double*, double*);
 __global__ void k_flushfix(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, double*, double*,
                            double*);
 int sweep_num_variants();
@@ -340,10 +339,10 @@ int enqueue(hawkes_batch* b, const hawkes_params* d_params, double* d_out, bool 
     HB_CUDA(launch_sweep_batch(st, b->plan, b->sms, b->variant, b->grid, b->d_probs, P, b->d_items,
                                b->nitems, b->d_ctr, bgt, (b->flags & HAWKES_LOGLIK_ONLY) != 0));
     if (time_sweep) HB_CUDA(cudaEventRecord(b->ev[1], st));
-    launch_finalize(st, dim3(final_grid(nmax, b->sms, P), P), EvalDesc{}, b->d_eval, 0, 0, 1, d_out,
-                    nullptr, nullptr);
+    launch_finalize(st, dim3(final_grid(nmax, b->sms, P), P), EvalDesc{}, b->d_eval, 0, 0, 1, nullptr,
+                    1, d_out, nullptr, nullptr);
     const int fix = std::max(2 * b->sms / P, 8);  // blocks per problem for the fix-ups (usually idle)
-    k_rows64<<<dim3(fix, P), 256, 0, st>>>(EvalDesc{}, b->d_eval, model, 0, 0, 1, d_out, nullptr);
+    k_rows64<<<dim3(fix, P), 256, 0, st>>>(EvalDesc{}, b->d_eval, model, 0, d_out, nullptr);
     k_flushfix<<<dim3(fix, P), 256, 0, st>>>(EvalDesc{}, b->d_eval, model, 0, 0, d_out, nullptr, nullptr);
     HB_CUDA(cudaGetLastError());
     return HAWKES_OK;

@@ -356,6 +356,7 @@ struct hawkes_ctx {
     double* acc = nullptr;     // [6 * npad] per-row moment sums (natural units)
     double* partials = nullptr;// [BPSM * sms * PART_STRIDE]
     double* fix7 = nullptr;    // [FIX_DOUBLES]
+    double* parts64 = nullptr; // [rows64_scratch] FP64 path: column segments' sums of few rows
     int* fixlist = nullptr;    // [npad]
     int* ctr = nullptr;        // [CT_COUNT]
     double* cc = nullptr;      // [CC_COUNT]

@@ -430,11 +430,14 @@ __device__ __forceinline__ void finish_outputs(const double* tot, const volatile
 // then a third as long, which is what few rows wait for (N = 2,000: 57 us as
 // 8 blocks of 256 whole rows, 19.5 in blocks of 64); many rows are bound by
 // the FP64 rate either way.
+// nparts > 1 (FP64 path): the moment sums are in nparts pieces, parts64[piece][6]
+// [rows rounded up to 32] (see k_pairs64).
 // err_out (optional): receives the latched error status as a double.
 template <bool ROWS>
 __global__ void __launch_bounds__(FINAL_THREADS)
     k_finalize(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs, int64_t rb,
-               int64_t re, int check, double* out, double* rows9, double* err_out) {
+               int64_t re, int check, const double* __restrict__ parts64, int nparts, double* out,
+               double* rows9, double* err_out) {
     const EvalDesc& d = probs ? probs[blockIdx.y] : one;
     if (probs) {
         rb = 0;
@@ -456,8 +459,17 @@ __global__ void __launch_bounds__(FINAL_THREADS)
         const double ti = d.t[i], mu = cc[CC_MU], th = cc[CC_TH];
         if (part == 0) {
             double S[6];
+            if (nparts > 1) {
+                const int64_t stride = (re - rb + 31) / 32 * 32;
 #pragma unroll
-            for (int q = 0; q < 6; ++q) S[q] = d.acc[q * npad + i];
+                for (int q = 0; q < 6; ++q) S[q] = parts64[q * stride + i - rb];
+                for (int k = 1; k < nparts; ++k)
+#pragma unroll
+                    for (int q = 0; q < 6; ++q) S[q] += parts64[(6 * k + q) * stride + i - rb];
+            } else {
+#pragma unroll
+                for (int q = 0; q < 6; ++q) S[q] = d.acc[q * npad + i];
+            }
             const bool queue = check && LB * S[0] + LE * S[3] < thr;
             if (queue) {
                 const int k = atomicAdd(ctr + CT_FIX, 1);
@@ -550,11 +562,14 @@ __global__ void __launch_bounds__(FINAL_THREADS)
 }
 
 void launch_finalize(cudaStream_t st, dim3 grid, const EvalDesc& one, const EvalDesc* probs, int64_t rb,
-                     int64_t re, int check, double* out, double* rows9, double* err_out) {
+                     int64_t re, int check, const double* parts64, int nparts, double* out, double* rows9,
+                     double* err_out) {
     if (rows9)
-        k_finalize<true><<<grid, FINAL_THREADS, 0, st>>>(one, probs, rb, re, check, out, rows9, err_out);
+        k_finalize<true><<<grid, FINAL_THREADS, 0, st>>>(one, probs, rb, re, check, parts64, nparts, out, rows9,
+                                                         err_out);
     else
-        k_finalize<false><<<grid, FINAL_THREADS, 0, st>>>(one, probs, rb, re, check, out, rows9, err_out);
+        k_finalize<false><<<grid, FINAL_THREADS, 0, st>>>(one, probs, rb, re, check, parts64, nparts, out, rows9,
+                                                          err_out);
 }
 
 // This thread's share (sources j = threadIdx.x + k blockDim.x) of row i's six
@@ -586,20 +601,18 @@ __device__ __forceinline__ void row_sums64(const EvalDesc& d, int64_t i, bool mo
 }
 
 // ---------------------------------------------------------------------------
-// FP64 pair rows: one CTA per row, threads stride over all sources.
-// mode 0: rows row_begin + [0, count) -> write natural-unit sums to acc
-// mode 1: the queued rows fixlist[0 .. ctr[CT_FIX]) -> finalise, add into fix7;
-//         the last block then writes the outputs (see k_finalize).  Returns at
-//         once when no row is queued.
+// The rows that k_finalize queued, in FP64: one CTA per row, threads stride over
+// all sources; the rows' lambda terms are added into fix7, and the last block
+// writes the outputs (see k_finalize).  Returns at once when no row is queued.
+// nrows: rows of the call (batches: all of the problem).
 // ---------------------------------------------------------------------------
 __global__ void k_rows64(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs,
-                         int model, int64_t row_begin, int64_t count, int mode, double* out,
-                         double* rows9) {
+                         int model, int64_t nrows, double* out, double* rows9) {
     const EvalDesc& d = probs ? probs[blockIdx.y] : one;
-    const int64_t n = d.n, npad = d.npad;
+    const int64_t n = d.n;
     double* cc = d.cc;
     int* ctr = d.ctr;
-    const int64_t total = mode ? static_cast<int64_t>(ctr[CT_FIX]) : count;
+    const int64_t total = ctr[CT_FIX];
     if (cc[CC_VALID] == 0.0 || total == 0) return;
     const bool model1 = (model & HAWKES_MODEL1) != 0;
     const double tx = cc[CC_TX], tt = cc[CC_TT], om = cc[CC_OM], h = cc[CC_H];
@@ -608,8 +621,8 @@ __global__ void k_rows64(const __grid_constant__ EvalDesc one, const EvalDesc* _
     const double it2 = 1.0 / (2.0 * tt * tt), ih2 = 1.0 / (2.0 * h * h);
     __shared__ double sums[8];
     for (int64_t k = blockIdx.x; k < total; k += gridDim.x) {
-        const int64_t i = mode ? d.fixlist[k] : row_begin + k;
-        if (kDebug && !(i >= 0 && i < n && (mode || k < npad))) {
+        const int64_t i = d.fixlist[k];
+        if (kDebug && !(i >= 0 && i < n)) {
             if (threadIdx.x == 0) set_error(ctr, HAWKES_ERR_BOUNDS);
             continue;  // uniform over the block: i depends on k only
         }
@@ -618,23 +631,18 @@ __global__ void k_rows64(const __grid_constant__ EvalDesc one, const EvalDesc* _
         block_reduce_store<6>(v, sums);
         __syncthreads();
         if (threadIdx.x == 0) {
-            if (mode == 0) {
-                for (int q = 0; q < 6; ++q) d.acc[q * npad + i] = sums[q];
-            } else {
-                // (k_finalize has the row's Lambda terms)
-                double o[9], b[7], loglam, dl[6];
-                row_lambda<false>(sums, d.t[i], 0.0, 0.0, 0.0, cc, loglam, dl, b);
-                atomicAdd(d.fix7, loglam);
-                for (int q = 0; q < 6; ++q) atomicAdd(d.fix7 + 1 + q, dl[q]);
-                if (rows9) {
-                    row_eval<false>(sums, d.t[i], 0.0, 0.0, 0.0, cc, o, b);
-                    for (int q = 0; q < 9; ++q) rows9[9 * i + q] = o[q];
-                }
+            // (k_finalize has the row's Lambda terms)
+            double o[9], b[7], loglam, dl[6];
+            row_lambda<false>(sums, d.t[i], 0.0, 0.0, 0.0, cc, loglam, dl, b);
+            atomicAdd(d.fix7, loglam);
+            for (int q = 0; q < 6; ++q) atomicAdd(d.fix7 + 1 + q, dl[q]);
+            if (rows9) {
+                row_eval<false>(sums, d.t[i], 0.0, 0.0, 0.0, cc, o, b);
+                for (int q = 0; q < 9; ++q) rows9[9 * i + q] = o[q];
             }
         }
         __syncthreads();
     }
-    if (mode == 0) return;
     __shared__ bool s_last;
     if (threadIdx.x == 0) {
         __threadfence();
@@ -642,7 +650,7 @@ __global__ void k_rows64(const __grid_constant__ EvalDesc one, const EvalDesc* _
         __threadfence();
     }
     __syncthreads();
-    if (s_last) finish_outputs(d.fix7 + 16, d.fix7, cc, probs ? n : count, out + (probs ? 7 * blockIdx.y : 0), ctr);
+    if (s_last) finish_outputs(d.fix7 + 16, d.fix7, cc, probs ? n : nrows, out + (probs ? 7 * blockIdx.y : 0), ctr);
 }
 
 // Recompute in FP64 the rows that the flush thresholds (finish_outputs) select

@@ -29,9 +29,8 @@ __global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const 
                        const __grid_constant__ hawkes_params,
                        int, int, int, int, const uint64_t*, int*);
 void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
-                     double*, double*, double*);
-__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, int, double*,
-                         double*);
+                     const double*, int, double*, double*, double*);
+__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, double*, double*);
 __global__ void k_flushfix(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, double*, double*,
                            double*);
 cudaError_t sweep_setup_attributes();
@@ -265,9 +264,9 @@ extern "C" int hawkes_loglik_grad_noalloc(const double* d_t, const double* d_x, 
     k_prep<<<g.blocks, g.threads, 0, st>>>(e, nullptr, d_params, hawkes_params{}, model, 1, 0, 0, nullptr,
                                            nullptr);
     if (launch_sweep(&c, true, 0, n, (flags & HAWKES_BG_TIME) != 0, false) != cudaSuccess) return HAWKES_ERR_CUDA;
-    launch_finalize(st, final_grid(n, d->sms < kMaxSms ? d->sms : kMaxSms), e, nullptr, 0, n, 1, d_out,
-                    nullptr, nullptr);
-    k_rows64<<<c.sms, 256, 0, st>>>(e, nullptr, model, 0, n, 1, d_out, nullptr);
+    launch_finalize(st, final_grid(n, d->sms < kMaxSms ? d->sms : kMaxSms), e, nullptr, 0, n, 1, nullptr,
+                    1, d_out, nullptr, nullptr);
+    k_rows64<<<c.sms, 256, 0, st>>>(e, nullptr, model, n, d_out, nullptr);
     k_flushfix<<<c.sms, 256, 0, st>>>(e, nullptr, model, 0, n, d_out, nullptr, nullptr);
     k_na_nan_on_error<<<1, 32, 0, st>>>(c.ctr, d_out);
     return cudaGetLastError() == cudaSuccess ? HAWKES_OK : HAWKES_ERR_CUDA;
