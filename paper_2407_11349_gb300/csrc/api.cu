@@ -215,11 +215,11 @@ int enqueue_finalize32(hawkes_ctx* c, int model, int64_t rb, int64_t re, double*
     const EvalDesc d = eval_desc(c);
     HK_TRY(enqueue_rows(c, rb, re, 1, 1, d_out, d_rows9, nullptr));
     HK_TRY(timed(c, HAWKES_K_ROWS64, [&] {
-        k_rows64<<<c->sms, 256, 0, c->stream>>>(d, nullptr, model, re - rb, d_out, d_rows9);
+        launch_chained(k_rows64, c->sms, 256, 0, c->stream, d, nullptr, model, re - rb, d_out, d_rows9);
     }));
     return timed(c, HAWKES_K_ROWS64, [&] {
-        k_flushfix<<<grid_for(c, re - rb, 2), 256, 0, c->stream>>>(d, nullptr, model, rb, re, d_out,
-                                                                   d_rows9, d_err);
+        launch_chained(k_flushfix, grid_for(c, re - rb, 2), 256, 0, c->stream, d, nullptr, model, rb, re, d_out,
+                       d_rows9, d_err);
     });
 }
 

@@ -342,8 +342,9 @@ int enqueue(hawkes_batch* b, const hawkes_params* d_params, double* d_out, bool 
     launch_finalize(st, dim3(final_grid(nmax, b->sms, P), P), EvalDesc{}, b->d_eval, 0, 0, 1, nullptr,
                     1, d_out, nullptr, nullptr);
     const int fix = std::max(2 * b->sms / P, 8);  // blocks per problem for the fix-ups (usually idle)
-    k_rows64<<<dim3(fix, P), 256, 0, st>>>(EvalDesc{}, b->d_eval, model, 0, d_out, nullptr);
-    k_flushfix<<<dim3(fix, P), 256, 0, st>>>(EvalDesc{}, b->d_eval, model, 0, 0, d_out, nullptr, nullptr);
+    HB_CUDA(launch_chained(k_rows64, dim3(fix, P), 256, 0, st, EvalDesc{}, b->d_eval, model, 0, d_out, nullptr));
+    HB_CUDA(launch_chained(k_flushfix, dim3(fix, P), 256, 0, st, EvalDesc{}, b->d_eval, model, 0, 0, d_out, nullptr,
+                           nullptr));
     HB_CUDA(cudaGetLastError());
     return HAWKES_OK;
 }

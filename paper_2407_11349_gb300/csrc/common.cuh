@@ -317,8 +317,36 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
+// Chained launches: a kernel of a call starts while its predecessor ends.
+// chain_wait comes before the first read of what an earlier kernel wrote, in
+// every thread (the predecessor has then finished, and all before it);
+// chain_next lets the successor's blocks take the SMs that this kernel leaves.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void set_error(int* ctr, int code) {
     atomicCAS(ctr + CT_ERR, 0, code);
+}
+
+// Launch a kernel that begins with chain_wait: it may start before the one
+// ahead of it in the stream has ended.  Saves the launch gaps between a call's
+// kernels: 68 -> 56 us for a synchronous call at N = 2,000, 441 -> 429 at 30,000
+// (time-only background).  The first kernel of a call (k_prep) is launched
+// plainly, so calls still follow one another.
+template <typename... Args, typename... Given>
+cudaError_t launch_chained(void (*kern)(Args...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                           const Given&... given) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<Args>(given)...);
 }
 
 }  // namespace hk

@@ -146,6 +146,7 @@ __global__ void k_prep(const __grid_constant__ EvalDesc one, const EvalDesc* __r
     const EvalDesc& d = probs ? probs[blockIdx.y] : one;
     const bool model1 = (model & HAWKES_MODEL1) != 0;
     const int64_t n = d.n, npad = d.npad;
+    chain_next();
     __shared__ double s_kx, s_kt, s_beta0;
     if (threadIdx.x < 32) {
         const bool bgt = (model & HAWKES_BG_TIME) != 0;
@@ -438,6 +439,8 @@ __global__ void __launch_bounds__(FINAL_THREADS)
     k_finalize(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs, int64_t rb,
                int64_t re, int check, const double* __restrict__ parts64, int nparts, double* out,
                double* rows9, double* err_out) {
+    chain_next();
+    chain_wait();
     const EvalDesc& d = probs ? probs[blockIdx.y] : one;
     if (probs) {
         rb = 0;
@@ -564,12 +567,8 @@ __global__ void __launch_bounds__(FINAL_THREADS)
 void launch_finalize(cudaStream_t st, dim3 grid, const EvalDesc& one, const EvalDesc* probs, int64_t rb,
                      int64_t re, int check, const double* parts64, int nparts, double* out, double* rows9,
                      double* err_out) {
-    if (rows9)
-        k_finalize<true><<<grid, FINAL_THREADS, 0, st>>>(one, probs, rb, re, check, parts64, nparts, out, rows9,
-                                                         err_out);
-    else
-        k_finalize<false><<<grid, FINAL_THREADS, 0, st>>>(one, probs, rb, re, check, parts64, nparts, out, rows9,
-                                                          err_out);
+    launch_chained(rows9 ? k_finalize<true> : k_finalize<false>, grid, FINAL_THREADS, 0, st, one, probs, rb, re, check,
+                   parts64, nparts, out, rows9, err_out);
 }
 
 // This thread's share (sources j = threadIdx.x + k blockDim.x) of row i's six
@@ -608,6 +607,8 @@ __device__ __forceinline__ void row_sums64(const EvalDesc& d, int64_t i, bool mo
 // ---------------------------------------------------------------------------
 __global__ void k_rows64(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs,
                          int model, int64_t nrows, double* out, double* rows9) {
+    chain_next();
+    chain_wait();
     const EvalDesc& d = probs ? probs[blockIdx.y] : one;
     const int64_t n = d.n;
     double* cc = d.cc;
@@ -663,6 +664,8 @@ __global__ void k_rows64(const __grid_constant__ EvalDesc one, const EvalDesc* _
 __global__ void k_flushfix(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs,
                            int model, int64_t rb, int64_t re, double* out, double* rows9,
                            double* err_out) {
+    chain_next();
+    chain_wait();
     const EvalDesc& d = probs ? probs[blockIdx.y] : one;
     if (probs) {
         rb = 0;

@@ -266,8 +266,8 @@ extern "C" int hawkes_loglik_grad_noalloc(const double* d_t, const double* d_x, 
     if (launch_sweep(&c, true, 0, n, (flags & HAWKES_BG_TIME) != 0, false) != cudaSuccess) return HAWKES_ERR_CUDA;
     launch_finalize(st, final_grid(n, d->sms < kMaxSms ? d->sms : kMaxSms), e, nullptr, 0, n, 1, nullptr,
                     1, d_out, nullptr, nullptr);
-    k_rows64<<<c.sms, 256, 0, st>>>(e, nullptr, model, n, d_out, nullptr);
-    k_flushfix<<<c.sms, 256, 0, st>>>(e, nullptr, model, 0, n, d_out, nullptr, nullptr);
+    launch_chained(k_rows64, c.sms, 256, 0, st, e, nullptr, model, n, d_out, nullptr);
+    launch_chained(k_flushfix, c.sms, 256, 0, st, e, nullptr, model, 0, n, d_out, nullptr, nullptr);
     k_na_nan_on_error<<<1, 32, 0, st>>>(c.ctr, d_out);
     return cudaGetLastError() == cudaSuccess ? HAWKES_OK : HAWKES_ERR_CUDA;
 }

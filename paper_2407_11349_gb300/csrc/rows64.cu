@@ -105,7 +105,10 @@ __global__ void __launch_bounds__(32 * R64_WARPS, 1)
         int item = 0;
         if (lane == 0) item = atomicAdd(d.ctr + CT_WORK, 1);
         item = __shfl_sync(ALL, item, 0);
-        if (item >= groups * segments) return;
+        if (item >= groups * segments) {
+            chain_next();
+            return;
+        }
         const int g = item / segments, sg = item % segments;
         const int64_t i = row_begin + 32 * static_cast<int64_t>(g) + lane;
         const bool live = i < row_end;
@@ -216,6 +219,8 @@ cudaError_t launch_pairs64(const hawkes_ctx* c, bool model1, bool bgt, int64_t r
     const int64_t items = static_cast<int64_t>(groups) * segments;
     const int warps = static_cast<int>(std::min<int64_t>((items + c->sms - 1) / c->sms, R64_WARPS));
     const int grid = static_cast<int>(std::min<int64_t>((items + warps - 1) / warps, c->sms));
+    // (Not chained to k_prep: while that runs, the blocks would land unevenly, two
+    // on some SMs and none on others: N = 2,000 344 us for 290.)
     (bgt ? k_pairs64<true> : k_pairs64<false>)<<<grid, 32 * warps, EXP_N * sizeof(double2) + warps * sizeof(R64Warp),
                                                  c->stream>>>(
         eval_desc(c), model1 ? 1 : 0, rb, re, groups, segments, out,

@@ -139,9 +139,8 @@ cudaError_t launch_sweep_list(hawkes_ctx* c, const int4* items, int nitems, bool
     const int grid_cap = c->sms * c->variant_bpsm;
     const int grid = nitems < grid_cap ? nitems : grid_cap;
     if (grid <= 0) return cudaSuccess;
-    v.sym<<<grid, THREADS, v.smem, c->stream>>>(desc_of(c), nullptr, items, nitems, c->ctr, 0,
-                                                c->n, 0, 0);
-    return cudaGetLastError();
+    return launch_chained(v.sym, grid, THREADS, v.smem, c->stream, desc_of(c), nullptr, items, nitems, c->ctr,
+                          0, c->n, 0, 0);
 }
 
 cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row_end, bool bgt,
@@ -162,10 +161,9 @@ cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row
         const int nitems = nrt * nch;
         const int grid = nitems < grid_cap ? nitems : grid_cap;
         if (grid <= 0) return cudaSuccess;
-        v.win<<<grid, THREADS, v.smem, c->stream>>>(one, nullptr, nullptr, nitems, c->ctr, row_begin,
-                                                    row_end, item0, nch);
+        return launch_chained(v.win, grid, THREADS, v.smem, c->stream, one, nullptr, nullptr, nitems, c->ctr,
+                              row_begin, row_end, item0, nch);
     }
-    return cudaGetLastError();
 }
 
 // One persistent launch over the items of many problems; ctr[CT_WORK] must be
@@ -179,8 +177,7 @@ cudaError_t launch_sweep_batch(cudaStream_t st, const SweepPlan& pl, int sms, in
     if (grid > nitems) grid = nitems;
     if (grid <= 0) return cudaSuccess;
     ProbDesc none{};
-    v.batch<<<grid, THREADS, v.smem, st>>>(none, probs, items, nitems, ctr, 0, 0, 0, nprobs);
-    return cudaGetLastError();
+    return launch_chained(v.batch, grid, THREADS, v.smem, st, none, probs, items, nitems, ctr, 0, 0, 0, nprobs);
 }
 
 }  // namespace hk

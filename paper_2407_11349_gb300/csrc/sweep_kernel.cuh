@@ -256,6 +256,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
     volatile ProbDesc* vpd = &s_pd;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    chain_wait();
     if (MODE != MODE_BATCH && one.cc[CC_VALID] == 0.0) return;
     if (tid == 0) {
         mbar_init(&bars[0], 1);
@@ -287,7 +288,10 @@ __global__ void __launch_bounds__(THREADS, MINB)
         }
         __syncthreads();
         const int item = s_item;
-        if (item >= nitems || s_abort) break;
+        if (item >= nitems || s_abort) {
+            chain_next();
+            break;
+        }
         int64_t I;
         int jb, je;
 #define HK_PD(field) (MODE == MODE_BATCH ? vpd->field : one.field)

@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
     volatile ProbDesc* vpd = &s_pd;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    chain_wait();
     if (MODE != MODE_BATCH && one.cc[CC_VALID] == 0.0) return;
     if (tid == 0) {
         mbar_init(&bars[0], 1);
@@ -95,7 +96,10 @@ __global__ void __launch_bounds__(THREADS, MINB)
         }
         __syncthreads();
         const int item = s_item;
-        if (item >= nitems || s_abort) break;
+        if (item >= nitems || s_abort) {
+            chain_next();
+            break;
+        }
 #define HK_PD(field) (MODE == MODE_BATCH ? vpd->field : one.field)
         const int4 it = items[item];
         const int64_t r0 = static_cast<int64_t>(it.x) * ROWS;
@@ -297,8 +301,8 @@ cudaError_t launch_sweep_split(cudaStream_t st, int sms, const ProbDesc& one, co
     const SplitKernel& k = kSplit[bgt ? 1 : ll ? 2 : 0];
     const int grid = std::min(nitems, sms * SPLIT_BPSM);
     if (grid <= 0) return cudaSuccess;
-    (probs ? k.batch : k.sym)<<<grid, THREADS, k.smem, st>>>(one, probs, items, nitems, ctr, nprobs);
-    return cudaGetLastError();
+    return launch_chained(probs ? k.batch : k.sym, grid, THREADS, k.smem, st, one, probs, items, nitems, ctr,
+                          nprobs);
 }
 
 }  // namespace hk
