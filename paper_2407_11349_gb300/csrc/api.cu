@@ -18,9 +18,10 @@ __global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const 
                        int, int, int, int, const uint64_t*, int*);
 void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
                      const double*, int, double*, double*, double*);
-__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, double*, double*);
-__global__ void k_flushfix(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, double*, double*,
-                           double*);
+void launch_rows64(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, double*, double*);
+cudaError_t rows_setup_attributes();
+void launch_flushfix(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, int64_t, double*, double*,
+                     double*);
 __global__ void k_tri_area(const double*, int32_t, double*, int*);
 __global__ void k_tri_county(const int32_t*, int32_t, int32_t, double*, int32_t*, int32_t*, int*);
 __global__ void k_tri_check(const int32_t*, int32_t, int32_t, int*);
@@ -39,6 +40,7 @@ int sweep_variant_rows(int v);
 // rows64.cu
 int rows64_segments(int64_t rows, int sms);
 size_t rows64_scratch(int sms);
+cudaError_t pairs64_setup_attributes();
 cudaError_t launch_pairs64(const hawkes_ctx* c, bool model1, bool bgt, int64_t rb, int64_t re, double* out);
 // sweep_spatial.cu
 int spatial_build(hawkes_ctx* c, const hawkes_params* p, const hawkes_params* d_p);
@@ -215,11 +217,10 @@ int enqueue_finalize32(hawkes_ctx* c, int model, int64_t rb, int64_t re, double*
     const EvalDesc d = eval_desc(c);
     HK_TRY(enqueue_rows(c, rb, re, 1, 1, d_out, d_rows9, nullptr));
     HK_TRY(timed(c, HAWKES_K_ROWS64, [&] {
-        launch_chained(k_rows64, c->sms, 256, 0, c->stream, d, nullptr, model, re - rb, d_out, d_rows9);
+        launch_rows64(c->stream, c->sms, c->sms, d, nullptr, model, re - rb, d_out, d_rows9);
     }));
     return timed(c, HAWKES_K_ROWS64, [&] {
-        launch_chained(k_flushfix, grid_for(c, re - rb, 2), 256, 0, c->stream, d, nullptr, model, rb, re, d_out,
-                       d_rows9, d_err);
+        launch_flushfix(c->stream, grid_for(c, re - rb, 2), c->sms, d, nullptr, model, rb, re, d_out, d_rows9, d_err);
     });
 }
 
@@ -336,7 +337,10 @@ int hawkes_create(hawkes_ctx** out, int device, void* cuda_stream) {
             }
             c->own_stream = true;
         }
-        if (sweep_setup_attributes() != cudaSuccess) { rc = HAWKES_ERR_CUDA; break; }
+        if (sweep_setup_attributes() != cudaSuccess || rows_setup_attributes() != cudaSuccess || pairs64_setup_attributes() != cudaSuccess) {
+            rc = HAWKES_ERR_CUDA;
+            break;
+        }
         c->variant = 0;
         c->variant_bpsm = sweep_blocks_per_sm(0);
         if ((rc = dalloc(&c->ctr, CT_COUNT)) != HAWKES_OK) break;

@@ -23,9 +23,9 @@ __global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const 
                        int, int, int, int, const uint64_t*, int*);
 void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
                      const double*, int, double*, double*, double*);
-__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, double*, double*);
-__global__ void k_flushfix(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, double*, double*,
-                           double*);
+void launch_rows64(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, double*, double*);
+void launch_flushfix(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, int64_t, double*, double*,
+                     double*);
 int sweep_num_variants();
 int sweep_blocks_per_sm(int v);
 struct GroupDesc;
@@ -342,9 +342,8 @@ int enqueue(hawkes_batch* b, const hawkes_params* d_params, double* d_out, bool 
     launch_finalize(st, dim3(final_grid(nmax, b->sms, P), P), EvalDesc{}, b->d_eval, 0, 0, 1, nullptr,
                     1, d_out, nullptr, nullptr);
     const int fix = std::max(2 * b->sms / P, 8);  // blocks per problem for the fix-ups (usually idle)
-    HB_CUDA(launch_chained(k_rows64, dim3(fix, P), 256, 0, st, EvalDesc{}, b->d_eval, model, 0, d_out, nullptr));
-    HB_CUDA(launch_chained(k_flushfix, dim3(fix, P), 256, 0, st, EvalDesc{}, b->d_eval, model, 0, 0, d_out, nullptr,
-                           nullptr));
+    launch_rows64(st, dim3(fix, P), b->sms, EvalDesc{}, b->d_eval, model, 0, d_out, nullptr);
+    launch_flushfix(st, dim3(fix, P), b->sms, EvalDesc{}, b->d_eval, model, 0, 0, d_out, nullptr, nullptr);
     HB_CUDA(cudaGetLastError());
     return HAWKES_OK;
 }

@@ -328,6 +328,15 @@ __device__ __forceinline__ void set_error(int* ctr, int code) {
     atomicCAS(ctr + CT_ERR, 0, code);
 }
 
+// Dynamic shared memory that keeps more than ceil(blocks / sms) blocks from one
+// SM.  A chained kernel's blocks are placed while its predecessor still holds
+// some SMs, and would otherwise crowd on the others.
+constexpr int SPREAD_MAX = 4;
+inline size_t spread_smem(int64_t blocks, int sms) {
+    const int64_t per = (blocks + sms - 1) / sms;
+    return per > SPREAD_MAX ? 0 : static_cast<size_t>(228 * 1024 / (per + 1));
+}
+
 // Launch a kernel that begins with chain_wait: it may start before the one
 // ahead of it in the stream has ended.  Saves the launch gaps between a call's
 // kernels: 68 -> 56 us for a synchronous call at N = 2,000, 441 -> 429 at 30,000

@@ -439,7 +439,6 @@ __global__ void __launch_bounds__(FINAL_THREADS)
     k_finalize(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs, int64_t rb,
                int64_t re, int check, const double* __restrict__ parts64, int nparts, double* out,
                double* rows9, double* err_out) {
-    chain_next();
     chain_wait();
     const EvalDesc& d = probs ? probs[blockIdx.y] : one;
     if (probs) {
@@ -524,6 +523,7 @@ __global__ void __launch_bounds__(FINAL_THREADS)
             v[5] -= th * gap * ea;
         }
     }
+    chain_next();
     constexpr int NW = FINAL_THREADS / 32;
     __shared__ double red[NW][16];  // per warp; then the totals in red[0]
     __shared__ bool s_last;
@@ -607,8 +607,8 @@ __device__ __forceinline__ void row_sums64(const EvalDesc& d, int64_t i, bool mo
 // ---------------------------------------------------------------------------
 __global__ void k_rows64(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs,
                          int model, int64_t nrows, double* out, double* rows9) {
-    chain_next();
     chain_wait();
+    chain_next();
     const EvalDesc& d = probs ? probs[blockIdx.y] : one;
     const int64_t n = d.n;
     double* cc = d.cc;
@@ -664,7 +664,6 @@ __global__ void k_rows64(const __grid_constant__ EvalDesc one, const EvalDesc* _
 __global__ void k_flushfix(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs,
                            int model, int64_t rb, int64_t re, double* out, double* rows9,
                            double* err_out) {
-    chain_next();
     chain_wait();
     const EvalDesc& d = probs ? probs[blockIdx.y] : one;
     if (probs) {
@@ -757,6 +756,28 @@ __global__ void k_flushfix(const __grid_constant__ EvalDesc one, const EvalDesc*
         if (!finite) set_error(ctr, HAWKES_ERR_NONFINITE);
         if (err_out) *err_out = static_cast<double>(*static_cast<volatile int*>(ctr + CT_ERR));
     }
+}
+
+// Chained and spread over the SMs: where rows are recomputed, their FP64 work
+// needs every SM (N = 5,000, sparse: 322 us for the call with the blocks as they
+// fall, 252 spread).
+void launch_rows64(cudaStream_t st, dim3 grid, int sms, const EvalDesc& one, const EvalDesc* probs, int model,
+                   int64_t nrows, double* out, double* rows9) {
+    launch_chained(k_rows64, grid, 256, spread_smem(static_cast<int64_t>(grid.x) * grid.y, sms), st, one, probs, model,
+                   nrows, out, rows9);
+}
+
+void launch_flushfix(cudaStream_t st, dim3 grid, int sms, const EvalDesc& one, const EvalDesc* probs, int model,
+                     int64_t rb, int64_t re, double* out, double* rows9, double* err_out) {
+    launch_chained(k_flushfix, grid, 256, spread_smem(static_cast<int64_t>(grid.x) * grid.y, sms), st, one, probs, model,
+                   rb, re, out, rows9, err_out);
+}
+
+cudaError_t rows_setup_attributes() {
+    const int most = static_cast<int>(spread_smem(1, 1));
+    const cudaError_t e = cudaFuncSetAttribute(k_rows64, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(k_flushfix, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 // ---------------------------------------------------------------------------

@@ -30,9 +30,10 @@ __global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const 
                        int, int, int, int, const uint64_t*, int*);
 void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
                      const double*, int, double*, double*, double*);
-__global__ void k_rows64(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, double*, double*);
-__global__ void k_flushfix(const __grid_constant__ EvalDesc, const EvalDesc*, int, int64_t, int64_t, double*, double*,
-                           double*);
+void launch_rows64(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, double*, double*);
+cudaError_t rows_setup_attributes();
+void launch_flushfix(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, int64_t, double*, double*,
+                     double*);
 cudaError_t sweep_setup_attributes();
 int sweep_blocks_per_sm(int v);
 int sweep_variant_rows(int v);
@@ -180,7 +181,7 @@ int device_setup(int dev, DeviceSetup** out) {
             cudaGetLastError();
             return HAWKES_ERR_CUDA;
         }
-        if (sweep_setup_attributes() != cudaSuccess ||
+        if (sweep_setup_attributes() != cudaSuccess || rows_setup_attributes() != cudaSuccess ||
             cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
             cudaGetLastError();
             return HAWKES_ERR_CUDA;
@@ -266,8 +267,8 @@ extern "C" int hawkes_loglik_grad_noalloc(const double* d_t, const double* d_x, 
     if (launch_sweep(&c, true, 0, n, (flags & HAWKES_BG_TIME) != 0, false) != cudaSuccess) return HAWKES_ERR_CUDA;
     launch_finalize(st, final_grid(n, d->sms < kMaxSms ? d->sms : kMaxSms), e, nullptr, 0, n, 1, nullptr,
                     1, d_out, nullptr, nullptr);
-    launch_chained(k_rows64, c.sms, 256, 0, st, e, nullptr, model, n, d_out, nullptr);
-    launch_chained(k_flushfix, c.sms, 256, 0, st, e, nullptr, model, 0, n, d_out, nullptr, nullptr);
+    launch_rows64(st, c.sms, c.sms, e, nullptr, model, n, d_out, nullptr);
+    launch_flushfix(st, c.sms, c.sms, e, nullptr, model, 0, n, d_out, nullptr, nullptr);
     k_na_nan_on_error<<<1, 32, 0, st>>>(c.ctr, d_out);
     return cudaGetLastError() == cudaSuccess ? HAWKES_OK : HAWKES_ERR_CUDA;
 }

@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(32 * R64_WARPS, 1)
     double2* tab = reinterpret_cast<double2*>(smem);
     R64Warp* warps = reinterpret_cast<R64Warp*>(smem + EXP_N * sizeof(double2));
     const double* cc = d.cc;
+    chain_wait();
     if (cc[CC_VALID] == 0.0) return;
     for (int k = threadIdx.x; k < EXP_N; k += blockDim.x) tab[k] = kExpTable[k];
     __syncthreads();
@@ -219,13 +220,19 @@ cudaError_t launch_pairs64(const hawkes_ctx* c, bool model1, bool bgt, int64_t r
     const int64_t items = static_cast<int64_t>(groups) * segments;
     const int warps = static_cast<int>(std::min<int64_t>((items + c->sms - 1) / c->sms, R64_WARPS));
     const int grid = static_cast<int>(std::min<int64_t>((items + warps - 1) / warps, c->sms));
-    // (Not chained to k_prep: while that runs, the blocks would land unevenly, two
-    // on some SMs and none on others: N = 2,000 344 us for 290.)
-    (bgt ? k_pairs64<true> : k_pairs64<false>)<<<grid, 32 * warps, EXP_N * sizeof(double2) + warps * sizeof(R64Warp),
-                                                 c->stream>>>(
-        eval_desc(c), model1 ? 1 : 0, rb, re, groups, segments, out,
-        segments > 1 ? static_cast<int64_t>(groups) * 32 : c->npad, segments > 1 ? rb : 0);
-    return cudaGetLastError();
+    const size_t smem = std::max(EXP_N * sizeof(double2) + warps * sizeof(R64Warp), spread_smem(grid, c->sms));
+    return launch_chained(bgt ? k_pairs64<true> : k_pairs64<false>, grid, 32 * warps, smem, c->stream, eval_desc(c),
+                          model1 ? 1 : 0, rb, re, groups, segments, out,
+                          segments > 1 ? static_cast<int64_t>(groups) * 32 : c->npad, segments > 1 ? rb : 0);
+}
+
+cudaError_t pairs64_setup_attributes() {
+    for (auto* k : {k_pairs64<false>, k_pairs64<true>}) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   static_cast<int>(spread_smem(1, 1)));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace hk
