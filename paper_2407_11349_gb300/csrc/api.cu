@@ -43,6 +43,7 @@ size_t rows64_scratch(int sms);
 cudaError_t pairs64_setup_attributes();
 cudaError_t launch_pairs64(const hawkes_ctx* c, bool model1, bool bgt, int64_t rb, int64_t re, double* out);
 // sweep_spatial.cu
+cudaError_t spatial_setup_attributes();
 int spatial_build(hawkes_ctx* c, const hawkes_params* p, const hawkes_params* d_p);
 cudaError_t spatial_launch(hawkes_ctx* c, int model1, int llonly);
 void spatial_free(hawkes_ctx* c);
@@ -337,7 +338,8 @@ int hawkes_create(hawkes_ctx** out, int device, void* cuda_stream) {
             }
             c->own_stream = true;
         }
-        if (sweep_setup_attributes() != cudaSuccess || rows_setup_attributes() != cudaSuccess || pairs64_setup_attributes() != cudaSuccess) {
+        if (sweep_setup_attributes() != cudaSuccess || spatial_setup_attributes() != cudaSuccess ||
+            rows_setup_attributes() != cudaSuccess || pairs64_setup_attributes() != cudaSuccess) {
             rc = HAWKES_ERR_CUDA;
             break;
         }

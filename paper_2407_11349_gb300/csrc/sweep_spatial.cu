@@ -13,27 +13,38 @@
 //     builds the order.  Locations that will be redrawn inside their counties
 //     say little beyond the county, so they enter as the county's mean plus a
 //     fifth of the offset from it.
-//   - Per call: records in that order and the bounding box, time range and
-//     largest excitation reach of every chunk and tile (a resample moves them
-//     with the events).
+//   - Per call: records in that order, relative to their chunk's centre, and the
+//     bounding box, time range and largest excitation reach of every chunk, tile
+//     and block of 32 tiles (a resample moves them with the events).
 //   - Sweep: one warp per group of 32 rows (one chunk of the order, a row per
-//     lane).  It tests tiles, then chunks, against its rows' box, then the
-//     chunk's 32 events, one per lane, and appends the survivors to two small
-//     buffers in shared memory (background, excitation).  A full buffer is
-//     evaluated, two columns per packed f32x2 register.
+//     lane).  It tests blocks, tiles and chunks against its rows' box and lists
+//     the chunks that can matter, for the background and for the excitation.
+//     Then it tests a listed chunk's 32 events, one per lane, and appends the
+//     survivors to a buffer in shared memory; every 32 of them are evaluated, two
+//     columns per packed f32x2 register.
 // Every test keeps 2 units of margin on the base-2 exponent, and the boxes are
 // widened by the FP32 rounding of the coordinates, so what is left out is an
 // exact FP32 zero; the rest is the full sweep's sum in another order.
 //
-// What bounds it: shared-memory reads (a column's 24 bytes go to every lane;
-// 74% of the wavefronts) and instruction issue (67%) in the evaluation of the
-// columns that pass the point test; the FP32 pipe is 46% busy.  Two rows per
-// lane would halve the reads, but the box of 64 rows keeps 48% more columns.
-// At N = 1,000,000 (3,143 counties, 1,200 days) a row has 1,811
-// columns with a nonzero background and 14 with a nonzero excitation; point
-// tests against the box of 32 rows leave 4,070 and 1,210, in 4.1 ms.  (The former
-// design, 256 x 256 tile pairs kept whole by box tests and swept through
-// shared-memory tiles, left about 40,000 with both terms: 45 ms.)
+// Coordinates: a background term between rows in a box of at most 8 scaled units
+// takes one FP32 word per coordinate, from the centre of the rows' box (3
+// differences and 12 bytes a column instead of 9 operations and 24 bytes).  Wider
+// groups, and every excitation term (whose length scale is a source's h s), take
+// two.  Up to 12 or 16 units one word would save another 11%, but log lambda's
+// rms error at N = 120,000 would rise from 1.3e-7 to 2.0e-7 (whole tiles swept
+// with two words: 1.5e-7).
+//
+// What bounds it: instruction dispatch.  A packed FP32 instruction takes two
+// dispatch cycles, any other one; at N = 1,000,000 (3,143 counties, 1,200 days)
+// a group takes 93,000 such cycles of the 97,000 it has, half of them in the
+// evaluation of the columns that pass the point test.  A row has 1,811 columns
+// with a nonzero background and 14 with a nonzero excitation; point tests
+// against the box of 32 rows leave 3,770 and 620.  Sweep 3.39 ms; 4.05 with two
+// words throughout, one list, and buffers moved down after each evaluation; the
+// former design, 256 x 256 tile pairs kept whole by box tests and swept through
+// shared-memory tiles, 45 ms (40,000 columns with both terms).  Two rows per lane
+// would halve the shared-memory reads, but the box of 64 rows keeps 48% more
+// columns.
 // Tie and causality indicators come from each event's index in the time order,
 // carried beside its record, and are only tested for columns that can share a
 // time with the rows.  Row sums go to the FP64 accumulators of the events'
@@ -52,22 +63,35 @@ namespace hk {
 
 constexpr int SP_CH = 32;              // events per chunk: a row group, and the finest column unit
 constexpr int SP_WARPS = 8, SP_THREADS = 32 * SP_WARPS;
-// Resident CTAs per SM.  At N = 1,000,000: 2 4.30 ms, 3 4.07, 4 (64 registers,
-// spills) 4.52, 5 6.3.
+// Resident CTAs per SM.  At N = 1,000,000: 2 3.49 ms, 3 3.41, 4 (64 registers,
+// spills) 3.59.
 constexpr int SP_BPSM = 3;
 constexpr int SP_BUF = 64;             // buffered columns (32 evaluated at a time)
-constexpr int SP_LIST = 128;           // chunks listed before they are read
+constexpr int SP_LIST = 128;           // chunks listed before their events are tested
 constexpr int SP_B_PLANES = 7, SP_E_PLANES = 9;
 constexpr int32_t SP_TIED = 1 << 30;   // flag in a position's rank: other events share the time
+constexpr float SP_REL = 8.f;          // widest row group (scaled units) with one-word coordinates
+// The point tests allow for the rounding of the points: 2^-24 of their distance
+// from the reference point, and of half a chunk's width.
+constexpr float SP_EPS = 4.76837158203125e-07f;
+constexpr float SP_OUT = 1.f + 9.5367431640625e-07f, SP_IN = 1.f - 9.5367431640625e-07f;
 constexpr float SP_ZERO = 128.f;       // exponent beyond which a term counts as zero (126 + margin)
 static_assert(NPAD_MULT % TC == 0 && TC == 8 * SP_CH, "a tile is 8 chunks");
+
+// Boxes and centres of the order's units, one allocation: SpBox (two float4) of
+// every chunk, tile and block of 32 tiles, then the chunks' centres.
+constexpr int SP_TB = 32;
+constexpr int sp_blocks(int ntiles) { return (ntiles + SP_TB - 1) / SP_TB; }
+constexpr size_t sp_meta_f4(int ntiles) {
+    return 2 * (static_cast<size_t>(9) * ntiles + sp_blocks(ntiles)) + static_cast<size_t>(8) * ntiles;
+}
 
 struct SpatialState {
     int64_t window = 131072;  // target events per time window
     bool built = false;
     int ntiles = 0;           // npad / TC
     int32_t* rank = nullptr;  // [npad] time-order index at each position, | SP_TIED (-1: padding)
-    float4* meta = nullptr;   // [2 x chunks], then [2 x tiles]: SpBox of each
+    float4* meta = nullptr;   // SpMeta's arrays
 };
 
 void spatial_free(hawkes_ctx* c) {
@@ -183,7 +207,7 @@ static int build_order(hawkes_ctx* c, double tau_x, double tau_t) {
         sp->rank = nullptr;
         sp->meta = nullptr;
         if (cudaMalloc(&sp->rank, npad * sizeof(int32_t)) != cudaSuccess ||
-            cudaMalloc(&sp->meta, 2 * static_cast<size_t>(9 * ntiles) * sizeof(float4)) != cudaSuccess) {
+            cudaMalloc(&sp->meta, sp_meta_f4(ntiles) * sizeof(float4)) != cudaSuccess) {
             cudaGetLastError();
             return HAWKES_ERR_OOM;
         }
@@ -251,13 +275,59 @@ __device__ __forceinline__ void sp_widen(float& lo, float& hi) {
     hi += s;
 }
 
-// Stage the records in the spatial order (negated column values): planes
-// ra[npad] = (-x hi, -x lo, -y hi, -y lo), rb[npad] = (-t hi, -t lo, -beta, ce),
-// with t~ = (t - t_1) sqrt(a_t) in two FP32 words like the coordinates, and
-// the boxes of the chunks and tiles (one block per tile).
+__device__ __forceinline__ SpBox sp_warp_join(SpBox box) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        SpBox q;
+        q.x0 = __shfl_xor_sync(0xffffffffu, box.x0, o); q.x1 = __shfl_xor_sync(0xffffffffu, box.x1, o);
+        q.y0 = __shfl_xor_sync(0xffffffffu, box.y0, o); q.y1 = __shfl_xor_sync(0xffffffffu, box.y1, o);
+        q.t0 = __shfl_xor_sync(0xffffffffu, box.t0, o); q.t1 = __shfl_xor_sync(0xffffffffu, box.t1, o);
+        q.ce = __shfl_xor_sync(0xffffffffu, box.ce, o); q.beta = __shfl_xor_sync(0xffffffffu, box.beta, o);
+        sp_join(box, q);
+    }
+    return box;
+}
+
+// Middle of a range on a grid of 1/16, so that differences of neighbouring
+// chunks' centres are exact in FP32 (beyond 2^20 FP32's own grid is coarser).
+__device__ __forceinline__ float sp_mid(float a, float b) {
+    const float m = 0.5f * a + 0.5f * b;
+    return fabsf(m) < 1048576.f ? rintf(m * 16.f) * 0.0625f : m;
+}
+
+// hi + lo = a + d exactly, lo0 added to lo.
+__device__ __forceinline__ void sp_two_sum(float a, float d, float lo0, float& hi, float& lo) {
+    hi = a + d;
+    const float z = hi - a;
+    lo = ((a - (hi - z)) + (d - z)) + lo0;
+}
+
+// First word of a two-word coordinate: on a grid of 2^-14 for |a| < 256, so that
+// first words' differences are exact.  (FP32 has steps of 2^-14 from 512 to 1,024.)
+__device__ __forceinline__ float sp_grid(float a) { return (a + 768.f) - 768.f; }
+
+// c - (xh + xl), and what sp_grid leaves of it.  (In FP32: FP64 arithmetic is what
+// staging waits for.)
+__device__ __forceinline__ void sp_recentre(float c, float xh, float xl, float& hi, float& lo) {
+    float h, l;
+    sp_two_sum(-xh, c, -xl, h, l);
+    sp_two_sum(h, l, 0.f, hi, lo);
+    lo += hi - sp_grid(hi);
+}
+
+// Stage the records in the spatial order: negated distances from the chunk's
+// centre in two FP32 words each,
+//   ra[npad] = (-x, -y, -t, rank bits), rb[npad] = (-x lo, -y lo, -t lo, -beta), rc[npad] = ce
+// (the second words belong to the first ones on sp_grid's grid),
+// in scaled units (t~ = (t - t_1) sqrt(a_t)), the centres, and the boxes of the
+// chunks and tiles (one block per tile).
 __global__ void __launch_bounds__(TC) k_sp_prep(EvalDesc d, const int32_t* __restrict__ rank, int model1,
                                                 float4* __restrict__ ra, float4* __restrict__ rb,
-                                                float4* __restrict__ meta, int ntiles) {
+                                                float* __restrict__ rc, float4* __restrict__ cmeta,
+                                                float4* __restrict__ tmeta, float4* __restrict__ centre,
+                                                int ntiles) {
+    chain_next();
+    chain_wait();
     if (d.cc[CC_VALID] == 0.0) return;
     const double kx = d.cc[CC_KX], kt = d.cc[CC_KT], tf = d.t[0];
     const double beta0 = (d.cc[CC_TX] * d.cc[CC_TX]) / (d.cc[CC_H] * d.cc[CC_H]);
@@ -266,58 +336,78 @@ __global__ void __launch_bounds__(TC) k_sp_prep(EvalDesc d, const int32_t* __res
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int64_t p = static_cast<int64_t>(tile) * TC + threadIdx.x;
         const int32_t r = rank[p];
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = make_float4(-PAD_T, 0.f, 0.f, -1e30f);
+        float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f, th = 0.f, tl = 0.f, beta = 0.f, ce = -1e30f;
         SpBox box = sp_empty();
         if (r >= 0) {
             const int32_t e = r & ~SP_TIED;
             const double ts = (d.t[e] - tf) * kt, xs = d.x[e] * kx, ys = d.y[e] * kx;
-            const float th = static_cast<float>(ts), xh = static_cast<float>(xs), yh = static_cast<float>(ys);
-            const float beta = static_cast<float>(model1 ? beta0 : beta0 * d.is2[e]);
-            const float ce = model1 ? 0.f : d.ce[e];
-            a = make_float4(-xh, -static_cast<float>(xs - static_cast<double>(xh)), -yh,
-                            -static_cast<float>(ys - static_cast<double>(yh)));
-            b = make_float4(-th, -static_cast<float>(ts - static_cast<double>(th)), -beta, ce);
+            th = static_cast<float>(ts);
+            xh = static_cast<float>(xs);
+            yh = static_cast<float>(ys);
+            tl = static_cast<float>(ts - static_cast<double>(th));
+            xl = static_cast<float>(xs - static_cast<double>(xh));
+            yl = static_cast<float>(ys - static_cast<double>(yh));
+            beta = static_cast<float>(model1 ? beta0 : beta0 * d.is2[e]);
+            ce = model1 ? 0.f : d.ce[e];
             box = SpBox{xh, xh, yh, yh, th, th, ce, beta};
+        }
+        box = sp_warp_join(box);
+        const bool any = box.x0 <= box.x1;
+        const float cx = any ? sp_mid(box.x0, box.x1) : 0.f, cy = any ? sp_mid(box.y0, box.y1) : 0.f,
+                    ct = any ? sp_mid(box.t0, box.t1) : 0.f;
+        float4 a = make_float4(0.f, 0.f, -PAD_T, __int_as_float(-1)), b = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r >= 0) {
+            a.w = __int_as_float(r);
+            b.w = -beta;
+            sp_recentre(cx, xh, xl, a.x, b.x);
+            sp_recentre(cy, yh, yl, a.y, b.y);
+            sp_recentre(ct, th, tl, a.z, b.z);
         }
         ra[p] = a;
         rb[p] = b;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            SpBox q;
-            q.x0 = __shfl_xor_sync(0xffffffffu, box.x0, o); q.x1 = __shfl_xor_sync(0xffffffffu, box.x1, o);
-            q.y0 = __shfl_xor_sync(0xffffffffu, box.y0, o); q.y1 = __shfl_xor_sync(0xffffffffu, box.y1, o);
-            q.t0 = __shfl_xor_sync(0xffffffffu, box.t0, o); q.t1 = __shfl_xor_sync(0xffffffffu, box.t1, o);
-            q.ce = __shfl_xor_sync(0xffffffffu, box.ce, o); q.beta = __shfl_xor_sync(0xffffffffu, box.beta, o);
-            sp_join(box, q);
-        }
+        rc[p] = ce;
         if (lane == 0) {
-            if (box.x0 <= box.x1) {
+            if (any) {
                 sp_widen(box.x0, box.x1);
                 sp_widen(box.y0, box.y1);
                 sp_widen(box.t0, box.t1);
             }
             boxes[warp] = box;
-            sp_store(meta, tile * (TC / SP_CH) + warp, box);
+            sp_store(cmeta, tile * (TC / SP_CH) + warp, box);
+            centre[tile * (TC / SP_CH) + warp] = make_float4(cx, cy, ct, 0.f);
         }
         __syncthreads();
         if (threadIdx.x == 0) {
             for (int k = 1; k < TC / SP_CH; ++k) sp_join(box, boxes[k]);
-            sp_store(meta, ntiles * (TC / SP_CH) + tile, box);
+            sp_store(tmeta, tile, box);
         }
         __syncthreads();
     }
 }
 
+// Boxes of the blocks of 32 tiles, one warp each.
+__global__ void k_sp_blocks(const float4* __restrict__ tmeta, float4* __restrict__ bmeta, int ntiles,
+                            const double* __restrict__ cc) {
+    chain_next();
+    chain_wait();
+    if (cc[CC_VALID] == 0.0) return;
+    const int t = blockIdx.x * SP_TB + threadIdx.x;
+    const SpBox box = sp_warp_join(t < ntiles ? sp_load(tmeta, t) : sp_empty());
+    if (threadIdx.x == 0) sp_store(bmeta, blockIdx.x, box);
+}
+
 struct SpArgs {
     const float4* ra;
     const float4* rb;
-    const int32_t* rank;
+    const float* rc;
     const int32_t* lo;
     const int32_t* hi;
     const double* cc;
     double* acc;
     const float4* cmeta;
     const float4* tmeta;
+    const float4* bmeta;
+    const float4* centre;
     int64_t npad;
     int ntiles, groups, parts;
 };
@@ -334,55 +424,93 @@ __device__ __forceinline__ void sp_near(const SpBox& w, const SpBox& c, float om
     ne = c.t0 <= w.t1 && !(c.ce - omt * fmaxf(0.f, w.t0 - c.t1) - c.beta * r2 < -SP_ZERO);
 }
 
-// A lane's row (values doubled for packed arithmetic) and its sums over the
-// even and odd columns.
+// A lane's row: its coordinates from the group's reference point, and its sums
+// over the even and odd columns.  (The two-word coordinates are in the warp's
+// shared memory.)
 struct SpRow {
-    float2 th, tl, xh, xl, yh, yl;
+    float x, y, t;
     float2 sB, sBr, sBt, sE, sEt, sEq;
     int lo, hi;
 };
 
+// Shared memory of a warp: the two column buffers, the rows' two-word
+// coordinates (x hi, x lo, y hi, y lo, t hi, t lo) and the chunk list.
+struct SpWarp {
+    float b[SP_B_PLANES * SP_BUF];
+    float e[SP_E_PLANES * SP_BUF];
+    float row[6 * SP_CH];
+    float4 list[SP_LIST];
+};
+
+// The differences of a pair of columns to the lane's row, from two-word
+// coordinates (planes 0 to 5).
+struct SpRow2 {
+    float2 xh, xl, yh, yl, th, tl;
+    __device__ __forceinline__ explicit SpRow2(const float* __restrict__ r) {
+        const float* q = r + (threadIdx.x & 31);
+        xh = f2(q[0], q[0]); xl = f2(q[32], q[32]); yh = f2(q[64], q[64]);
+        yl = f2(q[96], q[96]); th = f2(q[128], q[128]); tl = f2(q[160], q[160]);
+    }
+};
+
 __device__ __forceinline__ float2 half4(const float4& v, int h) { return h ? f2(v.z, v.w) : f2(v.x, v.y); }
 
-// Background of `quads` x 4 buffered columns against the lane's row.
 template <bool MASK, bool LL>
-__device__ __forceinline__ void sp_eval_b(const float* __restrict__ buf, int quads, SpRow& w) {
+__device__ __forceinline__ void sp_add_b(float2 dx, float2 dy, float2 dt, int r0, int r1, SpRow& w) {
+    const float2 r2 = fma2(dy, dy, mul2(dx, dx));
+    const float2 dt2 = mul2(dt, dt);
+    const float2 aB = add2(dt2, r2);
+    float2 B = f2(ex2(-aB.x), ex2(-aB.y));
+    if (MASK) {  // t_j != t_i
+        B.x = (r0 < w.lo || r0 >= w.hi) ? B.x : 0.f;
+        B.y = (r1 < w.lo || r1 >= w.hi) ? B.y : 0.f;
+    }
+    w.sB = add2(w.sB, B);
+    if (!LL) {
+        w.sBr = fma2(B, r2, w.sBr);
+        w.sBt = fma2(B, dt2, w.sBt);
+    }
+}
+
+// Background of `quads` x 4 buffered columns against the lane's row.  REL:
+// planes 0 to 2 hold the columns' x, y, t from the group's reference point.
+template <bool REL, bool MASK, bool LL>
+__device__ __forceinline__ void sp_eval_b(const SpWarp& sw, int first, int quads, SpRow& w) {
+    constexpr int P = SP_BUF / 4;
+    const float4* p = reinterpret_cast<const float4*>(sw.b + first);
+    int4 rk = make_int4(0, 0, 0, 0);
+    if (REL) {
+        const float2 x = f2(w.x, w.x), y = f2(w.y, w.y), t = f2(w.t, w.t);
+#pragma unroll 2
+        for (int q = 0; q < quads; ++q, ++p) {
+            const float4 X = p[0 * P], Y = p[1 * P], T = p[2 * P];
+            if (MASK) rk = *reinterpret_cast<const int4*>(p + 6 * P);
+            sp_add_b<MASK, LL>(add2(x, half4(X, 0)), add2(y, half4(Y, 0)), add2(t, half4(T, 0)), rk.x, rk.y, w);
+            sp_add_b<MASK, LL>(add2(x, half4(X, 1)), add2(y, half4(Y, 1)), add2(t, half4(T, 1)), rk.z, rk.w, w);
+        }
+    } else {
+        const SpRow2 r(sw.row);
 #pragma unroll 4
-    for (int q = 0; q < quads; ++q) {
-        const float4* p = reinterpret_cast<const float4*>(buf) + q;
-        const float4 xh = p[0 * SP_BUF / 4], xl = p[1 * SP_BUF / 4], yh = p[2 * SP_BUF / 4],
-                     yl = p[3 * SP_BUF / 4], th = p[4 * SP_BUF / 4], tl = p[5 * SP_BUF / 4];
-        int4 rk;
-        if (MASK) rk = *reinterpret_cast<const int4*>(p + 6 * SP_BUF / 4);
+        for (int q = 0; q < quads; ++q, ++p) {
+            const float4 xh = p[0 * P], xl = p[1 * P], yh = p[2 * P], yl = p[3 * P], th = p[4 * P], tl = p[5 * P];
+            if (MASK) rk = *reinterpret_cast<const int4*>(p + 6 * P);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float2 dt = add2(add2(w.th, half4(th, h)), add2(w.tl, half4(tl, h)));
-            const float2 dx = add2(add2(w.xh, half4(xh, h)), add2(w.xl, half4(xl, h)));
-            const float2 dy = add2(add2(w.yh, half4(yh, h)), add2(w.yl, half4(yl, h)));
-            const float2 r2 = fma2(dy, dy, mul2(dx, dx));
-            const float2 dt2 = mul2(dt, dt);
-            const float2 aB = add2(dt2, r2);
-            float2 B = f2(ex2(-aB.x), ex2(-aB.y));
-            if (MASK) {  // t_j != t_i
-                const int r0 = h ? rk.z : rk.x, r1 = h ? rk.w : rk.y;
-                B.x = (r0 < w.lo || r0 >= w.hi) ? B.x : 0.f;
-                B.y = (r1 < w.lo || r1 >= w.hi) ? B.y : 0.f;
-            }
-            w.sB = add2(w.sB, B);
-            if (!LL) {
-                w.sBr = fma2(B, r2, w.sBr);
-                w.sBt = fma2(B, dt2, w.sBt);
-            }
+            for (int h = 0; h < 2; ++h)
+                sp_add_b<MASK, LL>(add2(add2(r.xh, half4(xh, h)), add2(r.xl, half4(xl, h))),
+                                   add2(add2(r.yh, half4(yh, h)), add2(r.yl, half4(yl, h))),
+                                   add2(add2(r.th, half4(th, h)), add2(r.tl, half4(tl, h))),
+                                   h ? rk.z : rk.x, h ? rk.w : rk.y, w);
         }
     }
 }
 
 // Excitation of `quads` x 4 buffered columns (planes as above, then -beta, ce).
 template <bool MASK, bool LL>
-__device__ __forceinline__ void sp_eval_e(const float* __restrict__ buf, int quads, float2 nomt, SpRow& w) {
+__device__ __forceinline__ void sp_eval_e(const SpWarp& sw, int first, int quads, float2 nomt, SpRow& w) {
+    const SpRow2 r(sw.row);
 #pragma unroll 1
     for (int q = 0; q < quads; ++q) {
-        const float4* p = reinterpret_cast<const float4*>(buf) + q;
+        const float4* p = reinterpret_cast<const float4*>(sw.e + first) + q;
         const float4 xh = p[0 * SP_BUF / 4], xl = p[1 * SP_BUF / 4], yh = p[2 * SP_BUF / 4],
                      yl = p[3 * SP_BUF / 4], th = p[4 * SP_BUF / 4], tl = p[5 * SP_BUF / 4],
                      nb = p[7 * SP_BUF / 4], ce = p[8 * SP_BUF / 4];
@@ -390,9 +518,9 @@ __device__ __forceinline__ void sp_eval_e(const float* __restrict__ buf, int qua
         if (MASK) rk = *reinterpret_cast<const int4*>(p + 6 * SP_BUF / 4);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const float2 dt = add2(add2(w.th, half4(th, h)), add2(w.tl, half4(tl, h)));
-            const float2 dx = add2(add2(w.xh, half4(xh, h)), add2(w.xl, half4(xl, h)));
-            const float2 dy = add2(add2(w.yh, half4(yh, h)), add2(w.yl, half4(yl, h)));
+            const float2 dt = add2(add2(r.th, half4(th, h)), add2(r.tl, half4(tl, h)));
+            const float2 dx = add2(add2(r.xh, half4(xh, h)), add2(r.xl, half4(xl, h)));
+            const float2 dy = add2(add2(r.yh, half4(yh, h)), add2(r.yl, half4(yl, h)));
             const float2 r2 = fma2(dy, dy, mul2(dx, dx));
             const float2 nv = mul2(half4(nb, h), r2);
             const float2 arg = add2(fma2(nomt, dt, nv), half4(ce, h));
@@ -411,12 +539,165 @@ __device__ __forceinline__ void sp_eval_e(const float* __restrict__ buf, int qua
     }
 }
 
-// Shared memory of a warp: the two column buffers and the chunk list.
-struct SpWarp {
-    float b[SP_B_PLANES * SP_BUF];
-    float e[SP_E_PLANES * SP_BUF];
-    int list[SP_LIST];
+template <bool LL>
+__device__ __forceinline__ void sp_background(const SpWarp& sw, int first, int quads, bool rel, bool mask, SpRow& w) {
+    if (rel) {
+        if (mask) sp_eval_b<true, true, LL>(sw, first, quads, w);
+        else sp_eval_b<true, false, LL>(sw, first, quads, w);
+    } else {
+        if (mask) sp_eval_b<false, true, LL>(sw, first, quads, w);
+        else sp_eval_b<false, false, LL>(sw, first, quads, w);
+    }
+}
+
+template <bool LL>
+__device__ __forceinline__ void sp_excitation(const SpWarp& sw, int first, int quads, bool mask, float2 nomt, SpRow& w) {
+    if (mask) sp_eval_e<true, LL>(sw, first, quads, nomt, w);
+    else sp_eval_e<false, LL>(sw, first, quads, nomt, w);
+}
+
+// A row group as the column tests see it: half widths of its rows about its
+// centre, and the range of time-order indices that some row must be compared
+// with one by one (ties; the excitation's first later event).
+struct SpGroup {
+    float hx, hy, ht;
+    int lo_min, ties;  // [lo_min, lo_min + ties)
+    int self;          // its own chunk
 };
+
+// A listed chunk: offset of its centre from the group's, then its number, and
+// SP_WIDE if one word per coordinate is not enough for its events, SP_FAR if
+// the sum of a first word and the offset may not be exact (above 512).
+constexpr int SP_FAR = 1 << 27, SP_WIDE = 1 << 28, SP_ID = SP_FAR - 1;
+
+// Distance beyond the group's half width, not above the true one.
+__device__ __forceinline__ float sp_beyond(float d, float half) { return fmaxf(0.f, fmaf(fabsf(d), SP_IN, -half)); }
+
+// A column's coordinates from the group's centre in two words each.
+__device__ __forceinline__ void sp_two_words(const float4& a, const float4& b, const float4& off, float& xh, float& yh,
+                                             float& th, float& xl, float& yl, float& tl) {
+    if (__float_as_int(off.w) & SP_FAR) {
+        sp_two_sum(sp_grid(a.x), off.x, b.x, xh, xl);
+        sp_two_sum(sp_grid(a.y), off.y, b.y, yh, yl);
+        sp_two_sum(sp_grid(a.z), off.z, b.z, th, tl);
+    } else {
+        xh = sp_grid(a.x) + off.x;
+        yh = sp_grid(a.y) + off.y;
+        th = sp_grid(a.z) + off.z;
+        xl = b.x;
+        yl = b.y;
+        tl = b.z;
+    }
+}
+
+// Test the events of the n listed chunks, one per lane, for a nonzero
+// background, and evaluate the survivors 32 at a time.  count: survivors so far
+// (the buffer is a ring of two halves); mask: the current half holds a column
+// that may share a time with a row.
+template <bool REL, bool LL>
+__device__ __forceinline__ void sp_columns_b(const SpArgs& a, SpWarp& sw, int n, const SpGroup& gr, SpRow& w,
+                                             int& count, bool& mask) {
+    constexpr unsigned ALL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const float4* ra = a.ra + lane;
+    const float4* rb = a.rb + lane;
+    int64_t p = static_cast<int64_t>(__float_as_int(sw.list[0].w) & SP_ID) * SP_CH;
+    float4 next = ra[p], nextl = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!REL) nextl = rb[p];
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+        const float4 q = next, off = sw.list[k];
+        float4 lo = nextl;
+        p = static_cast<int64_t>(__float_as_int(sw.list[min(k + 1, n - 1)].w) & SP_ID) * SP_CH;
+        next = ra[p];
+        if (!REL) nextl = rb[p];
+        const int id = __float_as_int(off.w), rk = __float_as_int(q.w);
+        float nx = q.x + off.x, ny = q.y + off.y, nt = q.z + off.z;  // negated, from the group's centre
+        float hx = nx, hy = ny, ht = nt;                             // first of two words
+        if (!REL || (id & SP_WIDE)) {
+            if (REL) lo = rb[static_cast<int64_t>(id & SP_ID) * SP_CH];
+            sp_two_words(q, lo, off, hx, hy, ht, lo.x, lo.y, lo.z);
+            nx = hx + lo.x;
+            ny = hy + lo.y;
+            nt = ht + lo.z;
+        }
+        const float dx = sp_beyond(nx, gr.hx), dy = sp_beyond(ny, gr.hy), dt = sp_beyond(nt, gr.ht);
+        // (a padding event's time is far from any; negated: a NaN is kept)
+        const bool keep = !(fmaf(dt, dt, fmaf(dx, dx, dy * dy)) > SP_ZERO);
+        const unsigned bal = __ballot_sync(ALL, keep);
+        const bool any = __any_sync(ALL, keep && static_cast<unsigned>(rk - (gr.lo_min | SP_TIED)) <
+                                                     static_cast<unsigned>(gr.ties)) ||
+                         (id & SP_ID) == gr.self;
+        mask |= any;
+        if (keep) {
+            float* b = sw.b + ((count + __popc(bal & below)) & (SP_BUF - 1));
+            if (REL) {
+                b[0 * SP_BUF] = nx; b[1 * SP_BUF] = ny; b[2 * SP_BUF] = nt;
+            } else {
+                b[0 * SP_BUF] = hx; b[1 * SP_BUF] = lo.x; b[2 * SP_BUF] = hy; b[3 * SP_BUF] = lo.y;
+                b[4 * SP_BUF] = ht; b[5 * SP_BUF] = lo.z;
+            }
+            b[6 * SP_BUF] = __int_as_float(rk & ~SP_TIED);
+        }
+        const int before = count;
+        count += __popc(bal);
+        if ((before ^ count) & 32) {
+            __syncwarp();
+            sp_background<LL>(sw, before & 32, 8, REL, mask, w);
+            mask = any;
+            __syncwarp();
+        }
+    }
+}
+
+// The same for the excitation (the listed chunks from the end of the list).
+template <bool LL>
+__device__ __forceinline__ void sp_columns_e(const SpArgs& a, SpWarp& sw, int n, const SpGroup& gr, float omt,
+                                             SpRow& w, int& count, bool& mask) {
+    constexpr unsigned ALL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const float2 nomt = f2(-omt, -omt);
+    const float4* list = sw.list + SP_LIST - 1;
+    int64_t p = static_cast<int64_t>(__float_as_int(list[0].w) & SP_ID) * SP_CH + lane;
+    float4 na = a.ra[p], nl = a.rb[p];
+    float nc = a.rc[p];
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+        const float4 q = na, l = nl, off = list[-k];
+        const float ce = nc;
+        p = static_cast<int64_t>(__float_as_int(list[-min(k + 1, n - 1)].w) & SP_ID) * SP_CH + lane;
+        na = a.ra[p];
+        nl = a.rb[p];
+        nc = a.rc[p];
+        const int rank = __float_as_int(q.w) & ~SP_TIED;
+        float hx, hy, ht, lx, ly, lt;
+        sp_two_words(q, l, off, hx, hy, ht, lx, ly, lt);
+        const float nx = hx + lx, ny = hy + ly, nt = ht + lt;
+        const float dx = sp_beyond(nx, gr.hx), dy = sp_beyond(ny, gr.hy);
+        const float gap = fmaxf(0.f, fmaf(nt, SP_IN, -gr.ht));  // (nt > 0: earlier than the centre)
+        const bool keep = -nt <= gr.ht + fabsf(nt) * SP_EPS &&
+                          !(ce - omt * gap + l.w * fmaf(dx, dx, dy * dy) < -SP_ZERO);
+        const unsigned bal = __ballot_sync(ALL, keep);
+        const bool any = __any_sync(ALL, keep && rank >= gr.lo_min);
+        mask |= any;
+        if (keep) {
+            float* b = sw.e + ((count + __popc(bal & below)) & (SP_BUF - 1));
+            b[0 * SP_BUF] = hx; b[1 * SP_BUF] = lx; b[2 * SP_BUF] = hy; b[3 * SP_BUF] = ly;
+            b[4 * SP_BUF] = ht; b[5 * SP_BUF] = lt; b[6 * SP_BUF] = __int_as_float(rank);
+            b[7 * SP_BUF] = l.w; b[8 * SP_BUF] = ce;
+        }
+        const int before = count;
+        count += __popc(bal);
+        if ((before ^ count) & 32) {
+            __syncwarp();
+            sp_excitation<LL>(sw, before & 32, 8, mask, nomt, w);
+            mask = any;
+            __syncwarp();
+        }
+    }
+}
 
 // Persistent warps over items (row group, part of the column tiles).
 template <bool LL>
@@ -425,9 +706,9 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
     const int lane = threadIdx.x & 31;
     SpWarp& sw = reinterpret_cast<SpWarp*>(smem)[threadIdx.x >> 5];
     const double* cc = a.cc;
+    chain_wait();
     if (cc[CC_VALID] == 0.0) return;
     const float omt = static_cast<float>(cc[CC_OMT]);
-    const float2 nomt = f2(-omt, -omt);
     const unsigned below = (1u << lane) - 1u;
     constexpr unsigned ALL = 0xffffffffu;
 
@@ -435,43 +716,76 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
         int item = 0;
         if (lane == 0) item = atomicAdd(ctr + CT_WORK, 1);
         item = __shfl_sync(ALL, item, 0);
-        if (item >= nitems) return;
+        if (item >= nitems) {
+            chain_next();
+            return;
+        }
         const int g = item / a.parts, part = item % a.parts;
-        const int64_t p0 = static_cast<int64_t>(g) * SP_CH;
         const SpBox box = sp_load(a.cmeta, g);
         if (!(box.x0 <= box.x1)) continue;  // padding only
+        const bool rel = fmaxf(fmaxf(box.x1 - box.x0, box.y1 - box.y0), box.t1 - box.t0) <= SP_REL;
+        const float4 ref = a.centre[g];
         SpRow w;
-        const int rr = a.rank[p0 + lane];
-        const int e = rr >= 0 ? rr & ~SP_TIED : -1;
+        SpGroup gr;
+        gr.self = g;
+        int e;
         {
-            const float4 qa = a.ra[p0 + lane], qb = a.rb[p0 + lane];
-            w.xh = f2(-qa.x, -qa.x); w.xl = f2(-qa.y, -qa.y);
-            w.yh = f2(-qa.z, -qa.z); w.yl = f2(-qa.w, -qa.w);
-            w.th = f2(-qb.x, -qb.x); w.tl = f2(-qb.y, -qb.y);
+            const int64_t p = static_cast<int64_t>(g) * SP_CH + lane;
+            const float4 qa = a.ra[p], qb = a.rb[p];
+            const int rk = __float_as_int(qa.w);
+            e = rk >= 0 ? rk & ~SP_TIED : -1;
+            float* r = sw.row + lane;
+            r[0] = -sp_grid(qa.x); r[32] = -qb.x; r[64] = -sp_grid(qa.y); r[96] = -qb.y;
+            r[128] = -sp_grid(qa.z); r[160] = -qb.z;
+            w.x = -qa.x;
+            w.y = -qa.y;
+            w.t = -qa.z;
+            // (as integers: the order of nonnegative floats)
+            auto half = [&](float v) {
+                return __uint_as_float(__reduce_max_sync(ALL, e >= 0 ? __float_as_uint(fabsf(v)) : 0u)) * SP_OUT +
+                       SP_EPS;
+            };
+            gr.hx = half(qa.x);
+            gr.hy = half(qa.y);
+            gr.ht = half(qa.z);
         }
         w.lo = e >= 0 ? a.lo[e] : 0;
         w.hi = e >= 0 ? a.hi[e] : 0;
         w.sB = w.sBr = w.sBt = w.sE = w.sEt = w.sEq = f2(0.f, 0.f);
-        // time-order indices that some row must be compared with one by one
-        const int lo_min = __reduce_min_sync(ALL, e >= 0 ? w.lo : 0x7fffffff);
-        const int hi_max = __reduce_max_sync(ALL, e >= 0 ? w.hi : 0);
+        gr.lo_min = __reduce_min_sync(ALL, e >= 0 ? w.lo : 0x7fffffff);
+        gr.ties = __reduce_max_sync(ALL, e >= 0 ? w.hi : 0) - gr.lo_min;
 
-        int nB = 0, nE = 0;            // buffered columns
+        int nB = 0, nE = 0;            // columns buffered so far
         bool maskB = false, maskE = false;
-        int tile0 = 0;                 // next round of 32 tiles (of this part)
-        unsigned mT = 0;               // surviving tiles of the current round
-        int nlist = 0;
+        int next = 0;                  // next 32 tiles (of this part) or, unsplit, 32 blocks of tiles
+        int tile0 = 0;                 // current 32 tiles
+        unsigned mS = 0, mT = 0;       // surviving blocks of the round, tiles of the current 32
         for (;;) {
-            // list chunks that can hold a nonzero term
-            while (nlist <= SP_LIST - 32) {
+            // list chunks that can hold a nonzero background (from the front) and
+            // excitation (from the back)
+            int lB = 0, lE = 0;
+            while (lB + lE <= SP_LIST - 64) {
                 if (mT == 0) {
-                    const int first = tile0 * a.parts + part;
-                    if (first >= a.ntiles) break;
+                    if (a.parts == 1) {
+                        const int nblk = sp_blocks(a.ntiles);
+                        while (mS == 0 && next < nblk) {
+                            bool nb = false, ne = false;
+                            if (next + lane < nblk) sp_near(box, sp_load(a.bmeta, next + lane), omt, nb, ne);
+                            mS = __ballot_sync(ALL, nb || ne);
+                            next += 32;
+                        }
+                        if (mS == 0) break;
+                        tile0 = (next - 32 + __ffs(mS) - 1) * SP_TB;
+                        mS &= mS - 1;
+                    } else {
+                        tile0 = next;
+                        if (tile0 * a.parts + part >= a.ntiles) break;
+                        next += 32;
+                    }
                     const int t = (tile0 + lane) * a.parts + part;
                     bool nb = false, ne = false;
                     if (t < a.ntiles) sp_near(box, sp_load(a.tmeta, t), omt, nb, ne);
                     mT = __ballot_sync(ALL, nb || ne);
-                    if (mT == 0) tile0 += 32;
                     continue;
                 }
                 // the 8 chunks of the next (up to) 4 surviving tiles
@@ -482,104 +796,48 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
                 const int t = has ? (tile0 + __ffs(m) - 1) * a.parts + part : 0;
                 const int ch = t * (TC / SP_CH) + (lane & 7);
                 bool nb = false, ne = false;
-                if (has) sp_near(box, sp_load(a.cmeta, ch), omt, nb, ne);
-                const unsigned keep = __ballot_sync(ALL, nb || ne);
-                if (nb || ne) sw.list[nlist + __popc(keep & below)] = ch | (nb ? 1 << 29 : 0) | (ne ? 1 << 30 : 0);
-                nlist += __popc(keep);
-                if (mT == 0) tile0 += 32;
+                float4 entry = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (has) {
+                    const SpBox q = sp_load(a.cmeta, ch);
+                    sp_near(box, q, omt, nb, ne);
+                    const float width = fmaxf(fmaxf(q.x1 - q.x0, q.y1 - q.y0), q.t1 - q.t0);
+                    const float4 c = a.centre[ch];
+                    entry = make_float4(ref.x - c.x, ref.y - c.y, ref.z - c.z, 0.f);
+                    const float far = fmaxf(fmaxf(fabsf(entry.x), fabsf(entry.y)), fabsf(entry.z));
+                    entry.w = __int_as_float(ch | (width <= SP_REL ? 0 : SP_WIDE) | (width + far <= 256.f ? 0 : SP_FAR));
+                }
+                const unsigned kb = __ballot_sync(ALL, nb), ke = __ballot_sync(ALL, ne);
+                if (nb) sw.list[lB + __popc(kb & below)] = entry;
+                if (ne) sw.list[SP_LIST - 1 - lE - __popc(ke & below)] = entry;
+                lB += __popc(kb);
+                lE += __popc(ke);
             }
             __syncwarp();
-            if (nlist == 0) break;
-            // read the listed chunks, one event per lane, the next one ahead
-            int cur = sw.list[0];
-            int64_t p = static_cast<int64_t>(cur & ((1 << 29) - 1)) * SP_CH + lane;
-            float4 qa = a.ra[p], qb = a.rb[p];
-            int rk = a.rank[p];
-            for (int k = 0; k < nlist; ++k) {
-                const int id = cur;
-                const float4 ca = qa, cb = qb;
-                const int rank = rk & ~SP_TIED;
-                const bool real = rk >= 0;
-                const bool tied = (rk & SP_TIED) != 0 || (id & ((1 << 29) - 1)) == g;
-                if (k + 1 < nlist) {
-                    cur = sw.list[k + 1];
-                    p = static_cast<int64_t>(cur & ((1 << 29) - 1)) * SP_CH + lane;
-                    qa = a.ra[p];
-                    qb = a.rb[p];
-                    rk = a.rank[p];
-                }
-                const float dx = sp_gap(box.x0, box.x1, -ca.x, -ca.x), dy = sp_gap(box.y0, box.y1, -ca.z, -ca.z);
-                const float r2 = fmaf(dx, dx, dy * dy);
-                if (id & (1 << 29)) {
-                    const float gap = sp_gap(box.t0, box.t1, -cb.x, -cb.x);
-                    const bool keep = real && !(fmaf(gap, gap, r2) > SP_ZERO);
-                    const unsigned bal = __ballot_sync(ALL, keep);
-                    maskB |= __any_sync(ALL, keep && tied && rank >= lo_min && rank < hi_max);
-                    if (keep) {
-                        float* b = sw.b + nB + __popc(bal & below);
-                        b[0 * SP_BUF] = ca.x; b[1 * SP_BUF] = ca.y; b[2 * SP_BUF] = ca.z; b[3 * SP_BUF] = ca.w;
-                        b[4 * SP_BUF] = cb.x; b[5 * SP_BUF] = cb.y; b[6 * SP_BUF] = __int_as_float(rank);
-                    }
-                    nB += __popc(bal);
-                    if (nB >= 32) {
-                        __syncwarp();
-                        if (maskB) sp_eval_b<true, LL>(sw.b, 8, w);
-                        else sp_eval_b<false, LL>(sw.b, 8, w);
-                        nB -= 32;
-                        maskB = maskB && nB > 0;
-                        __syncwarp();
-                        if (lane < nB)
-#pragma unroll
-                            for (int q = 0; q < SP_B_PLANES; ++q) sw.b[q * SP_BUF + lane] = sw.b[q * SP_BUF + 32 + lane];
-                        __syncwarp();
-                    }
-                }
-                if (id & (1 << 30)) {
-                    const float tj = -cb.x;
-                    const bool keep = real && tj <= box.t1 &&
-                                      !(cb.w - omt * fmaxf(0.f, box.t0 - tj) + cb.z * r2 < -SP_ZERO);
-                    const unsigned bal = __ballot_sync(ALL, keep);
-                    maskE |= __any_sync(ALL, keep && rank >= lo_min);
-                    if (keep) {
-                        float* b = sw.e + nE + __popc(bal & below);
-                        b[0 * SP_BUF] = ca.x; b[1 * SP_BUF] = ca.y; b[2 * SP_BUF] = ca.z; b[3 * SP_BUF] = ca.w;
-                        b[4 * SP_BUF] = cb.x; b[5 * SP_BUF] = cb.y; b[6 * SP_BUF] = __int_as_float(rank);
-                        b[7 * SP_BUF] = cb.z; b[8 * SP_BUF] = cb.w;
-                    }
-                    nE += __popc(bal);
-                    if (nE >= 32) {
-                        __syncwarp();
-                        if (maskE) sp_eval_e<true, LL>(sw.e, 8, nomt, w);
-                        else sp_eval_e<false, LL>(sw.e, 8, nomt, w);
-                        nE -= 32;
-                        maskE = maskE && nE > 0;
-                        __syncwarp();
-                        if (lane < nE)
-#pragma unroll
-                            for (int q = 0; q < SP_E_PLANES; ++q) sw.e[q * SP_BUF + lane] = sw.e[q * SP_BUF + 32 + lane];
-                        __syncwarp();
-                    }
-                }
+            if (lB + lE == 0) break;
+            if (lB > 0) {
+                if (rel) sp_columns_b<true, LL>(a, sw, lB, gr, w, nB, maskB);
+                else sp_columns_b<false, LL>(a, sw, lB, gr, w, nB, maskB);
             }
-            nlist = 0;
+            if (lE > 0) sp_columns_e<LL>(a, sw, lE, gr, omt, w, nE, maskE);
             __syncwarp();
         }
         // what is left in the buffers, filled up to quads with columns whose
         // terms are zero
+        const int hB = nB & 32, hE = nE & 32;
+        nB &= 31;
+        nE &= 31;
         const int qB = (nB + 3) >> 2, qE = (nE + 3) >> 2;
         if (nB + lane < 4 * qB) {
-            for (int q = 0; q < SP_B_PLANES; ++q) sw.b[q * SP_BUF + nB + lane] = 0.f;
-            sw.b[4 * SP_BUF + nB + lane] = -PAD_T;
+            for (int q = 0; q < SP_B_PLANES; ++q) sw.b[q * SP_BUF + hB + nB + lane] = 0.f;
+            sw.b[(rel ? 2 : 4) * SP_BUF + hB + nB + lane] = -PAD_T;
         }
         if (nE + lane < 4 * qE) {
-            for (int q = 0; q < SP_E_PLANES; ++q) sw.e[q * SP_BUF + nE + lane] = 0.f;
-            sw.e[8 * SP_BUF + nE + lane] = -1e30f;
+            for (int q = 0; q < SP_E_PLANES; ++q) sw.e[q * SP_BUF + hE + nE + lane] = 0.f;
+            sw.e[8 * SP_BUF + hE + nE + lane] = -1e30f;
         }
         __syncwarp();
-        if (maskB) sp_eval_b<true, LL>(sw.b, qB, w);
-        else sp_eval_b<false, LL>(sw.b, qB, w);
-        if (maskE) sp_eval_e<true, LL>(sw.e, qE, nomt, w);
-        else sp_eval_e<false, LL>(sw.e, qE, nomt, w);
+        sp_background<LL>(sw, hB, qB, rel, maskB, w);
+        sp_excitation<LL>(sw, hE, qE, maskE, f2(-omt, -omt), w);
         __syncwarp();
         if (e >= 0) {
             const float v[6] = {w.sB.x + w.sB.y, w.sBr.x + w.sBr.y, w.sBt.x + w.sBt.y,
@@ -602,14 +860,20 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
 // of the staged records of the other paths.
 cudaError_t spatial_launch(hawkes_ctx* c, int model1, int llonly) {
     SpatialState* sp = c->sp;
+    SpArgs a;
     float4* ra = reinterpret_cast<float4*>(c->rec);
     float4* rb = ra + c->npad;
-    k_sp_prep<<<std::min(sp->ntiles, 8 * c->sms), TC, 0, c->stream>>>(eval_desc(c), sp->rank, model1, ra, rb,
-                                                                      sp->meta, sp->ntiles);
-    SpArgs a;
-    a.ra = ra; a.rb = rb; a.rank = sp->rank; a.lo = c->lo; a.hi = c->hi; a.cc = c->cc; a.acc = c->acc;
-    a.cmeta = sp->meta;
-    a.tmeta = sp->meta + 2 * static_cast<size_t>(sp->ntiles) * (TC / SP_CH);
+    float* rc = reinterpret_cast<float*>(rb + c->npad);
+    float4* cmeta = sp->meta;
+    float4* tmeta = cmeta + 16 * static_cast<size_t>(sp->ntiles);
+    float4* bmeta = tmeta + 2 * static_cast<size_t>(sp->ntiles);
+    const int nblk = sp_blocks(sp->ntiles);
+    float4* centre = bmeta + 2 * static_cast<size_t>(nblk);
+    cudaError_t err = launch_chained(k_sp_prep, std::min(sp->ntiles, 8 * c->sms), TC, 0, c->stream, eval_desc(c),
+                                     sp->rank, model1, ra, rb, rc, cmeta, tmeta, centre, sp->ntiles);
+    if (err != cudaSuccess) return err;
+    a.ra = ra; a.rb = rb; a.rc = rc; a.lo = c->lo; a.hi = c->hi; a.cc = c->cc; a.acc = c->acc;
+    a.cmeta = cmeta; a.tmeta = tmeta; a.bmeta = bmeta; a.centre = centre;
     a.npad = c->npad;
     a.ntiles = sp->ntiles;
     a.groups = static_cast<int>((c->n + SP_CH - 1) / SP_CH);
@@ -617,16 +881,27 @@ cudaError_t spatial_launch(hawkes_ctx* c, int model1, int llonly) {
     // resident CTA's worth of warps for every SM.
     const size_t smem = SP_WARPS * sizeof(SpWarp);
     auto* kern = llonly ? k_sweep_sp<true> : k_sweep_sp<false>;
-    static_assert(SP_WARPS * sizeof(SpWarp) <= 48 * 1024, "below the default dynamic limit");
     a.parts = 1;
     while (a.parts < 64 && 2 * a.parts <= a.ntiles &&
            static_cast<int64_t>(a.groups) * a.parts < static_cast<int64_t>(c->sms) * SP_BPSM * SP_WARPS)
         a.parts *= 2;
+    if (a.parts == 1) {
+        err = launch_chained(k_sp_blocks, nblk, SP_TB, 0, c->stream, tmeta, bmeta, sp->ntiles, c->cc);
+        if (err != cudaSuccess) return err;
+    }
     const int64_t nitems = static_cast<int64_t>(a.groups) * a.parts;
     const int grid = static_cast<int>(std::min<int64_t>((nitems + SP_WARPS - 1) / SP_WARPS,
                                                         static_cast<int64_t>(c->sms) * SP_BPSM));
-    kern<<<grid, SP_THREADS, smem, c->stream>>>(a, c->ctr, static_cast<int>(nitems));
-    return cudaGetLastError();
+    return launch_chained(kern, grid, SP_THREADS, smem, c->stream, a, c->ctr, static_cast<int>(nitems));
+}
+
+cudaError_t spatial_setup_attributes() {
+    for (auto* k : {k_sweep_sp<false>, k_sweep_sp<true>}) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   static_cast<int>(SP_WARPS * sizeof(SpWarp)));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace hk
