@@ -292,7 +292,7 @@ int hawkes_profile_read(hawkes_ctx* ctx, hawkes_profile* out);
  * Kernel variants of the FP32 pair sweep (rows per thread, resident CTAs per
  * SM).  All give the same result up to FP32 summation order; they differ in
  * speed by problem size.  They hold for row windows, shards and whole sums of
- * about 36,000 events and more; smaller whole sums, whose variants' row tiles
+ * about 28,000 events and more; smaller whole sums, whose variants' row tiles
  * would leave most SMs idle, are swept with smaller tiles.  hawkes_sweep_variants() is their number;
  * hawkes_set_sweep_variant selects one (synchronous; rebuilds the work list).
  */
@@ -404,8 +404,7 @@ int hawkes_batch_wait(hawkes_batch* batch);
 
 /*
  * Autotune the batch over the sweep variant, the column-chunk length of a
- * work item (16, 32 or 64 tiles of 256 sources, or the length chosen for the
- * problems' sizes when the batch is made), the item order (0: all
+ * work item (16, 32 or 64 tiles of 256 sources), the item order (0: all
  * items longest first; 1: problem by problem, largest problem first, each
  * longest first) and the chains per CTA (1, 2 or 4; see
  * hawkes_batch_set_chains_per_cta).  Each configuration's sweep launches
@@ -420,9 +419,11 @@ int hawkes_batch_tune(hawkes_batch* batch, const hawkes_params* d_params, double
 
 /*
  * Select the sweep variant, chunk length and item order directly (drops a
- * captured graph).  Batches of small problems (below about 36,000 events) are
- * swept by a kernel with smaller row tiles whatever the variant; the chunk
- * length and order hold for it too.
+ * captured graph).  A chunk length up to 16 is the longest that items have:
+ * small problems take shorter ones, so that every SM has several; a length
+ * above 16 is taken as it is.  Batches of few events (one problem below about
+ * 28,000) are swept by a kernel with smaller row tiles whatever the variant; the
+ * chunk length and order hold for it too.
  */
 int hawkes_batch_set_config(hawkes_batch* batch, int variant, int chunk, int order);
 

@@ -31,11 +31,13 @@ __global__ void k_wait_selftest(int*);
 cudaError_t sweep_setup_attributes();
 int sweep_num_variants();
 int sweep_blocks_per_sm(int v);
-SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk);
+SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk, bool band);
 std::vector<int4> sweep_items(int64_t n, const SweepPlan& pl, int v);
 cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row_end, bool bgt,
                          bool ll);
-cudaError_t launch_sweep_list(hawkes_ctx* c, const int4* items, int nitems, bool bgt, bool ll);
+cudaError_t launch_sweep_list(hawkes_ctx* c, const int4* items, int nitems, int nband, bool bgt, bool ll);
+int split_rows();
+std::vector<int4> sweep_band(const std::vector<int64_t>& ns, const SweepPlan& pl, int v);
 int sweep_variant_rows(int v);
 // rows64.cu
 int rows64_segments(int64_t rows, int sms);
@@ -123,7 +125,7 @@ int grid_for(hawkes_ctx* c, int64_t items, int per_sm = 8) {
 
 void drop_shard_items(hawkes_ctx* c) {
     dfree(c->shard_items);
-    c->shard_nitems = 0;
+    c->shard_nitems = c->shard_nband = 0;
     c->shard_key[0] = c->shard_key[1] = c->shard_key[2] = -1;
 }
 
@@ -166,13 +168,17 @@ bool params_ok(const hawkes_params* p) {
 int ensure_items(hawkes_ctx* c) {
     if (c->items && c->items_variant == c->variant) return HAWKES_OK;
     dfree(c->items);
-    c->plan = sweep_plan({c->n}, c->sms, c->variant, 0);
-    const std::vector<int4> items = sweep_items(c->n, c->plan, c->variant);
+    c->plan = sweep_plan({c->n}, c->sms, c->variant, 0, true);
+    std::vector<int4> items = sweep_items(c->n, c->plan, c->variant);
+    const std::vector<int4> band = sweep_band({c->n}, c->plan, c->variant);
+    const size_t nitems = items.size();
+    items.insert(items.end(), band.begin(), band.end());
     HK_TRY(dalloc(&c->items, items.size()));
     HK_CUDA(cudaMemcpyAsync(c->items, items.data(), items.size() * sizeof(int4),
                             cudaMemcpyHostToDevice, c->stream));
     HK_CUDA(cudaStreamSynchronize(c->stream));
-    c->nitems = static_cast<int>(items.size());
+    c->nitems = static_cast<int>(nitems);
+    c->nband = static_cast<int>(band.size());
     c->items_variant = c->variant;
     return HAWKES_OK;
 }
@@ -623,16 +629,22 @@ int hawkes_shard_moments(hawkes_ctx* c, const hawkes_params* d_params, uint32_t 
         HK_TRY(hawkes_shard_bounds(c->n, tr, nshards, b.data()));
         const int64_t I0 = b[shard] / tr, I1 = (b[shard + 1] + tr - 1) / tr;
         std::vector<int4> mine;
-        // (row tiles in the whole sweep's item lengths, where it runs on row tiles:
-        // the same FP32 partial sums)
-        const SweepPlan pl{false, c->plan.split ? CHUNK : c->plan.chunk};
+        // (the whole sweep's items, where it runs on row tiles: the same FP32 partial
+        // sums)
+        const SweepPlan pl = c->plan.split ? SweepPlan{false, CHUNK, false} : c->plan;
         for (const int4& it : sweep_items(c->n, pl, c->variant))
             if (it.x >= I0 && it.x < I1) mine.push_back(it);
+        const size_t nitems = mine.size();
+        for (const int4& it : sweep_band({c->n}, pl, c->variant)) {
+            const int64_t I = static_cast<int64_t>(it.x) * split_rows() / tr;
+            if (I >= I0 && I < I1) mine.push_back(it);
+        }
         HK_TRY(dalloc(&c->shard_items, mine.size()));
         HK_CUDA(cudaMemcpyAsync(c->shard_items, mine.data(), mine.size() * sizeof(int4),
                                 cudaMemcpyHostToDevice, c->stream));
         HK_CUDA(cudaStreamSynchronize(c->stream));
-        c->shard_nitems = static_cast<int>(mine.size());
+        c->shard_nitems = static_cast<int>(nitems);
+        c->shard_nband = static_cast<int>(mine.size() - nitems);
         for (int q = 0; q < 3; ++q) c->shard_key[q] = key[q];
     }
     const int model = static_cast<int>(flags & kModelBits);
@@ -640,7 +652,7 @@ int hawkes_shard_moments(hawkes_ctx* c, const hawkes_params* d_params, uint32_t 
     HK_TRY(enqueue_prep(c, CallParams{d_params, {}}, model, 1, skip));
     cudaError_t se = cudaSuccess;
     HK_TRY(timed(c, HAWKES_K_SWEEP, [&] {
-        se = launch_sweep_list(c, c->shard_items, c->shard_nitems, (flags & HAWKES_BG_TIME) != 0,
+        se = launch_sweep_list(c, c->shard_items, c->shard_nitems, c->shard_nband, (flags & HAWKES_BG_TIME) != 0,
                                (flags & HAWKES_LOGLIK_ONLY) != 0);
     }));
     HK_CUDA(se);

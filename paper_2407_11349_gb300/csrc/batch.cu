@@ -38,11 +38,12 @@ cudaError_t launch_group_stage(cudaStream_t st, int sms, const GroupDesc& gd,
                                const Rec* const* recs, const double* t, int kc, float4* out);
 cudaError_t launch_sweep_group(cudaStream_t st, int kc, int grid, const GroupDesc* groups,
                                int ngroups, const int4* items, int nitems, int* ctr);
-SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk);
+SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk, bool band);
+std::vector<int4> sweep_band(const std::vector<int64_t>& ns, const SweepPlan& pl, int v);
 std::vector<int4> sweep_items_batch(const std::vector<int64_t>& ns, const SweepPlan& pl, int v,
                                     int order);
 cudaError_t launch_sweep_batch(cudaStream_t st, const SweepPlan& pl, int sms, int variant, int grid,
-                               const ProbDesc* probs, int nprobs, const int4* items, int nitems,
+                               const ProbDesc* probs, int nprobs, const int4* items, int nitems, int nband,
                                int* ctr, bool bgt, bool ll);
 
 __global__ void k_set_u64(uint64_t* dst, uint64_t v) {
@@ -90,11 +91,11 @@ struct hawkes_batch {
     EvalDesc* d_eval = nullptr;
     std::vector<EvalDesc> h_eval;  // what d_eval holds
     int4* d_items = nullptr;
-    int nitems = 0;
+    int nitems = 0, nband = 0;  // one-problem items, then those of the diagonal band
     int variant = 0;
     int chunk = CHUNK;
     int order = 1;
-    SweepPlan plan{false, CHUNK};  // how the one-problem items are cut
+    SweepPlan plan{false, CHUNK, false};  // how the one-problem items are cut
     int grid = 0;
     int* d_ctr = nullptr;        // [2 CT_COUNT]: work cursor, latched error (batch kernel, group kernel)
     uint64_t* d_iter = nullptr;  // iteration read by the resample kernels
@@ -259,13 +260,16 @@ int build_groups(hawkes_batch* b, int chunk) {
     return HAWKES_OK;
 }
 
-// chunk 0: chosen for the problems' sizes (sweep_plan); only without groups.
+// chunk: as in sweep_plan; the group kernel's items are that long.
 int build_items(hawkes_batch* b, int variant, int chunk, int order) {
     HB_TRY(build_groups(b, chunk));
     std::vector<int64_t> ns;
     for (int p : b->singles) ns.push_back(b->probs[p]->n);
-    b->plan = sweep_plan(ns, b->sms, variant, chunk);
+    b->plan = sweep_plan(ns, b->sms, variant, chunk, true);
     std::vector<int4> items = sweep_items_batch(ns, b->plan, variant, order);
+    const size_t nitems = items.size();
+    const std::vector<int4> band = sweep_band(ns, b->plan, variant);
+    items.insert(items.end(), band.begin(), band.end());
     for (int4& it : items) it.w = b->singles[it.w];  // index into all problems
     if (b->d_items) cudaFree(b->d_items);
     b->d_items = nullptr;
@@ -273,9 +277,10 @@ int build_items(hawkes_batch* b, int variant, int chunk, int order) {
     HB_CUDA(cudaMemcpyAsync(b->d_items, items.data(), items.size() * sizeof(int4),
                             cudaMemcpyHostToDevice, b->stream));
     HB_CUDA(cudaStreamSynchronize(b->stream));
-    b->nitems = static_cast<int>(items.size());
+    b->nitems = static_cast<int>(nitems);
+    b->nband = static_cast<int>(band.size());
     b->variant = variant;
-    b->chunk = b->plan.chunk;
+    b->chunk = chunk;
     b->order = order;
     b->grid = b->sms * sweep_blocks_per_sm(variant);
     drop_graph(b);  // a captured graph refers to the old work list
@@ -337,7 +342,7 @@ int enqueue(hawkes_batch* b, const hawkes_params* d_params, double* d_out, bool 
                                    static_cast<int>(b->h_groups.size()), b->d_gitems, b->ngitems,
                                    b->d_ctr + CT_COUNT));
     HB_CUDA(launch_sweep_batch(st, b->plan, b->sms, b->variant, b->grid, b->d_probs, P, b->d_items,
-                               b->nitems, b->d_ctr, bgt, (b->flags & HAWKES_LOGLIK_ONLY) != 0));
+                               b->nitems, b->nband, b->d_ctr, bgt, (b->flags & HAWKES_LOGLIK_ONLY) != 0));
     if (time_sweep) HB_CUDA(cudaEventRecord(b->ev[1], st));
     launch_finalize(st, dim3(final_grid(nmax, b->sms, P), P), EvalDesc{}, b->d_eval, 0, 0, 1, nullptr,
                     1, d_out, nullptr, nullptr);
@@ -422,7 +427,7 @@ int hawkes_batch_create(hawkes_batch** out, hawkes_ctx* const* problems, int32_t
             if ((rc = st_of(cudaStreamSynchronize(c->stream)))) break;
         if (rc) break;
         if ((rc = time_classes(b))) break;
-        rc = build_items(b, 0, 0, 1);
+        rc = build_items(b, 0, CHUNK, 1);
     } while (0);
     if (rc != HAWKES_OK) {
         hawkes_batch_destroy(b);
@@ -508,7 +513,7 @@ int hawkes_batch_tune(hawkes_batch* b, const hawkes_params* d_params, double* d_
     if (!b || !d_params || !d_out || !aligned8(d_params) || !aligned8(d_out) || reps < 1)
         return HAWKES_ERR_ARG;
     DeviceGuard g(b->device);
-    static const int kChunks[] = {0, 16, 32, 64};  // 0: by the problems' sizes
+    static const int kChunks[] = {16, 32, 64};
     int bv = -1, bc = 0, bo = 0, bk = 1;
     double bms = 0.0;
     auto time_one = [&](int v, int ch, int o, double* t) -> int {
@@ -535,7 +540,7 @@ int hawkes_batch_tune(hawkes_batch* b, const hawkes_params* d_params, double* d_
                 HB_TRY(time_one(v, ch, o, &t));
                 if (bv < 0 || t < bms) {
                     bv = v;
-                    bc = b->chunk;
+                    bc = ch;
                     bo = o;
                     bms = t;
                 }
@@ -549,7 +554,6 @@ int hawkes_batch_tune(hawkes_batch* b, const hawkes_params* d_params, double* d_
             if (!group_kc_supported(kc) || largest_class(b) < static_cast<size_t>(kc)) continue;
             b->kc = kc;
             for (int ch : kChunks) {
-                if (ch == 0) continue;
                 double t = 0.0;
                 HB_TRY(time_one(bv, ch, bo, &t));
                 if (t < bms) {

@@ -165,10 +165,13 @@ inline int final_grid(int64_t rows, int sms, int problems = 1) {
 
 // How the symmetric sweep of a problem (or of a batch) is cut into work items
 // of `chunk` column tiles: by the row-tile kernel of the selected variant
-// (k_sweep), or by the column-split kernel (k_sweep_cs).
+// (k_sweep), or by the column-split kernel (k_sweep_cs); with `band`, the row
+// tiles leave out the columns of their own rows, which the column-split kernel
+// takes.
 struct SweepPlan {
     bool split;
     int chunk;
+    bool band;
 };
 
 // A group of chains with identical event times, swept kc at a time by the
@@ -239,6 +242,7 @@ enum {
     CT_CEMAX,       // bits of max(0, max_j -2 log2 s_j), set when the events are loaded
     CT_FDONE,       // finished blocks of k_finalize
     CT_RDONE,       // finished blocks of k_rows64 (fix-up rows)
+    CT_BAND,        // work-queue cursor of the diagonal band
     CT_COUNT = 8
 };
 
@@ -386,8 +390,9 @@ struct hawkes_ctx {
     hk::Rec* rec = nullptr;    // [npad] staged FP32 records
     int4* items = nullptr;     // symmetric-sweep work list
     int nitems = 0;
+    int nband = 0;             // items of the diagonal band, behind the nitems others
     int items_variant = -1;    // variant the work list was built for
-    hk::SweepPlan plan{false, 0};  // how the work list cuts the symmetric sweep
+    hk::SweepPlan plan{false, 0, false};  // how the work list cuts the symmetric sweep
     int variant = 0;           // sweep kernel variant in use
     int variant_bpsm = 1;      // its resident CTAs per SM
     double* acc = nullptr;     // [6 * npad] per-row moment sums (natural units)
@@ -419,7 +424,7 @@ struct hawkes_ctx {
     // Work list of one shard of the symmetric sweep (hawkes_shard_moments),
     // for (nshards, shard, variant) = shard_key; rebuilt when any changes.
     int4* shard_items = nullptr;
-    int shard_nitems = 0;
+    int shard_nitems = 0, shard_nband = 0;
     int shard_key[3] = {-1, -1, -1};
 };
 

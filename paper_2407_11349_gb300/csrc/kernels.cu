@@ -156,6 +156,7 @@ __global__ void k_prep(const __grid_constant__ EvalDesc one, const EvalDesc* __r
         s_beta0 = k.beta0;
         if (threadIdx.x == 0 && bctr && blockIdx.x == 0 && blockIdx.y == 0) {
             bctr[CT_WORK] = 0;
+            bctr[CT_BAND] = 0;
             bctr[CT_COUNT + CT_WORK] = 0;
         }
         if (threadIdx.x == 0 && blockIdx.x == 0) {
@@ -203,6 +204,7 @@ __global__ void k_prep(const __grid_constant__ EvalDesc one, const EvalDesc* __r
             cc[CC_F0 + 5] = LE * F * ((cemax + 127.0) * k.seq * ih3 + 2.0 * ih);
             cc[CC_F0 + 6] = LE * F;
             ctr[CT_WORK] = 0;
+            ctr[CT_BAND] = 0;
             ctr[CT_FIX] = 0;
             ctr[CT_DONE] = 0;
             ctr[CT_FDONE] = 0;

@@ -3,6 +3,7 @@
 // space-time background's kernels; sweep_bgt.cu the time-only background's
 // and sweep_ll.cu the log-likelihood-only ones.
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 #include "sweep_kernel.cuh"
@@ -13,7 +14,7 @@ namespace hk {
 cudaError_t split_setup_attributes();
 int split_rows();
 cudaError_t launch_sweep_split(cudaStream_t st, int sms, const ProbDesc& one, const ProbDesc* probs,
-                               int nprobs, const int4* items, int nitems, int* ctr, bool bgt, bool ll);
+                               int nprobs, const int4* items, int nitems, int* ctr, bool bgt, bool ll, bool band);
 
 static const Variant kVariants[] = HK_SWEEP_VARIANTS(false, false);
 static_assert(sizeof(kVariants) / sizeof(kVariants[0]) == kNumVariants, "variant count");
@@ -62,32 +63,55 @@ static int pow2_floor(double v, int cap) {
     return p;
 }
 
-// The plan for problems of sizes ns[] swept in one launch on variant v.
-//   chunk > 0: that many column tiles per item; 0: chosen here.
-// Kernel: a row tile's units that lie partly above the diagonal leave warps
-// idle.  Where the row tiles cover more than 1.1 times the pairs that the
-// column-split kernel's 128-row items cover (N below about 36,000), the
-// latter runs: 0.402 against 0.434 ms at N = 30,000; at N = 50,000 (1.08
-// times) it would be 1.056 against 1.042.  30 chains of 20,000 events (1.14
-// times): 4.29 against 4.52 ms per step.
-// Chunk: small enough for 16 items per SM (the tail), large enough to
-// amortise an item's row flush.  Row tiles: N = 100,000 3.95 ms with 4 against
-// 4.07 with 16; 250,000 23.2 with 16 against 23.5 with 4.  Column split: from
-// three items per SM up to 4 tiles (N = 17,103: 0.144 ms with 4, 0.163 with
-// 1; N = 5,000: 0.023 with 1, 0.028 with 2), and 8 where 64 items per SM are
-// left (30 x 20,000: 4.29 with 8, 4.44 with 4).
-SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk) {
-    double rows = 0.0, split = 0.0;
+// The plan for problems of sizes ns[] swept together on variant v.
+//   chunk: most column tiles per item, up to CHUNK (0: CHUNK); above CHUNK that many.
+//   band: the work list may have a diagonal band (SweepPlan).
+//
+// With a band.  A row tile's units that lie partly above the diagonal leave
+// warps idle, and a persistent kernel ends on whole items of up to CHUNK units
+// (N = 100,000: 62 units per SM).  So the row tiles take only the columns
+// below their own rows, and the column-split kernel takes the band between;
+// it starts while the row tiles' last items run and fills the SMs they leave:
+// N = 100,000 3.96 -> 3.75 ms, 50,000 1.047 -> 0.965, 30,000 0.402 -> 0.379.
+// Items are as long as the rounds over the SMs come out shortest, in units of
+// one row tile x one column tile; an item's row flush costs 0.07 of one.  The
+// column-split kernel alone takes 1.1 times the pairs' units and 0.35 (measured
+// within 3% from N = 12,000 to 30,000), and is chosen where that is less (N below
+// about 28,000).
+//
+// Without: column split where the row tiles cover more than 1.1 times its pairs
+// (N below about 36,000); items for 16 per SM.
+//
+// Column-split items: from three items per SM up to 4 tiles (N = 17,103:
+// 0.144 ms with 4, 0.163 with 1; N = 5,000: 0.023 with 1, 0.028 with 2), and 8
+// where 64 items per SM are left.
+SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk, bool band) {
+    const int tr = kVariants[v].tr;
+    double rows = 0.0, split = 0.0, below = 0.0;  // units: tr x TC, split_rows() x TC, tr x TC
     for (int64_t n : ns) {
-        rows += static_cast<double>(plan_units(n, kVariants[v].tr)) * kVariants[v].tr;
-        split += static_cast<double>(plan_units(n, split_rows())) * split_rows();
+        const double full = static_cast<double>((n - 1) / tr);  // row tiles with columns below them
+        rows += static_cast<double>(plan_units(n, tr));
+        split += static_cast<double>(plan_units(n, split_rows()));
+        below += full * (full + 1.0) / 2.0 * (tr / TC);
     }
-    SweepPlan pl{rows > 1.1 * split, chunk};
-    if (chunk <= 0) {
-        const double u = pl.split ? split / split_rows() : rows / kVariants[v].tr;  // items of one tile
-        pl.chunk = pl.split ? std::max(pow2_floor(u / (3.0 * sms), 4), pow2_floor(u / (64.0 * sms), 8))
-                            : pow2_floor(u / (16.0 * sms), CHUNK);
+    SweepPlan pl{rows * tr > 1.1 * split * split_rows(), chunk, false};
+    int best = pow2_floor(rows / (16.0 * sms), CHUNK);
+    if (band) {
+        const double slots = static_cast<double>(sms) * kVariants[v].minb, all = split * split_rows() / tr, flush = 0.07;
+        double least = 1e300;
+        for (int c = CHUNK; c >= 1; c /= 2) {
+            const double items = below / c;
+            const double t = std::max(std::ceil(items / slots) * (c + flush), (all + flush * items) / slots);
+            if (t < least) {
+                least = t;
+                best = c;
+            }
+        }
+        pl.split = below == 0.0 || 1.1 * all / slots + 0.35 < least;
+        pl.band = !pl.split;
     }
+    if (pl.split) best = std::max(pow2_floor(split / (3.0 * sms), 4), pow2_floor(split / (64.0 * sms), 8));
+    if (chunk <= CHUNK) pl.chunk = chunk <= 0 ? best : std::min(best, chunk);
     return pl;
 }
 
@@ -113,7 +137,7 @@ std::vector<int4> sweep_items_batch(const std::vector<int64_t>& ns, const SweepP
         const int64_t nI = (n + tr - 1) / tr;
         const size_t first = items.size();
         for (int64_t I = 0; I < nI; ++I) {
-            const int nJ = static_cast<int>((std::min<int64_t>((I + 1) * tr, n) + TC - 1) / TC);
+            const int nJ = static_cast<int>(pl.band ? I * tr / TC : (std::min<int64_t>((I + 1) * tr, n) + TC - 1) / TC);
             for (int jb = 0; jb < nJ; jb += chunk)
                 items.push_back(make_int4(static_cast<int>(I), jb, std::min(jb + chunk, nJ),
                                           static_cast<int>(p)));
@@ -121,6 +145,21 @@ std::vector<int4> sweep_items_batch(const std::vector<int64_t>& ns, const SweepP
         if (order == 1) std::stable_sort(items.begin() + first, items.end(), longest_first);
     }
     if (order == 0) std::stable_sort(items.begin(), items.end(), longest_first);
+    return items;
+}
+
+// Items of the diagonal band, for the column-split kernel: the columns that the
+// row tiles of a plan with `band` leave out.
+std::vector<int4> sweep_band(const std::vector<int64_t>& ns, const SweepPlan& pl, int v) {
+    std::vector<int4> items;
+    if (!pl.band) return items;
+    const int tr = kVariants[v].tr, rows = split_rows();
+    for (size_t p = 0; p < ns.size(); ++p)
+        for (int64_t r = 0; r < ns[p]; r += rows)
+            items.push_back(make_int4(static_cast<int>(r / rows), static_cast<int>(r / tr * (tr / TC)),
+                                      static_cast<int>((std::min<int64_t>(r + rows, ns[p]) + TC - 1) / TC),
+                                      static_cast<int>(p)));
+    std::stable_sort(items.begin(), items.end(), [](const int4& a, const int4& b) { return a.z - a.y > b.z - b.y; });
     return items;
 }
 
@@ -132,15 +171,20 @@ static ProbDesc desc_of(const hawkes_ctx* c) {
     return ProbDesc{c->t, c->rec, c->lo, c->hi, c->tb, c->cc, c->acc, c->n, c->npad};
 }
 
-// Row-tile sweep of one problem over the work list items[0, nitems) (the whole
-// list, or one shard's part of it).
-cudaError_t launch_sweep_list(hawkes_ctx* c, const int4* items, int nitems, bool bgt, bool ll) {
+// Row-tile sweep of one problem over the work list items[0, nitems) and the
+// diagonal band's items behind it (the whole lists, or one shard's part of them).
+cudaError_t launch_sweep_list(hawkes_ctx* c, const int4* items, int nitems, int nband, bool bgt, bool ll) {
     const Variant& v = variant_of(c->variant, bgt, ll);
     const int grid_cap = c->sms * c->variant_bpsm;
     const int grid = nitems < grid_cap ? nitems : grid_cap;
-    if (grid <= 0) return cudaSuccess;
-    return launch_chained(v.sym, grid, THREADS, v.smem, c->stream, desc_of(c), nullptr, items, nitems, c->ctr,
-                          0, c->n, 0, 0);
+    if (grid > 0) {
+        const cudaError_t e = launch_chained(v.sym, grid, THREADS, v.smem, c->stream, desc_of(c), nullptr, items,
+                                             nitems, c->ctr, 0, c->n, nband > 0 ? 1 : 0, 0);
+        if (e != cudaSuccess) return e;
+    }
+    if (nband == 0) return cudaSuccess;
+    return launch_sweep_split(c->stream, c->sms, desc_of(c), nullptr, 0, items + nitems, nband, c->ctr, bgt, ll,
+                              nitems > 0);
 }
 
 cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row_end, bool bgt,
@@ -150,9 +194,9 @@ cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row
     const ProbDesc one = desc_of(c);
     if (sym && c->plan.split) {
         return launch_sweep_split(c->stream, c->sms, one, nullptr, 0, c->items, c->nitems, c->ctr, bgt,
-                                  ll);
+                                  ll, false);
     } else if (sym) {
-        return launch_sweep_list(c, c->items, c->nitems, bgt, ll);
+        return launch_sweep_list(c, c->items, c->nitems, c->nband, bgt, ll);
     } else {
         const int item0 = static_cast<int>(row_begin / v.tr);
         const int nrt = static_cast<int>((row_end + v.tr - 1) / v.tr) - item0;
@@ -166,18 +210,23 @@ cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row
     }
 }
 
-// One persistent launch over the items of many problems; ctr[CT_WORK] must be
-// zero when it starts.
+// Persistent launches over the items of many problems; ctr[CT_WORK] and
+// ctr[CT_BAND] must be zero when they start.
 cudaError_t launch_sweep_batch(cudaStream_t st, const SweepPlan& pl, int sms, int variant, int grid,
-                               const ProbDesc* probs, int nprobs, const int4* items, int nitems,
+                               const ProbDesc* probs, int nprobs, const int4* items, int nitems, int nband,
                                int* ctr, bool bgt, bool ll) {
     if (pl.split)
-        return launch_sweep_split(st, sms, ProbDesc{}, probs, nprobs, items, nitems, ctr, bgt, ll);
+        return launch_sweep_split(st, sms, ProbDesc{}, probs, nprobs, items, nitems, ctr, bgt, ll, false);
     const Variant& v = variant_of(variant, bgt, ll);
     if (grid > nitems) grid = nitems;
-    if (grid <= 0) return cudaSuccess;
     ProbDesc none{};
-    return launch_chained(v.batch, grid, THREADS, v.smem, st, none, probs, items, nitems, ctr, 0, 0, 0, nprobs);
+    if (grid > 0) {
+        const cudaError_t e = launch_chained(v.batch, grid, THREADS, v.smem, st, none, probs, items, nitems, ctr, 0, 0,
+                                             nband > 0 ? 1 : 0, nprobs);
+        if (e != cudaSuccess) return e;
+    }
+    if (nband == 0) return cudaSuccess;
+    return launch_sweep_split(st, sms, none, probs, nprobs, items + nitems, nband, ctr, bgt, ll, nitems > 0);
 }
 
 }  // namespace hk

@@ -231,6 +231,8 @@ enum { MODE_WIN = 0, MODE_SYM = 1, MODE_BATCH = 2 };
 //               launch, one queue)
 //   MODE_WIN:   item k -> row tile item0 + k / nch, column chunk k % nch of
 //               problem `one`, rows [row_begin, row_end) only
+// MODE_SYM and MODE_BATCH: item0 != 0 lets the next kernel in the stream (the
+// diagonal band) take each SM as it falls idle.
 // In MODE_BATCH, nch is the number of problems (checked in debug builds).
 template <int RP, int MINB, int UNROLL, int MODE, bool BGT, bool LL>
 __global__ void __launch_bounds__(THREADS, MINB)
@@ -257,6 +259,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     chain_wait();
+    if (SYM && item0 != 0) chain_next();
     if (MODE != MODE_BATCH && one.cc[CC_VALID] == 0.0) return;
     if (tid == 0) {
         mbar_init(&bars[0], 1);

@@ -52,7 +52,7 @@ static_assert(TC == 32 * WARPS, "one 32-column chunk of a tile per warp");
 template <int RP, int MINB, int MODE, bool BGT, bool LL>
 __global__ void __launch_bounds__(THREADS, MINB)
     k_sweep_cs(ProbDesc one, const ProbDesc* __restrict__ probs, const int4* __restrict__ items,
-               int nitems, int* __restrict__ ctr, int nprobs) {
+               int nitems, int* __restrict__ ctr, int nprobs, int band) {
     using G = SGeo<RP>;
     constexpr int R = G::R, ROWS = G::ROWS;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -67,8 +67,13 @@ __global__ void __launch_bounds__(THREADS, MINB)
     volatile ProbDesc* vpd = &s_pd;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    chain_wait();
-    if (MODE != MODE_BATCH && one.cc[CC_VALID] == 0.0) return;
+    // As the band of a row-tile sweep, this kernel starts while that one runs: its
+    // inputs were complete when that one started, and its end waits for that one's.
+    if (!band) chain_wait();
+    if (MODE != MODE_BATCH && one.cc[CC_VALID] == 0.0) {
+        if (band) chain_wait();
+        return;
+    }
     if (tid == 0) {
         mbar_init(&bars[0], 1);
         mbar_init(&bars[1], 1);
@@ -82,7 +87,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
 
     for (;;) {
         if (tid == 0) {
-            const int k = atomicAdd(ctr + CT_WORK, 1);
+            const int k = atomicAdd(ctr + (band ? CT_BAND : CT_WORK), 1);
             s_item = k;
             if (kDebug) s_bad = 0;
             if (kDebug && MODE == MODE_BATCH && k < nitems &&
@@ -267,9 +272,10 @@ __global__ void __launch_bounds__(THREADS, MINB)
     if (tid == 0)
         for (int q = 0; q < 2; ++q)
             if ((pendbits >> q) & 1u) (void)mbar_wait(&bars[q], (parbits >> q) & 1u);
+    if (band) chain_wait();
 }
 
-using SplitFn = void (*)(ProbDesc, const ProbDesc*, const int4*, int, int*, int);
+using SplitFn = void (*)(ProbDesc, const ProbDesc*, const int4*, int, int*, int, int);
 
 struct SplitKernel {
     SplitFn sym, batch;
@@ -295,14 +301,15 @@ cudaError_t split_setup_attributes() {
 
 int split_rows() { return SGeo<SPLIT_RP>::ROWS; }
 
-// One problem (probs null) or the items of many.
+// One problem (probs null) or the items of many; band: launched behind a row-tile
+// sweep of the same problems that lets it start early.
 cudaError_t launch_sweep_split(cudaStream_t st, int sms, const ProbDesc& one, const ProbDesc* probs,
-                               int nprobs, const int4* items, int nitems, int* ctr, bool bgt, bool ll) {
+                               int nprobs, const int4* items, int nitems, int* ctr, bool bgt, bool ll, bool band) {
     const SplitKernel& k = kSplit[bgt ? 1 : ll ? 2 : 0];
     const int grid = std::min(nitems, sms * SPLIT_BPSM);
     if (grid <= 0) return cudaSuccess;
     return launch_chained(probs ? k.batch : k.sym, grid, THREADS, k.smem, st, one, probs, items, nitems, ctr,
-                          nprobs);
+                          nprobs, band ? 1 : 0);
 }
 
 }  // namespace hk
