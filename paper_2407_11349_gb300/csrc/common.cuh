@@ -314,6 +314,20 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     return false;
 }
 
+// Lower bounds for the proof that an FP64 term is zero.
+// FP32 form of a scale factor, not above it, and small enough that the rounding
+// of a subnormal difference stays below 2^-40 when scaled.
+__device__ __forceinline__ float bound_scale(double a) {
+    return a > 1e30 ? 1e30f : __double2float_rd(a);
+}
+
+// |a| in FP32, 0 where its square could overflow.  (Rounded to nearest: the
+// callers' thresholds leave 0.6% for it.)
+__device__ __forceinline__ float bound_diff(double a) {
+    const float f = fabsf(static_cast<float>(a));
+    return f < 1e18f ? f : 0.f;
+}
+
 // 2^x on the special-function unit; results below 2^-126 flush to zero.
 __device__ __forceinline__ float ex2(float x) {
     float y;

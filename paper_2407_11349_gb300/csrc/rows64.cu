@@ -73,12 +73,6 @@ __device__ __forceinline__ float low_diff(float a, float b) {
 __device__ __forceinline__ float bound_coord(double a) {
     return fabs(a) < 1e18 ? static_cast<float>(a) : __int_as_float(0x7fc00000);
 }
-// FP32 form of a scale factor, not above it, and small enough that the rounding
-// of a subnormal difference stays below 2^-40 when scaled.
-__device__ __forceinline__ float bound_scale(double a) {
-    return a > 1e30 ? 1e30f : __double2float_rd(a);
-}
-
 // Items: (group of 32 rows from row_begin, segment of the columns).  Sums go to
 // out[(segment * 6 + moment) * stride + row - origin].
 template <bool BGT>
