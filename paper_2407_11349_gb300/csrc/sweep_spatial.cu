@@ -35,16 +35,17 @@
 // with two words: 1.5e-7).
 //
 // What bounds it: instruction dispatch.  A packed FP32 instruction takes two
-// dispatch cycles, any other one; at N = 1,000,000 (3,143 counties, 1,200 days)
-// a group takes 93,000 such cycles of the 97,000 it has, half of them in the
-// evaluation of the columns that pass the point test.  A row has 1,811 columns
-// with a nonzero background and 14 with a nonzero excitation; point tests
-// against the box of 32 rows leave 3,770 and 620.  Sweep 3.39 ms; 4.05 with two
-// words throughout, one list, and buffers moved down after each evaluation; the
-// former design, 256 x 256 tile pairs kept whole by box tests and swept through
-// shared-memory tiles, 45 ms (40,000 columns with both terms).  Two rows per lane
-// would halve the shared-memory reads, but the box of 64 rows keeps 48% more
-// columns.
+// dispatch cycles, any other one.  At N = 1,000,000 (3,143 counties, 1,200 days;
+// order built at the evaluated locations) a group takes 92,500 such cycles of
+// about 94,000, half of them in the evaluation of the columns that pass the point
+// test: 2.48 ms, 3.29 with two words throughout, one list for both terms, and
+// buffers moved down after each evaluation.  After a resample the boxes are wider:
+// a row has 1,811 columns with a nonzero background and 14 with a nonzero
+// excitation, point tests against the box of 32 rows leave 3,770 and 620, in 3.39
+// ms (4.05).  The design before that, 256 x 256 tile pairs kept whole by box tests
+// and swept through shared-memory tiles, took 45 ms (40,000 columns with both
+// terms).  Two rows per lane would halve the shared-memory reads, but the box of
+// 64 rows keeps 48% more columns.
 // Tie and causality indicators come from each event's index in the time order,
 // carried beside its record, and are only tested for columns that can share a
 // time with the rows.  Row sums go to the FP64 accumulators of the events'
