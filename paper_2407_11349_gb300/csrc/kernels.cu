@@ -1,7 +1,7 @@
 // O(N) kernels around the pair sweep: event set-up (validation, tie ranges,
-// time blocks), per-call staging of the FP32 event table, the FP64 pair rows,
-// per-row finalisation (lambda_i, Lambda_i, the gradient of eq. 4), the
-// global reduction, and the cut-posterior location resample (Sec. 2.2).
+// time blocks), per-call staging of the FP32 event table, per-row finalisation
+// (lambda_i, Lambda_i, the gradient of eq. 4) with the global reduction, the rows
+// recomputed in FP64, and the cut-posterior location resample (Sec. 2.2).
 #include <math_constants.h>
 
 #include "common.cuh"

@@ -11,7 +11,9 @@
 // (chunk_pass), plus the row flush below once per item.  Sweep times before
 // (row tiles, 16 column tiles per item) and after, space-time background:
 // N = 2,000 0.425 -> 0.014 ms, 10,000 0.945 -> 0.062, 17,103 0.943 -> 0.144,
-// 30,000 0.87 -> 0.40.  sweep_plan (sweep.cu) says which kernel runs.
+// 30,000 0.87 -> 0.40.  sweep_plan (sweep.cu) says which kernel runs.  Larger
+// sums take the row-tile kernel below the diagonal and this one for the band of
+// each row tile's own columns.
 // What changes:
 //   - a column belongs to one warp: its sums go from the warp's registers to
 //     the FP64 accumulators, without the shared-memory pass;
@@ -27,8 +29,8 @@ namespace hk {
 
 // 2 row pairs per lane (128 rows) and 2 CTAs per SM: measured against 4 pairs
 // and one CTA it was 0.0143 to 0.0208 ms at N = 2,000, 0.0622 to 0.0786 at
-// 10,000, 0.402 to 0.410 at 30,000 and 1.056 to 1.040 at 50,000, where the
-// row-tile kernel takes over.
+// 10,000, 0.402 to 0.410 at 30,000 and 1.056 to 1.040 at 50,000 (where the two
+// kernels together take 0.956).
 constexpr int SPLIT_RP = 2, SPLIT_BPSM = 2;
 constexpr int STAGE = 2;  // column tiles per shared-memory buffer (one CTA barrier each)
 
