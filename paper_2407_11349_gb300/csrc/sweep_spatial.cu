@@ -26,26 +26,20 @@
 // widened by the FP32 rounding of the coordinates, so what is left out is an
 // exact FP32 zero; the rest is the full sweep's sum in another order.
 //
-// Coordinates: a background term between rows in a box of at most 8 scaled units
-// takes one FP32 word per coordinate, from the centre of the rows' box (3
-// differences and 12 bytes a column instead of 9 operations and 24 bytes).  Wider
-// groups, and every excitation term (whose length scale is a source's h s), take
-// two.  Up to 12 or 16 units one word would save another 11%, but log lambda's
-// rms error at N = 120,000 would rise from 1.3e-7 to 2.0e-7 (whole tiles swept
-// with two words: 1.5e-7).
+// Coordinates: two FP32 words each, rows and columns, from the centre of the rows'
+// box, as in the dense sweep.  (One word for the background of row groups up to 8
+// scaled units wide took 13% less time but put up to 2^-24 of the group's width
+// into every difference.)
 //
 // What bounds it: instruction dispatch.  A packed FP32 instruction takes two
-// dispatch cycles, any other one.  At N = 1,000,000 (3,143 counties, 1,200 days;
-// order built at the evaluated locations) a group takes 92,500 such cycles of
-// about 94,000, half of them in the evaluation of the columns that pass the point
-// test: 2.48 ms, 3.29 with two words throughout, one list for both terms, and
-// buffers moved down after each evaluation.  After a resample the boxes are wider:
-// a row has 1,811 columns with a nonzero background and 14 with a nonzero
-// excitation, point tests against the box of 32 rows leave 3,770 and 620, in 3.39
-// ms (4.05).  The design before that, 256 x 256 tile pairs kept whole by box tests
-// and swept through shared-memory tiles, took 45 ms (40,000 columns with both
-// terms).  Two rows per lane would halve the shared-memory reads, but the box of
-// 64 rows keeps 48% more columns.
+// dispatch cycles, any other one; half of the cycles go to the evaluation of the
+// columns that pass the point test.  At N = 1,000,000 (3,143 counties, 1,200 days)
+// after a resample, which widens the boxes, a row has 1,811 columns with a nonzero
+// background and 14 with a nonzero excitation; point tests against the box of 32
+// rows leave 3,770 and 620, in 3.82 ms.  256 x 256 tile pairs kept whole by box
+// tests and swept through shared-memory tiles took 45 ms (40,000 columns with both
+// terms).  Two rows per lane would halve the shared-memory reads, but the box of 64
+// rows keeps 48% more columns.
 // Tie and causality indicators come from each event's index in the time order,
 // carried beside its record, and are only tested for columns that can share a
 // time with the rows.  Row sums go to the FP64 accumulators of the events'
@@ -76,10 +70,9 @@ constexpr int SP_B_PLANES = 7, SP_E_PLANES = 9;
 // length: with bandwidths that keep every pair of 200,000 events on integer
 // days, one chain to the end left the log-likelihood 4.2e-6 and the gradient
 // 9.5e-5 off; folded, 2.2e-8 and 1.5e-6.  The usual bandwidths keep about 4,000
-// columns of a row and seldom come here (N = 1,000,000: 3.38 -> 3.44 ms).
+// columns of a row and seldom come here (N = 1,000,000: 1.5% of the sweep).
 constexpr int SP_FOLD = 8192;
 constexpr int32_t SP_TIED = 1 << 30;   // flag in a position's rank: other events share the time
-constexpr float SP_REL = 8.f;          // widest row group (scaled units) with one-word coordinates
 // The point tests allow for the rounding of the points: 2^-24 of their distance
 // from the reference point, and of half a chunk's width.
 constexpr float SP_EPS = 4.76837158203125e-07f;
@@ -433,11 +426,9 @@ __device__ __forceinline__ void sp_near(const SpBox& w, const SpBox& c, float om
     ne = c.t0 <= w.t1 && !(c.ce - omt * fmaxf(0.f, w.t0 - c.t1) - c.beta * r2 < -SP_ZERO);
 }
 
-// A lane's row: its coordinates from the group's reference point, and its sums
-// over the even and odd columns.  (The two-word coordinates are in the warp's
-// shared memory.)
+// A lane's row: its sums over the even and odd columns.  (Its coordinates are in
+// the warp's shared memory.)
 struct SpRow {
-    float x, y, t;
     float2 sB, sBr, sBt, sE, sEt, sEq;
     int lo, hi;
 };
@@ -481,35 +472,23 @@ __device__ __forceinline__ void sp_add_b(float2 dx, float2 dy, float2 dt, int r0
     }
 }
 
-// Background of `quads` x 4 buffered columns against the lane's row.  REL:
-// planes 0 to 2 hold the columns' x, y, t from the group's reference point.
-template <bool REL, bool MASK, bool LL>
+// Background of `quads` x 4 buffered columns against the lane's row.
+template <bool MASK, bool LL>
 __device__ __forceinline__ void sp_eval_b(const SpWarp& sw, int first, int quads, SpRow& w) {
     constexpr int P = SP_BUF / 4;
     const float4* p = reinterpret_cast<const float4*>(sw.b + first);
+    const SpRow2 r(sw.row);
     int4 rk = make_int4(0, 0, 0, 0);
-    if (REL) {
-        const float2 x = f2(w.x, w.x), y = f2(w.y, w.y), t = f2(w.t, w.t);
 #pragma unroll 2
-        for (int q = 0; q < quads; ++q, ++p) {
-            const float4 X = p[0 * P], Y = p[1 * P], T = p[2 * P];
-            if (MASK) rk = *reinterpret_cast<const int4*>(p + 6 * P);
-            sp_add_b<MASK, LL>(add2(x, half4(X, 0)), add2(y, half4(Y, 0)), add2(t, half4(T, 0)), rk.x, rk.y, w);
-            sp_add_b<MASK, LL>(add2(x, half4(X, 1)), add2(y, half4(Y, 1)), add2(t, half4(T, 1)), rk.z, rk.w, w);
-        }
-    } else {
-        const SpRow2 r(sw.row);
-#pragma unroll 4
-        for (int q = 0; q < quads; ++q, ++p) {
-            const float4 xh = p[0 * P], xl = p[1 * P], yh = p[2 * P], yl = p[3 * P], th = p[4 * P], tl = p[5 * P];
-            if (MASK) rk = *reinterpret_cast<const int4*>(p + 6 * P);
+    for (int q = 0; q < quads; ++q, ++p) {
+        const float4 xh = p[0 * P], xl = p[1 * P], yh = p[2 * P], yl = p[3 * P], th = p[4 * P], tl = p[5 * P];
+        if (MASK) rk = *reinterpret_cast<const int4*>(p + 6 * P);
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
-                sp_add_b<MASK, LL>(add2(add2(r.xh, half4(xh, h)), add2(r.xl, half4(xl, h))),
-                                   add2(add2(r.yh, half4(yh, h)), add2(r.yl, half4(yl, h))),
-                                   add2(add2(r.th, half4(th, h)), add2(r.tl, half4(tl, h))),
-                                   h ? rk.z : rk.x, h ? rk.w : rk.y, w);
-        }
+        for (int h = 0; h < 2; ++h)
+            sp_add_b<MASK, LL>(add2(add2(r.xh, half4(xh, h)), add2(r.xl, half4(xl, h))),
+                               add2(add2(r.yh, half4(yh, h)), add2(r.yl, half4(yl, h))),
+                               add2(add2(r.th, half4(th, h)), add2(r.tl, half4(tl, h))),
+                               h ? rk.z : rk.x, h ? rk.w : rk.y, w);
     }
 }
 
@@ -549,14 +528,9 @@ __device__ __forceinline__ void sp_eval_e(const SpWarp& sw, int first, int quads
 }
 
 template <bool LL>
-__device__ __forceinline__ void sp_background(const SpWarp& sw, int first, int quads, bool rel, bool mask, SpRow& w) {
-    if (rel) {
-        if (mask) sp_eval_b<true, true, LL>(sw, first, quads, w);
-        else sp_eval_b<true, false, LL>(sw, first, quads, w);
-    } else {
-        if (mask) sp_eval_b<false, true, LL>(sw, first, quads, w);
-        else sp_eval_b<false, false, LL>(sw, first, quads, w);
-    }
+__device__ __forceinline__ void sp_background(const SpWarp& sw, int first, int quads, bool mask, SpRow& w) {
+    if (mask) sp_eval_b<true, LL>(sw, first, quads, w);
+    else sp_eval_b<false, LL>(sw, first, quads, w);
 }
 
 template <bool LL>
@@ -575,9 +549,8 @@ struct SpGroup {
 };
 
 // A listed chunk: offset of its centre from the group's, then its number, and
-// SP_WIDE if one word per coordinate is not enough for its events, SP_FAR if
-// the sum of a first word and the offset may not be exact (above 512).
-constexpr int SP_FAR = 1 << 27, SP_WIDE = 1 << 28, SP_ID = SP_FAR - 1;
+// SP_FAR if the sum of a first word and the offset may not be exact (above 512).
+constexpr int SP_FAR = 1 << 27, SP_ID = SP_FAR - 1;
 
 // Distance beyond the group's half width, not above the true one.
 __device__ __forceinline__ float sp_beyond(float d, float half) { return fmaxf(0.f, fmaf(fabsf(d), SP_IN, -half)); }
@@ -603,7 +576,7 @@ __device__ __forceinline__ void sp_two_words(const float4& a, const float4& b, c
 // background, and evaluate the survivors 32 at a time.  count: survivors so far
 // (the buffer is a ring of two halves); mask: the current half holds a column
 // that may share a time with a row.
-template <bool REL, bool LL>
+template <bool LL>
 __device__ __forceinline__ void sp_columns_b(const SpArgs& a, SpWarp& sw, int n, const SpGroup& gr, SpRow& w,
                                              int& count, bool& mask) {
     constexpr unsigned ALL = 0xffffffffu;
@@ -612,25 +585,17 @@ __device__ __forceinline__ void sp_columns_b(const SpArgs& a, SpWarp& sw, int n,
     const float4* ra = a.ra + lane;
     const float4* rb = a.rb + lane;
     int64_t p = static_cast<int64_t>(__float_as_int(sw.list[0].w) & SP_ID) * SP_CH;
-    float4 next = ra[p], nextl = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!REL) nextl = rb[p];
+    float4 next = ra[p], nextl = rb[p];
 #pragma unroll 1
     for (int k = 0; k < n; ++k) {
-        const float4 q = next, off = sw.list[k];
-        float4 lo = nextl;
+        const float4 q = next, l = nextl, off = sw.list[k];
         p = static_cast<int64_t>(__float_as_int(sw.list[min(k + 1, n - 1)].w) & SP_ID) * SP_CH;
         next = ra[p];
-        if (!REL) nextl = rb[p];
+        nextl = rb[p];
         const int id = __float_as_int(off.w), rk = __float_as_int(q.w);
-        float nx = q.x + off.x, ny = q.y + off.y, nt = q.z + off.z;  // negated, from the group's centre
-        float hx = nx, hy = ny, ht = nt;                             // first of two words
-        if (!REL || (id & SP_WIDE)) {
-            if (REL) lo = rb[static_cast<int64_t>(id & SP_ID) * SP_CH];
-            sp_two_words(q, lo, off, hx, hy, ht, lo.x, lo.y, lo.z);
-            nx = hx + lo.x;
-            ny = hy + lo.y;
-            nt = ht + lo.z;
-        }
+        float hx, hy, ht, lx, ly, lt;  // negated, from the group's centre
+        sp_two_words(q, l, off, hx, hy, ht, lx, ly, lt);
+        const float nx = hx + lx, ny = hy + ly, nt = ht + lt;
         const float dx = sp_beyond(nx, gr.hx), dy = sp_beyond(ny, gr.hy), dt = sp_beyond(nt, gr.ht);
         // (a padding event's time is far from any; negated: a NaN is kept)
         const bool keep = !(fmaf(dt, dt, fmaf(dx, dx, dy * dy)) > SP_ZERO);
@@ -641,19 +606,15 @@ __device__ __forceinline__ void sp_columns_b(const SpArgs& a, SpWarp& sw, int n,
         mask |= any;
         if (keep) {
             float* b = sw.b + ((count + __popc(bal & below)) & (SP_BUF - 1));
-            if (REL) {
-                b[0 * SP_BUF] = nx; b[1 * SP_BUF] = ny; b[2 * SP_BUF] = nt;
-            } else {
-                b[0 * SP_BUF] = hx; b[1 * SP_BUF] = lo.x; b[2 * SP_BUF] = hy; b[3 * SP_BUF] = lo.y;
-                b[4 * SP_BUF] = ht; b[5 * SP_BUF] = lo.z;
-            }
+            b[0 * SP_BUF] = hx; b[1 * SP_BUF] = lx; b[2 * SP_BUF] = hy; b[3 * SP_BUF] = ly;
+            b[4 * SP_BUF] = ht; b[5 * SP_BUF] = lt;
             b[6 * SP_BUF] = __int_as_float(rk & ~SP_TIED);
         }
         const int before = count;
         count += __popc(bal);
         if ((before ^ count) & 32) {
             __syncwarp();
-            sp_background<LL>(sw, before & 32, 8, REL, mask, w);
+            sp_background<LL>(sw, before & 32, 8, mask, w);
             mask = any;
             __syncwarp();
         }
@@ -730,11 +691,9 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
             return;
         }
         const int g = item / a.parts, part = item % a.parts;
-        bool rel;
         {
-            const SpBox box = sp_load(a.cmeta, g);
-            if (!(box.x0 <= box.x1)) continue;  // padding only
-            rel = fmaxf(fmaxf(box.x1 - box.x0, box.y1 - box.y0), box.t1 - box.t0) <= SP_REL;
+            const float4 x = a.cmeta[2 * g];
+            if (!(x.x <= x.y)) continue;  // padding only
         }
         SpRow w;
         SpGroup gr;
@@ -748,9 +707,6 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
             float* r = sw.row + lane;
             r[0] = -sp_grid(qa.x); r[32] = -qb.x; r[64] = -sp_grid(qa.y); r[96] = -qb.y;
             r[128] = -sp_grid(qa.z); r[160] = -qb.z;
-            w.x = -qa.x;
-            w.y = -qa.y;
-            w.t = -qa.z;
             // (as integers: the order of nonnegative floats)
             auto half = [&](float v) {
                 return __uint_as_float(__reduce_max_sync(ALL, e >= 0 ? __float_as_uint(fabsf(v)) : 0u)) * SP_OUT +
@@ -835,7 +791,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
                     const float4 c = a.centre[ch];
                     entry = make_float4(ref.x - c.x, ref.y - c.y, ref.z - c.z, 0.f);
                     const float far = fmaxf(fmaxf(fabsf(entry.x), fabsf(entry.y)), fabsf(entry.z));
-                    entry.w = __int_as_float(ch | (width <= SP_REL ? 0 : SP_WIDE) | (width + far <= 256.f ? 0 : SP_FAR));
+                    entry.w = __int_as_float(ch | (width + far <= 256.f ? 0 : SP_FAR));
                 }
                 const unsigned kb = __ballot_sync(ALL, nb), ke = __ballot_sync(ALL, ne);
                 if (nb) sw.list[lB + __popc(kb & below)] = entry;
@@ -845,10 +801,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
             }
             __syncwarp();
             if (lB + lE == 0) break;
-            if (lB > 0) {
-                if (rel) sp_columns_b<true, LL>(a, sw, lB, gr, w, nB, maskB);
-                else sp_columns_b<false, LL>(a, sw, lB, gr, w, nB, maskB);
-            }
+            if (lB > 0) sp_columns_b<LL>(a, sw, lB, gr, w, nB, maskB);
             if (lE > 0) sp_columns_e<LL>(a, sw, lE, gr, omt, w, nE, maskE);
             __syncwarp();
             if (nB + nE > SP_FOLD) {
@@ -865,14 +818,14 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
         const int qB = (nB + 3) >> 2, qE = (nE + 3) >> 2;
         if (nB + lane < 4 * qB) {
             for (int q = 0; q < SP_B_PLANES; ++q) sw.b[q * SP_BUF + hB + nB + lane] = 0.f;
-            sw.b[(rel ? 2 : 4) * SP_BUF + hB + nB + lane] = -PAD_T;
+            sw.b[4 * SP_BUF + hB + nB + lane] = -PAD_T;
         }
         if (nE + lane < 4 * qE) {
             for (int q = 0; q < SP_E_PLANES; ++q) sw.e[q * SP_BUF + hE + nE + lane] = 0.f;
             sw.e[8 * SP_BUF + hE + nE + lane] = -1e30f;
         }
         __syncwarp();
-        sp_background<LL>(sw, hB, qB, rel, maskB, w);
+        sp_background<LL>(sw, hB, qB, maskB, w);
         sp_excitation<LL>(sw, hE, qE, maskE, f2(-omt, -omt), w);
         __syncwarp();
         flush_rows();
