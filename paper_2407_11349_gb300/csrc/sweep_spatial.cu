@@ -48,15 +48,13 @@
 #include <cmath>
 #include <cstring>
 #include <new>
-#include <system_error>
-#include <thread>
 #include <vector>
 
+#include "spatial_order.h"
 #include "sweep_kernel.cuh"
 
 namespace hk {
 
-constexpr int SP_CH = 32;              // events per chunk: a row group, and the finest column unit
 constexpr int SP_WARPS = 8, SP_THREADS = 32 * SP_WARPS;
 // Resident CTAs per SM.  At N = 1,000,000: 2 3.49 ms, 3 3.41, 4 (64 registers,
 // spills) 3.59.
@@ -78,7 +76,7 @@ constexpr int32_t SP_TIED = 1 << 30;   // flag in a position's rank: other event
 constexpr float SP_EPS = 4.76837158203125e-07f;
 constexpr float SP_OUT = 1.f + 9.5367431640625e-07f, SP_IN = 1.f - 9.5367431640625e-07f;
 constexpr float SP_ZERO = 128.f;       // exponent beyond which a term counts as zero (126 + margin)
-static_assert(NPAD_MULT % TC == 0 && TC == 8 * SP_CH, "a tile is 8 chunks");
+static_assert(NPAD_MULT % TC == 0 && TC == SP_TILE && TC == 8 * SP_CH, "a tile is 8 chunks");
 
 // Boxes and centres of the order's units, one allocation: SpBox (two float4) of
 // every chunk, tile and block of 32 tiles, then the chunks' centres.
@@ -122,34 +120,6 @@ int spatial_set_window(hawkes_ctx* c, int64_t window) {
     return HAWKES_OK;
 }
 
-// Split [a, b) of the permutation at medians of its widest side, down to
-// chunks; parts stay whole tiles while larger than a tile.
-struct SpPoint {
-    float c[3];
-    int32_t e;
-};
-static void sp_split(SpPoint* a, SpPoint* b) {
-    while (b - a > SP_CH) {
-        const int64_t len = b - a, unit = len > TC ? TC : SP_CH;
-        float lo[3], hi[3];
-        for (int k = 0; k < 3; ++k) lo[k] = hi[k] = a->c[k];
-        for (const SpPoint* p = a + 1; p < b; ++p)
-            for (int k = 0; k < 3; ++k) {
-                lo[k] = std::min(lo[k], p->c[k]);
-                hi[k] = std::max(hi[k], p->c[k]);
-            }
-        int ax = 0;
-        for (int k = 1; k < 3; ++k)
-            if (hi[k] - lo[k] > hi[ax] - lo[ax]) ax = k;
-        SpPoint* m = a + std::min((len / 2 + unit - 1) / unit * unit, (len - 1) / unit * unit);
-        std::nth_element(a, m, b, [ax](const SpPoint& u, const SpPoint& v) {
-            return u.c[ax] < v.c[ax] || (u.c[ax] == v.c[ax] && u.e < v.e);
-        });
-        sp_split(m, b);
-        b = m;
-    }
-}
-
 static int build_order(hawkes_ctx* c, double tau_x, double tau_t) {
     SpatialState* sp = c->sp;
     const int64_t n = c->n, npad = c->npad;
@@ -181,22 +151,7 @@ static int build_order(hawkes_ctx* c, double tau_x, double tau_t) {
         pt[i] = SpPoint{{static_cast<float>((x[i] - x[0]) / tau_x), static_cast<float>((y[i] - y[0]) / tau_x),
                          static_cast<float>((t[i] - t[0]) / tau_t)},
                         static_cast<int32_t>(i)};
-    // time windows (whole tiles), split independently on a few host threads
-    const int64_t w = (sp->window + TC - 1) / TC * TC;
-    const int64_t nw = (n + w - 1) / w;
-    auto work = [&](int64_t k0, int64_t step) {
-        for (int64_t k = k0; k < nw; k += step) sp_split(pt.data() + k * w, pt.data() + std::min(n, (k + 1) * w));
-    };
-    const int64_t nth = std::min<int64_t>(nw, n > 50000 ? 8 : 1);
-    std::vector<std::thread> th;
-    int64_t started = 1;  // this thread takes window 0, nth, 2 nth, ...
-    try {
-        for (; started < nth; ++started) th.emplace_back(work, started, nth);
-    } catch (const std::system_error&) {  // no more threads: the rest runs here
-    }
-    work(0, nth);
-    for (int64_t k = started; k < nth; ++k) work(k, nth);
-    for (std::thread& q : th) q.join();
+    sp_split_windows(pt, sp->window);
     std::vector<int32_t> rank(npad, -1);
     for (int64_t p = 0; p < n; ++p) {
         const int32_t e = pt[p].e;
