@@ -20,6 +20,40 @@ struct SpPoint {
     int32_t e;
 };
 
+// A point's coordinate: finite, so that the points can be ordered.  (Sums and
+// differences of coordinates near the end of the FP64 range are not.)
+inline float sp_coord(double v) {
+    return v != v ? 0.f : static_cast<float>(std::min(std::max(v, -1e30), 1e30));
+}
+
+// The events as points of the tree.  Locations that will be redrawn inside their
+// counties (n_counties > 0) enter as the county's mean plus a fifth of the offset
+// from it.  x and y are overwritten.
+inline std::vector<SpPoint> sp_points(const std::vector<double>& t, std::vector<double>& x, std::vector<double>& y,
+                                      const std::vector<int32_t>& county, int32_t n_counties, double tau_x,
+                                      double tau_t) {
+    const size_t n = t.size();
+    if (n_counties > 0) {
+        std::vector<double> mx(n_counties, 0.0), my(n_counties, 0.0), cnt(n_counties, 0.0);
+        for (size_t i = 0; i < n; ++i) {
+            mx[county[i]] += x[i];
+            my[county[i]] += y[i];
+            cnt[county[i]] += 1.0;
+        }
+        for (size_t i = 0; i < n; ++i) {
+            const double cx = mx[county[i]] / cnt[county[i]], cy = my[county[i]] / cnt[county[i]];
+            x[i] = cx + 0.2 * (x[i] - cx);
+            y[i] = cy + 0.2 * (y[i] - cy);
+        }
+    }
+    std::vector<SpPoint> pt(n);
+    for (size_t i = 0; i < n; ++i)
+        pt[i] = SpPoint{{sp_coord((x[i] - x[0]) / tau_x), sp_coord((y[i] - y[0]) / tau_x),
+                         sp_coord((t[i] - t[0]) / tau_t)},
+                        static_cast<int32_t>(i)};
+    return pt;
+}
+
 // Split [a, b) at medians of its widest side, down to chunks; parts stay whole
 // tiles while larger than a tile.
 inline void sp_split(SpPoint* a, SpPoint* b) {

@@ -133,24 +133,7 @@ static int build_order(hawkes_ctx* c, double tau_x, double tau_t) {
         cudaMemcpy(lo.data(), c->lo, n * sizeof(int32_t), cudaMemcpyDeviceToHost) != cudaSuccess ||
         cudaMemcpy(hi.data(), c->hi, n * sizeof(int32_t), cudaMemcpyDeviceToHost) != cudaSuccess)
         return HAWKES_ERR_CUDA;
-    if (c->counties_ok) {  // a resample can move the events inside their counties
-        std::vector<double> mx(c->n_counties, 0.0), my(c->n_counties, 0.0), cnt(c->n_counties, 0.0);
-        for (int64_t i = 0; i < n; ++i) {
-            mx[cty[i]] += x[i];
-            my[cty[i]] += y[i];
-            cnt[cty[i]] += 1.0;
-        }
-        for (int64_t i = 0; i < n; ++i) {
-            const double cx = mx[cty[i]] / cnt[cty[i]], cy = my[cty[i]] / cnt[cty[i]];
-            x[i] = cx + 0.2 * (x[i] - cx);
-            y[i] = cy + 0.2 * (y[i] - cy);
-        }
-    }
-    std::vector<SpPoint> pt(n);
-    for (int64_t i = 0; i < n; ++i)
-        pt[i] = SpPoint{{static_cast<float>((x[i] - x[0]) / tau_x), static_cast<float>((y[i] - y[0]) / tau_x),
-                         static_cast<float>((t[i] - t[0]) / tau_t)},
-                        static_cast<int32_t>(i)};
+    std::vector<SpPoint> pt = sp_points(t, x, y, cty, c->counties_ok ? c->n_counties : 0, tau_x, tau_t);
     sp_split_windows(pt, sp->window);
     std::vector<int32_t> rank(npad, -1);
     for (int64_t p = 0; p < n; ++p) {

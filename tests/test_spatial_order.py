@@ -54,3 +54,37 @@ def test_out_of_memory_while_threads_run(tmp_path, fail_at):
         }
         """, fail_at)
     assert r.returncode == 0 and r.stdout.strip() in ("bad_alloc", "ordered"), (r.returncode, r.stdout, r.stderr)
+
+
+@pytest.mark.parametrize("size", [1e3, 1.7e308])
+def test_order_is_a_permutation_at_any_finite_coordinate(tmp_path, size):
+    """County means, and differences, of finite coordinates may overflow; the
+    points keep an order all the same (a NaN would leave none, and the split could
+    then run outside its range)."""
+    r = run_cpp(tmp_path, """
+        #include <cmath>
+        #include <cstdio>
+        #include <cstdlib>
+        #include "spatial_order.h"
+        int main(int, char** argv) {
+            const int n = 5000;
+            const double size = std::atof(argv[1]);
+            std::vector<double> t(n), x(n), y(n);
+            std::vector<int32_t> county(n);
+            for (int i = 0; i < n; ++i) {
+                t[i] = 1.0 + i / 3;
+                x[i] = size * (((i * 7919) % 1000) / 500.0 - 1.0);
+                y[i] = (i % 5 ? size : -size) * 0.9;
+                county[i] = i % 7;
+            }
+            std::vector<hk::SpPoint> pt = hk::sp_points(t, x, y, county, 7, 1.0, 1.0);
+            for (const auto& p : pt)
+                for (float c : p.c)
+                    if (!std::isfinite(c)) return 2;
+            hk::sp_split_windows(pt, 1024);
+            std::vector<char> seen(n, 0);
+            for (const auto& p : pt) seen[p.e] = 1;
+            for (char s : seen) if (!s) return 1;
+        }
+        """, repr(size))
+    assert r.returncode == 0, r.returncode
