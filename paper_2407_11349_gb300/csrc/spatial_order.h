@@ -15,6 +15,18 @@ namespace hk {
 constexpr int SP_CH = 32;     // events per chunk: a row group, and the finest column unit
 constexpr int SP_TILE = 256;  // events per tile
 
+// A position's entry in the order: the event's index in time order, and whether
+// other events share its time; SP_PAD for padding.  (Indices end below 2^31 - 4,096,
+// hawkes_set_events, so no event's entry is SP_PAD.)
+#ifdef __CUDACC__
+#define SP_HD __host__ __device__ __forceinline__
+#else
+#define SP_HD inline
+#endif
+constexpr uint32_t SP_TIED = 1u << 31, SP_PAD = ~0u;
+SP_HD uint32_t sp_rank(int32_t e, bool tied) { return static_cast<uint32_t>(e) | (tied ? SP_TIED : 0u); }
+SP_HD int32_t sp_event(uint32_t rank) { return static_cast<int32_t>(rank & ~SP_TIED); }
+
 struct SpPoint {
     float c[3];
     int32_t e;

@@ -70,7 +70,6 @@ constexpr int SP_B_PLANES = 7, SP_E_PLANES = 9;
 // 9.5e-5 off; folded, 2.2e-8 and 1.5e-6.  The usual bandwidths keep about 4,000
 // columns of a row and seldom come here (N = 1,000,000: 1.5% of the sweep).
 constexpr int SP_FOLD = 8192;
-constexpr int32_t SP_TIED = 1 << 30;   // flag in a position's rank: other events share the time
 // The point tests allow for the rounding of the points: 2^-24 of their distance
 // from the reference point, and of half a chunk's width.
 constexpr float SP_EPS = 4.76837158203125e-07f;
@@ -90,7 +89,7 @@ struct SpatialState {
     int64_t window = 131072;  // target events per time window
     bool built = false;
     int ntiles = 0;           // npad / TC
-    int32_t* rank = nullptr;  // [npad] time-order index at each position, | SP_TIED (-1: padding)
+    uint32_t* rank = nullptr; // [npad] event at each position (sp_rank)
     float4* meta = nullptr;   // SpMeta's arrays
 };
 
@@ -135,10 +134,10 @@ static int build_order(hawkes_ctx* c, double tau_x, double tau_t) {
         return HAWKES_ERR_CUDA;
     std::vector<SpPoint> pt = sp_points(t, x, y, cty, c->counties_ok ? c->n_counties : 0, tau_x, tau_t);
     sp_split_windows(pt, sp->window);
-    std::vector<int32_t> rank(npad, -1);
+    std::vector<uint32_t> rank(npad, SP_PAD);
     for (int64_t p = 0; p < n; ++p) {
         const int32_t e = pt[p].e;
-        rank[p] = hi[e] - lo[e] > 1 ? (e | SP_TIED) : e;
+        rank[p] = sp_rank(e, hi[e] - lo[e] > 1);
     }
     const int ntiles = static_cast<int>(npad / TC);
     if (sp->ntiles != ntiles || !sp->rank || !sp->meta) {
@@ -146,14 +145,14 @@ static int build_order(hawkes_ctx* c, double tau_x, double tau_t) {
         if (sp->meta) cudaFree(sp->meta);
         sp->rank = nullptr;
         sp->meta = nullptr;
-        if (cudaMalloc(&sp->rank, npad * sizeof(int32_t)) != cudaSuccess ||
+        if (cudaMalloc(&sp->rank, npad * sizeof(uint32_t)) != cudaSuccess ||
             cudaMalloc(&sp->meta, sp_meta_f4(ntiles) * sizeof(float4)) != cudaSuccess) {
             cudaGetLastError();
             return HAWKES_ERR_OOM;
         }
         sp->ntiles = ntiles;
     }
-    if (cudaMemcpy(sp->rank, rank.data(), npad * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess)
+    if (cudaMemcpy(sp->rank, rank.data(), npad * sizeof(uint32_t), cudaMemcpyHostToDevice) != cudaSuccess)
         return HAWKES_ERR_CUDA;
     sp->built = true;
     return HAWKES_OK;
@@ -168,7 +167,6 @@ int spatial_build(hawkes_ctx* c, const hawkes_params* p, const hawkes_params* d_
         if (rc != HAWKES_OK) return rc;
     }
     if (c->sp->built) return HAWKES_OK;
-    if (c->n >= SP_TIED) return HAWKES_ERR_ARG;
     hawkes_params q{};
     if (p)
         q = *p;
@@ -261,7 +259,7 @@ __device__ __forceinline__ void sp_recentre(float c, float xh, float xl, float& 
 // (the second words belong to the first ones on sp_grid's grid),
 // in scaled units (t~ = (t - t_1) sqrt(a_t)), the centres, and the boxes of the
 // chunks and tiles (one block per tile).
-__global__ void __launch_bounds__(TC) k_sp_prep(EvalDesc d, const int32_t* __restrict__ rank, int model1,
+__global__ void __launch_bounds__(TC) k_sp_prep(EvalDesc d, const uint32_t* __restrict__ rank, int model1,
                                                 float4* __restrict__ ra, float4* __restrict__ rb,
                                                 float* __restrict__ rc, float4* __restrict__ cmeta,
                                                 float4* __restrict__ tmeta, float4* __restrict__ centre,
@@ -275,11 +273,11 @@ __global__ void __launch_bounds__(TC) k_sp_prep(EvalDesc d, const int32_t* __res
     __shared__ SpBox boxes[TC / SP_CH];
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int64_t p = static_cast<int64_t>(tile) * TC + threadIdx.x;
-        const int32_t r = rank[p];
+        const uint32_t r = rank[p];
         float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f, th = 0.f, tl = 0.f, beta = 0.f, ce = -1e30f;
         SpBox box = sp_empty();
-        if (r >= 0) {
-            const int32_t e = r & ~SP_TIED;
+        if (r != SP_PAD) {
+            const int32_t e = sp_event(r);
             const double ts = (d.t[e] - tf) * kt, xs = d.x[e] * kx, ys = d.y[e] * kx;
             th = static_cast<float>(ts);
             xh = static_cast<float>(xs);
@@ -295,9 +293,9 @@ __global__ void __launch_bounds__(TC) k_sp_prep(EvalDesc d, const int32_t* __res
         const bool any = box.x0 <= box.x1;
         const float cx = any ? sp_mid(box.x0, box.x1) : 0.f, cy = any ? sp_mid(box.y0, box.y1) : 0.f,
                     ct = any ? sp_mid(box.t0, box.t1) : 0.f;
-        float4 a = make_float4(0.f, 0.f, -PAD_T, __int_as_float(-1)), b = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r >= 0) {
-            a.w = __int_as_float(r);
+        float4 a = make_float4(0.f, 0.f, -PAD_T, __uint_as_float(SP_PAD)), b = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r != SP_PAD) {
+            a.w = __uint_as_float(r);
             b.w = -beta;
             sp_recentre(cx, xh, xl, a.x, b.x);
             sp_recentre(cy, yh, yl, a.y, b.y);
@@ -530,7 +528,8 @@ __device__ __forceinline__ void sp_columns_b(const SpArgs& a, SpWarp& sw, int n,
         p = static_cast<int64_t>(__float_as_int(sw.list[min(k + 1, n - 1)].w) & SP_ID) * SP_CH;
         next = ra[p];
         nextl = rb[p];
-        const int id = __float_as_int(off.w), rk = __float_as_int(q.w);
+        const int id = __float_as_int(off.w);
+        const uint32_t rk = __float_as_uint(q.w);
         float hx, hy, ht, lx, ly, lt;  // negated, from the group's centre
         sp_two_words(q, l, off, hx, hy, ht, lx, ly, lt);
         const float nx = hx + lx, ny = hy + ly, nt = ht + lt;
@@ -538,7 +537,7 @@ __device__ __forceinline__ void sp_columns_b(const SpArgs& a, SpWarp& sw, int n,
         // (a padding event's time is far from any; negated: a NaN is kept)
         const bool keep = !(fmaf(dt, dt, fmaf(dx, dx, dy * dy)) > SP_ZERO);
         const unsigned bal = __ballot_sync(ALL, keep);
-        const bool any = __any_sync(ALL, keep && static_cast<unsigned>(rk - (gr.lo_min | SP_TIED)) <
+        const bool any = __any_sync(ALL, keep && rk - (static_cast<uint32_t>(gr.lo_min) | SP_TIED) <
                                                      static_cast<unsigned>(gr.ties)) ||
                          (id & SP_ID) == gr.self;
         mask |= any;
@@ -546,7 +545,7 @@ __device__ __forceinline__ void sp_columns_b(const SpArgs& a, SpWarp& sw, int n,
             float* b = sw.b + ((count + __popc(bal & below)) & (SP_BUF - 1));
             b[0 * SP_BUF] = hx; b[1 * SP_BUF] = lx; b[2 * SP_BUF] = hy; b[3 * SP_BUF] = ly;
             b[4 * SP_BUF] = ht; b[5 * SP_BUF] = lt;
-            b[6 * SP_BUF] = __int_as_float(rk & ~SP_TIED);
+            b[6 * SP_BUF] = __int_as_float(sp_event(rk));
         }
         const int before = count;
         count += __popc(bal);
@@ -579,7 +578,7 @@ __device__ __forceinline__ void sp_columns_e(const SpArgs& a, SpWarp& sw, int n,
         na = a.ra[p];
         nl = a.rb[p];
         nc = a.rc[p];
-        const int rank = __float_as_int(q.w) & ~SP_TIED;
+        const int rank = sp_event(__float_as_uint(q.w));
         float hx, hy, ht, lx, ly, lt;
         sp_two_words(q, l, off, hx, hy, ht, lx, ly, lt);
         const float nx = hx + lx, ny = hy + ly, nt = ht + lt;
@@ -640,8 +639,8 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
         {
             const int64_t p = static_cast<int64_t>(g) * SP_CH + lane;
             const float4 qa = a.ra[p], qb = a.rb[p];
-            const int rk = __float_as_int(qa.w);
-            e = rk >= 0 ? rk & ~SP_TIED : -1;
+            const uint32_t rk = __float_as_uint(qa.w);
+            e = rk != SP_PAD ? sp_event(rk) : -1;
             float* r = sw.row + lane;
             r[0] = -sp_grid(qa.x); r[32] = -qb.x; r[64] = -sp_grid(qa.y); r[96] = -qb.y;
             r[128] = -sp_grid(qa.z); r[160] = -qb.z;

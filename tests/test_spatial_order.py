@@ -88,3 +88,20 @@ def test_order_is_a_permutation_at_any_finite_coordinate(tmp_path, size):
         }
         """, repr(size))
     assert r.returncode == 0, r.returncode
+
+
+def test_every_event_index_has_an_entry(tmp_path):
+    """Indices up to the largest that hawkes_set_events accepts (n at most
+    2^31 - 4,096), tied or not, come back whole and are never the padding."""
+    r = run_cpp(tmp_path, """
+        #include "spatial_order.h"
+        int main() {
+            const int64_t last = (int64_t(1) << 31) - 4097;
+            for (int64_t e : {int64_t(0), int64_t(1), (int64_t(1) << 30) - 1, int64_t(1) << 30, last})
+                for (bool tied : {false, true}) {
+                    const uint32_t r = hk::sp_rank(int32_t(e), tied);
+                    if (hk::sp_event(r) != e || r == hk::SP_PAD || bool(r & hk::SP_TIED) != tied) return 1;
+                }
+        }
+        """)
+    assert r.returncode == 0
