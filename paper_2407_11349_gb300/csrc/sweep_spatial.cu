@@ -50,6 +50,7 @@
 #include <new>
 #include <vector>
 
+#include "spatial_bounds.h"
 #include "spatial_order.h"
 #include "sweep_kernel.cuh"
 
@@ -70,11 +71,6 @@ constexpr int SP_B_PLANES = 7, SP_E_PLANES = 9;
 // 9.5e-5 off; folded, 2.2e-8 and 1.5e-6.  The usual bandwidths keep about 4,000
 // columns of a row and seldom come here (N = 1,000,000: 1.5% of the sweep).
 constexpr int SP_FOLD = 8192;
-// The point tests allow for the rounding of the points: 2^-24 of their distance
-// from the reference point, and of half a chunk's width.
-constexpr float SP_EPS = 4.76837158203125e-07f;
-constexpr float SP_OUT = 1.f + 9.5367431640625e-07f, SP_IN = 1.f - 9.5367431640625e-07f;
-constexpr float SP_ZERO = 128.f;       // exponent beyond which a term counts as zero (126 + margin)
 static_assert(NPAD_MULT % TC == 0 && TC == SP_TILE && TC == 8 * SP_CH, "a tile is 8 chunks");
 
 // Boxes and centres of the order's units, one allocation: SpBox (two float4) of
@@ -182,12 +178,6 @@ int spatial_build(hawkes_ctx* c, const hawkes_params* p, const hawkes_params* d_
     }
 }
 
-// Bounds of a set of events, in scaled units: box, time range, largest ce,
-// smallest beta.  Empty: x0 > x1.
-struct SpBox {
-    float x0, x1, y0, y1, t0, t1, ce, beta;
-};
-
 __device__ __forceinline__ SpBox sp_load(const float4* __restrict__ meta, int k) {
     const float4 a = meta[2 * k], b = meta[2 * k + 1];
     return SpBox{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
@@ -196,23 +186,6 @@ __device__ __forceinline__ void sp_store(float4* meta, int k, const SpBox& v) {
     meta[2 * k] = make_float4(v.x0, v.x1, v.y0, v.y1);
     meta[2 * k + 1] = make_float4(v.t0, v.t1, v.ce, v.beta);
 }
-__device__ __forceinline__ SpBox sp_empty() {
-    return SpBox{1e30f, -1e30f, 1e30f, -1e30f, 1e30f, -1e30f, -1e30f, 1e30f};
-}
-__device__ __forceinline__ void sp_join(SpBox& a, const SpBox& b) {
-    a.x0 = fminf(a.x0, b.x0); a.x1 = fmaxf(a.x1, b.x1);
-    a.y0 = fminf(a.y0, b.y0); a.y1 = fmaxf(a.y1, b.y1);
-    a.t0 = fminf(a.t0, b.t0); a.t1 = fmaxf(a.t1, b.t1);
-    a.ce = fmaxf(a.ce, b.ce); a.beta = fminf(a.beta, b.beta);
-}
-// Widen [lo, hi] by 2^-22 of its magnitude: more than the rounding to FP32 of
-// its own ends and of any point compared with it nearby.
-__device__ __forceinline__ void sp_widen(float& lo, float& hi) {
-    const float s = 2.384185791015625e-07f * fmaxf(fabsf(lo), fabsf(hi));
-    lo -= s;
-    hi += s;
-}
-
 __device__ __forceinline__ SpBox sp_warp_join(SpBox box) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -224,33 +197,6 @@ __device__ __forceinline__ SpBox sp_warp_join(SpBox box) {
         sp_join(box, q);
     }
     return box;
-}
-
-// Middle of a range on a grid of 1/16, so that differences of neighbouring
-// chunks' centres are exact in FP32 (beyond 2^20 FP32's own grid is coarser).
-__device__ __forceinline__ float sp_mid(float a, float b) {
-    const float m = 0.5f * a + 0.5f * b;
-    return fabsf(m) < 1048576.f ? rintf(m * 16.f) * 0.0625f : m;
-}
-
-// hi + lo = a + d exactly, lo0 added to lo.
-__device__ __forceinline__ void sp_two_sum(float a, float d, float lo0, float& hi, float& lo) {
-    hi = a + d;
-    const float z = hi - a;
-    lo = ((a - (hi - z)) + (d - z)) + lo0;
-}
-
-// First word of a two-word coordinate: on a grid of 2^-14 for |a| < 256, so that
-// first words' differences are exact.  (FP32 has steps of 2^-14 from 512 to 1,024.)
-__device__ __forceinline__ float sp_grid(float a) { return (a + 768.f) - 768.f; }
-
-// c - (xh + xl), and what sp_grid leaves of it.  (In FP32: FP64 arithmetic is what
-// staging waits for.)
-__device__ __forceinline__ void sp_recentre(float c, float xh, float xl, float& hi, float& lo) {
-    float h, l;
-    sp_two_sum(-xh, c, -xl, h, l);
-    sp_two_sum(h, l, 0.f, hi, lo);
-    lo += hi - sp_grid(hi);
 }
 
 // Stage the records in the spatial order: negated distances from the chunk's
@@ -349,18 +295,6 @@ struct SpArgs {
     int64_t npad;
     int ntiles, groups, parts;
 };
-
-// Can a column of box (or point) c hold a nonzero background / excitation term
-// for some row of box w?
-__device__ __forceinline__ float sp_gap(float lo, float hi, float a0, float a1) {
-    return fmaxf(0.f, fmaxf(a0 - hi, lo - a1));
-}
-__device__ __forceinline__ void sp_near(const SpBox& w, const SpBox& c, float omt, bool& nb, bool& ne) {
-    const float dx = sp_gap(w.x0, w.x1, c.x0, c.x1), dy = sp_gap(w.y0, w.y1, c.y0, c.y1);
-    const float r2 = fmaf(dx, dx, dy * dy), g = sp_gap(w.t0, w.t1, c.t0, c.t1);
-    nb = !(fmaf(g, g, r2) > SP_ZERO);  // (negated: a NaN is kept, and reported as ever)
-    ne = c.t0 <= w.t1 && !(c.ce - omt * fmaxf(0.f, w.t0 - c.t1) - c.beta * r2 < -SP_ZERO);
-}
 
 // A lane's row: its sums over the even and odd columns.  (Its coordinates are in
 // the warp's shared memory.)
@@ -475,37 +409,17 @@ __device__ __forceinline__ void sp_excitation(const SpWarp& sw, int first, int q
     else sp_eval_e<false, LL>(sw, first, quads, nomt, w);
 }
 
-// A row group as the column tests see it: half widths of its rows about its
-// centre, and the range of time-order indices that some row must be compared
-// with one by one (ties; the excitation's first later event).
-struct SpGroup {
-    float hx, hy, ht;
-    int lo_min, ties;  // [lo_min, lo_min + ties)
-    int self;          // its own chunk
-};
-
 // A listed chunk: offset of its centre from the group's, then its number, and
 // SP_FAR if the sum of a first word and the offset may not be exact (above 512).
 constexpr int SP_FAR = 1 << 27, SP_ID = SP_FAR - 1;
 
-// Distance beyond the group's half width, not above the true one.
-__device__ __forceinline__ float sp_beyond(float d, float half) { return fmaxf(0.f, fmaf(fabsf(d), SP_IN, -half)); }
-
 // A column's coordinates from the group's centre in two words each.
 __device__ __forceinline__ void sp_two_words(const float4& a, const float4& b, const float4& off, float& xh, float& yh,
                                              float& th, float& xl, float& yl, float& tl) {
-    if (__float_as_int(off.w) & SP_FAR) {
-        sp_two_sum(sp_grid(a.x), off.x, b.x, xh, xl);
-        sp_two_sum(sp_grid(a.y), off.y, b.y, yh, yl);
-        sp_two_sum(sp_grid(a.z), off.z, b.z, th, tl);
-    } else {
-        xh = sp_grid(a.x) + off.x;
-        yh = sp_grid(a.y) + off.y;
-        th = sp_grid(a.z) + off.z;
-        xl = b.x;
-        yl = b.y;
-        tl = b.z;
-    }
+    const bool far = (__float_as_int(off.w) & SP_FAR) != 0;
+    sp_shift(a.x, b.x, off.x, far, xh, xl);
+    sp_shift(a.y, b.y, off.y, far, yh, yl);
+    sp_shift(a.z, b.z, off.z, far, th, tl);
 }
 
 // Test the events of the n listed chunks, one per lane, for a nonzero
@@ -533,9 +447,7 @@ __device__ __forceinline__ void sp_columns_b(const SpArgs& a, SpWarp& sw, int n,
         float hx, hy, ht, lx, ly, lt;  // negated, from the group's centre
         sp_two_words(q, l, off, hx, hy, ht, lx, ly, lt);
         const float nx = hx + lx, ny = hy + ly, nt = ht + lt;
-        const float dx = sp_beyond(nx, gr.hx), dy = sp_beyond(ny, gr.hy), dt = sp_beyond(nt, gr.ht);
-        // (a padding event's time is far from any; negated: a NaN is kept)
-        const bool keep = !(fmaf(dt, dt, fmaf(dx, dx, dy * dy)) > SP_ZERO);
+        const bool keep = sp_keep_b(gr, nx, ny, nt);  // (a padding event's time is far from any)
         const unsigned bal = __ballot_sync(ALL, keep);
         const bool any = __any_sync(ALL, keep && rk - (static_cast<uint32_t>(gr.lo_min) | SP_TIED) <
                                                      static_cast<unsigned>(gr.ties)) ||
@@ -582,10 +494,7 @@ __device__ __forceinline__ void sp_columns_e(const SpArgs& a, SpWarp& sw, int n,
         float hx, hy, ht, lx, ly, lt;
         sp_two_words(q, l, off, hx, hy, ht, lx, ly, lt);
         const float nx = hx + lx, ny = hy + ly, nt = ht + lt;
-        const float dx = sp_beyond(nx, gr.hx), dy = sp_beyond(ny, gr.hy);
-        const float gap = fmaxf(0.f, fmaf(nt, SP_IN, -gr.ht));  // (nt > 0: earlier than the centre)
-        const bool keep = -nt <= gr.ht + fabsf(nt) * SP_EPS &&
-                          !(ce - omt * gap + l.w * fmaf(dx, dx, dy * dy) < -SP_ZERO);
+        const bool keep = sp_keep_e(gr, nx, ny, nt, omt, ce, l.w);
         const unsigned bal = __ballot_sync(ALL, keep);
         const bool any = __any_sync(ALL, keep && rank >= gr.lo_min);
         mask |= any;
@@ -646,8 +555,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
             r[128] = -sp_grid(qa.z); r[160] = -qb.z;
             // (as integers: the order of nonnegative floats)
             auto half = [&](float v) {
-                return __uint_as_float(__reduce_max_sync(ALL, e >= 0 ? __float_as_uint(fabsf(v)) : 0u)) * SP_OUT +
-                       SP_EPS;
+                return sp_half(__uint_as_float(__reduce_max_sync(ALL, e >= 0 ? __float_as_uint(fabsf(v)) : 0u)));
             };
             gr.hx = half(qa.x);
             gr.hy = half(qa.y);
@@ -728,7 +636,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_BPSM) k_sweep_sp(SpArgs a, int*
                     const float4 c = a.centre[ch];
                     entry = make_float4(ref.x - c.x, ref.y - c.y, ref.z - c.z, 0.f);
                     const float far = fmaxf(fmaxf(fabsf(entry.x), fabsf(entry.y)), fabsf(entry.z));
-                    entry.w = __int_as_float(ch | (width + far <= 256.f ? 0 : SP_FAR));
+                    entry.w = __int_as_float(ch | (sp_is_far(width, far) ? SP_FAR : 0));
                 }
                 const unsigned kb = __ballot_sync(ALL, nb), ke = __ballot_sync(ALL, ne);
                 if (nb) sw.list[lB + __popc(kb & below)] = entry;
