@@ -18,10 +18,10 @@ __global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const 
                        int, int, int, int, const uint64_t*, int*);
 void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
                      const double*, int, double*, double*, double*);
-void launch_rows64(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, double*, double*);
+void launch_rows64(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, double*, double*);
 cudaError_t rows_setup_attributes();
-void launch_flushfix(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, int64_t, double*, double*,
-                     double*);
+void launch_flushfix(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, int64_t, double*,
+                     double*, double*);
 __global__ void k_tri_area(const double*, int32_t, double*, int*);
 __global__ void k_tri_county(const int32_t*, int32_t, int32_t, double*, int32_t*, int32_t*, int*);
 __global__ void k_tri_check(const int32_t*, int32_t, int32_t, int*);
@@ -224,10 +224,10 @@ int enqueue_finalize32(hawkes_ctx* c, int model, int64_t rb, int64_t re, double*
     const EvalDesc d = eval_desc(c);
     HK_TRY(enqueue_rows(c, rb, re, 1, 1, d_out, d_rows9, nullptr));
     HK_TRY(timed(c, HAWKES_K_ROWS64, [&] {
-        launch_rows64(c->stream, c->sms, c->sms, d, nullptr, model, re - rb, d_out, d_rows9);
+        launch_rows64(c->stream, c->sms, c->sms, d, nullptr, 1, model, re - rb, d_out, d_rows9);
     }));
     return timed(c, HAWKES_K_ROWS64, [&] {
-        launch_flushfix(c->stream, grid_for(c, re - rb, 2), c->sms, d, nullptr, model, rb, re, d_out, d_rows9, d_err);
+        launch_flushfix(c->stream, grid_for(c, re - rb, 2), c->sms, d, nullptr, 1, model, rb, re, d_out, d_rows9, d_err);
     });
 }
 

@@ -23,9 +23,9 @@ __global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const 
                        int, int, int, int, const uint64_t*, int*);
 void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
                      const double*, int, double*, double*, double*);
-void launch_rows64(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, double*, double*);
-void launch_flushfix(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, int64_t, double*, double*,
-                     double*);
+void launch_rows64(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, double*, double*);
+void launch_flushfix(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, int64_t, double*,
+                     double*, double*);
 int sweep_num_variants();
 int sweep_blocks_per_sm(int v);
 struct GroupDesc;
@@ -346,9 +346,9 @@ int enqueue(hawkes_batch* b, const hawkes_params* d_params, double* d_out, bool 
     if (time_sweep) HB_CUDA(cudaEventRecord(b->ev[1], st));
     launch_finalize(st, dim3(final_grid(nmax, b->sms, P), P), EvalDesc{}, b->d_eval, 0, 0, 1, nullptr,
                     1, d_out, nullptr, nullptr);
-    const int fix = std::max(2 * b->sms / P, 8);  // blocks per problem for the fix-ups (usually idle)
-    launch_rows64(st, dim3(fix, P), b->sms, EvalDesc{}, b->d_eval, model, 0, d_out, nullptr);
-    launch_flushfix(st, dim3(fix, P), b->sms, EvalDesc{}, b->d_eval, model, 0, 0, d_out, nullptr, nullptr);
+    const int fix = 2 * b->sms;  // blocks of the fix-ups (usually idle), whatever the problems
+    launch_rows64(st, fix, b->sms, EvalDesc{}, b->d_eval, P, model, 0, d_out, nullptr);
+    launch_flushfix(st, fix, b->sms, EvalDesc{}, b->d_eval, P, model, 0, 0, d_out, nullptr, nullptr);
     HB_CUDA(cudaGetLastError());
     return HAWKES_OK;
 }

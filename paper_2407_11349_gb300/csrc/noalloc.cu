@@ -30,10 +30,10 @@ __global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const 
                        int, int, int, int, const uint64_t*, int*);
 void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
                      const double*, int, double*, double*, double*);
-void launch_rows64(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, double*, double*);
+void launch_rows64(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, double*, double*);
 cudaError_t rows_setup_attributes();
-void launch_flushfix(cudaStream_t, dim3, int, const EvalDesc&, const EvalDesc*, int, int64_t, int64_t, double*, double*,
-                     double*);
+void launch_flushfix(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, int64_t, double*,
+                     double*, double*);
 cudaError_t sweep_setup_attributes();
 int sweep_blocks_per_sm(int v);
 int sweep_variant_rows(int v);
@@ -267,8 +267,8 @@ extern "C" int hawkes_loglik_grad_noalloc(const double* d_t, const double* d_x, 
     if (launch_sweep(&c, true, 0, n, (flags & HAWKES_BG_TIME) != 0, false) != cudaSuccess) return HAWKES_ERR_CUDA;
     launch_finalize(st, final_grid(n, d->sms < kMaxSms ? d->sms : kMaxSms), e, nullptr, 0, n, 1, nullptr,
                     1, d_out, nullptr, nullptr);
-    launch_rows64(st, c.sms, c.sms, e, nullptr, model, n, d_out, nullptr);
-    launch_flushfix(st, c.sms, c.sms, e, nullptr, model, 0, n, d_out, nullptr, nullptr);
+    launch_rows64(st, c.sms, c.sms, e, nullptr, 1, model, n, d_out, nullptr);
+    launch_flushfix(st, c.sms, c.sms, e, nullptr, 1, model, 0, n, d_out, nullptr, nullptr);
     k_na_nan_on_error<<<1, 32, 0, st>>>(c.ctr, d_out);
     return cudaGetLastError() == cudaSuccess ? HAWKES_OK : HAWKES_ERR_CUDA;
 }
