@@ -287,6 +287,10 @@ int build_items(hawkes_batch* b, int variant, int chunk, int order) {
     return HAWKES_OK;
 }
 
+// Most problems in one launch (gridDim.y); few in the debug build, so that small
+// batches take several launches there.
+constexpr int kGridY = kDebug ? 4 : 65535;
+
 static_assert(sizeof(EvalDesc) % 8 == 0, "compared as bytes: no padding");
 
 // Bring the device's problem descriptors up to date (hawkes_set_counties on a
@@ -315,7 +319,8 @@ int refresh_eval(hawkes_batch* b) {
 
 // Queue one batched evaluation.  d_params[P], d_out[7 P]; the iteration is read
 // from b->d_iter.  One launch per stage covers all problems (blockIdx.y): the
-// resample and staging, the sweeps, the finalisation and its two fix-ups.  (As
+// resample and staging, the sweeps, the finalisation and its two fix-ups (beyond
+// kGridY problems the first and third in several launches).  (As
 // one kernel per problem and stage over four side streams, 30 chains of 20,000
 // events took 180 launches, 0.5 ms of a 4.4 ms evaluation.)
 int enqueue(hawkes_batch* b, const hawkes_params* d_params, double* d_out, bool time_sweep) {
@@ -326,10 +331,11 @@ int enqueue(hawkes_batch* b, const hawkes_params* d_params, double* d_out, bool 
     cudaStream_t st = b->stream;
     int64_t nmax = 0;
     for (const hawkes_ctx* c : b->probs) nmax = std::max(nmax, c->n);
-    const EventGrid g = event_grid(nmax, b->sms, P);
-    const dim3 grid(g.blocks, P);
-    k_prep<<<grid, g.threads, 0, st>>>(EvalDesc{}, b->d_eval, d_params, hawkes_params{}, model, 1, skip,
-                                       b->resample ? 1 : 0, b->d_iter, b->d_ctr);
+    const EventGrid g = event_grid(nmax, b->sms, std::min(P, kGridY));
+    for (int p = 0; p < P; p += kGridY)
+        k_prep<<<dim3(g.blocks, std::min(P - p, kGridY)), g.threads, 0, st>>>(
+            EvalDesc{}, b->d_eval + p, d_params + p, hawkes_params{}, model, 1, skip, b->resample ? 1 : 0, b->d_iter,
+            p == 0 ? b->d_ctr : nullptr);
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
         const Rec* recs[KMAX] = {nullptr, nullptr, nullptr, nullptr};
         for (int k = 0; k < b->kc; ++k) recs[k] = b->probs[b->groups[gi][k]]->rec;
@@ -344,8 +350,9 @@ int enqueue(hawkes_batch* b, const hawkes_params* d_params, double* d_out, bool 
     HB_CUDA(launch_sweep_batch(st, b->plan, b->sms, b->variant, b->grid, b->d_probs, P, b->d_items,
                                b->nitems, b->nband, b->d_ctr, bgt, (b->flags & HAWKES_LOGLIK_ONLY) != 0));
     if (time_sweep) HB_CUDA(cudaEventRecord(b->ev[1], st));
-    launch_finalize(st, dim3(final_grid(nmax, b->sms, P), P), EvalDesc{}, b->d_eval, 0, 0, 1, nullptr,
-                    1, d_out, nullptr, nullptr);
+    for (int p = 0; p < P; p += kGridY)
+        launch_finalize(st, dim3(final_grid(nmax, b->sms, std::min(P, kGridY)), std::min(P - p, kGridY)), EvalDesc{},
+                        b->d_eval + p, 0, 0, 1, nullptr, 1, d_out + 7 * static_cast<int64_t>(p), nullptr, nullptr);
     const int fix = 2 * b->sms;  // blocks of the fix-ups (usually idle), whatever the problems
     launch_rows64(st, fix, b->sms, EvalDesc{}, b->d_eval, P, model, 0, d_out, nullptr);
     launch_flushfix(st, fix, b->sms, EvalDesc{}, b->d_eval, P, model, 0, 0, d_out, nullptr, nullptr);

@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(FINAL_THREADS)
     if (probs) {
         rb = 0;
         re = d.n;
-        out += 7 * blockIdx.y;
+        out += 7 * static_cast<int64_t>(blockIdx.y);
     }
     const int64_t n = d.n, npad = d.npad;
     double* cc = d.cc;
@@ -689,7 +689,7 @@ __global__ void __launch_bounds__(FIX_THREADS)
                 __threadfence();
             }
             __syncthreads();
-            if (s_last) finish_outputs(d.fix7 + 16, d.fix7, cc, probs ? d.n : nrows, out + (probs ? 7 * p : 0), ctr);
+            if (s_last) finish_outputs(d.fix7 + 16, d.fix7, cc, probs ? d.n : nrows, out + (probs ? 7 * static_cast<int64_t>(p) : 0), ctr);
             __syncthreads();
         }
         __syncthreads();
@@ -736,7 +736,7 @@ __global__ void __launch_bounds__(FIX_THREADS)
             const EvalDesc& d = probs ? probs[p] : one;
             const int64_t n = d.n, npad = d.npad;
             const int64_t r0 = probs ? 0 : rb, r1 = probs ? n : re;
-            double* o = out + (probs ? 7 * p : 0);
+            double* o = out + (probs ? 7 * static_cast<int64_t>(p) : 0);
             const double* cc = d.cc;
             int* ctr = d.ctr;
             const double tx = cc[CC_TX], tt = cc[CC_TT], om = cc[CC_OM], h = cc[CC_H];
