@@ -50,6 +50,10 @@ __global__ void k_set_u64(uint64_t* dst, uint64_t v) {
     if (threadIdx.x == 0 && blockIdx.x == 0) *dst = v;
 }
 
+__global__ void k_set_eval(EvalDesc* dst, const __grid_constant__ EvalDesc v) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) *dst = v;
+}
+
 // First latched error of the batch (its own counters, then the problems' in
 // order); clears them all.  One warp.
 __global__ void k_take_errors(int* bctr, const EvalDesc* __restrict__ probs, int P, int* out) {
@@ -293,27 +297,30 @@ constexpr int kGridY = kDebug ? 4 : 65535;
 
 static_assert(sizeof(EvalDesc) % 8 == 0, "compared as bytes: no padding");
 
+EvalDesc problem_desc(const hawkes_batch* b, size_t p) {
+    EvalDesc d = eval_desc(b->probs[p]);
+    if (b->resample) {
+        d.seed = b->seeds[p];
+        d.stream = b->streams[p];
+    }
+    return d;
+}
+
 // Bring the device's problem descriptors up to date (hawkes_set_counties on a
-// member replaces its triangles).  Not under stream capture.
+// member replaces its triangles), by kernels on the batch's stream.  Under stream
+// capture they become part of the graph, and the host's copy stays behind: the
+// device's changes when the graph is launched.
 int refresh_eval(hawkes_batch* b) {
-    std::vector<EvalDesc> now;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    HB_CUDA(cudaStreamIsCapturing(b->stream, &cap));
     for (size_t p = 0; p < b->probs.size(); ++p) {
         if (b->resample && !b->probs[p]->counties_ok) return HAWKES_ERR_STATE;
-        EvalDesc d = eval_desc(b->probs[p]);
-        if (b->resample) {
-            d.seed = b->seeds[p];
-            d.stream = b->streams[p];
-        }
-        now.push_back(d);
+        const EvalDesc d = problem_desc(b, p);
+        if (std::memcmp(&d, &b->h_eval[p], sizeof(d)) == 0) continue;
+        k_set_eval<<<1, 32, 0, b->stream>>>(b->d_eval + p, d);
+        HB_CUDA(cudaGetLastError());
+        if (cap == cudaStreamCaptureStatusNone) b->h_eval[p] = d;
     }
-    if (now.size() == b->h_eval.size() &&
-        std::memcmp(now.data(), b->h_eval.data(), now.size() * sizeof(EvalDesc)) == 0)
-        return HAWKES_OK;
-    HB_CUDA(cudaStreamSynchronize(b->stream));
-    HB_CUDA(cudaMemcpyAsync(b->d_eval, now.data(), now.size() * sizeof(EvalDesc), cudaMemcpyHostToDevice,
-                            b->stream));
-    HB_CUDA(cudaStreamSynchronize(b->stream));
-    b->h_eval = now;
     return HAWKES_OK;
 }
 
@@ -428,7 +435,10 @@ int hawkes_batch_create(hawkes_batch** out, hawkes_ctx* const* problems, int32_t
                                         cudaMemcpyHostToDevice, b->stream))))
             break;
         if ((rc = st_of(cudaMalloc(&b->d_eval, b->probs.size() * sizeof(EvalDesc))))) break;
-        if ((rc = refresh_eval(b))) break;
+        for (size_t p = 0; p < b->probs.size(); ++p) b->h_eval.push_back(problem_desc(b, p));
+        if ((rc = st_of(cudaMemcpyAsync(b->d_eval, b->h_eval.data(), b->h_eval.size() * sizeof(EvalDesc),
+                                        cudaMemcpyHostToDevice, b->stream))))
+            break;
         // the contexts' own queued work must finish before the batch touches their buffers
         for (auto* c : b->probs)
             if ((rc = st_of(cudaStreamSynchronize(c->stream)))) break;
