@@ -41,7 +41,7 @@ std::vector<int4> sweep_band(const std::vector<int64_t>& ns, const SweepPlan& pl
 int sweep_variant_rows(int v);
 // rows64.cu
 int rows64_segments(int64_t rows, int sms);
-size_t rows64_scratch(int sms);
+size_t rows64_scratch(int64_t n, int sms);
 cudaError_t pairs64_setup_attributes();
 cudaError_t launch_pairs64(const hawkes_ctx* c, bool model1, bool bgt, int64_t rb, int64_t re, double* out);
 // sweep_spatial.cu
@@ -132,6 +132,7 @@ void drop_shard_items(hawkes_ctx* c) {
 void free_events(hawkes_ctx* c) {
     dfree(c->t); dfree(c->x); dfree(c->y); dfree(c->is2); dfree(c->ce); dfree(c->scale_c); dfree(c->county);
     dfree(c->lo); dfree(c->hi); dfree(c->tb); dfree(c->rec); dfree(c->acc); dfree(c->fixlist);
+    dfree(c->parts64);
     dfree(c->items);
     drop_shard_items(c);
     c->nitems = 0;
@@ -355,7 +356,6 @@ int hawkes_create(hawkes_ctx** out, int device, void* cuda_stream) {
         if ((rc = dalloc(&c->cc, CC_COUNT)) != HAWKES_OK) break;
         if ((rc = dalloc(&c->out_dev, 8)) != HAWKES_OK) break;
         if ((rc = dalloc(&c->fix7, FIX_DOUBLES)) != HAWKES_OK) break;
-        if ((rc = dalloc(&c->parts64, rows64_scratch(c->sms))) != HAWKES_OK) break;
         if ((rc = dalloc(&c->partials, static_cast<size_t>(PART_STRIDE * BPSM * c->sms))) != HAWKES_OK)
             break;
         if (cudaMallocHost(reinterpret_cast<void**>(&c->out_host), 8 * sizeof(double)) != cudaSuccess) {
@@ -392,7 +392,6 @@ void hawkes_destroy(hawkes_ctx* c) {
     spatial_free(c);
     dfree(c->ctr); dfree(c->cc); dfree(c->out_dev); dfree(c->fix7);
     dfree(c->partials);
-    dfree(c->parts64);
     if (c->out_host) cudaFreeHost(c->out_host);
     for (auto& e : c->pev)
         if (e) cudaEventDestroy(e);
@@ -432,7 +431,7 @@ int hawkes_set_events(hawkes_ctx* c, int64_t n, const double* t, const double* x
             (rc = dalloc(&c->county, n)) || (rc = dalloc(&c->lo, npad)) ||
             (rc = dalloc(&c->hi, npad)) || (rc = dalloc(&c->tb, c->nblk)) ||
             (rc = dalloc(&c->rec, npad)) || (rc = dalloc(&c->acc, 6 * npad)) ||
-            (rc = dalloc(&c->fixlist, npad)))
+            (rc = dalloc(&c->fixlist, npad)) || (rc = dalloc(&c->parts64, rows64_scratch(n, c->sms))))
             return fail(rc);
     }
     cudaStream_t st = c->stream;

@@ -412,8 +412,8 @@ struct hawkes_ctx {
     double* acc = nullptr;     // [6 * npad] per-row moment sums (natural units)
     double* partials = nullptr;// [BPSM * sms * PART_STRIDE]
     double* fix7 = nullptr;    // [FIX_DOUBLES]
-    double* parts64 = nullptr; // [rows64_scratch] FP64 path: column segments' sums of few rows
     int* fixlist = nullptr;    // [npad]
+    double* parts64 = nullptr; // [rows64_scratch] FP64 path: column segments' sums of few rows
     int* ctr = nullptr;        // [CT_COUNT]
     double* cc = nullptr;      // [CC_COUNT]
     double* out_dev = nullptr; // [8]

@@ -199,12 +199,15 @@ __global__ void __launch_bounds__(32 * R64_WARPS, 1)
 // Column segments per row group: up to 32, for four items per warp of a full
 // chip, so that few rows still fill it and uneven items even out (N = 2,000: 63
 // groups x 32).  More than one segment needs at most rows64_scratch doubles for
-// the partial sums.
+// the partial sums of any rows of n events: 1.5 KB an event, up to 7.5 MB (152 SMs).
 int rows64_segments(int64_t rows, int sms) {
     const int64_t groups = (rows + 31) / 32, s = 4ll * R64_WARPS * sms / groups;
     return static_cast<int>(std::min<int64_t>(std::max<int64_t>(s, 1), 32));
 }
-size_t rows64_scratch(int sms) { return static_cast<size_t>(4 * R64_WARPS * sms) * 32 * 6; }
+size_t rows64_scratch(int64_t n, int sms) {
+    const int64_t groups = (n + 31) / 32;
+    return static_cast<size_t>(std::min<int64_t>(32 * groups, 4ll * R64_WARPS * sms)) * 32 * 6;
+}
 
 // Rows [rb, re) into out (one segment: the accumulators, [6][npad]; else the
 // scratch, [segment][6][rows rounded up to 32]); ctr[CT_WORK] must be zero.
