@@ -980,6 +980,7 @@ int hawkes_mlp_create(hawkes_mlp** out, int device, void* cuda_stream, uint64_t 
         k_refresh<<<DH * DH / 256, 256, 0, m->stream>>>(m->P, m->W1p, m->W3p, m->W2s, m->W2Ts);
         if ((rc = st_of(cudaMemsetAsync(m->M, 0, NPARAMS * sizeof(float), m->stream))) ||
             (rc = st_of(cudaMemsetAsync(m->V, 0, NPARAMS * sizeof(float), m->stream))) ||
+            (rc = st_of(cudaMemsetAsync(m->loss, 0, sizeof(double), m->stream))) ||
             (rc = st_of(cudaStreamSynchronize(m->stream))))
             break;
     } while (0);
@@ -1078,7 +1079,7 @@ int hawkes_mlp_train(hawkes_mlp* m, int64_t steps, int batch, double lr, uint64_
     a.n = m->n;
     a.seed = seed;
     a.nrec = ~0ull / static_cast<uint64_t>(m->n);
-    HM_CUDA(cudaMemsetAsync(m->loss, 0, sizeof(double), m->stream));
+    if (steps > 0) HM_CUDA(cudaMemsetAsync(m->loss, 0, sizeof(double), m->stream));  // (no step: the last loss stays)
     for (int64_t s = 0; s < steps; ++s) {
         a.step = m->step;
         a.loss = s == steps - 1 ? m->loss : nullptr;  // the last minibatch's
