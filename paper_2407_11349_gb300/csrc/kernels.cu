@@ -465,11 +465,20 @@ __global__ void __launch_bounds__(FINAL_THREADS)
             double S[6];
             if (nparts > 1) {
                 const int64_t stride = (re - rb + 31) / 32 * 32;
+                double T[6];  // (two chains, of the first and the last half: less rounding, and side by side)
 #pragma unroll
-                for (int q = 0; q < 6; ++q) S[q] = parts64[q * stride + i - rb];
-                for (int k = 1; k < nparts; ++k)
+                for (int q = 0; q < 6; ++q) S[q] = parts64[q * stride + i - rb], T[q] = 0.0;
+                const int half = nparts / 2;
+#pragma unroll 4
+                for (int k = 1; k < nparts - half; ++k)
 #pragma unroll
                     for (int q = 0; q < 6; ++q) S[q] += parts64[(6 * k + q) * stride + i - rb];
+#pragma unroll 4
+                for (int k = nparts - half; k < nparts; ++k)
+#pragma unroll
+                    for (int q = 0; q < 6; ++q) T[q] += parts64[(6 * k + q) * stride + i - rb];
+#pragma unroll
+                for (int q = 0; q < 6; ++q) S[q] += T[q];
             } else {
 #pragma unroll
                 for (int q = 0; q < 6; ++q) S[q] = d.acc[q * npad + i];

@@ -16,9 +16,9 @@
 //     pairs and not of every column that some row needs.
 //   - exp by a table of 2^(j/512) in two words and a polynomial of degree 4:
 //     10 FP64 instructions.
-// Every row's terms are added in column order, segment by segment, and
-// k_finalize adds the segments in order, so the path is reproducible to the
-// last bit.
+// Every row's terms are added in a fixed order, queue by queue and segment by
+// segment, and k_finalize adds the segments in order, so the path is reproducible
+// to the last bit.
 // Measured at N = 2,000 (100 days, 1,000 x 1,000 km, 82% of the background terms nonzero):
 // 424 us as one CTA per row with CUDA's exp over all pairs, 233 here; at
 // N = 12,000 over 1,200 days 13.1 ms and 0.92 ms.
@@ -56,6 +56,7 @@ __device__ __forceinline__ double exp_neg(double x, const double2* __restrict__ 
 
 constexpr int R64_WARPS = 8;  // most warps per CTA (one CTA per SM)
 constexpr int R64_QB = 16, R64_QE = 8;  // queued columns per lane
+constexpr int R64_FOLD = 16;            // queues per second-level sum
 constexpr float R64_ZERO = 750.f;
 
 struct R64Warp {
@@ -113,8 +114,19 @@ __global__ void __launch_bounds__(32 * R64_WARPS, 1)
         // reference point of the FP32 tests: the group's first row
         const double x0 = __shfl_sync(ALL, xi, 0), y0 = __shfl_sync(ALL, yi, 0), t0 = __shfl_sync(ALL, ti, 0);
         const float xf = bound_coord(xi - x0), yf = bound_coord(yi - y0), tf = bound_coord(ti - t0);
-        double v[6] = {0, 0, 0, 0, 0, 0};
+        // The row's sums, in two levels so that no chain of additions grows with the
+        // events: R64_FOLD queues (v), and those (total).
+        double v[6] = {0, 0, 0, 0, 0, 0}, total[6] = {0, 0, 0, 0, 0, 0};
+        int queues = 0;      // evaluated since the last fold
         int nb = 0, ne = 0;  // queued columns of this lane's row
+        auto add = [&]() {
+            if (++queues < R64_FOLD) return;
+            queues = 0;
+            for (int q = 0; q < 6; ++q) {
+                total[q] += v[q];
+                v[q] = 0.0;
+            }
+        };
 
         auto term_b = [&](int j) {
             const double dt = ti - d.t[j];
@@ -141,6 +153,7 @@ __global__ void __launch_bounds__(32 * R64_WARPS, 1)
                 for (int k = 0; k < m; ++k)
                     if (k < nb) term_b(w.qb[k][lane]);
             }
+            add();
             nb = 0;
             __syncwarp();
         };
@@ -157,6 +170,7 @@ __global__ void __launch_bounds__(32 * R64_WARPS, 1)
                     v[4] = fma(e, dt, v[4]);
                     v[5] = fma(e, q, v[5]);
                 }
+            add();
             ne = 0;
             __syncwarp();
         };
@@ -192,7 +206,7 @@ __global__ void __launch_bounds__(32 * R64_WARPS, 1)
         eval_b();
         eval_e();
         if (live)
-            for (int q = 0; q < 6; ++q) out[(static_cast<int64_t>(sg) * 6 + q) * stride + i - origin] = v[q];
+            for (int q = 0; q < 6; ++q) out[(static_cast<int64_t>(sg) * 6 + q) * stride + i - origin] = total[q] + v[q];
     }
 }
 
