@@ -249,6 +249,7 @@ enum {
 constexpr double LOG2E = 1.4426950408889634;
 constexpr double CLIP = 1e-40;
 constexpr double TWO_PI = 6.283185307179586;
+constexpr double SQRT_HALF = 0.7071067811865476;
 constexpr double SQRT_TWO_PI = 2.5066282746310002;
 
 // Bounded waits: a wait on an mbarrier gives up after WAIT_CYCLES SM clock

@@ -263,9 +263,8 @@ __global__ void k_prep(const __grid_constant__ EvalDesc one, const EvalDesc* __r
 //
 // FP64 arithmetic is the cost (1.7 lanes per clock and SM): the parameters'
 // quotients are formed once per call (k_prep), so a row needs one division,
-// one logarithm, the exponentials, and the normal CDF only near the ends of
-// the time range, where it is not 0 or 1 to the last bit: Phi(a) rounds to 1
-// for a > 8.5, and Phi(b) for b < -8.5 is below half an ulp of Phi(a) >= 1/2.
+// one logarithm, the exponentials, and the error function only near the ends of
+// the time range: erf(a / sqrt 2) rounds to 1 for a > 8.5.
 // An exponential whose argument is below -746 is exactly 0.
 //
 // row_lambda: log lambda_i and the partials of log lambda_i.  With BOUND, b[7] receives a bound on what the FP32 sweep's flushed terms can
@@ -321,16 +320,19 @@ __device__ __forceinline__ void row_lambda(const double* S, double ti, double t1
 }
 
 // Lambda_i's three parts (Sec. 2.1) and their derivatives: the Gaussian end
-// terms z = Phi(a), w = phi(a) a for a = (t_N - t_i)/tau_t (upper) or
-// -t_i/tau_t (lower), and the exponential e^{-omega (t_N - t_i)}.
+// terms z = Phi(a) - 1/2, w = phi(a) a for a = (t_N - t_i)/tau_t (upper) or
+// -t_i/tau_t (lower), and the exponential e^{-omega (t_N - t_i)}.  Only the
+// difference of the two z counts, and k_finalize sums each over all rows first:
+// without the 1/2 nothing is lost where tau_t is long against the time range and
+// the two Phi are nearly equal.
 __device__ __forceinline__ void lambda_upper(double ti, const double* __restrict__ cc, double& z, double& w) {
     const double a = (cc[CC_TN] - ti) * cc[CC_ITT], x = 0.5 * a * a;
-    z = a > 8.5 ? 1.0 : normcdf(a);
+    z = a > 8.5 ? 0.5 : 0.5 * erf(a * SQRT_HALF);
     w = x > 746.0 ? 0.0 : exp(-x) * 0.3989422804014327 * a;
 }
 __device__ __forceinline__ void lambda_lower(double ti, const double* __restrict__ cc, double& z, double& w) {
     const double b = -ti * cc[CC_ITT], x = 0.5 * b * b;
-    z = b < -8.5 ? 0.0 : normcdf(b);
+    z = b < -8.5 ? -0.5 : 0.5 * erf(b * SQRT_HALF);
     w = x > 746.0 ? 0.0 : exp(-x) * 0.3989422804014327 * b;
 }
 __device__ __forceinline__ double lambda_exp(double ti, const double* __restrict__ cc, double& gap) {
