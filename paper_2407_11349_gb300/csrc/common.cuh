@@ -243,7 +243,8 @@ enum {
     CT_FDONE,       // finished blocks of k_finalize
     CT_RDONE,       // finished blocks of k_rows64 (fix-up rows)
     CT_BAND,        // work-queue cursor of the diagonal band
-    CT_COUNT = 8
+    CT_READY,       // 1 once the row tiles' sweep has its inputs (publish_ready)
+    CT_COUNT = 16
 };
 
 constexpr double LOG2E = 1.4426950408889634;
@@ -342,6 +343,27 @@ __device__ __forceinline__ float ex2(float x) {
 // chain_next lets the successor's blocks take the SMs that this kernel leaves.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// A kernel that starts before its predecessor has ended and reads what came before
+// that one (the diagonal band behind the row tiles' sweep) has no wait of its own to
+// order those reads.  The predecessor publishes, after its own chain_wait, that its
+// inputs are there, and the successor acquires that before its first read (at once:
+// it only starts when every block ahead has passed chain_next, so after this).
+// False if the bounded wait gave up.
+__device__ __forceinline__ void publish_ready(int* ctr) {
+    asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(ctr + CT_READY) : "memory");
+}
+__device__ __forceinline__ bool acquire_ready(const int* ctr) {
+    const long long t0 = clock64();
+    for (;;) {
+        int v;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr + CT_READY) : "memory");
+        if (v != 0) break;
+        if (clock64() - t0 > WAIT_CYCLES) return false;
+    }
+    asm volatile("fence.proxy.async;" ::: "memory");  // bulk copies read the same data
+    return true;
+}
 
 __device__ __forceinline__ void set_error(int* ctr, int code) {
     atomicCAS(ctr + CT_ERR, 0, code);

@@ -157,6 +157,7 @@ __global__ void k_prep(const __grid_constant__ EvalDesc one, const EvalDesc* __r
         if (threadIdx.x == 0 && bctr && blockIdx.x == 0 && blockIdx.y == 0) {
             bctr[CT_WORK] = 0;
             bctr[CT_BAND] = 0;
+            bctr[CT_READY] = 0;
             bctr[CT_COUNT + CT_WORK] = 0;
         }
         if (threadIdx.x == 0 && blockIdx.x == 0) {
@@ -205,6 +206,7 @@ __global__ void k_prep(const __grid_constant__ EvalDesc one, const EvalDesc* __r
             cc[CC_F0 + 6] = LE * F;
             ctr[CT_WORK] = 0;
             ctr[CT_BAND] = 0;
+            ctr[CT_READY] = 0;
             ctr[CT_FIX] = 0;
             ctr[CT_DONE] = 0;
             ctr[CT_FDONE] = 0;

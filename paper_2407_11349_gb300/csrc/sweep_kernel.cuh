@@ -259,7 +259,10 @@ __global__ void __launch_bounds__(THREADS, MINB)
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     chain_wait();
-    if (SYM && item0 != 0) chain_next();
+    if (SYM && item0 != 0) {  // (in this order: the band's blocks read what this wait has ordered)
+        if (tid == 0) publish_ready(ctr);
+        chain_next();
+    }
     if (MODE != MODE_BATCH && one.cc[CC_VALID] == 0.0) return;
     if (tid == 0) {
         mbar_init(&bars[0], 1);

@@ -70,8 +70,17 @@ __global__ void __launch_bounds__(THREADS, MINB)
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // As the band of a row-tile sweep, this kernel starts while that one runs: its
-    // inputs were complete when that one started, and its end waits for that one's.
+    // inputs were complete when that one passed its chain_wait, which it publishes
+    // before the chain_next that lets this one start; this one's end waits for its.
     if (!band) chain_wait();
+    if (tid == 0) {
+        s_abort = 0;
+        if (band && !acquire_ready(ctr)) {
+            set_error(ctr, HAWKES_ERR_TIMEOUT);
+            s_abort = 1;
+        }
+    }
+    __syncthreads();
     if (MODE != MODE_BATCH && one.cc[CC_VALID] == 0.0) {
         if (band) chain_wait();
         return;
@@ -80,7 +89,6 @@ __global__ void __launch_bounds__(THREADS, MINB)
         mbar_init(&bars[0], 1);
         mbar_init(&bars[1], 1);
         fence_barrier_init();
-        s_abort = 0;
     }
     __syncthreads();
     uint32_t parbits = 0u;   // bit b: parity of the next phase of buffer b
