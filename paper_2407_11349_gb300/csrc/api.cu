@@ -31,7 +31,7 @@ __global__ void k_wait_selftest(int*);
 cudaError_t sweep_setup_attributes();
 int sweep_num_variants();
 int sweep_blocks_per_sm(int v);
-SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk, bool band);
+SweepPlan sweep_plan(const int64_t* ns, size_t count, int sms, int v, int chunk, bool band);
 std::vector<int4> sweep_items(int64_t n, const SweepPlan& pl, int v);
 cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row_end, bool bgt,
                          bool ll);
@@ -169,7 +169,7 @@ bool params_ok(const hawkes_params* p) {
 int ensure_items(hawkes_ctx* c) {
     if (c->items && c->items_variant == c->variant) return HAWKES_OK;
     dfree(c->items);
-    c->plan = sweep_plan({c->n}, c->sms, c->variant, 0, true);
+    c->plan = sweep_plan(&c->n, 1, c->sms, c->variant, 0, true);
     std::vector<int4> items = sweep_items(c->n, c->plan, c->variant);
     const std::vector<int4> band = sweep_band({c->n}, c->plan, c->variant);
     const size_t nitems = items.size();

@@ -38,7 +38,7 @@ cudaError_t launch_group_stage(cudaStream_t st, int sms, const GroupDesc& gd,
                                const Rec* const* recs, const double* t, int kc, float4* out);
 cudaError_t launch_sweep_group(cudaStream_t st, int kc, int grid, const GroupDesc* groups,
                                int ngroups, const int4* items, int nitems, int* ctr);
-SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk, bool band);
+SweepPlan sweep_plan(const int64_t* ns, size_t count, int sms, int v, int chunk, bool band);
 std::vector<int4> sweep_band(const std::vector<int64_t>& ns, const SweepPlan& pl, int v);
 std::vector<int4> sweep_items_batch(const std::vector<int64_t>& ns, const SweepPlan& pl, int v,
                                     int order);
@@ -269,7 +269,7 @@ int build_items(hawkes_batch* b, int variant, int chunk, int order) {
     HB_TRY(build_groups(b, chunk));
     std::vector<int64_t> ns;
     for (int p : b->singles) ns.push_back(b->probs[p]->n);
-    b->plan = sweep_plan(ns, b->sms, variant, chunk, true);
+    b->plan = sweep_plan(ns.data(), ns.size(), b->sms, variant, chunk, true);
     std::vector<int4> items = sweep_items_batch(ns, b->plan, variant, order);
     const size_t nitems = items.size();
     const std::vector<int4> band = sweep_band(ns, b->plan, variant);

@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include "hawkes.h"
+#include "sweep_plan.h"
 
 namespace hk {
 
@@ -57,6 +58,7 @@ constexpr int TC = 256;
 constexpr int TB = TC;
 constexpr int CHUNK = 16;
 constexpr int NPAD_MULT = 2048;
+static_assert(TC == PLAN_TC && CHUNK == PLAN_CHUNK, "the plans' tiles and items");
 static_assert(TC == THREADS, "column flush maps one thread to one column");
 
 // Staged per-event record (64 B), rebuilt every call from the FP64 inputs and
@@ -162,17 +164,6 @@ inline int final_grid(int64_t rows, int sms, int problems = 1) {
     if (g > cap) g = cap;
     return g < 1 ? 1 : static_cast<int>(g);
 }
-
-// How the symmetric sweep of a problem (or of a batch) is cut into work items
-// of `chunk` column tiles: by the row-tile kernel of the selected variant
-// (k_sweep), or by the column-split kernel (k_sweep_cs); with `band`, the row
-// tiles leave out the columns of their own rows, which the column-split kernel
-// takes.
-struct SweepPlan {
-    bool split;
-    int chunk;
-    bool band;
-};
 
 // A group of chains with identical event times, swept kc at a time by the
 // group kernel (sweep_group.cu): the group's tile records (TC / 2 + 3 kc TC

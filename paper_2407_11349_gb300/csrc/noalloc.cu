@@ -20,7 +20,6 @@
 // work overlaps on the GPU (other streams, other host threads) race on it.
 #include <cmath>
 #include <mutex>
-#include <vector>
 
 #include "common.cuh"
 
@@ -38,7 +37,7 @@ cudaError_t sweep_setup_attributes();
 int sweep_blocks_per_sm(int v);
 int sweep_variant_rows(int v);
 int split_rows();
-SweepPlan sweep_plan(const std::vector<int64_t>& ns, int sms, int v, int chunk, bool band);
+SweepPlan sweep_plan(const int64_t* ns, size_t count, int sms, int v, int chunk, bool band);
 cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row_end, bool bgt,
                          bool ll);
 }  // namespace hk
@@ -220,7 +219,7 @@ extern "C" int hawkes_loglik_grad_noalloc(const double* d_t, const double* d_x, 
 
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     unsigned char* base = d->scratch;
-    SweepPlan plan = sweep_plan({n}, d->sms, kVariant, 0, false);  // (k_na_items writes no band)
+    SweepPlan plan = sweep_plan(&n, 1, d->sms, kVariant, 0, false);  // (k_na_items writes no band)
     const int tr = plan.split ? split_rows() : sweep_variant_rows(kVariant);
     while (items_for(n, tr, plan.chunk) > kMaxItems) plan.chunk *= 2;
     const int64_t npad = (n + NPAD_MULT - 1) / NPAD_MULT * NPAD_MULT;
