@@ -293,7 +293,8 @@ int hawkes_profile_read(hawkes_ctx* ctx, hawkes_profile* out);
  * SM).  All give the same result up to FP32 summation order; they differ in
  * speed by problem size.  They hold for row windows, shards and whole sums of
  * about 28,000 events and more; smaller whole sums, whose variants' row tiles
- * would leave most SMs idle, are swept with smaller tiles.  hawkes_sweep_variants() is their number;
+ * would leave SMs idle, are mostly swept with smaller tiles (from 17,000 events
+ * by what the sizes come out at).  hawkes_sweep_variants() is their number;
  * hawkes_set_sweep_variant selects one (synchronous; rebuilds the work list).
  */
 int hawkes_sweep_variants(void);
@@ -421,8 +422,9 @@ int hawkes_batch_tune(hawkes_batch* batch, const hawkes_params* d_params, double
  * Select the sweep variant, chunk length and item order directly (drops a
  * captured graph).  A chunk length up to 16 is the longest that items have:
  * small problems take shorter ones, so that every SM has several; a length
- * above 16 is taken as it is.  Batches of few events (one problem below about
- * 28,000) are swept by a kernel with smaller row tiles whatever the variant; the
+ * above 16 is taken as it is.  Batches of few events (as much work as one
+ * problem below about 28,000) are mostly swept by a kernel with smaller row tiles
+ * whatever the variant; the
  * chunk length and order hold for it too.
  */
 int hawkes_batch_set_config(hawkes_batch* batch, int variant, int chunk, int order);

@@ -53,12 +53,25 @@ inline int pow2_floor(double v, int cap) {
 // (N = 100,000: 62 units per SM).  So the row tiles take only the columns
 // below their own rows, and the column-split kernel takes the band between;
 // it starts while the row tiles' last items run and fills the SMs they leave:
-// N = 100,000 3.96 -> 3.75 ms, 50,000 1.047 -> 0.965, 30,000 0.402 -> 0.379.
+// N = 100,000 3.96 -> 3.75 ms, 50,000 1.047 -> 0.956, 30,000 0.402 -> 0.379.
 // Items are as long as the rounds over the SMs come out shortest, in units of
-// one row tile x one column tile; an item's row flush costs 0.07 of one.  The
-// column-split kernel alone takes 1.1 times the pairs' units and 0.35 (measured
-// within 3% from N = 12,000 to 30,000), and is chosen where that is less (N below
-// about 28,000).
+// one row tile x one column tile (62 us of one SM); an item's row flush costs 0.07
+// of one.
+//
+// Row tiles with the band, or the column-split kernel alone, by what each takes in
+// these units, fitted to 50 sizes from 4,000 to 65,536 events at 152 SMs (within 4%
+// up to 25,000):
+//   - column split: 1.12 times the pairs' units per SM, and 0.2;
+//   - row tiles: 0.93 for each unit of an item and 0.06 for the item, in every round,
+//     and 0.3.  The band (1.1 times its pairs' units) runs beside them, on the SMs that
+//     the last round leaves idle and beside a last row tile with at most half of its
+//     warps' rows (0.58 of its time); what finds no room adds itself and 0.65.
+// From 4.9 units of pairs per SM (27,700 events) the row tiles are always taken: they
+// win by up to 11% there (43,000 events 0.722 ms for 0.801; 33,000, the one exception
+// seen, 0.481 for 0.478).  Below, they win where they fill their rounds: 17,103 events
+// 0.137 ms for 0.143, 24,550 0.248 for 0.275; but 10,250 0.064 for 0.075, 17,500
+// 0.144 for 0.181 and 22,000 0.226 for 0.243 are column split.  Of the sizes timed the
+// slower plan is taken at 27,000 (0.337 for 0.329) and where the two are within 2%.
 //
 // Without: column split where the row tiles cover more than 1.1 times its pairs
 // (N below about 36,000); items for 16 per SM.
@@ -68,13 +81,19 @@ inline int pow2_floor(double v, int cap) {
 // where 64 items per SM are left.
 inline SweepPlan sweep_plan(const int64_t* ns, size_t count, int sms, const PlanKernels& k, int chunk, bool band) {
     const int tr = k.tile_rows;
-    double rows = 0.0, split = 0.0, below = 0.0;  // units: tr x PLAN_TC, split_rows x PLAN_TC, tr x PLAN_TC
+    double rows = 0.0, split = 0.0;  // units: tr x PLAN_TC, split_rows x PLAN_TC
+    // units below the row tiles' own rows; those of them without rows (of a last row
+    // tile that is partly filled); and the SM time that such a tile leaves
+    double below = 0.0, dead = 0.0, thin = 0.0;
     for (size_t p = 0; p < count; ++p) {
         const int64_t n = ns[p];
         const double full = static_cast<double>((n - 1) / tr);  // row tiles with columns below them
         rows += static_cast<double>(plan_units(n, tr));
         split += static_cast<double>(plan_units(n, k.split_rows));
         below += full * (full + 1.0) / 2.0 * (tr / PLAN_TC);
+        const double last = static_cast<double>(n - static_cast<int64_t>(full) * tr) / tr;
+        dead += full * (tr / PLAN_TC) * (1.0 - last);
+        thin += last <= 0.5 ? 0.42 * full * (tr / PLAN_TC) : 0.0;
     }
     SweepPlan pl{rows * tr > 1.1 * split * k.split_rows, chunk, false};
     int best = pow2_floor(rows / (16.0 * sms), PLAN_CHUNK);
@@ -89,7 +108,11 @@ inline SweepPlan sweep_plan(const int64_t* ns, size_t count, int sms, const Plan
                 best = c;
             }
         }
-        pl.split = below == 0.0 || 1.1 * all / slots + 0.35 < least;
+        const double rounds = std::ceil(below / best / slots);
+        const double room = (slots * rounds - below / best) * (best + flush) + thin;
+        const double left = 1.1 * (all - below + dead) - room;  // of the band, when the row tiles end
+        const double tiles = rounds * (0.93 * best + 0.06) + 0.3 + (left > 0.0 ? left / slots + 0.65 : 0.0);
+        pl.split = below == 0.0 || (all < 4.9 * slots && 1.12 * all / slots + 0.2 < tiles);
         pl.band = !pl.split;
     }
     if (pl.split) best = std::max(pow2_floor(split / (3.0 * sms), 4), pow2_floor(split / (64.0 * sms), 8));

@@ -11,9 +11,9 @@
 // (chunk_pass), plus the row flush below once per item.  Sweep times before
 // (row tiles, 16 column tiles per item) and after, space-time background:
 // N = 2,000 0.425 -> 0.014 ms, 10,000 0.945 -> 0.062, 17,103 0.943 -> 0.144,
-// 30,000 0.87 -> 0.40.  sweep_plan (sweep.cu) says which kernel runs.  Larger
-// sums take the row-tile kernel below the diagonal and this one for the band of
-// each row tile's own columns.
+// 30,000 0.87 -> 0.40.  sweep_plan.h says which kernel runs.  Larger sums (and some of the
+// smaller, as 17,103) take the row-tile kernel below the diagonal and this one for
+// the band of each row tile's own columns.
 // What changes:
 //   - a column belongs to one warp: its sums go from the warp's registers to
 //     the FP64 accumulators, without the shared-memory pass;
