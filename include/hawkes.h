@@ -302,6 +302,14 @@ int hawkes_set_sweep_variant(hawkes_ctx* ctx, int variant);
 int hawkes_get_sweep_variant(const hawkes_ctx* ctx);
 
 /*
+ * How whole sums of the current events are swept (HAWKES_ERR_STATE without
+ * events): *column_split 1 if by the kernel with smaller row tiles alone, else 0;
+ * *band 1 if by the variant's row tiles below the diagonal and that kernel for the
+ * diagonal band; *chunk the column tiles per work item.  Null pointers are skipped.
+ */
+int hawkes_get_sweep_plan(const hawkes_ctx* ctx, int* column_split, int* band, int* chunk);
+
+/*
  * Autotune the sweep on the current events: run every variant `reps` times
  * (after one warm-up) at `params` (host pointer; flags as for
  * hawkes_loglik_grad, FP32 path), time the sweep kernel with CUDA events,

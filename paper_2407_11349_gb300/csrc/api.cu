@@ -689,6 +689,15 @@ int hawkes_set_sweep_variant(hawkes_ctx* c, int variant) {
 
 int hawkes_get_sweep_variant(const hawkes_ctx* c) { return c ? c->variant : HAWKES_ERR_ARG; }
 
+int hawkes_get_sweep_plan(const hawkes_ctx* c, int* column_split, int* band, int* chunk) {
+    if (!c) return HAWKES_ERR_ARG;
+    if (c->n == 0) return HAWKES_ERR_STATE;
+    if (column_split) *column_split = c->plan.split ? 1 : 0;
+    if (band) *band = c->plan.band ? 1 : 0;
+    if (chunk) *chunk = c->plan.chunk;
+    return HAWKES_OK;
+}
+
 int hawkes_tune(hawkes_ctx* c, const hawkes_params* p, uint32_t flags, int reps, int* chosen,
                 double* ms) {
     HK_NVTX("hawkes_tune");

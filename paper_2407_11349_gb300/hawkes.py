@@ -74,6 +74,7 @@ _SIGS = {
     "hawkes_debug_set_item": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
     "hawkes_set_sweep_variant": (ctypes.c_int, [_VP, ctypes.c_int]),
     "hawkes_get_sweep_variant": (ctypes.c_int, [_VP]),
+    "hawkes_get_sweep_plan": (ctypes.c_int, [_VP] + [ctypes.POINTER(ctypes.c_int)] * 3),
     "hawkes_tune": (ctypes.c_int, [_VP, ctypes.POINTER(hawkes_params), ctypes.c_uint32, ctypes.c_int,
                                    ctypes.POINTER(ctypes.c_int), _D]),
     "hawkes_tune_cached": (ctypes.c_int, [_VP, ctypes.POINTER(hawkes_params), ctypes.c_uint32, ctypes.c_int,
@@ -576,6 +577,12 @@ class Hawkes:
         sec = ctypes.c_double()
         _check(lib().hawkes_check_bounded_wait(self.ctx, ctypes.byref(sec)), "hawkes_check_bounded_wait")
         return sec.value
+
+    def sweep_plan(self):
+        """(column split, diagonal band, column tiles per item) of whole sums."""
+        v = [ctypes.c_int() for _ in range(3)]
+        _check(lib().hawkes_get_sweep_plan(self.ctx, *[ctypes.byref(k) for k in v]), "hawkes_get_sweep_plan")
+        return tuple(k.value for k in v)
 
     def tune(self, params, flags=HAWKES_F32, reps=2):
         return hawkes_tune(self.ctx, params, flags, reps)
