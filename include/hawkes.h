@@ -329,10 +329,14 @@ int hawkes_tune(hawkes_ctx* ctx, const hawkes_params* params, uint32_t flags, in
  *   ...
  *   }
  * The tuners below build the key as
- *   "<device name>|sm_<major><minor>|single|n<=2^<e>|flags=<flags>"
- *   "<device name>|sm_<major><minor>|batch|P=<P>|pairs<=2^<e>|flags=<flags>"
+ *   "<device name>|sm_<major><minor>|<kernels>|single|n<=2^<e>|flags=<flags>"
+ *   "<device name>|sm_<major><minor>|<kernels>|batch|P=<P>|pairs<=2^<e>|flags=<flags>"
  * where 2^e is the smallest power of two >= n (single problem) or >= the
- * batch's total number of unordered pairs.  Entries written by a build with a
+ * batch's total number of unordered pairs, and <kernels> is
+ * "kernels=<number>|plans=<a letter per variant>": a number that changes with the
+ * sweep's kernels, and how each variant would sweep these sizes (c the kernel with
+ * smaller row tiles alone, r the variant's own).  Variants with a c run one kernel;
+ * the tuners choose the first of them.  Entries written by a build with a
  * different number of sweep variants ("nvariants") are ignored, and lines
  * that do not parse are skipped, so a stale or damaged file only causes cache
  * misses.  Writes go to "<path>.tmp" and are renamed over the file.

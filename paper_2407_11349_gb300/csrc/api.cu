@@ -712,8 +712,13 @@ int hawkes_tune(hawkes_ctx* c, const hawkes_params* p, uint32_t flags, int reps,
     int best = -1;
     double best_ms = 0.0;
     double out7[7];
+    double split_ms = -1.0;  // variants whose plan is column split run one kernel: the first is timed for them
     for (int v = 0; v < sweep_num_variants(); ++v) {
         HK_TRY(select_variant(c, v));
+        if (c->plan.split && split_ms >= 0.0) {
+            if (ms) ms[v] = split_ms;
+            continue;
+        }
         HK_TRY(sync_loglik(c, p, flags, 0, c->n, out7, nullptr));  // warm-up
         c->prof = true;
         std::memset(&c->pacc, 0, sizeof(c->pacc));
@@ -721,6 +726,7 @@ int hawkes_tune(hawkes_ctx* c, const hawkes_params* p, uint32_t flags, int reps,
         const double t = c->pacc.ms[HAWKES_K_SWEEP] / reps;
         c->prof = prof;
         if (ms) ms[v] = t;
+        if (c->plan.split) split_ms = t;
         if (best < 0 || t < best_ms) {
             best = v;
             best_ms = t;
@@ -760,6 +766,7 @@ int tune_cache_put(const char* path, const char* key, int variant, int chunk, in
                    int kc);
 int log2_ceil(double v);
 std::string device_key();
+std::string sweep_plans_key(const int64_t* ns, size_t count, int sms);
 }  // namespace hk
 
 int hawkes_tune_cached(hawkes_ctx* c, const hawkes_params* p, uint32_t flags, int reps,
@@ -774,7 +781,7 @@ int hawkes_tune_cached(hawkes_ctx* c, const hawkes_params* p, uint32_t flags, in
     DeviceGuard g(c->device);
     const std::string dk = device_key();
     if (dk.empty()) return HAWKES_ERR_CUDA;
-    const std::string key = dk + "single|n<=2^" + std::to_string(log2_ceil(static_cast<double>(c->n))) +
+    const std::string key = dk + sweep_plans_key(&c->n, 1, c->sms) + "single|n<=2^" + std::to_string(log2_ceil(static_cast<double>(c->n))) +
                             "|flags=" + std::to_string(flags);
     int v = -1;
     if (tune_cache_get(cache_path, key.c_str(), &v, nullptr, nullptr, nullptr, nullptr) == 1) {

@@ -78,6 +78,7 @@ int tune_cache_put(const char* path, const char* key, int variant, int chunk, in
                    int kc);
 int log2_ceil(double v);
 std::string device_key();
+std::string sweep_plans_key(const int64_t* ns, size_t count, int sms);
 }  // namespace hk
 
 using namespace hk;
@@ -189,6 +190,12 @@ int time_classes(hawkes_batch* b) {
 // gradient, Model 1 or 2, no tile skipping.
 bool group_flags_ok(uint32_t flags) {
     return (flags & (HAWKES_BG_TIME | HAWKES_LOGLIK_ONLY | HAWKES_SKIP_UNDERFLOW)) == 0;
+}
+
+std::vector<int64_t> problem_sizes(const hawkes_batch* b) {
+    std::vector<int64_t> ns;
+    for (const hawkes_ctx* c : b->probs) ns.push_back(c->n);
+    return ns;
 }
 
 // Largest class of problems with identical event times.
@@ -548,9 +555,15 @@ int hawkes_batch_tune(hawkes_batch* b, const hawkes_params* d_params, double* d_
         return HAWKES_OK;
     };
     HB_TRY(refresh_eval(b));
-    // one problem per CTA: sweep variant x item order x chunk length
+    // one problem per CTA: sweep variant x item order x chunk length (variants whose
+    // plan is column split run one kernel: the first stands for them)
     b->kc = 1;
+    bool one_split = false;
     for (int v = 0; v < sweep_num_variants(); ++v) {
+        const std::vector<int64_t> ns = problem_sizes(b);
+        const bool split = sweep_plan(ns.data(), ns.size(), b->sms, v, CHUNK, true).split;
+        if (split && one_split) continue;
+        one_split = one_split || split;
         for (int o = 0; o < 2; ++o) {
             for (int ch : kChunks) {
                 double t = 0.0;
@@ -641,9 +654,10 @@ int hawkes_batch_tune_cached(hawkes_batch* b, const hawkes_params* d_params, dou
     DeviceGuard g(b->device);
     const std::string dk = device_key();
     if (dk.empty()) return HAWKES_ERR_CUDA;
+    const std::vector<int64_t> ns = problem_sizes(b);
     double pairs = 0.0;
     for (const hawkes_ctx* c : b->probs) pairs += 0.5 * static_cast<double>(c->n) * (c->n - 1);
-    const std::string key = dk + "batch|P=" + std::to_string(b->probs.size()) + "|pairs<=2^" +
+    const std::string key = dk + sweep_plans_key(ns.data(), ns.size(), b->sms) + "batch|P=" + std::to_string(b->probs.size()) + "|pairs<=2^" +
                             std::to_string(log2_ceil(pairs > 1.0 ? pairs : 1.0)) +
                             "|flags=" + std::to_string(b->flags);
     int v = -1, ch = 0, o = 0, kc = 1;

@@ -3,6 +3,7 @@
 // space-time background's kernels; sweep_bgt.cu the time-only background's
 // and sweep_ll.cu the log-likelihood-only ones.
 #include <algorithm>
+#include <string>
 #include <vector>
 
 #include "sweep_kernel.cuh"
@@ -52,6 +53,16 @@ int sweep_blocks_per_sm(int v) {
 // The plan (sweep_plan.h) on variant v.
 SweepPlan sweep_plan(const int64_t* ns, size_t count, int sms, int v, int chunk, bool band) {
     return sweep_plan(ns, count, sms, PlanKernels{kVariants[v].tr, kVariants[v].minb, split_rows()}, chunk, band);
+}
+
+// The tuning caches' part of a key that says which kernels the times are of: a
+// number to raise when the sweep's kernels or plans change, and each variant's plan
+// (c column split alone, r row tiles).  Sizes of one power of two may differ in it,
+// and on a c the variants' times are one kernel's.
+std::string sweep_plans_key(const int64_t* ns, size_t count, int sms) {
+    std::string key = "kernels=2|plans=";
+    for (int v = 0; v < kNumVariants; ++v) key += sweep_plan(ns, count, sms, v, CHUNK, true).split ? 'c' : 'r';
+    return key + "|";
 }
 
 // Symmetric work list over problems of sizes ns[] for plan pl (variant v on

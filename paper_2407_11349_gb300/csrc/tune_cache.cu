@@ -5,7 +5,7 @@
 // The file is written by this library as a JSON object with one entry per
 // line:
 //   {
-//   "NVIDIA GB300|sm_103|single|n<=2^20|flags=0": {"variant": 0, "chunk": 16, "order": 0, "ms": 365.359, "nvariants": 5, "kc": 1},
+//   "NVIDIA GB300|sm_103|kernels=2|plans=rrrrr|single|n<=2^20|flags=0": {"variant": 0, "chunk": 16, "order": 0, "ms": 365.359, "nvariants": 5, "kc": 1},
 //   ...
 //   }
 // The reader accepts exactly that shape and skips any line it cannot parse,
