@@ -330,7 +330,9 @@ __device__ __forceinline__ float ex2(float x) {
 
 // Chained launches: a kernel of a call starts while its predecessor ends.
 // chain_wait comes before the first read of what an earlier kernel wrote, in
-// every thread (the predecessor has then finished, and all before it);
+// every thread (the predecessor has then finished, and all before it); what it wrote
+// is not read through a `const __restrict__` parameter, whose loads the compiler may
+// take for invariant and move ahead of the wait;
 // chain_next lets the successor's blocks take the SMs that this kernel leaves.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

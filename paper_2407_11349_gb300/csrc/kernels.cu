@@ -443,7 +443,7 @@ __device__ __forceinline__ void finish_outputs(const double* tot, const volatile
 template <bool ROWS>
 __global__ void __launch_bounds__(FINAL_THREADS)
     k_finalize(const __grid_constant__ EvalDesc one, const EvalDesc* __restrict__ probs, int64_t rb,
-               int64_t re, int check, const double* __restrict__ parts64, int nparts, double* out,
+               int64_t re, int check, const double* parts64, int nparts, double* out,
                double* rows9, double* err_out) {
     chain_wait();
     const EvalDesc& d = probs ? probs[blockIdx.y] : one;

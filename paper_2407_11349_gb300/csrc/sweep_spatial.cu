@@ -270,8 +270,7 @@ __global__ void __launch_bounds__(TC) k_sp_prep(EvalDesc d, const uint32_t* __re
 }
 
 // Boxes of the blocks of 32 tiles, one warp each.
-__global__ void k_sp_blocks(const float4* __restrict__ tmeta, float4* __restrict__ bmeta, int ntiles,
-                            const double* __restrict__ cc) {
+__global__ void k_sp_blocks(const float4* tmeta, float4* bmeta, int ntiles, const double* cc) {
     chain_next();
     chain_wait();
     if (cc[CC_VALID] == 0.0) return;
