@@ -79,7 +79,11 @@ enum {
      * 1e-8 of its magnitude, the rows whose bound exceeds 1e-8 of that
      * magnitude divided by the row count are recomputed in FP64 (at normal
      * bandwidths none is; with bandwidths so small that every excitation
-     * term underflows, most are).
+     * term underflows, most are).  What FP32 keeps of a term is its exponent
+     * to 2^-24 of the exponent: where an output rests on terms with base-2
+     * exponents near 100 (a few hundred sparse events), it carries their
+     * relative error, about 1e-5, and a gradient component that their sum
+     * all but cancels, 1.2e-4 of itself.  HAWKES_F64 has neither.
      */
     HAWKES_F32 = 0,
     HAWKES_F64 = 1,      /* every pair term in FP64 (slow on GB300: reference path) */
@@ -117,7 +121,9 @@ enum {
      * full sum up to FP32 summation order.  The first call after
      * hawkes_set_events builds the order on the host (synchronous: make it
      * outside stream capture), weighing space against time by that call's
-     * tau_x and tau_t; a later call with other values gives the same result.
+     * tau_x and tau_t; a later call with other values gives the same result,
+     * if at another speed (with bandwidths far from those that built the order,
+     * call hawkes_set_events again).
      * Not for batches, HAWKES_F64, HAWKES_BG_TIME or row windows
      * (HAWKES_ERR_ARG).
      */
@@ -272,8 +278,8 @@ enum {
     HAWKES_K_PREP = 0,     /* per-call FP32 staging of the event table */
     HAWKES_K_SWEEP = 1,    /* FP32 pair sweep */
     HAWKES_K_ROWS64 = 2,   /* FP64 pair rows */
-    HAWKES_K_FINAL = 3,    /* per-row finalisation + block reduction */
-    HAWKES_K_REDUCE = 4,   /* global reduction */
+    HAWKES_K_FINAL = 3,    /* per-row finalisation and the reductions */
+    HAWKES_K_REDUCE = 4,   /* (no launches: HAWKES_K_FINAL reduces) */
     HAWKES_K_RESAMPLE = 5, /* location resample */
     HAWKES_K_OTHER = 6     /* set-up kernels */
 };

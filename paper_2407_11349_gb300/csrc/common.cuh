@@ -202,7 +202,7 @@ enum {
     CC_BGT,         // 1 for the time-only background
     CC_LLONLY,      // 1 when only the log-likelihood is evaluated
     CC_FTHR,        // [7] flush-bound thresholds per output (< 0: nothing to recompute)
-    // Row finalisation, linear in the raw moment sums S (see row_eval):
+    // Row finalisation, linear in the raw moment sums S (see row_lambda):
     CC_LB = CC_FTHR + 7,  // lambda = LB SB + LE SE
     CC_LE,
     CC_A1, CC_B1,   // d/dtau_x numerator A1 SBr - B1 SB

@@ -185,7 +185,7 @@ __global__ void k_prep(const __grid_constant__ EvalDesc one, const EvalDesc* __r
             cc[CC_BGT] = bgt ? 1.0 : 0.0;
             cc[CC_LLONLY] = (model & HAWKES_LOGLIK_ONLY) ? 1.0 : 0.0;
             for (int q = 0; q < 7; ++q) cc[CC_FTHR + q] = -1.0;
-            // coefficients of the row finalisation (see row_eval)
+            // coefficients of the row finalisation (see row_lambda)
             const double LB = k.mu * k.cB, LE = k.th * k.cE;
             const double itx = k.itx, itt = k.itt, iom = k.iom, ih = k.ih;
             const double itx3 = itx * itx * itx, itt3 = itt * itt * itt, ih3 = ih * ih * ih;
@@ -344,11 +344,9 @@ __device__ __forceinline__ double lambda_exp(double ti, const double* __restrict
 }
 
 // A whole row: ell_i, its six partials, log lambda_i, Lambda_i.
-template <bool BOUND>
-__device__ __forceinline__ void row_eval(const double* S, double ti, double t1, double nb, double ne,
-                                         const double* __restrict__ cc, double out[9], double b[7]) {
-    double d[6], Pa, Pb, wa, wb, gap;
-    row_lambda<BOUND>(S, ti, t1, nb, ne, cc, out[7], d, b);
+__device__ __forceinline__ void row_eval(const double* S, double ti, const double* __restrict__ cc, double out[9]) {
+    double d[6], b[7], Pa, Pb, wa, wb, gap;
+    row_lambda<false>(S, ti, 0.0, 0.0, 0.0, cc, out[7], d, b);
     lambda_upper(ti, cc, Pa, wa);
     lambda_lower(ti, cc, Pb, wb);
     const double ea = lambda_exp(ti, cc, gap);
@@ -511,8 +509,8 @@ __global__ void __launch_bounds__(FINAL_THREADS)
                     for (int q = 0; q < 7; ++q) v[7 + q] += bd[q];
             }
             if (ROWS && !queue) {  // queued rows are written by k_rows64
-                double o[9], b[7];
-                row_eval<false>(S, ti, t1, 0.0, 0.0, cc, o, b);
+                double o[9];
+                row_eval(S, ti, cc, o);
                 for (int q = 0; q < 9; ++q) rows9[9 * i + q] = o[q];
             }
         }
@@ -688,7 +686,7 @@ __global__ void __launch_bounds__(FIX_THREADS)
                     atomicAdd(d.fix7, loglam);
                     for (int m = 0; m < 6; ++m) atomicAdd(d.fix7 + 1 + m, dl[m]);
                     if (rows9) {
-                        row_eval<false>(sums, d.t[i], 0.0, 0.0, 0.0, cc, o, b);
+                        row_eval(sums, d.t[i], cc, o);
                         for (int m = 0; m < 9; ++m) rows9[9 * i + m] = o[m];
                     }
                 }
@@ -795,7 +793,7 @@ __global__ void __launch_bounds__(FIX_THREADS)
                         for (int q = 0; q < 6; ++q) mine[1 + q] += d64[q] - d32[q];
                         if (rows9) {
                             double o64[9];
-                            row_eval<false>(sums, d.t[r], 0.0, 0.0, 0.0, cc, o64, b);
+                            row_eval(sums, d.t[r], cc, o64);
                             for (int q = 0; q < 9; ++q) rows9[9 * r + q] = o64[q];
                         }
                     }

@@ -827,7 +827,7 @@ struct hawkes_mlp {
     float *X = nullptr, *T = nullptr, *Y = nullptr;  // one batch given by the caller
     unsigned char *h1op = nullptr, *dzop = nullptr;  // k_mlp to k_update (see MlpArgs)
     float *h2t = nullptr, *dz2t = nullptr, *dz1t = nullptr, *xin = nullptr, *dyo = nullptr;
-    double* hbuf = nullptr;  // pinned host scratch
+    double* hbuf = nullptr;  // pinned host copy of the loss
     int* err = nullptr;      // pinned host: latched device error (a wait that gave up)
 };
 
@@ -889,27 +889,9 @@ MlpArgs args_of(const hawkes_mlp* m, int B) {
     return a;
 }
 
-// Launch with programmatic serialisation: the kernel may start while the one
-// before it ends, and waits for it (griddepcontrol.wait) before it reads what
-// that one writes.
-template <typename... Args, typename... Given>
-int launch_chained(void (*kern)(Args...), int grid, size_t smem, cudaStream_t st, Given... given) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(MLP_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return st_of(cudaLaunchKernelEx(&cfg, kern, static_cast<Args>(given)...));
-}
-
 template <int MODE>
 int launch_mlp(hawkes_mlp* m, const MlpArgs& a) {
-    return launch_chained(k_mlp<MODE>, CL * ((a.B + MT - 1) / MT), sizeof(MlpSmem), m->stream, a);
+    return st_of(hk::launch_chained(k_mlp<MODE>, CL * ((a.B + MT - 1) / MT), MLP_THREADS, sizeof(MlpSmem), m->stream, a));
 }
 
 template <bool UPDATE>
@@ -925,7 +907,7 @@ int launch_update(hawkes_mlp* m, int B, float lr) {
     a.W1p = m->W1p; a.W3p = m->W3p;
     a.W2s = m->W2s; a.W2Ts = m->W2Ts;
     a.err = m->err;
-    return launch_chained(k_update<UPDATE>, UPDATE_BLOCKS, sizeof(UpdateSmem), m->stream, a);
+    return st_of(hk::launch_chained(k_update<UPDATE>, UPDATE_BLOCKS, MLP_THREADS, sizeof(UpdateSmem), m->stream, a));
 }
 
 }  // namespace
@@ -962,7 +944,7 @@ int hawkes_mlp_create(hawkes_mlp** out, int device, void* cuda_stream, uint64_t 
             (rc = alloc(&m->h2t, BMAX * DH)) || (rc = alloc(&m->dz2t, BMAX * DH)) ||
             (rc = alloc(&m->dz1t, BMAX * DH)) || (rc = alloc(&m->xin, BMAX * 8)) || (rc = alloc(&m->dyo, BMAX * 8)))
             break;
-        if ((rc = st_of(cudaMallocHost(reinterpret_cast<void**>(&m->hbuf), 64 * sizeof(double))))) break;
+        if ((rc = st_of(cudaMallocHost(reinterpret_cast<void**>(&m->hbuf), sizeof(double))))) break;
         if ((rc = st_of(cudaMallocHost(reinterpret_cast<void**>(&m->err), sizeof(int))))) break;
         *m->err = 0;
         for (const void* f : {reinterpret_cast<const void*>(k_mlp<MLP_PREDICT>),
