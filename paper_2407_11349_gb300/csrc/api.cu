@@ -7,51 +7,7 @@
 #include <string>
 #include <vector>
 
-#include "common.cuh"
-
-namespace hk {
-// kernels.cu
-__global__ void k_setup(double*, double*, double*, const int32_t*, int32_t, const double*, int64_t,
-                        int64_t, int, double*, float*, int32_t*, int32_t*, double*, int*);
-__global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const hawkes_params*,
-                       const __grid_constant__ hawkes_params,
-                       int, int, int, int, const uint64_t*, int*);
-void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
-                     const double*, int, double*, double*, double*);
-void launch_rows64(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, double*, double*);
-cudaError_t rows_setup_attributes();
-void launch_flushfix(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, int64_t, double*,
-                     double*, double*);
-__global__ void k_tri_area(const double*, int32_t, double*, int*);
-__global__ void k_tri_county(const int32_t*, int32_t, int32_t, double*, int32_t*, int32_t*, int*);
-__global__ void k_tri_check(const int32_t*, int32_t, int32_t, int*);
-__global__ void k_resample(const __grid_constant__ EvalDesc, uint64_t);
-__global__ void k_wait_selftest(int*);
-// sweep.cu
-cudaError_t sweep_setup_attributes();
-int sweep_num_variants();
-int sweep_blocks_per_sm(int v);
-SweepPlan sweep_plan(const int64_t* ns, size_t count, int sms, int v, int chunk, bool band);
-std::vector<int4> sweep_items(int64_t n, const SweepPlan& pl, int v);
-cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row_end, bool bgt,
-                         bool ll);
-cudaError_t launch_sweep_list(hawkes_ctx* c, const int4* items, int nitems, int nband, bool bgt, bool ll);
-int split_rows();
-std::vector<int4> sweep_band(const std::vector<int64_t>& ns, const SweepPlan& pl, int v);
-int sweep_variant_rows(int v);
-// rows64.cu
-int rows64_segments(int64_t rows, int sms);
-size_t rows64_scratch(int64_t n, int sms);
-cudaError_t pairs64_setup_attributes();
-cudaError_t launch_pairs64(const hawkes_ctx* c, bool model1, bool bgt, int64_t rb, int64_t re, double* out);
-// sweep_spatial.cu
-cudaError_t spatial_setup_attributes();
-int spatial_build(hawkes_ctx* c, const hawkes_params* p, const hawkes_params* d_p);
-cudaError_t spatial_launch(hawkes_ctx* c, int model1, int llonly);
-void spatial_free(hawkes_ctx* c);
-int spatial_set_window(hawkes_ctx* c, int64_t window);
-void spatial_invalidate(hawkes_ctx* c);
-}  // namespace hk
+#include "units.cuh"
 
 using namespace hk;
 
@@ -758,16 +714,6 @@ int hawkes_profile_read(hawkes_ctx* c, hawkes_profile* out) {
 }
 
 }  // extern "C"
-
-namespace hk {
-int tune_cache_get(const char* path, const char* key, int* variant, int* chunk, int* order,
-                   double* ms, int* kc);
-int tune_cache_put(const char* path, const char* key, int variant, int chunk, int order, double ms,
-                   int kc);
-int log2_ceil(double v);
-std::string device_key();
-std::string sweep_plans_key(const int64_t* ns, size_t count, int sms);
-}  // namespace hk
 
 int hawkes_tune_cached(hawkes_ctx* c, const hawkes_params* p, uint32_t flags, int reps,
                        const char* cache_path, int* chosen, int* from_cache) {

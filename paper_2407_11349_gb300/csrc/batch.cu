@@ -15,37 +15,9 @@
 #include <string>
 #include <vector>
 
-#include "common.cuh"
+#include "units.cuh"
 
 namespace hk {
-__global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const hawkes_params*,
-                       const __grid_constant__ hawkes_params,
-                       int, int, int, int, const uint64_t*, int*);
-void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
-                     const double*, int, double*, double*, double*);
-void launch_rows64(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, double*, double*);
-void launch_flushfix(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, int64_t, double*,
-                     double*, double*);
-int sweep_num_variants();
-int sweep_blocks_per_sm(int v);
-struct GroupDesc;
-bool group_kc_supported(int kc);
-int group_blocks_per_sm(int kc);
-size_t group_tile_bytes(int kc);
-cudaError_t group_setup_attributes();
-std::vector<int4> group_items(const std::vector<int64_t>& ns, int kc, int chunk);
-cudaError_t launch_group_stage(cudaStream_t st, int sms, const GroupDesc& gd,
-                               const Rec* const* recs, const double* t, int kc, float4* out);
-cudaError_t launch_sweep_group(cudaStream_t st, int kc, int grid, const GroupDesc* groups,
-                               int ngroups, const int4* items, int nitems, int* ctr);
-SweepPlan sweep_plan(const int64_t* ns, size_t count, int sms, int v, int chunk, bool band);
-std::vector<int4> sweep_band(const std::vector<int64_t>& ns, const SweepPlan& pl, int v);
-std::vector<int4> sweep_items_batch(const std::vector<int64_t>& ns, const SweepPlan& pl, int v,
-                                    int order);
-cudaError_t launch_sweep_batch(cudaStream_t st, const SweepPlan& pl, int sms, int variant, int grid,
-                               const ProbDesc* probs, int nprobs, const int4* items, int nitems, int nband,
-                               int* ctr, bool bgt, bool ll);
-
 __global__ void k_set_u64(uint64_t* dst, uint64_t v) {
     if (threadIdx.x == 0 && blockIdx.x == 0) *dst = v;
 }
@@ -72,13 +44,6 @@ __global__ void k_take_errors(int* bctr, const EvalDesc* __restrict__ probs, int
     }
     if (lane == 0) *out = err;
 }
-int tune_cache_get(const char* path, const char* key, int* variant, int* chunk, int* order,
-                   double* ms, int* kc);
-int tune_cache_put(const char* path, const char* key, int variant, int chunk, int order, double ms,
-                   int kc);
-int log2_ceil(double v);
-std::string device_key();
-std::string sweep_plans_key(const int64_t* ns, size_t count, int sms);
 }  // namespace hk
 
 using namespace hk;

@@ -4,7 +4,7 @@
 // recomputed in FP64, and the cut-posterior location resample (Sec. 2.2).
 #include <math_constants.h>
 
-#include "common.cuh"
+#include "units.cuh"
 
 namespace hk {
 

@@ -21,26 +21,7 @@
 #include <cmath>
 #include <mutex>
 
-#include "common.cuh"
-
-namespace hk {
-__global__ void k_prep(const __grid_constant__ EvalDesc, const EvalDesc*, const hawkes_params*,
-                       const __grid_constant__ hawkes_params,
-                       int, int, int, int, const uint64_t*, int*);
-void launch_finalize(cudaStream_t, dim3, const EvalDesc&, const EvalDesc*, int64_t, int64_t, int,
-                     const double*, int, double*, double*, double*);
-void launch_rows64(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, double*, double*);
-cudaError_t rows_setup_attributes();
-void launch_flushfix(cudaStream_t, int, int, const EvalDesc&, const EvalDesc*, int, int, int64_t, int64_t, double*,
-                     double*, double*);
-cudaError_t sweep_setup_attributes();
-int sweep_blocks_per_sm(int v);
-int sweep_variant_rows(int v);
-int split_rows();
-SweepPlan sweep_plan(const int64_t* ns, size_t count, int sms, int v, int chunk, bool band);
-cudaError_t launch_sweep(hawkes_ctx* c, bool sym, int64_t row_begin, int64_t row_end, bool bgt,
-                         bool ll);
-}  // namespace hk
+#include "units.cuh"
 
 using namespace hk;
 

@@ -24,7 +24,7 @@
 // N = 12,000 over 1,200 days 13.1 ms and 0.92 ms.
 #include <algorithm>
 
-#include "common.cuh"
+#include "units.cuh"
 #include "exp_table.cuh"
 
 namespace hk {

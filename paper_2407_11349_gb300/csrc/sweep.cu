@@ -7,14 +7,9 @@
 #include <vector>
 
 #include "sweep_kernel.cuh"
+#include "units.cuh"
 
 namespace hk {
-
-// The column-split kernels (sweep_split.cu).
-cudaError_t split_setup_attributes();
-int split_rows();
-cudaError_t launch_sweep_split(cudaStream_t st, int sms, const ProbDesc& one, const ProbDesc* probs,
-                               int nprobs, const int4* items, int nitems, int* ctr, bool bgt, bool ll, bool band);
 
 static const Variant kVariants[] = HK_SWEEP_VARIANTS(false, false);
 static_assert(sizeof(kVariants) / sizeof(kVariants[0]) == kNumVariants, "variant count");

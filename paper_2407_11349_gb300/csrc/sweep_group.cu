@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "sweep_kernel.cuh"
+#include "units.cuh"
 
 namespace hk {
 
@@ -418,7 +419,6 @@ static const GroupVariant* group_variant(int kc) {
 
 bool group_kc_supported(int kc) { return group_variant(kc) != nullptr; }
 int group_tile_rows(int kc) { return group_variant(kc)->tr; }
-size_t group_tile_bytes(int kc) { return static_cast<size_t>(gt_f4(kc)) * sizeof(float4); }
 
 cudaError_t group_setup_attributes() {
     for (const GroupVariant& v : kGroupVariants) {

@@ -36,7 +36,7 @@
 // columns that pass the point test.  At N = 1,000,000 (3,143 counties, 1,200 days)
 // after a resample, which widens the boxes, a row has 1,811 columns with a nonzero
 // background and 14 with a nonzero excitation; point tests against the box of 32
-// rows leave 3,770 and 620, in 3.82 ms.  256 x 256 tile pairs kept whole by box
+// rows leave 3,770 and 620, in 3.55 to 3.85 ms.  256 x 256 tile pairs kept whole by box
 // tests and swept through shared-memory tiles took 45 ms (40,000 columns with both
 // terms).  Two rows per lane would halve the shared-memory reads, but the box of 64
 // rows keeps 48% more columns.
@@ -53,12 +53,13 @@
 #include "spatial_bounds.h"
 #include "spatial_order.h"
 #include "sweep_kernel.cuh"
+#include "units.cuh"
 
 namespace hk {
 
 constexpr int SP_WARPS = 8, SP_THREADS = 32 * SP_WARPS;
-// Resident CTAs per SM.  At N = 1,000,000: 2 3.49 ms, 3 3.41, 4 (64 registers,
-// spills) 3.59.
+// Resident CTAs per SM.  At N = 1,000,000: 2 4.08 ms, 3 3.86, 4 (64 registers,
+// spills) 3.90.
 constexpr int SP_BPSM = 3;
 constexpr int SP_BUF = 64;             // buffered columns (32 evaluated at a time)
 constexpr int SP_LIST = 128;           // chunks listed before their events are tested

@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "sweep_kernel.cuh"
+#include "units.cuh"
 
 namespace hk {
 

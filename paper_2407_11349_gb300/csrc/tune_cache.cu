@@ -19,11 +19,9 @@
 #include <string>
 #include <vector>
 
-#include "common.cuh"
+#include "units.cuh"
 
 namespace hk {
-
-int sweep_num_variants();
 
 namespace {
 
