@@ -759,7 +759,7 @@ def main():
             "note": "tiles whose every pair term is an exact FP32 zero are skipped "
                     "(HAWKES_SKIP_UNDERFLOW); not the headline"}
 
-    # the same step evaluating only the tile pairs that can be nonzero in FP32
+    # the same step evaluating only the columns that can be nonzero in FP32
     # (space-ordered tiles inside time windows; reported separately)
     hk.loglik_grad(p, HAWKES_F32 | HAWKES_SKIP_SPATIAL)  # builds the order (untimed)
     sp_ms = []
@@ -781,8 +781,8 @@ def main():
                     "loglik_rel_diff_vs_full": abs(ll_x - ll_y) / abs(ll_y),
                     "grad_max_rel_diff_vs_full": float(np.max(np.abs(np.asarray(g_x) - np.asarray(g_y)) /
                                                               np.maximum(np.abs(np.asarray(g_y)), 1e-300))),
-                    "note": "only tile pairs whose terms can be nonzero in FP32 are evaluated "
-                            "(HAWKES_SKIP_SPATIAL: events ordered by location inside time windows of "
+                    "note": "only columns whose terms can be nonzero in FP32 are evaluated for a group of rows "
+                            "(HAWKES_SKIP_SPATIAL: events ordered by place and time inside time windows of "
                             "131,072 events); same result up to FP32 summation order; not the headline"}
 
     # the same step with eq. 2's time-only background (a model option, not the headline)
